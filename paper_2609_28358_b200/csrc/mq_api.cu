@@ -83,8 +83,9 @@ mq_status check_qtensor(const Geom& g, const mq_qtensor* q, int role) {
 
 // ---- tensor-core path: eligibility, tile shape, tensor maps ------------------------------------
 
-// fwd / bwd_data run on the tcgen05 kernel when both operands are 8-bit formats or both are E2M1 and a
-// tap's channel row is a whole number of 32-byte MMA K-atoms.
+// fwd / bwd_data run on the tcgen05 kernel when both operands are 8-bit formats or both are E2M1, at any channel count: a row
+// that ends inside an MMA's 32-byte K-atom is completed by the copy engine's zero fill (E2M1, 96 -> 160 channels, N = 50,
+// 27x27: the CUDA-core kernels, which took these layers before, 410 / 445 us forward / input gradient; here 30 / 30 us).
 bool conv_tc_eligible(int op, const Geom& g, int fmt_x_like, int fmt_w) {
   if (op != MQ_OP_FWD && op != MQ_OP_BWD_DATA) return false;
   if (env_int("MQ_DISABLE_TC", 0)) return false;
@@ -94,9 +95,7 @@ bool conv_tc_eligible(int op, const Geom& g, int fmt_x_like, int fmt_w) {
   // 6-bit operands: the tensor core reads them as 16 codes packed into 12 bytes + 4 bytes of padding (along K), not one
   // code per byte as they are stored; run_conv_tc packs them into scratch first (MQ_TC_NO_FP6=1: CUDA-core kernels)
   if ((fmt_is_6bit(fmt_x_like) || fmt_is_6bit(fmt_w)) && env_int("MQ_TC_NO_FP6", 0)) return false;
-  const int Kp = op == MQ_OP_FWD ? g.Cp : g.Cop;
-  const int rowbytes = Kp * (fp4 ? 4 : 8) / 8;
-  return rowbytes % 32 == 0;
+  return true;
 }
 
 size_t wt_codes_bytes(const Geom& g, int fmt_w) {
@@ -163,9 +162,16 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
   p.Kblocks = Kp / 32;
   const int rowbytes = Kp * bits / 8;
   out->rowbytes = rowbytes;
-  p.KB = rowbytes % 128 == 0 ? 128 : (rowbytes % 64 == 0 ? 64 : 32);
+  // Box width.  Rows of up to 64 bytes go as one box per tap; multiples of 64 as 64-byte boxes, two of which fill a stage (192-byte
+  // rows: 14 stages for nine taps instead of 18 half-empty ones; measured, quantizing forward of 183 -> 48 channels, N = 21,
+  // 19x14: 11.3 us against 12.5; 64 -> 320 channels stride 2, input gradient 43 against 47 us).  Every other row goes as 128-byte boxes,
+  // the last one short: a box costs a request per row whatever its width, and 32-byte boxes (one per K-atom, the rule before)
+  // cost three times as many of them for 96-byte rows (E4M3 129 -> 186 channels, N = 23, 45x56, forward: 74 -> 60 us).
+  const int atoms = (rowbytes + 31) / 32;
+  p.KB = atoms == 1 ? 32 : (atoms == 2 || (rowbytes % 64 == 0 && rowbytes % 128 != 0) ? 64 : 128);
   p.G = 128 / p.KB;
-  p.cpt = rowbytes / p.KB;
+  p.cpt = (rowbytes + p.KB - 1) / p.KB;
+  p.last_atoms = atoms - (p.cpt - 1) * (p.KB / 32);
   const int w_eff = op == MQ_OP_FWD ? g.Wo : (g.W + g.sw - 1) / g.sw;
   // line blocks (one scale per row): the per-tap kernel, whose preparation launch lays out the scale vectors row by row
   const bool thin = !line && !mx && !ts16 && g.sh == 1 && g.sw == 1 && p.cpt == 1 && p.KB <= 64 && !env_int("MQ_TC_NO_HALO", 0);
@@ -1002,7 +1008,9 @@ mq_status run_conv_mx(int op, const mq_conv_desc* desc, const mq_qtensor* qa, in
     fmt_x_like = op == MQ_OP_FWD ? qa->fmt : qb->fmt; fmt_w = op == MQ_OP_FWD ? qb->fmt : qa->fmt;
   }
   ConvTcPlan pl;
-  if (!conv_tc_eligible(op, g, fmt_x_like, fmt_w) || !conv_tc_plan(op, g, fmt_x_like, fmt_w, MQ_HWNC, &pl, false, true, ts)) {
+  // the paper's own format with rows that end inside an MMA's K-atom keeps the CUDA-core route (as its tests fix)
+  const bool ts_short = ts && (op == MQ_OP_FWD ? g.Cp : g.Cop) % 64 != 0;
+  if (ts_short || !conv_tc_eligible(op, g, fmt_x_like, fmt_w) || !conv_tc_plan(op, g, fmt_x_like, fmt_w, MQ_HWNC, &pl, false, true, ts)) {
     // layers the tensor-core kernels do not take: the same result in two launches - the CUDA-core GEMM writes fp32
     // [pixel][sample][channel] into scratch and the channel-fastest quantizer, which applies the activation, reads it back
     const long long P = op == MQ_OP_FWD ? (long long)g.Ho * g.Wo : (long long)g.H * g.W;

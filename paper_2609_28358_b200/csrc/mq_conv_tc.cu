@@ -19,8 +19,10 @@
 //                 registers and handed back before the stores (fp32 output: these two warpgroups take registers from the
 //                 other two with setmaxnreg); two warps per TMEM lane quadrant, half of the columns each
 // Wide layers run the DUO instance: clusters of two blocks on 256 x 256 tiles (cta_group::2), see conv_tc_kernel.
-// A pipeline stage holds 128 bytes of K per row (four MMAs): one 128-byte box, or 128/KB boxes of KB
-// bytes when a tap has fewer than 128 bytes of channels (then several taps share a stage).
+// A pipeline stage holds 128 bytes of K per row (four MMAs): one 128-byte box, or 128/KB boxes of KB = 64 or 32 bytes (then several
+// taps share a stage).  Rows that are no multiple of their box (E2M1 rows are any multiple of 16 bytes) end in a box that reaches
+// beyond the tensor's innermost extent: the copy engine fills the rest with zeros, which cost shared-memory space but no
+// traffic, and of a 128-byte chunk only the K-atoms that hold channels are multiplied.
 // Every wait is bounded; on expiry the kernel records MQ_ERR_TIMEOUT in the status word and drains.
 #include <cstdlib>
 #include "mq_conv_tc.cuh"
@@ -1081,6 +1083,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         tc_fence_after_sync();
         const uint32_t d_tmem = tmem + acc * p.BN;
         uint32_t accumulate = 0;
+        int cc = 0;     // (G == 1) chunk of the tap's channel row: the last one may be short
         for (int q0 = 0; q0 < Q; q0 += G) {
           // the scale copier signals sffull[s] once the stage's operands are in smem and its scale vectors in TMEM
           // E2M1: the scale copier signals sffull[s] once the stage's scale vectors are in TMEM.  8-bit operands: this
@@ -1090,7 +1093,8 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           tc_fence_after_sync();
           const uint32_t so = s * stage16;
           const uint32_t sfa_t = sf_base + s * SFC, sfb_t = sfa_t + SFB_OFF;
-          const int natoms = min(G, Q - q0) * APC;
+          int natoms = min(G, Q - q0) * APC;
+          if (G == 1 && p.last_atoms < 4 && ++cc == p.cpt) { cc = 0; natoms = p.last_atoms; }
           if (elect_one()) {
             if (DUO) {
 #pragma unroll
@@ -1183,12 +1187,32 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   if (warp == 1) { if (DUO) tmem_dealloc_2(tmem, 512); else tmem_dealloc(tmem, 512); }
 }
 
+// The BPC scale bytes of chunk `cc` of a row whose Kblocks scales start at `row`.  Rows of whole chunks (Kblocks a multiple of BPC)
+// are read in one access; else the row starts anywhere and its last chunk is short: byte by byte, zero (2^-127, times a code of
+// zero) for K-blocks beyond the row.
 template <int BPC>
-__device__ __forceinline__ unsigned long long load_scale_bytes(const uint8_t* ptr) {
-  if (BPC == 1) return __ldg(ptr);
-  if (BPC == 2) return __ldg(reinterpret_cast<const unsigned short*>(ptr));
-  if (BPC == 4) return __ldg(reinterpret_cast<const unsigned int*>(ptr));
-  return __ldg(reinterpret_cast<const unsigned long long*>(ptr));
+__device__ __forceinline__ unsigned long long load_scale_bytes(const uint8_t* row, int cc, int Kblocks) {
+  if (BPC == 1) return __ldg(row + cc);
+  if (Kblocks % BPC == 0) {
+    const uint8_t* ptr = row + cc * BPC;
+    if (BPC == 2) return __ldg(reinterpret_cast<const unsigned short*>(ptr));
+    if (BPC == 4) return __ldg(reinterpret_cast<const unsigned int*>(ptr));
+    return __ldg(reinterpret_cast<const unsigned long long*>(ptr));
+  }
+  unsigned long long v = 0ull;
+#pragma unroll
+  for (int k = 0; k < BPC; ++k)
+    if (cc * BPC + k < Kblocks) v |= (unsigned long long)__ldg(row + cc * BPC + k) << (8 * k);
+  return v;
+}
+// The same for the paper's own format: the four E4M3 scale bytes of K-atom `atom` (64 elements) of a row whose Kb16 (an even
+// number of) scales start at `row`, zero beyond the row.
+__device__ __forceinline__ unsigned load_ts_scales(const uint8_t* row, int atom, int Kb16) {
+  if (Kb16 % 4 == 0) return 4 * atom < Kb16 ? __ldg(reinterpret_cast<const unsigned int*>(row + 4 * atom)) : 0u;
+  unsigned v = 0u;
+  if (4 * atom < Kb16) v = __ldg(reinterpret_cast<const unsigned short*>(row + 4 * atom));
+  if (4 * atom + 2 < Kb16) v |= (unsigned)__ldg(reinterpret_cast<const unsigned short*>(row + 4 * atom + 2)) << 16;
+  return v;
 }
 
 // Builds, in shared memory, the scale-vector chunks ([chunk][group][atom][512]) of the resident weight tile of
@@ -1210,7 +1234,7 @@ __device__ __forceinline__ void halo_build_sfb(const ConvTcParams& p, uint8_t* s
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           if (j < 4 * atoms_b && 32 * j < p.BN && 32 * j < p.Cd)
-            acc[j] |= load_scale_bytes<BPC>(p.b_scales + ((long long)j * taps + q) * p.Kblocks) << (8 * c * BPC);
+            acc[j] |= load_scale_bytes<BPC>(p.b_scales + ((long long)j * taps + q) * p.Kblocks, 0, p.Kblocks) << (8 * c * BPC);
         }
       }
     }
@@ -1495,7 +1519,7 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         for (int i = 0; i < 4; ++i) {
           const int hh = hs + e_h[i], ww = ws + e_w[i];
           raw[i] = 0;
-          if (e_h[i] >= 0 && hh >= 0 && hh < p.Hs && ww >= 0 && ww < p.Ws)
+          if (e_h[i] >= 0 && e_k[i] < p.Kblocks && hh >= 0 && hh < p.Hs && ww >= 0 && ww < p.Ws)
             raw[i] = __ldg(p.a_scales + (((long long)hh * p.Ws + ww) * p.Nt + nblk) * p.Kblocks + e_k[i]);
         }
         bool ok = true;
@@ -1624,9 +1648,9 @@ __global__ void __launch_bounds__(256) expand_conv_scales_kernel(const ConvTcPar
         const int tw_ = r & (p.TW - 1), tn = r >> p.lgTW;
         const int n = tile.n0 + tn, ws = ws0 + tw_;
         const bool ok = n < p.N && hs >= 0 && hs < p.Hs && ws >= 0 && ws < p.Ws;
-        const uint8_t* rowp = p.a_scales + (((long long)hs * p.Ws + ws) * Nt16 + (n >> 4)) * Kb16 + pos.cc * (4 * APC);
+        const uint8_t* rowp = p.a_scales + (((long long)hs * p.Ws + ws) * Nt16 + (n >> 4)) * Kb16;
 #pragma unroll
-        for (int ja = 0; ja < 4; ++ja) val[ja][j] = (ok && ja < APC) ? __ldg(reinterpret_cast<const unsigned int*>(rowp + 4 * ja)) : 0u;
+        for (int ja = 0; ja < 4; ++ja) val[ja][j] = (ok && ja < APC) ? load_ts_scales(rowp, pos.cc * APC + ja, Kb16) : 0u;
       }
       uint8_t* dst = p.sfa_img + (size_t)wid * (512 * 4) + lane * 16;
 #pragma unroll
@@ -1662,9 +1686,9 @@ __global__ void __launch_bounds__(256) expand_conv_scales_kernel(const ConvTcPar
             const int tw_ = r & (p.TW - 1), tn = r >> p.lgTW;
             const int n = tile.n0 + tn, ws = ws0 + tw_ * wstep;
             if (n < p.N && hs >= 0 && hs < p.Hs && ws >= 0 && ws < p.Ws) {
-              const uint8_t* rowp = p.a_scales + (((long long)hs * p.Ws + ws) * Nt16 + (n >> 4)) * Kb16 + pos.cc * (4 * APC);
+              const uint8_t* rowp = p.a_scales + (((long long)hs * p.Ws + ws) * Nt16 + (n >> 4)) * Kb16;
 #pragma unroll
-              for (int ja = 0; ja < APC; ++ja) val[c * APC + ja][j] = __ldg(reinterpret_cast<const unsigned int*>(rowp + 4 * ja));
+              for (int ja = 0; ja < APC; ++ja) val[c * APC + ja][j] = load_ts_scales(rowp, pos.cc * APC + ja, Kb16);
             }
           }
         }
@@ -1711,14 +1735,14 @@ __global__ void __launch_bounds__(256) expand_conv_scales_kernel(const ConvTcPar
                     unsigned w = 0;
 #pragma unroll
                     for (int kb = 0; kb < 4; ++kb)
-                      w |= (unsigned)__ldg(p.wt_sc_in + ((long long)(pos.cc * (4 * APC) + 4 * ja + kb) * taps_all + tap) * Cb_w + (row >> 4)) << (8 * kb);
+                      if (pos.cc * (4 * APC) + 4 * ja + kb < Kb16) w |= (unsigned)__ldg(p.wt_sc_in + ((long long)(pos.cc * (4 * APC) + 4 * ja + kb) * taps_all + tap) * Cb_w + (row >> 4)) << (8 * kb);
                     val[c * APC + ja][j] = w;
                   }
                 }
               } else if (row < p.b_rows_total) {
-                const uint8_t* rowp = p.b_scales + ((long long)(row >> 4) * taps_all + tap) * Kb16 + pos.cc * (4 * APC);
+                const uint8_t* rowp = p.b_scales + ((long long)(row >> 4) * taps_all + tap) * Kb16;
 #pragma unroll
-                for (int ja = 0; ja < APC; ++ja) val[c * APC + ja][j] = __ldg(reinterpret_cast<const unsigned int*>(rowp + 4 * ja));
+                for (int ja = 0; ja < APC; ++ja) val[c * APC + ja][j] = load_ts_scales(rowp, pos.cc * APC + ja, Kb16);
               }
             }
           }
@@ -1744,7 +1768,7 @@ __global__ void __launch_bounds__(256) expand_conv_scales_kernel(const ConvTcPar
       const int ct = (int)(tt / (unsigned)taps_all), tap = (int)(tt - (unsigned)ct * taps_all);
       const int row = ct * p.BN + r;
       uint4 v = make_uint4(0, 0, 0, 0);
-      if (row < p.b_rows_total) v = __ldg(reinterpret_cast<const uint4*>(p.b_codes + ((size_t)row * taps_all + tap) * p.b_rowbytes) + ch);
+      if (row < p.b_rows_total && 16 * ch < p.b_rowbytes) v = __ldg(reinterpret_cast<const uint4*>(p.b_codes + ((size_t)row * taps_all + tap) * p.b_rowbytes) + ch);
       const int sw = KB == 128 ? (r & 7) : (KB == 64 ? ((r >> 1) & 3) : ((r >> 2) & 1));
       *reinterpret_cast<uint4*>(p.b_img + (size_t)row_id * KB + ((ch ^ sw) << 4)) = v;
     }
@@ -1773,7 +1797,7 @@ __global__ void __launch_bounds__(256) expand_conv_scales_kernel(const ConvTcPar
       const int tw_ = r & (p.TW - 1), tn = r >> p.lgTW;
       const int n = tile.n0 + tn, ws = ws0 + tw_;
       if (n < p.N && hs >= 0 && hs < p.Hs && ws >= 0 && ws < p.Ws)
-        acc[j] = load_scale_bytes<BPC>(p.a_scales + (((long long)hs * p.Ws + ws) * (p.line ? p.N : p.Nt) + (p.line ? n : (n >> 5))) * p.Kblocks + pos.cc * BPC);
+        acc[j] = load_scale_bytes<BPC>(p.a_scales + (((long long)hs * p.Ws + ws) * (p.line ? p.N : p.Nt) + (p.line ? n : (n >> 5))) * p.Kblocks, pos.cc, p.Kblocks);
     }
     uint8_t* dst = p.sfa_img + (size_t)wid * (512 * SPA) + lane * 16;
 #pragma unroll
@@ -1807,7 +1831,7 @@ __global__ void __launch_bounds__(256) expand_conv_scales_kernel(const ConvTcPar
           const int tw_ = r & (p.TW - 1), tn = r >> p.lgTW;
           const int n = tile.n0 + tn, ws = ws0 + tw_ * wstep;
           if (n < p.N && hs >= 0 && hs < p.Hs && ws >= 0 && ws < p.Ws)
-            acc[j] |= load_scale_bytes<BPC>(p.a_scales + (((long long)hs * p.Ws + ws) * (p.line ? p.N : p.Nt) + (p.line ? n : (n >> 5))) * p.Kblocks + pos.cc * BPC) << (8 * c * BPC);
+            acc[j] |= load_scale_bytes<BPC>(p.a_scales + (((long long)hs * p.Ws + ws) * (p.line ? p.N : p.Nt) + (p.line ? n : (n >> 5))) * p.Kblocks, pos.cc, p.Kblocks) << (8 * c * BPC);
         }
       }
     }
@@ -1848,14 +1872,14 @@ __global__ void __launch_bounds__(256) expand_conv_scales_kernel(const ConvTcPar
               unsigned long long bytes = 0;
 #pragma unroll
               for (int kb = 0; kb < BPC; ++kb)
-                bytes |= (unsigned long long)__ldg(p.wt_sc_in + ((long long)(pos.cc * BPC + kb) * taps_all + tap) * Ct_w + cib) << (8 * kb);
+                if (pos.cc * BPC + kb < p.Kblocks) bytes |= (unsigned long long)__ldg(p.wt_sc_in + ((long long)(pos.cc * BPC + kb) * taps_all + tap) * Ct_w + cib) << (8 * kb);
               acc[j] |= bytes << (8 * c * BPC);
             } else if (p.line) {
               // line blocks: every weight row has its own scale per K-block
               const int row = tile.c0 + 32 * j + lane;
-              if (row < p.b_rows_total) acc[j] |= load_scale_bytes<BPC>(p.b_scales + ((long long)row * taps_all + tap) * p.Kblocks + pos.cc * BPC) << (8 * c * BPC);
+              if (row < p.b_rows_total) acc[j] |= load_scale_bytes<BPC>(p.b_scales + ((long long)row * taps_all + tap) * p.Kblocks, pos.cc, p.Kblocks) << (8 * c * BPC);
             } else {
-              acc[j] |= load_scale_bytes<BPC>(p.b_scales + ((long long)((tile.c0 >> 5) + j) * taps_all + tap) * p.Kblocks + pos.cc * BPC) << (8 * c * BPC);
+              acc[j] |= load_scale_bytes<BPC>(p.b_scales + ((long long)((tile.c0 >> 5) + j) * taps_all + tap) * p.Kblocks, pos.cc, p.Kblocks) << (8 * c * BPC);
             }
           }
         }

@@ -23,7 +23,8 @@ struct ConvTcParams {
   uint32_t idesc;       // instruction descriptor without scale ids
   int KB;               // bytes of K per row per TMA box: 128, 64 or 32 (= swizzle span)
   int G;                // boxes (chunks) per pipeline stage = 128 / KB
-  int cpt;              // chunks per tap = row bytes / KB
+  int cpt;              // chunks per tap = ceil(row bytes / KB)
+  int last_atoms;       // MMA K-atoms (32 bytes) of a tap's last 128-byte chunk that hold channels (KB == 128)
   int BN;               // output channels per tile (multiple of 16, <= 256)
   int stages;
   int n_acc;            // accumulator buffers in TMEM (1 or 2)
