@@ -18,18 +18,20 @@ void count_launches(int n) { g_launches.fetch_add((unsigned long long)n, std::me
 // environment knobs, read once each (see mq_internal.cuh)
 static std::mutex g_env_mutex;
 static std::map<std::string, std::pair<bool, int>> g_env;   // name -> (set in the environment, value)
-int env_int(const char* name, int dflt) {
+std::atomic<uint32_t> g_env_generation{1};
+uint64_t env_lookup(const char* name) {
   std::lock_guard<std::mutex> lock(g_env_mutex);
   auto it = g_env.find(name);
   if (it == g_env.end()) {
     const char* v = std::getenv(name);
     it = g_env.emplace(name, std::make_pair(v != nullptr, v ? std::atoi(v) : 0)).first;
   }
-  return it->second.first ? it->second.second : dflt;
+  return ((uint64_t)g_env_generation.load(std::memory_order_relaxed) << 33) | (it->second.first ? 1ull << 32 : 0ull) | (uint32_t)it->second.second;
 }
 static void env_forget() {
   std::lock_guard<std::mutex> lock(g_env_mutex);
   g_env.clear();
+  g_env_generation.fetch_add(1, std::memory_order_release);
 }
 
 namespace {
@@ -88,13 +90,13 @@ mq_status check_qtensor(const Geom& g, const mq_qtensor* q, int role) {
 // 27x27: the CUDA-core kernels, which took these layers before, 410 / 445 us forward / input gradient; here 30 / 30 us).
 bool conv_tc_eligible(int op, const Geom& g, int fmt_x_like, int fmt_w) {
   if (op != MQ_OP_FWD && op != MQ_OP_BWD_DATA) return false;
-  if (env_int("MQ_DISABLE_TC", 0)) return false;
+  if (MQ_ENV("MQ_DISABLE_TC", 0)) return false;
   const bool fp4 = fmt_x_like == MQ_E2M1 && fmt_w == MQ_E2M1;
   const bool fp8 = fmt_x_like != MQ_E2M1 && fmt_w != MQ_E2M1;
   if (!fp4 && !fp8) return false;
   // 6-bit operands: the tensor core reads them as 16 codes packed into 12 bytes + 4 bytes of padding (along K), not one
   // code per byte as they are stored; run_conv_tc packs them into scratch first (MQ_TC_NO_FP6=1: CUDA-core kernels)
-  if ((fmt_is_6bit(fmt_x_like) || fmt_is_6bit(fmt_w)) && env_int("MQ_TC_NO_FP6", 0)) return false;
+  if ((fmt_is_6bit(fmt_x_like) || fmt_is_6bit(fmt_w)) && MQ_ENV("MQ_TC_NO_FP6", 0)) return false;
   return true;
 }
 
@@ -112,7 +114,7 @@ size_t up256(size_t v) { return (v + 255) / 256 * 256; }
 //   pair: the tiles of the even and the odd output columns are stored together (stride-2 input gradient): runs of
 //   2 tw floats, and the two accumulators belong to one pair, so the store is not overlapped either.
 int choose_tw(int w_eff, int N, int layout, double k_bytes, int bn, bool thin, bool serial, bool pair) {
-  const int forced = env_int("MQ_TC_TW", 0);
+  const int forced = MQ_ENV("MQ_TC_TW", 0);
   if (forced > 0) return forced;
   if (thin) return 8;   // the whole-tile kernel (8-column tiles): its per-tile loads beat any per-tap shape on thin layers
   const double t_mma = k_bytes / 32.0 * 107.0 * (bn / 128.0 < 0.5 ? 0.5 : bn / 128.0);
@@ -174,7 +176,7 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
   p.last_atoms = atoms - (p.cpt - 1) * (p.KB / 32);
   const int w_eff = op == MQ_OP_FWD ? g.Wo : (g.W + g.sw - 1) / g.sw;
   // line blocks (one scale per row): the per-tap kernel, whose preparation launch lays out the scale vectors row by row
-  const bool thin = !line && !mx && !ts16 && g.sh == 1 && g.sw == 1 && p.cpt == 1 && p.KB <= 64 && !env_int("MQ_TC_NO_HALO", 0);
+  const bool thin = !line && !mx && !ts16 && g.sh == 1 && g.sw == 1 && p.cpt == 1 && p.KB <= 64 && !MQ_ENV("MQ_TC_NO_HALO", 0);
   p.line = line ? 1 : 0;
   const int cd16 = mx ? (p.Cd + 31) / 32 * 32 : (p.Cd + 15) / 16 * 16;
   p.BN = cd16 <= 128 ? cd16 : 128;
@@ -187,19 +189,19 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
   // (measured, N = 256, 8-bit, fp32 / quantized output: 256 channels 56x56 324 -> 207 us / 217 -> 196 us; 512 channels 56x56
   // 531 -> 528 / 464 -> 410 us; 512 channels 28x28 181 -> 175 / 133 -> 127 us)
   // E2M1 likewise: 512 channels 56x56 550 -> 364 us, 256 channels 56x56 290 -> 173 us
-  if (p.Cd >= 256 && taps == 1 && g.sh == 1 && g.sw == 1 && !env_int("MQ_TC_1X1_BN128", 0)) p.BN = 256;
+  if (p.Cd >= 256 && taps == 1 && g.sh == 1 && g.sw == 1 && !MQ_ENV("MQ_TC_1X1_BN128", 0)) p.BN = 256;
   // E2M1: the same trade (measured with the tile widths chosen below: 256 channels 28x28 -13 %, 512 channels 14x14 -6 %,
   // 56x56 -10 %)
   const double act_bytes = (double)p.Hs * p.Ws * g.N * rowbytes;
-  if (fp4 && p.Cd >= 256 && (double)taps * rowbytes >= 1024.0 && (op == MQ_OP_FWD || (g.sh == 1 && g.sw == 1)) && !env_int("MQ_TC_FP4_BN128", 0)) p.BN = 256;
+  if (fp4 && p.Cd >= 256 && (double)taps * rowbytes >= 1024.0 && (op == MQ_OP_FWD || (g.sh == 1 && g.sw == 1)) && !MQ_ENV("MQ_TC_FP4_BN128", 0)) p.BN = 256;
   {
-    const int forced_bn_ = env_int("MQ_TC_BN", 0);
+    const int forced_bn_ = MQ_ENV("MQ_TC_BN", 0);
     const int bn_ = (forced_bn_ >= 32 && forced_bn_ <= 256 && forced_bn_ % 32 == 0) ? (forced_bn_ < cd16 ? forced_bn_ : cd16) : p.BN;
     const int nkh_ = op == MQ_OP_FWD ? g.Kh : (g.Kh + g.sh - 1) / g.sh, nkw_ = op == MQ_OP_FWD ? g.Kw : (g.Kw + g.sw - 1) / g.sw;
     // with a single accumulator the store time adds to the tile's time instead of hiding behind the next tile: wider
     // tiles (longer store runs) then win - as long as the activations stay in L2 (measured: 28x28 -11 %, 56x56 +11 %)
     const bool serial = bn_ > 128 && act_bytes <= 110e6;
-    const bool pair_hint = !mx && op == MQ_OP_BWD_DATA && g.sw == 2 && layout == MQ_NCHW && p.Wd % 2 == 0 && bn_ <= 128 && !env_int("MQ_TC_NO_PAIR", 0);
+    const bool pair_hint = !mx && op == MQ_OP_BWD_DATA && g.sw == 2 && layout == MQ_NCHW && p.Wd % 2 == 0 && bn_ <= 128 && !MQ_ENV("MQ_TC_NO_PAIR", 0);
     p.TW = choose_tw(w_eff, g.N, layout, (double)nkh_ * nkw_ * rowbytes, bn_ < 128 ? bn_ : (serial ? bn_ : 128), thin, serial, pair_hint);
     if (mx) {   // a sample tile (32 samples) must lie inside a GEMM tile: 1, 2 or 4 columns; the least edge padding wins, then the
                 // narrowest: with one column a warp's 32 rows ARE a sample tile, and the epilogue needs no exchange between warps
@@ -210,7 +212,7 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
         const double waste = (double)((w_eff + tw - 1) / tw * tw) / w_eff * (double)((g.N + tn - 1) / tn * tn) / g.N;
         if (waste < best * (1.0 - 1e-9)) { best = waste; p.TW = tw; }
       }
-      const int ftw = env_int("MQ_TC_MX_TW", 0);
+      const int ftw = MQ_ENV("MQ_TC_MX_TW", 0);
       if (ftw == 1 || ftw == 2 || (ftw == 4 && !ts16)) p.TW = ftw;
     }
   }
@@ -218,7 +220,7 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
   p.TN = 128 / p.TW;
   p.lgTW = 0;
   while ((1 << p.lgTW) < p.TW) ++p.lgTW;
-  const int forced_bn = env_int("MQ_TC_BN", 0);
+  const int forced_bn = MQ_ENV("MQ_TC_BN", 0);
   if (forced_bn >= 32 && forced_bn <= 256 && forced_bn % 32 == 0) p.BN = forced_bn < cd16 ? forced_bn : cd16;
   if (mx && (p.BN % 32 != 0 || p.TW > (ts16 ? 2 : 4))) return false;
   p.tiles_c = (p.Cd + p.BN - 1) / p.BN;
@@ -247,7 +249,7 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
   // pixels along W.  Not for NCHW: there W is the innermost axis and a class's first column (x = 1 for the odd one) would be
   // a TMA coordinate that is not on a 16-byte boundary, which the hardware refuses; NCHW keeps the paired direct stores.
   const bool strided_out = op == MQ_OP_BWD_DATA && (g.sh != 1 || g.sw != 1);
-  const bool s2_tma_ok = strided_out && layout == MQ_HWNC && g.sw <= 8 && !env_int("MQ_TC_NO_S2_TMA", 0);
+  const bool s2_tma_ok = strided_out && layout == MQ_HWNC && g.sw <= 8 && !MQ_ENV("MQ_TC_NO_S2_TMA", 0);
   const bool tma_store_ok = (!strided_out || s2_tma_ok) && p.TW <= 32 &&
                             (layout == MQ_NCHW ? (p.TW >= 4 && p.Wd % 4 == 0) : (p.Cd % 4 == 0 && p.BN % 64 == 0));
   // ... and for 1x1 layers, whose main loop is a handful of stages: the tile's time is its store (measured 4-12 % faster, 28x28 and
@@ -255,7 +257,7 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
   // ... and for the channel-fastest output order, where a direct store is one 16-byte request per row and instruction - the request
   // count, not the bytes, bounds the store path (measured, N = 256, 512 channels: 1x1 56x56 841 -> 443 us, 3x3 28x28 447 -> 396 us,
   // the latter 2.39 PFLOP/s against 2.15 for the NCHW order)
-  p.tma_store = !mx && tma_store_ok && (env_int("MQ_TC_TMA_STORE", 0) || ((taps == 1 || layout == MQ_HWNC || strided_out) && !env_int("MQ_TC_NO_TMA_STORE", 0))) ? 1 : 0;
+  p.tma_store = !mx && tma_store_ok && (MQ_ENV("MQ_TC_TMA_STORE", 0) || ((taps == 1 || layout == MQ_HWNC || strided_out) && !MQ_ENV("MQ_TC_NO_TMA_STORE", 0))) ? 1 : 0;
   const size_t stage_bytes = 128 * 128 + (size_t)p.BN * 128 + (ts16 ? 6144 : 3072);
   const int sf_cols = ts16 ? 48 : 24;
   int stages = (int)((227 * 1024 - 2048 - (p.tma_store ? 65536 : 0)) / stage_bytes);
@@ -267,22 +269,22 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
   p.stages = stages;
   p.n_acc = (2 * p.BN + sf_cols * stages <= 512) ? 2 : 1;
   if (p.n_acc * p.BN + sf_cols * stages > 512) return false;
-  p.mma_cp = env_int("MQ_TC_NO_MMA_CP", 0) ? 0 : 1;   // E2M1 too: the bubble behind a copier warp costs more than the lane's extra issues
+  p.mma_cp = MQ_ENV("MQ_TC_NO_MMA_CP", 0) ? 0 : 1;   // E2M1 too: the bubble behind a copier warp costs more than the lane's extra issues
   p.pair = !mx && !p.tma_store && op == MQ_OP_BWD_DATA && g.sw == 2 && layout == MQ_NCHW && p.Wd % 2 == 0 && p.n_acc == 2 && p.total_tiles % 2 == 0 &&
-           !env_int("MQ_TC_NO_PAIR", 0);
+           !MQ_ENV("MQ_TC_NO_PAIR", 0);
   const int nkh = op == MQ_OP_FWD ? g.Kh : (g.Kh + g.sh - 1) / g.sh, nkw = op == MQ_OP_FWD ? g.Kw : (g.Kw + g.sw - 1) / g.sw;
   p.max_stages = (nkh * nkw * p.cpt + p.G - 1) / p.G;
   // one 256-column accumulator: the epilogue copies it into registers and frees it before storing (with the staged TMA
   // stores only when a tile has at least MQ_TC_SNAP_MIN_STAGES pipeline stages of MMAs to overlap: E2M1 1x1 512 channels, two
   // stages per tile, measured 384-407 us without and 517-601 us with it; E4M3, four stages, 562-567 against 521 us)
-  p.snap = (!mx && ((p.BN == 256 && p.n_acc == 1 && !p.pair) || (p.pair && p.BN == 128)) && !env_int("MQ_TC_NO_SNAP", 0) &&
-            (!p.tma_store || p.max_stages >= env_int("MQ_TC_SNAP_MIN_STAGES", 4))) ? 1 : 0;
+  p.snap = (!mx && ((p.BN == 256 && p.n_acc == 1 && !p.pair) || (p.pair && p.BN == 128)) && !MQ_ENV("MQ_TC_NO_SNAP", 0) &&
+            (!p.tma_store || p.max_stages >= MQ_ENV("MQ_TC_SNAP_MIN_STAGES", 4))) ? 1 : 0;
   const uint32_t fa = fp4 ? 1u : fmt_mma_code(fmt_x_like);   // kind::mxf4: 1 = E2M1; kind::mxf8f6f4: E4M3 0, E5M2 1, E2M3 3, E3M2 4
   const uint32_t fb = fp4 ? 1u : fmt_mma_code(fmt_w);
   // pairs of blocks on 256 x 256 tiles (see conv_tc_kernel's DUO): tiles 2k and 2k + 1 must exist and share the channel tile
   // (and have at least eight pipeline stages of MMAs per tile: 1x1 layers, four stages, measured 538-548 us without, 609 us with it)
   p.duo = (p.snap && !p.halo && p.KB == 128 && p.classes == 1 && p.mma_cp && p.total_tiles % 2 == 0 &&
-           (p.tiles_w * p.tiles_h) % 2 == 0 && !fmt_is_6bit(fmt_x_like) && !fmt_is_6bit(fmt_w) && p.max_stages >= 8 && !env_int("MQ_TC_NO_DUO", 0)) ? 1 : 0;
+           (p.tiles_w * p.tiles_h) % 2 == 0 && !fmt_is_6bit(fmt_x_like) && !fmt_is_6bit(fmt_w) && p.max_stages >= 8 && !MQ_ENV("MQ_TC_NO_DUO", 0)) ? 1 : 0;
   if (p.duo) {   // half of the weight tile per block: a stage is 16 KB smaller, the ring two stages deeper
     int st = (int)((227 * 1024 - 2048 - (p.tma_store ? 65536 : 0)) / (stage_bytes - (size_t)p.BN * 64));
     if (st > 8) st = 8;
@@ -294,7 +296,7 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
   // whole-tile-per-stage variant: stride 1, one chunk per tap (<= 64 bytes of channels).  One box with the column
   // halo needs 8-column tiles; one box per column shift takes 8, 16 or 32 columns (longer NCHW store runs).
   p.halo = 0;
-  if (!line && !mx && !ts16 && g.sh == 1 && g.sw == 1 && p.cpt == 1 && p.KB <= 64 && taps <= 64 && !env_int("MQ_TC_NO_HALO", 0)) {
+  if (!line && !mx && !ts16 && g.sh == 1 && g.sw == 1 && p.cpt == 1 && p.KB <= 64 && taps <= 64 && !MQ_ENV("MQ_TC_NO_HALO", 0)) {
     const int spa = fp4 ? 2 : 1, atoms_b = (p.BN + 127) / 128;
     if (p.TW == 8) {
       p.WH = p.TW + g.Kw - 1;
@@ -302,7 +304,7 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
       p.halo_a_bytes = (p.halo_box_bytes + 1023) / 1024 * 1024;
       p.halo_stage_bytes = (p.halo_a_bytes + p.max_stages * 512 * spa + 1023) / 1024 * 1024;
       p.halo_b_bytes = (taps * p.BN * p.KB + p.max_stages * 512 * spa * atoms_b + 1023) / 1024 * 1024;
-      const int halo_tma = tma_store_ok && !env_int("MQ_TC_NO_TMA_STORE", 0) ? 1 : 0;
+      const int halo_tma = tma_store_ok && !MQ_ENV("MQ_TC_NO_TMA_STORE", 0) ? 1 : 0;
       int hst = (227 * 1024 - 4096 - p.halo_b_bytes - (halo_tma ? 65536 : 0)) / p.halo_stage_bytes;
       if (hst > 4) hst = 4;
       // TMEM: accumulator(s), 16 columns per chunk of resident weight scales, 8 per chunk per stage
@@ -310,7 +312,7 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
       if (hst >= 2 && p.WH <= 256) {
         p.halo = 1;
         p.tma_store = halo_tma;
-        p.fused = p.tiles_c == 1 && p.TN <= 32 && g.Kh * (p.TW + g.Kw - 1) * (p.KB / 32) * spa <= 128 && !env_int("MQ_TC_NO_FUSED", 0);
+        p.fused = p.tiles_c == 1 && p.TN <= 32 && g.Kh * (p.TW + g.Kw - 1) * (p.KB / 32) * spa <= 128 && !MQ_ENV("MQ_TC_NO_FUSED", 0);
         p.stages = hst;
         p.n_acc = (2 * p.BN + 16 * p.max_stages + 8 * p.max_stages * hst <= 512) ? 2 : 1;
       }
@@ -318,7 +320,7 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
   }
   // unit strides and one 128-byte chunk per stage: the activation-side scale chunk of (tile, kh) equals that of the tile one
   // output row further with kh - 1, so chunks are stored per source row - Kh times fewer to expand
-  p.sfa_dedup = (!p.halo && p.KB == 128 && g.sh == 1 && g.sw == 1 && !env_int("MQ_TC_NO_SFA_DEDUP", 0)) ? 1 : 0;
+  p.sfa_dedup = (!p.halo && p.KB == 128 && g.sh == 1 && g.sw == 1 && !MQ_ENV("MQ_TC_NO_SFA_DEDUP", 0)) ? 1 : 0;
   p.sfa_hk = p.tiles_h + g.Kh - 1;
   out->p = p;
   size_t o = 0;
@@ -371,7 +373,7 @@ mq_status run_conv_tc(int op, const Geom& g, ConvTcPlan& pl, const mq_qtensor* q
     p.b_scales = qw->scales;
   } else {
     // per-tap kernel, operands that need no repacking: the re-layout rides in the scale-expansion launch
-    p.wt_fused = (!p.halo && !fmt_is_6bit(fw) && (p.kind_fp4 == 2 || !env_int("MQ_TC_NO_WT_FUSED", 0))) ? 1 : 0;   // kind 2: this route only
+    p.wt_fused = (!p.halo && !fmt_is_6bit(fw) && (p.kind_fp4 == 2 || !MQ_ENV("MQ_TC_NO_WT_FUSED", 0))) ? 1 : 0;   // kind 2: this route only
     if (p.wt_fused) {
       p.wt_in = w_stored; p.wt_out = base; p.wt_sc_in = qw->scales;
       p.wt_Cout = g.Cout; p.wt_Cop = g.Cop; p.wt_Cp = g.Cp; p.wt_bx = g.Cp / 32; p.wt_by = g.Cop / 32;
@@ -397,7 +399,7 @@ mq_status run_conv_tc(int op, const Geom& g, ConvTcPlan& pl, const mq_qtensor* q
     const uint32_t es[4] = {1u, wst, 1u, 1u};
     // a packed activation / gradient tensor with rows of whole 128-code boxes is read where it is stored (the copy engine pads
     // each 12-byte group on its way into shared memory): no scratch copy, no pass over the tensor before the GEMM
-    if (pk_x && p.KB == 128 && rb % 128 == 0 && !env_int("MQ_TC_NO_P6_DIRECT", 0)) {
+    if (pk_x && p.KB == 128 && rb % 128 == 0 && !MQ_ENV("MQ_TC_NO_P6_DIRECT", 0)) {
       const uint64_t ps[3] = {strides[0] * 3 / 4, strides[1] * 3 / 4, strides[2] * 3 / 4};
       direct_x = encode_tensor_map_p6(&map_a, x_stored, 4, dims, ps, box, es);
     }
@@ -481,27 +483,27 @@ struct WgradPlan {
 // ts16: the paper's own format (E4M3 scales per 16 x 16 block): the two E2M1 modes with kind::mxf4nvf4
 WgradPlan wgrad_plan(const Geom& g, int fmt_x, int fmt_g, bool ts16 = false) {
   WgradPlan w{};
-  if (ts16 && (fmt_x != MQ_E2M1 || fmt_g != MQ_E2M1 || env_int("MQ_TC_NO_TS16", 0))) return w;
-  if (env_int("MQ_DISABLE_TC", 0) || env_int("MQ_DISABLE_TC_WGRAD", 0)) return w;
+  if (ts16 && (fmt_x != MQ_E2M1 || fmt_g != MQ_E2M1 || MQ_ENV("MQ_TC_NO_TS16", 0))) return w;
+  if (MQ_ENV("MQ_DISABLE_TC", 0) || MQ_ENV("MQ_DISABLE_TC_WGRAD", 0)) return w;
   const bool fp4_in = fmt_x == MQ_E2M1 && fmt_g == MQ_E2M1;
   const bool fp8_in = fmt_x != MQ_E2M1 && fmt_g != MQ_E2M1;
   if (!fp4_in && !fp8_in) return w;
   // E2M1 layers that the flat mode below does not take (stride 2, batches that are not 1, 2, 4 or 8 sample tiles): every
   // E2M1 value is an E4M3 value, so the codes are re-encoded exactly as E4M3 bytes in scratch and the 8-bit path (stored
   // order read MN-major, block pairs) runs - faster than the per-pixel E2M1 mode (MQ_WGRAD_FP4_PIXEL=1 keeps that mode)
-  const bool flat_ok = fp4_in && g.sh == 1 && g.sw == 1 && (g.Nt == 1 || g.Nt == 2 || g.Nt == 4 || g.Nt == 8) && !env_int("MQ_WGRAD_NO_FLAT", 0);
-  const bool recode4 = fp4_in && !flat_ok && !ts16 && !env_int("MQ_WGRAD_FP4_PIXEL", 0);   // (E4M3 block scales are no E8M0 scales: not for ts16)
+  const bool flat_ok = fp4_in && g.sh == 1 && g.sw == 1 && (g.Nt == 1 || g.Nt == 2 || g.Nt == 4 || g.Nt == 8) && !MQ_ENV("MQ_WGRAD_NO_FLAT", 0);
+  const bool recode4 = fp4_in && !flat_ok && !ts16 && !MQ_ENV("MQ_WGRAD_FP4_PIXEL", 0);   // (E4M3 block scales are no E8M0 scales: not for ts16)
   const bool fp4 = fp4_in && !recode4;
   const bool fp8 = fp8_in || recode4;
   w.recode4 = recode4;
   // 6-bit operands: this GEMM reads its operands MN-major (K = samples), where the MMA's packed 6-bit container (packed
   // along K) does not apply; every E3M2 / E2M3 value is also an E4M3 value, so the codes are re-encoded exactly as
   // E4M3 bytes in scratch and the 8-bit path runs unchanged (MQ_TC_NO_FP6=1: CUDA-core kernels)
-  if ((fmt_is_6bit(fmt_x) || fmt_is_6bit(fmt_g)) && env_int("MQ_TC_NO_FP6", 0)) return w;
+  if ((fmt_is_6bit(fmt_x) || fmt_is_6bit(fmt_g)) && MQ_ENV("MQ_TC_NO_FP6", 0)) return w;
   WgradTcParams& p = w.p;
   p.N = g.N; p.Nt = g.Nt; p.Ho = g.Ho; p.Wo = g.Wo; p.H = g.H; p.W = g.W; p.Cout = g.Cout; p.Cp = g.Cp; p.Ct = g.Ct; p.Cot = g.Cot;
   p.Kh = g.Kh; p.Kw = g.Kw; p.sh = g.sh; p.sw = g.sw; p.ph = g.ph; p.pw = g.pw;
-  const bool flat = fp4 && g.sh == 1 && g.sw == 1 && (g.Nt == 1 || g.Nt == 2 || g.Nt == 4 || g.Nt == 8) && !env_int("MQ_WGRAD_NO_FLAT", 0);
+  const bool flat = fp4 && g.sh == 1 && g.sw == 1 && (g.Nt == 1 || g.Nt == 2 || g.Nt == 4 || g.Nt == 8) && !MQ_ENV("MQ_WGRAD_NO_FLAT", 0);
   p.mode = fp8 ? MQ_WG_FP8 : (flat ? MQ_WG_FP4_FLAT : MQ_WG_FP4_PIXEL);
   p.kind = ts16 ? 2 : (fp4 ? 1 : 0);
   const int sf_cols1 = ts16 ? 16 : 8;       // TMEM columns and shared-memory bytes of one 128-row scale chunk
@@ -515,17 +517,17 @@ WgradPlan wgrad_plan(const Geom& g, int fmt_x, int fmt_g, bool ts16 = false) {
   p.groups_w = (g.Wo + p.KPX - 1) / p.KPX;
   p.Wp = g.W + 2 * g.pw;
   p.Hp = g.H + 2 * g.ph;
-  p.mma_cp = env_int("MQ_WGRAD_MMA_CP", 0);
+  p.mma_cp = MQ_ENV("MQ_WGRAD_MMA_CP", 0);
   p.stages_total = flat ? (g.Ho * p.Wp + p.KPX - 1) / p.KPX : g.Ho * p.groups_w * p.nchunks;
   p.b_rows = flat ? (g.Cp < 128 ? g.Cp : 128) : 128;
   // 8-bit operands: 256 input channels per MMA when the layer has them (the kernel is bound by the tensor core's
   // shared-memory operand reads, and a wider N reads the G_Y tile once for twice the work)
-  if (fp8 && g.Cp >= 256 && !env_int("MQ_WGRAD_N128", 0)) p.b_rows = 256;
+  if (fp8 && g.Cp >= 256 && !MQ_ENV("MQ_WGRAD_N128", 0)) p.b_rows = 256;
   p.m_tiles = (g.Cout + 127) / 128;
   p.m_tiles128 = p.m_tiles;
   // Pairs of blocks on 256 x 256 tiles (cta_group::2) when both channel counts allow it: half the X bytes per block
   // and stage, so six pipeline stages instead of four, and one MMA instruction per 256 x 256 x 32 for the issuing lane.
-  p.cta2 = fp8 && p.b_rows == 256 && g.Cout >= 256 && !env_int("MQ_WGRAD_NO_CTA2", 0);
+  p.cta2 = fp8 && p.b_rows == 256 && g.Cout >= 256 && !MQ_ENV("MQ_WGRAD_NO_CTA2", 0);
   if (p.cta2) { p.m_tiles = (g.Cout + 255) / 256; p.m_tiles128 = 2 * p.m_tiles; }
   // Thin 8-bit layers (32 or 64 input channels, unit strides): with one tap per block a 128-row B tile is mostly zero
   // fill.  Instead the Kw taps of a kernel row form one B operand of Kw * Cp rows: a stage loads a strip of
@@ -533,18 +535,18 @@ WgradPlan wgrad_plan(const Geom& g, int fmt_x, int fmt_g, bool ts16 = false) {
   // further - Kw times fewer stages, G_Y loads and MMA instructions.
   // (With a column stride the strip is the contiguous run of (KPX - 1) sw + Kw input pixels: output pixel a's tap kw is
   // input pixel a sw + kw of the strip, so panels stay one pixel apart and K slices sw pixels apart.)
-  p.grp8 = (fp8 && !p.cta2 && g.Kw > 1 && (g.Cp == 32 || g.Cp == 64) && g.Kw * g.Cp <= 256 && !env_int("MQ_WGRAD_NO_GROUP8", 0)) ? 1 : 0;
+  p.grp8 = (fp8 && !p.cta2 && g.Kw > 1 && (g.Cp == 32 || g.Cp == 64) && g.Kw * g.Cp <= 256 && !MQ_ENV("MQ_WGRAD_NO_GROUP8", 0)) ? 1 : 0;
   if (p.grp8) p.b_rows = g.Cp;
   p.cb_tiles = (g.Cp + p.b_rows - 1) / p.b_rows;
   // taps per block: a whole kernel row in the flat mode when its accumulators fit in tensor memory
   p.TG = p.grp8 ? g.Kw : 1;
-  if (flat && g.Kw > 1 && g.Kw * p.b_rows + 2 * sf_cols1 * (1 + (g.Kw * p.b_rows + 127) / 128) <= 512 && !env_int("MQ_WGRAD_NO_GROUP", 0)) p.TG = g.Kw;
+  if (flat && g.Kw > 1 && g.Kw * p.b_rows + 2 * sf_cols1 * (1 + (g.Kw * p.b_rows + 127) / 128) <= 512 && !MQ_ENV("MQ_WGRAD_NO_GROUP", 0)) p.TG = g.Kw;
   p.NB = (p.TG * p.b_rows + 127) / 128;
   p.n0 = p.TG * p.b_rows < 256 ? p.TG * p.b_rows : 256;
   p.n1 = p.TG * p.b_rows - p.n0;
   p.j_tiles = (g.Kh * g.Kw / p.TG) * p.cb_tiles;
   const int items = p.m_tiles * p.j_tiles;
-  int splits = env_int("MQ_WGRAD_SPLITS", 0);
+  int splits = MQ_ENV("MQ_WGRAD_SPLITS", 0);
   const int units = p.cta2 ? sm_count() / 2 : sm_count();   // blocks, or pairs of blocks, that run at once
   if (splits <= 0) splits = items >= units ? 1 : units / items;
   if (splits > p.stages_total) splits = p.stages_total;
@@ -558,7 +560,7 @@ WgradPlan wgrad_plan(const Geom& g, int fmt_x, int fmt_g, bool ts16 = false) {
     if (st > 6) st = 6;
     int slots = st;
     // kind 2: the scale buffers are twice as wide; rather than giving up pipeline stages, fewer buffers are used in turn
-    if (ts16 && !env_int("MQ_WGRAD_TS_NO_SLOTS", 0)) { while (slots > 2 && p.TG * p.b_rows + slots * sf_cols1 * (1 + p.NB) > 512) --slots; }
+    if (ts16 && !MQ_ENV("MQ_WGRAD_TS_NO_SLOTS", 0)) { while (slots > 2 && p.TG * p.b_rows + slots * sf_cols1 * (1 + p.NB) > 512) --slots; }
     else { while (st > 2 && p.TG * p.b_rows + st * sf_cols1 * (1 + p.NB) > 512) --st; slots = st; }
     p.stages = st;
     p.sf_slots = slots;
@@ -572,7 +574,7 @@ WgradPlan wgrad_plan(const Geom& g, int fmt_x, int fmt_g, bool ts16 = false) {
   size_t o = up256((size_t)splits * g.Cout * g.Kh * g.Kw * g.Cp * sizeof(float));
   w.off_sfa = o; o += up256((size_t)p.m_tiles128 * p.stages_total * 512 * spa);
   // flat mode with whole 128-channel tap panels: the X-side scale chunks once per padded start pixel (Kh Kw / KPX times fewer)
-  p.sfb_S = (flat && p.b_rows == 128 && !env_int("MQ_WGRAD_NO_SFB_DEDUP", 0)) ? w.P_b : 0;
+  p.sfb_S = (flat && p.b_rows == 128 && !MQ_ENV("MQ_WGRAD_NO_SFB_DEDUP", 0)) ? w.P_b : 0;
   w.off_sfb = o; o += up256(fp8 ? (size_t)p.cb_tiles * p.Hp * p.Wp * p.nchunks * p.NB * 512
                                 : p.sfb_S > 0 ? ((size_t)p.cb_tiles * p.sfb_S + p.NB) * 512 * spa
                                               : (size_t)p.cb_tiles * (g.Kh * g.Kw / p.TG) * p.stages_total * p.NB * 512 * spa);
@@ -716,7 +718,7 @@ mq_status check_conv_args(int op, const mq_conv_desc* desc, const mq_qtensor* qa
 
 // Does a forward / input-gradient call of this layer, formats and output layout run on the tensor cores?  (formats: one code per byte)
 bool conv_takes_tc(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, bool line, bool ts16, ConvTcPlan* pl) {
-  return (!ts16 || !env_int("MQ_TC_NO_TS16", 0)) && (op == MQ_OP_FWD || op == MQ_OP_BWD_DATA) && conv_tc_eligible(op, g, fmt_x_like, fmt_w) &&
+  return (!ts16 || !MQ_ENV("MQ_TC_NO_TS16", 0)) && (op == MQ_OP_FWD || op == MQ_OP_BWD_DATA) && conv_tc_eligible(op, g, fmt_x_like, fmt_w) &&
          conv_tc_plan(op, g, fmt_x_like, fmt_w, layout, pl, line, false, ts16);
 }
 
@@ -815,7 +817,7 @@ mq_status run_conv(int op, const mq_conv_desc* desc, const mq_qtensor* qa_in, in
 
 }  // namespace
 
-bool pdl_enabled() { return env_int("MQ_NO_PDL", 0) == 0; }
+bool pdl_enabled() { return MQ_ENV("MQ_NO_PDL", 0) == 0; }
 
 }  // namespace mq
 
@@ -898,7 +900,7 @@ static mq_status quantize_impl(const mq_conv_desc* desc, const void* src, int sr
   a.sr = sr;
   a.sr_seed_lo = (unsigned)seed; a.sr_seed_hi = (unsigned)(seed >> 32);
   a.sr_key0 = sr_mix32(a.sr_seed_lo ^ sr_mix32(a.sr_seed_hi ^ sr_mix32(0u)));
-  a.sr_wide = ((unsigned long long)v.P * (unsigned long long)v.R * (unsigned long long)v.C >= (1ull << 32) || env_int("MQ_SR_WIDE", 0)) ? 1 : 0;
+  a.sr_wide = ((unsigned long long)v.P * (unsigned long long)v.R * (unsigned long long)v.C >= (1ull << 32) || MQ_ENV("MQ_SR_WIDE", 0)) ? 1 : 0;
   cudaError_t e = ts16 ? launch_quantize_ts(a, amax_in, dst->tensor_scale, static_cast<cudaStream_t>(stream)) : launch_quantize(a, static_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? MQ_OK : MQ_ERR_CUDA;
 }
@@ -1133,7 +1135,7 @@ LayerArena layer_arena(const mq_conv_desc* desc, const int fmts[3]) {
   auto take = [&](size_t n) { size_t r = o; o += up256(n); return r; };
   L.off_x = take(L.nx); L.off_w = take(L.nw); L.off_g = take(L.ng);
   L.off_y = take(L.ng); L.off_dx = take(L.nx); L.off_dw = take(L.nw);
-  int max_slabs = env_int("MQ_HOST_SLABS", 8);
+  int max_slabs = MQ_ENV("MQ_HOST_SLABS", 8);
   max_slabs = max_slabs < 1 ? 1 : (max_slabs > 8 ? 8 : max_slabs);
   const int tiles_per_slab = (g.Nt + max_slabs - 1) / max_slabs;
   L.slab_n = 32 * tiles_per_slab;

@@ -8,6 +8,8 @@
 #include <cuda_fp6.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "mq.h"
 
 namespace mq {
@@ -75,7 +77,27 @@ inline int sm_count() {
 // Integer value of an MQ_* environment knob.  Each knob is read from the environment ONCE, on its first use in the
 // process, and answered from a table afterwards, so that a size query and the call it sizes always see the same plan;
 // mq_reload_env() (a diagnostic entry point) empties the table.
-int env_int(const char* name, int dflt);
+// A call asks for some dozens of knobs, so every place that asks keeps the table's answer beside it, stamped with the
+// table's generation: one atomic load instead of a lock, a string and a map (the latter were 1-2 us of each call).
+extern std::atomic<uint32_t> g_env_generation;   // 31 bits, advanced by mq_reload_env
+uint64_t env_lookup(const char* name);           // generation << 33 | set << 32 | value, from the table
+class EnvKnob {
+ public:
+  constexpr explicit EnvKnob(const char* name) : name_(name) {}
+  int get(int dflt) {
+    uint64_t c = cell_.load(std::memory_order_acquire);
+    if ((uint32_t)(c >> 33) != (g_env_generation.load(std::memory_order_acquire) & 0x7fffffffu)) {
+      c = env_lookup(name_);
+      cell_.store(c, std::memory_order_release);
+    }
+    return (c >> 32) & 1u ? (int)(uint32_t)c : dflt;
+  }
+
+ private:
+  const char* name_;
+  std::atomic<uint64_t> cell_{0};
+};
+#define MQ_ENV(name, dflt) ([]() -> ::mq::EnvKnob& { static ::mq::EnvKnob knob(name); return knob; }().get(dflt))
 
 // ---- launchers (defined in the .cu files) ---------------------------------------------------
 struct QuantArgs {

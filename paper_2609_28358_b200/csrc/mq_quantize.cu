@@ -811,7 +811,7 @@ cudaError_t launch_q(const QuantArgs& a, int n_pstrips, int Ct, long long n_item
 bool quantize_ts_tma_eligible(const QuantArgs& a) {
   const bool vec = (a.P % 4 == 0) && ((reinterpret_cast<uintptr_t>(a.src) & 15) == 0);
   const long long elems = (long long)a.P * a.R * a.C;
-  const int tv = env_int("MQ_QUANT_TMA", -1);   // 1 / 0 force the choice
+  const int tv = MQ_ENV("MQ_QUANT_TMA", -1);   // 1 / 0 force the choice
   return vec && a.src_stride_r == 0 && a.fmt == MQ_E2M1 && (tv >= 0 ? tv != 0 : elems >= (1ll << 22));
 }
 
@@ -851,7 +851,7 @@ cudaError_t launch_quantize_ts_tma(const QuantArgs& a0, const float* amax_src, f
 cudaError_t launch_quantize(const QuantArgs& a, cudaStream_t s) {
   const bool vec = (a.P % 4 == 0) && ((reinterpret_cast<uintptr_t>(a.src) & 15) == 0);
   // at most 16 rows (e.g. a batch of 16 samples): items of 16 positions, see quantize_pipe_kernel
-  const bool r16 = vec && !a.line && a.src_stride_r == 0 && a.R <= 16 && !env_int("MQ_QUANT_NO_R16", 0);
+  const bool r16 = vec && !a.line && a.src_stride_r == 0 && a.R <= 16 && !MQ_ENV("MQ_QUANT_NO_R16", 0);
   const int psi = r16 ? 2 * PS : PS;
   const int n_pstrips = (a.P + psi - 1) / psi;
   const int Rt = (a.R + 31) / 32, Ct = a.Cp / 32;
@@ -873,7 +873,7 @@ cudaError_t launch_quantize(const QuantArgs& a, cudaStream_t s) {
   // large tensors with 16-byte rows: whole-line TMA boxes (items of 32 positions); small ones keep the 8-position items,
   // which give a small tensor more blocks to spread over
   const long long elems = (long long)a.P * a.R * a.C;
-  const int tv = env_int("MQ_QUANT_TMA", -1);   // 1 / 0 force the choice
+  const int tv = MQ_ENV("MQ_QUANT_TMA", -1);   // 1 / 0 force the choice
   const bool tma = vec && (a.debug_skip_loads || (tv >= 0 ? tv != 0 : (elems >= (1ll << 22) || (a.line && elems >= (1ll << 18)))));
   if (a.debug_skip_loads && !tma) return cudaErrorInvalidValue;
   if (tma) {

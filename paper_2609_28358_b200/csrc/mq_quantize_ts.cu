@@ -138,7 +138,7 @@ cudaError_t launch_quantize_ts(const QuantArgs& a, const float* amax_in, float* 
   if (a.act && a.src_stride_r == 0) return cudaErrorInvalidValue;   // the activation rides on the channel-fastest source only
   // maximum supplied from outside and the whole-line kernel applies: ONE pass - the quantizer collects this tensor's own
   // maximum for the next step while it works (MQ_QUANT_TS_TWO_PASS=1 keeps the separate reduction)
-  if (amax_in && quantize_ts_tma_eligible(a) && !env_int("MQ_QUANT_TS_TWO_PASS", 0)) {
+  if (amax_in && quantize_ts_tma_eligible(a) && !MQ_ENV("MQ_QUANT_TS_TWO_PASS", 0)) {
     count_launches(1);
     return launch_quantize_ts_tma(a, amax_in, stats, s, true);
   }

@@ -836,7 +836,7 @@ static bool make_flat_args(FlatArgs* fa, const uint8_t* in, uint8_t* out, int Hs
                            int nblocks, int KBn) {
   fa->in = in; fa->out = out; fa->Hs = Hs; fa->Ws = Ws; fa->N = N; fa->Cs_p = Cs_p; fa->P_out = P_out; fa->Wp = Wp; fa->off_h = off_h; fa->off_w = off_w;
   fa->rows = rows; fa->nblocks = nblocks; fa->KBn = KBn;
-  fa->wide = (KBn == 128 && nblocks * rows >= 256 && N <= 256 && !env_int("MQ_WGRAD_NO_WIDE_PREP", 0)) ? 1 : 0;
+  fa->wide = (KBn == 128 && nblocks * rows >= 256 && N <= 256 && !MQ_ENV("MQ_WGRAD_NO_WIDE_PREP", 0)) ? 1 : 0;
   if (fa->wide) {
     fa->ncg = (nblocks * rows + 255) / 256;
     const long long units = (long long)P_out * fa->ncg;

@@ -1,7 +1,7 @@
 """Python binding of ``libmq.so``: the same names as the C ABI (``include/mq.h``), argument
-marshalling only.  PyTorch supplies device memory and the current CUDA stream; every step of the
-path runs in the library's kernels.  There is no fallback: if the library is missing or a call
-fails, an exception is raised.
+marshalling only, and that of the per-step calls natively (``csrc/mq_torch.cpp``, module ``_mq_torch``).  PyTorch
+supplies device memory and the current CUDA stream; every step of the path runs in the library's kernels.  There is
+no fallback: if the library is missing or a call fails, an exception is raised.
 """
 from __future__ import annotations
 
@@ -29,6 +29,7 @@ DEBUG_FILL = False
 
 _LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "libmq.so")
 _lib = None
+_n = None      # the native marshalling module
 
 
 class MqError(RuntimeError):
@@ -59,6 +60,20 @@ def lib():
         _lib.mq_kernel_launch_count.restype = ctypes.c_ulonglong
         _lib.mq_reload_env.restype = None
     return _lib
+
+
+def _native():
+    """The native marshalling module, loaded on first use.  Raises if it has not been built, as lib() does."""
+    global _n
+    lib()
+    try:
+        from . import _mq_torch
+    except ImportError as e:
+        raise RuntimeError(f"the binding of {_LIB_PATH} cannot be loaded ({e}): build it with `python -m paper_2609_28358_b200.build`; "
+                           "there is no fallback path") from e
+    _mq_torch.set_error(MqError)
+    _n = _mq_torch
+    return _n
 
 
 def status_string(status):
@@ -126,41 +141,26 @@ def empty_qtensor(desc, role, fmt, device="cuda", block=TILE32):
 _DTYPES = {torch.float32: F32, torch.bfloat16: BF16}
 
 
+def _stored(created, out, fmt, role, block):
+    """`out`, or the stored tensor made of the buffers the native call created."""
+    return out if created is None else QTensor(created[0], created[1], fmt, role, block, created[2])
+
+
 def quantize(desc, role, fmt, src, out=None, src_layout=NCHW, stream=None, block=TILE32):
     """mq_quantize: device tensor (NCHW / OIHW, or channel-fastest with src_layout=HWNC) -> stored MX tensor."""
-    assert src.is_cuda and src.dtype in _DTYPES and src.is_contiguous()
-    if out is None:
-        out = empty_qtensor(desc, role, fmt, src.device, block)
-    q = out._c()
-    _check("mq_quantize", lib().mq_quantize(ctypes.byref(_d(desc)), ctypes.c_void_p(src.data_ptr()), _DTYPES[src.dtype], src_layout, ctypes.byref(q),
-                                           _stream(stream)))
-    return out
+    return _stored((_n or _native()).quantize(0, desc, role, fmt, block, src, src_layout, out, None, None, stream, DEBUG_FILL), out, fmt, role, block)
 
 
 def quantize_sr(desc, role, fmt, src, seed, out=None, src_layout=NCHW, stream=None, block=TILE32):
     """mq_quantize_sr: as quantize(), with stochastic rounding of the elements (the gradient's rounding); `seed` is a 64-bit integer."""
-    assert src.is_cuda and src.dtype in _DTYPES and src.is_contiguous()
-    if out is None:
-        out = empty_qtensor(desc, role, fmt, src.device, block)
-    q = out._c()
-    _check("mq_quantize_sr", lib().mq_quantize_sr(ctypes.byref(_d(desc)), ctypes.c_void_p(src.data_ptr()), _DTYPES[src.dtype], src_layout, ctypes.byref(q),
-                                                 ctypes.c_uint64(int(seed) & 0xFFFFFFFFFFFFFFFF), _stream(stream)))
-    return out
+    return _stored((_n or _native()).quantize(1, desc, role, fmt, block, src, src_layout, out, int(seed), None, stream, DEBUG_FILL), out, fmt, role, block)
 
 
 def quantize_ts(desc, role, src, out=None, src_layout=NCHW, amax_in=None, seed=None, stream=None):
     """mq_quantize_ts: the paper's own format (fp32 tensor scale, E4M3 scale per 16 x 16 block, E2M1 elements).  amax_in: a
     device float tensor holding the maximum Eq. 4 should use (e.g. an earlier tensor's tensor_scale[1:2]); None = this
     tensor's own (two passes).  seed: stochastic rounding with that 64-bit seed."""
-    assert src.is_cuda and src.dtype in _DTYPES and src.is_contiguous()
-    if out is None:
-        out = empty_qtensor(desc, role, E2M1, src.device, TS16)
-    q = out._c()
-    sd = ctypes.c_uint64(int(seed) & 0xFFFFFFFFFFFFFFFF) if seed is not None else None
-    _check("mq_quantize_ts", lib().mq_quantize_ts(ctypes.byref(_d(desc)), ctypes.c_void_p(src.data_ptr()), _DTYPES[src.dtype], src_layout, ctypes.byref(q),
-                                                 ctypes.c_void_p(amax_in.data_ptr()) if amax_in is not None else None,
-                                                 ctypes.byref(sd) if sd is not None else None, _stream(stream)))
-    return out
+    return _stored((_n or _native()).quantize(2, desc, role, E2M1, TS16, src, src_layout, out, seed, amax_in, stream, DEBUG_FILL), out, E2M1, role, TS16)
 
 
 def selftest_wait_timeout(desc, role, fmt, src, polls=2000, stream=None):
@@ -175,47 +175,15 @@ def selftest_wait_timeout(desc, role, fmt, src, polls=2000, stream=None):
 
 def cbf_im2col(desc, xq, out_codes=None, out_scales=None, stream=None):
     """mq_cbf_im2col: stored quantized activation -> (codes, scales) of X'."""
-    cb, sb = im2col_sizes(desc, xq.fmt, xq.block)
-    if out_codes is None:
-        out_codes = _new(cb, torch.uint8, xq.codes.device)
-    if out_scales is None:
-        out_scales = _new(sb, torch.uint8, xq.codes.device)
-    q = xq._c()
-    _check("mq_cbf_im2col", lib().mq_cbf_im2col(ctypes.byref(_d(desc)), ctypes.byref(q), ctypes.c_void_p(out_codes.data_ptr()),
-                                               ctypes.c_void_p(out_scales.data_ptr()), _stream(stream)))
-    return out_codes, out_scales
-
-
-def _out_hw(desc):
-    d = ConvDesc(*desc)
-    return ((d.H + 2 * d.pad_h - d.Kh) // d.stride_h + 1, (d.W + 2 * d.pad_w - d.Kw) // d.stride_w + 1)
-
-
-def _conv(name, op, desc, qa, qb, out, shape_nchw, shape_hwnc, layout, workspace, stream, dtype=torch.float32):
-    dev = qa.codes.device
-    if out is None:
-        out = _new(shape_nchw if layout == NCHW else shape_hwnc, dtype, dev)
-    need = workspace_size(desc, op, qa.fmt, qb.fmt, qa.block)
-    if workspace is None and need > 0:
-        workspace = _new(need, torch.uint8, dev)
-    wp = ctypes.c_void_p(workspace.data_ptr()) if workspace is not None else None
-    wn = workspace.numel() * workspace.element_size() if workspace is not None else 0
-    a, b = qa._c(), qb._c()
-    fn = getattr(lib(), name)
-    _check(name, fn(ctypes.byref(_d(desc)), ctypes.byref(a), ctypes.byref(b), ctypes.c_void_p(out.data_ptr()), _DTYPES[out.dtype], layout, wp,
-                    ctypes.c_size_t(wn), _stream(stream)))
-    return out
+    return (_n or _native()).im2col(desc, xq, out_codes, out_scales, stream, DEBUG_FILL)
 
 
 def conv_fwd(desc, xq, wq, y=None, layout=NCHW, workspace=None, stream=None, dtype=torch.float32):
-    d = ConvDesc(*desc)
-    ho, wo = _out_hw(d)
-    return _conv("mq_conv_fwd", OP_FWD, desc, xq, wq, y, (d.N, d.C_out, ho, wo), (ho, wo, d.N, d.C_out), layout, workspace, stream, dtype)
+    return (_n or _native()).conv(OP_FWD, desc, xq, wq, y, layout, workspace, stream, dtype, DEBUG_FILL)
 
 
 def conv_bwd_data(desc, wq, dyq, dx=None, layout=NCHW, workspace=None, stream=None, dtype=torch.float32):
-    d = ConvDesc(*desc)
-    return _conv("mq_conv_bwd_data", OP_BWD_DATA, desc, wq, dyq, dx, (d.N, d.C_in, d.H, d.W), (d.H, d.W, d.N, d.C_in), layout, workspace, stream, dtype)
+    return (_n or _native()).conv(OP_BWD_DATA, desc, wq, dyq, dx, layout, workspace, stream, dtype, DEBUG_FILL)
 
 
 ACT_NONE, ACT_RELU, ACT_SILU = 0, 1, 2
@@ -227,41 +195,21 @@ def conv_mx_workspace_size(desc, op, fmt_a, fmt_b):
     return b.value
 
 
-def _mx_out(desc, op, fmt, role, device):
-    """An empty stored tensor of what the quantizing epilogue emits: the forward result as a role-X tensor of
-    N x C_out x Ho x Wo, the input gradient as a role-DY tensor of N x C_in x H x W."""
-    d = ConvDesc(*desc)
-    ho, wo = _out_hw(d)
-    c, h, w = (d.C_out, ho, wo) if op == OP_FWD else (d.C_in, d.H, d.W)
-    cp = (c + 31) // 32 * 32
-    cb = h * w * d.N * cp * (4 if fmt == E2M1 else 8) // 8
-    sb = h * w * ((d.N + 31) // 32) * (cp // 32)
-    return QTensor(_new(cb, torch.uint8, device), _new(sb, torch.uint8, device), fmt, role)
-
-
-def _conv_mx(name, op, desc, qa, qb, out, extra, workspace, stream):
-    need = conv_mx_workspace_size(desc, op, qa.fmt, qb.fmt)
-    if workspace is None and need > 0:
-        workspace = _new(need, torch.uint8, qa.codes.device)
-    wp = ctypes.c_void_p(workspace.data_ptr()) if workspace is not None else None
-    wn = workspace.numel() * workspace.element_size() if workspace is not None else 0
-    a, b, o = qa._c(), qb._c(), out._c()
-    _check(name, getattr(lib(), name)(ctypes.byref(_d(desc)), ctypes.byref(a), ctypes.byref(b), *extra, ctypes.byref(o), wp, ctypes.c_size_t(wn), _stream(stream)))
-    return out
+def _conv_emit(op, desc, qa, qb, fmt, act, amax, out, workspace, stream):
+    """The quantizing producer epilogue.  The forward result is created as a role-X tensor of N x C_out x Ho x Wo, the input
+    gradient as a role-DY tensor of N x C_in x H x W; amax None: MX tiles of format `fmt`, else the paper's own format."""
+    created = (_n or _native()).conv_emit(op, desc, qa, qb, fmt, act, amax, out, workspace, stream, DEBUG_FILL)
+    return _stored(created, out, fmt, ROLE_X if op == OP_FWD else ROLE_DY, TILE32 if amax is None else TS16)
 
 
 def conv_fwd_mx(desc, xq, wq, fmt, act=ACT_NONE, yq=None, workspace=None, stream=None):
     """mq_conv_fwd_mx: act(conv(X, W)) emitted as the next layer's stored activation (element format `fmt`)."""
-    if yq is None:
-        yq = _mx_out(desc, OP_FWD, fmt, ROLE_X, xq.codes.device)
-    return _conv_mx("mq_conv_fwd_mx", OP_FWD, desc, xq, wq, yq, (ctypes.c_int(act),), workspace, stream)
+    return _conv_emit(OP_FWD, desc, xq, wq, fmt, act, None, yq, workspace, stream)
 
 
 def conv_bwd_data_mx(desc, wq, dyq, fmt, dxq=None, workspace=None, stream=None):
     """mq_conv_bwd_data_mx: the input gradient emitted as the previous layer's stored output gradient."""
-    if dxq is None:
-        dxq = _mx_out(desc, OP_BWD_DATA, fmt, ROLE_DY, wq.codes.device)
-    return _conv_mx("mq_conv_bwd_data_mx", OP_BWD_DATA, desc, wq, dyq, dxq, (), workspace, stream)
+    return _conv_emit(OP_BWD_DATA, desc, wq, dyq, fmt, ACT_NONE, None, dxq, workspace, stream)
 
 
 def conv_ts_workspace_size(desc, op):
@@ -270,42 +218,17 @@ def conv_ts_workspace_size(desc, op):
     return b.value
 
 
-def _ts_out(desc, op, role, device):
-    """An empty stored tensor in the paper's own format of what the quantizing epilogue emits (see _mx_out)."""
-    d = ConvDesc(*desc)
-    ho, wo = _out_hw(d)
-    c, h, w = (d.C_out, ho, wo) if op == OP_FWD else (d.C_in, d.H, d.W)
-    cp = (c + 31) // 32 * 32
-    return QTensor(_new(h * w * d.N * cp // 2, torch.uint8, device), _new(h * w * ((d.N + 15) // 16) * (cp // 16), torch.uint8, device), E2M1, role, TS16,
-                   _new(2, torch.float32, device))
-
-
-def _conv_ts(name, op, desc, qa, qb, out, extra, workspace, stream):
-    need = conv_ts_workspace_size(desc, op)
-    if workspace is None and need > 0:
-        workspace = _new(need, torch.uint8, qa.codes.device)
-    wp = ctypes.c_void_p(workspace.data_ptr()) if workspace is not None else None
-    wn = workspace.numel() * workspace.element_size() if workspace is not None else 0
-    a, b, o = qa._c(), qb._c(), out._c()
-    _check(name, getattr(lib(), name)(ctypes.byref(_d(desc)), ctypes.byref(a), ctypes.byref(b), *extra, ctypes.byref(o), wp, ctypes.c_size_t(wn), _stream(stream)))
-    return out
-
-
 def conv_fwd_ts(desc, xq, wq, amax_in, act=ACT_NONE, yq=None, workspace=None, stream=None):
     """mq_conv_fwd_ts: act(conv(X, W)) emitted as the next layer's stored activation in the paper's own format; amax_in: a
     device float tensor holding the maximum Eq. 4 uses (an earlier step's tensor_scale[1:2])."""
     assert amax_in.is_cuda and amax_in.dtype == torch.float32 and amax_in.numel() >= 1
-    if yq is None:
-        yq = _ts_out(desc, OP_FWD, ROLE_X, xq.codes.device)
-    return _conv_ts("mq_conv_fwd_ts", OP_FWD, desc, xq, wq, yq, (ctypes.c_int(act), ctypes.c_void_p(amax_in.data_ptr())), workspace, stream)
+    return _conv_emit(OP_FWD, desc, xq, wq, E2M1, act, amax_in, yq, workspace, stream)
 
 
 def conv_bwd_data_ts(desc, wq, dyq, amax_in, dxq=None, workspace=None, stream=None):
     """mq_conv_bwd_data_ts: the input gradient emitted as the previous layer's stored output gradient in the paper's own format."""
     assert amax_in.is_cuda and amax_in.dtype == torch.float32 and amax_in.numel() >= 1
-    if dxq is None:
-        dxq = _ts_out(desc, OP_BWD_DATA, ROLE_DY, wq.codes.device)
-    return _conv_ts("mq_conv_bwd_data_ts", OP_BWD_DATA, desc, wq, dyq, dxq, (ctypes.c_void_p(amax_in.data_ptr()),), workspace, stream)
+    return _conv_emit(OP_BWD_DATA, desc, wq, dyq, E2M1, ACT_NONE, amax_in, dxq, workspace, stream)
 
 
 STATIC_SCRATCH_BYTES = 16 << 20
@@ -326,8 +249,7 @@ def conv_bwd_data_static(desc, wq, dyq, dx=None, layout=NCHW, stream=None):
 
 
 def conv_bwd_weight(desc, xq, dyq, dw=None, layout=NCHW, workspace=None, stream=None):
-    d = ConvDesc(*desc)
-    return _conv("mq_conv_bwd_weight", OP_BWD_WEIGHT, desc, xq, dyq, dw, (d.C_out, d.C_in, d.Kh, d.Kw), (d.C_out, d.Kh, d.Kw, d.C_in), layout, workspace, stream)
+    return (_n or _native()).conv(OP_BWD_WEIGHT, desc, xq, dyq, dw, layout, workspace, stream, torch.float32, DEBUG_FILL)
 
 
 def reload_env():
