@@ -1187,13 +1187,14 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   if (warp == 1) { if (DUO) tmem_dealloc_2(tmem, 512); else tmem_dealloc(tmem, 512); }
 }
 
-// The BPC scale bytes of chunk `cc` of a row whose Kblocks scales start at `row`.  Rows of whole chunks (Kblocks a multiple of BPC)
-// are read in one access; else the row starts anywhere and its last chunk is short: byte by byte, zero (2^-127, times a code of
-// zero) for K-blocks beyond the row.
-template <int BPC>
+// The BPC scale bytes of chunk `cc` of a row whose Kblocks scales start at `row`.  WHOLE: rows of whole chunks (Kblocks a multiple of
+// BPC), read in one access; else the row starts anywhere and its last chunk is short: byte by byte, zero (2^-127, times a code
+// of zero) for K-blocks beyond the row.  (A template parameter and not a test here: with a branch around every load the loads
+// of a chunk go one after the other - the paper's format, 256 channels 28x28: the forward call 97 -> 107 us.)
+template <int BPC, bool WHOLE>
 __device__ __forceinline__ unsigned long long load_scale_bytes(const uint8_t* row, int cc, int Kblocks) {
   if (BPC == 1) return __ldg(row + cc);
-  if (Kblocks % BPC == 0) {
+  if (WHOLE) {
     const uint8_t* ptr = row + cc * BPC;
     if (BPC == 2) return __ldg(reinterpret_cast<const unsigned short*>(ptr));
     if (BPC == 4) return __ldg(reinterpret_cast<const unsigned int*>(ptr));
@@ -1207,8 +1208,9 @@ __device__ __forceinline__ unsigned long long load_scale_bytes(const uint8_t* ro
 }
 // The same for the paper's own format: the four E4M3 scale bytes of K-atom `atom` (64 elements) of a row whose Kb16 (an even
 // number of) scales start at `row`, zero beyond the row.
+template <bool WHOLE>
 __device__ __forceinline__ unsigned load_ts_scales(const uint8_t* row, int atom, int Kb16) {
-  if (Kb16 % 4 == 0) return 4 * atom < Kb16 ? __ldg(reinterpret_cast<const unsigned int*>(row + 4 * atom)) : 0u;
+  if (WHOLE) return __ldg(reinterpret_cast<const unsigned int*>(row + 4 * atom));
   unsigned v = 0u;
   if (4 * atom < Kb16) v = __ldg(reinterpret_cast<const unsigned short*>(row + 4 * atom));
   if (4 * atom + 2 < Kb16) v |= (unsigned)__ldg(reinterpret_cast<const unsigned short*>(row + 4 * atom + 2)) << 16;
@@ -1218,7 +1220,7 @@ __device__ __forceinline__ unsigned load_ts_scales(const uint8_t* row, int atom,
 // Builds, in shared memory, the scale-vector chunks ([chunk][group][atom][512]) of the resident weight tile of
 // the whole-tile kernel (channel tile 0).  Called by all threads of the block before the roles start (stride 1:
 // tap q of the walk is weight tap q).
-template <int KB, bool FP4>
+template <int KB, bool FP4, bool WHOLE>
 __device__ __forceinline__ void halo_build_sfb(const ConvTcParams& p, uint8_t* s_sfb) {
   constexpr int G = 128 / KB, APC = KB / 32, SPA = FP4 ? 2 : 1, BPC = APC * SPA;
   const int taps = p.Kh * p.Kw;
@@ -1234,7 +1236,7 @@ __device__ __forceinline__ void halo_build_sfb(const ConvTcParams& p, uint8_t* s
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           if (j < 4 * atoms_b && 32 * j < p.BN && 32 * j < p.Cd)
-            acc[j] |= load_scale_bytes<BPC>(p.b_scales + ((long long)j * taps + q) * p.Kblocks, 0, p.Kblocks) << (8 * c * BPC);
+            acc[j] |= load_scale_bytes<BPC, WHOLE>(p.b_scales + ((long long)j * taps + q) * p.Kblocks, 0, p.Kblocks) << (8 * c * BPC);
         }
       }
     }
@@ -1326,7 +1328,10 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   }
   if (warp == 1) { tmem_alloc(tmem_slot, 512); tmem_relinquish(); }
   pdl_wait();
-  if (p.fused) halo_build_sfb<KB, FP4>(p, smem + b_bytes);
+  if (p.fused) {
+    if (p.Kblocks == APC * SPA) halo_build_sfb<KB, FP4, true>(p, smem + b_bytes);
+    else halo_build_sfb<KB, FP4, false>(p, smem + b_bytes);
+  }
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
@@ -1574,7 +1579,8 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
 // row r of the tile at byte (r % 32) * 16 + (r / 32) * 4, four consecutive K-blocks per 32-bit word --
 // from the compact tile scales.  A-side chunks exist per tile (without its channel index), B-side
 // chunks per (stride class, channel tile).
-template <int MODE, int KB, int KIND>
+// WHOLE: every row is a whole number of chunks (see load_scale_bytes).
+template <int MODE, int KB, int KIND, bool WHOLE>
 __global__ void __launch_bounds__(256) expand_conv_scales_kernel(const ConvTcParams p, unsigned n_tile_m) {
   constexpr bool FP4 = KIND != 0;
   pdl_wait();
@@ -1650,7 +1656,7 @@ __global__ void __launch_bounds__(256) expand_conv_scales_kernel(const ConvTcPar
         const bool ok = n < p.N && hs >= 0 && hs < p.Hs && ws >= 0 && ws < p.Ws;
         const uint8_t* rowp = p.a_scales + (((long long)hs * p.Ws + ws) * Nt16 + (n >> 4)) * Kb16;
 #pragma unroll
-        for (int ja = 0; ja < 4; ++ja) val[ja][j] = (ok && ja < APC) ? load_ts_scales(rowp, pos.cc * APC + ja, Kb16) : 0u;
+        for (int ja = 0; ja < 4; ++ja) val[ja][j] = (ok && ja < APC) ? load_ts_scales<WHOLE>(rowp, pos.cc * APC + ja, Kb16) : 0u;
       }
       uint8_t* dst = p.sfa_img + (size_t)wid * (512 * 4) + lane * 16;
 #pragma unroll
@@ -1688,7 +1694,7 @@ __global__ void __launch_bounds__(256) expand_conv_scales_kernel(const ConvTcPar
             if (n < p.N && hs >= 0 && hs < p.Hs && ws >= 0 && ws < p.Ws) {
               const uint8_t* rowp = p.a_scales + (((long long)hs * p.Ws + ws) * Nt16 + (n >> 4)) * Kb16;
 #pragma unroll
-              for (int ja = 0; ja < APC; ++ja) val[c * APC + ja][j] = load_ts_scales(rowp, pos.cc * APC + ja, Kb16);
+              for (int ja = 0; ja < APC; ++ja) val[c * APC + ja][j] = load_ts_scales<WHOLE>(rowp, pos.cc * APC + ja, Kb16);
             }
           }
         }
@@ -1735,14 +1741,14 @@ __global__ void __launch_bounds__(256) expand_conv_scales_kernel(const ConvTcPar
                     unsigned w = 0;
 #pragma unroll
                     for (int kb = 0; kb < 4; ++kb)
-                      if (pos.cc * (4 * APC) + 4 * ja + kb < Kb16) w |= (unsigned)__ldg(p.wt_sc_in + ((long long)(pos.cc * (4 * APC) + 4 * ja + kb) * taps_all + tap) * Cb_w + (row >> 4)) << (8 * kb);
+                      if (WHOLE || pos.cc * (4 * APC) + 4 * ja + kb < Kb16) w |= (unsigned)__ldg(p.wt_sc_in + ((long long)(pos.cc * (4 * APC) + 4 * ja + kb) * taps_all + tap) * Cb_w + (row >> 4)) << (8 * kb);
                     val[c * APC + ja][j] = w;
                   }
                 }
               } else if (row < p.b_rows_total) {
                 const uint8_t* rowp = p.b_scales + ((long long)(row >> 4) * taps_all + tap) * Kb16;
 #pragma unroll
-                for (int ja = 0; ja < APC; ++ja) val[c * APC + ja][j] = load_ts_scales(rowp, pos.cc * APC + ja, Kb16);
+                for (int ja = 0; ja < APC; ++ja) val[c * APC + ja][j] = load_ts_scales<WHOLE>(rowp, pos.cc * APC + ja, Kb16);
               }
             }
           }
@@ -1797,7 +1803,7 @@ __global__ void __launch_bounds__(256) expand_conv_scales_kernel(const ConvTcPar
       const int tw_ = r & (p.TW - 1), tn = r >> p.lgTW;
       const int n = tile.n0 + tn, ws = ws0 + tw_;
       if (n < p.N && hs >= 0 && hs < p.Hs && ws >= 0 && ws < p.Ws)
-        acc[j] = load_scale_bytes<BPC>(p.a_scales + (((long long)hs * p.Ws + ws) * (p.line ? p.N : p.Nt) + (p.line ? n : (n >> 5))) * p.Kblocks, pos.cc, p.Kblocks);
+        acc[j] = load_scale_bytes<BPC, WHOLE>(p.a_scales + (((long long)hs * p.Ws + ws) * (p.line ? p.N : p.Nt) + (p.line ? n : (n >> 5))) * p.Kblocks, pos.cc, p.Kblocks);
     }
     uint8_t* dst = p.sfa_img + (size_t)wid * (512 * SPA) + lane * 16;
 #pragma unroll
@@ -1831,7 +1837,7 @@ __global__ void __launch_bounds__(256) expand_conv_scales_kernel(const ConvTcPar
           const int tw_ = r & (p.TW - 1), tn = r >> p.lgTW;
           const int n = tile.n0 + tn, ws = ws0 + tw_ * wstep;
           if (n < p.N && hs >= 0 && hs < p.Hs && ws >= 0 && ws < p.Ws)
-            acc[j] |= load_scale_bytes<BPC>(p.a_scales + (((long long)hs * p.Ws + ws) * (p.line ? p.N : p.Nt) + (p.line ? n : (n >> 5))) * p.Kblocks, pos.cc, p.Kblocks) << (8 * c * BPC);
+            acc[j] |= load_scale_bytes<BPC, WHOLE>(p.a_scales + (((long long)hs * p.Ws + ws) * (p.line ? p.N : p.Nt) + (p.line ? n : (n >> 5))) * p.Kblocks, pos.cc, p.Kblocks) << (8 * c * BPC);
         }
       }
     }
@@ -1872,14 +1878,14 @@ __global__ void __launch_bounds__(256) expand_conv_scales_kernel(const ConvTcPar
               unsigned long long bytes = 0;
 #pragma unroll
               for (int kb = 0; kb < BPC; ++kb)
-                if (pos.cc * BPC + kb < p.Kblocks) bytes |= (unsigned long long)__ldg(p.wt_sc_in + ((long long)(pos.cc * BPC + kb) * taps_all + tap) * Ct_w + cib) << (8 * kb);
+                if (WHOLE || pos.cc * BPC + kb < p.Kblocks) bytes |= (unsigned long long)__ldg(p.wt_sc_in + ((long long)(pos.cc * BPC + kb) * taps_all + tap) * Ct_w + cib) << (8 * kb);
               acc[j] |= bytes << (8 * c * BPC);
             } else if (p.line) {
               // line blocks: every weight row has its own scale per K-block
               const int row = tile.c0 + 32 * j + lane;
-              if (row < p.b_rows_total) acc[j] |= load_scale_bytes<BPC>(p.b_scales + ((long long)row * taps_all + tap) * p.Kblocks, pos.cc, p.Kblocks) << (8 * c * BPC);
+              if (row < p.b_rows_total) acc[j] |= load_scale_bytes<BPC, WHOLE>(p.b_scales + ((long long)row * taps_all + tap) * p.Kblocks, pos.cc, p.Kblocks) << (8 * c * BPC);
             } else {
-              acc[j] |= load_scale_bytes<BPC>(p.b_scales + ((long long)((tile.c0 >> 5) + j) * taps_all + tap) * p.Kblocks, pos.cc, p.Kblocks) << (8 * c * BPC);
+              acc[j] |= load_scale_bytes<BPC, WHOLE>(p.b_scales + ((long long)((tile.c0 >> 5) + j) * taps_all + tap) * p.Kblocks, pos.cc, p.Kblocks) << (8 * c * BPC);
             }
           }
         }
@@ -2029,14 +2035,17 @@ cudaError_t launch_expand_inst(const ConvTcParams& p, cudaStream_t s) {
   unsigned long long warps = (unsigned long long)conv_tc_sfa_chunks(p) + (unsigned long long)p.classes * p.tiles_c * p.max_stages;
   if (p.halo) warps += ((unsigned long long)p.tiles_c * p.Kh * p.Kw * p.BN * (KB / 16) + 31) / 32;
   const unsigned blocks = (unsigned)((warps + 7) / 8);
+  // scales per chunk of KB bytes: KB / 32 K-blocks of 32 bytes, each one scale (8-bit) or two (E2M1; in the paper's format four halves)
+  const bool whole = p.Kblocks % (KB / 32 * (FP4 ? 2 : 1)) == 0;
+  auto kernel = whole ? expand_conv_scales_kernel<MODE, KB, FP4, true> : expand_conv_scales_kernel<MODE, KB, FP4, false>;
   count_launches(1);
   if (p.wt_fused) {
     ConvTcParams q = p;
     q.expand_blocks = blocks;
     const unsigned extra = (unsigned)(p.wt_bx * p.wt_by * p.Kh * p.Kw);
-    return launch_pdl(expand_conv_scales_kernel<MODE, KB, FP4>, dim3(blocks + extra), dim3(256), 0, s, q, n_tile_m);
+    return launch_pdl(kernel, dim3(blocks + extra), dim3(256), 0, s, q, n_tile_m);
   }
-  return launch_pdl(expand_conv_scales_kernel<MODE, KB, FP4>, dim3(blocks), dim3(256), 0, s, p, n_tile_m);
+  return launch_pdl(kernel, dim3(blocks), dim3(256), 0, s, p, n_tile_m);
 }
 
 cudaError_t launch_expand_conv_scales(const ConvTcParams& p, cudaStream_t s) {
