@@ -1738,10 +1738,10 @@ __global__ void __launch_bounds__(256) expand_conv_scales_kernel(const ConvTcPar
                   const int Cb_w = p.wt_Cp >> 4;
 #pragma unroll
                   for (int ja = 0; ja < APC; ++ja) {
-                    unsigned w = 0;
+                    unsigned w = 0;      // (the stored scales end with the last 16-channel block that holds output channels, not at C_out_p)
 #pragma unroll
                     for (int kb = 0; kb < 4; ++kb)
-                      if (WHOLE || pos.cc * (4 * APC) + 4 * ja + kb < Kb16) w |= (unsigned)__ldg(p.wt_sc_in + ((long long)(pos.cc * (4 * APC) + 4 * ja + kb) * taps_all + tap) * Cb_w + (row >> 4)) << (8 * kb);
+                      if (16 * (pos.cc * (4 * APC) + 4 * ja + kb) < p.wt_Cout) w |= (unsigned)__ldg(p.wt_sc_in + ((long long)(pos.cc * (4 * APC) + 4 * ja + kb) * taps_all + tap) * Cb_w + (row >> 4)) << (8 * kb);
                     val[c * APC + ja][j] = w;
                   }
                 }
