@@ -269,32 +269,101 @@ template <int FMT>
 __device__ __forceinline__ float sr_value(float x, unsigned lo, unsigned key) {
   constexpr int M = (FMT == MQ_E4M3 || FMT == MQ_E2M3) ? 3 : (FMT == MQ_E2M1 ? 1 : 2);                      // mantissa bits
   constexpr int EMIN = FMT == MQ_E4M3 ? -6 : (FMT == MQ_E5M2 ? -14 : (FMT == MQ_E3M2 ? -2 : 0));           // smallest normal exponent
-  // fp32 pattern of the largest magnitude: 448, 57344, 6, 28, 7.5
-  constexpr unsigned MAXBITS = FMT == MQ_E4M3 ? 0x43E00000u : (FMT == MQ_E5M2 ? 0x47600000u : (FMT == MQ_E2M1 ? 0x40C00000u : (FMT == MQ_E3M2 ? 0x41E00000u : 0x40F00000u)));
   const unsigned b = __float_as_uint(x) & 0x7fffffffu;       // |x|; patterns of non-negative floats order like their values
-  const unsigned r23 = sr_mix32(lo ^ key) >> 9;
-  // normal range of the format: the grid keeps M mantissa bits of the fp32 pattern.  The dropped field f (23 - M bits)
-  // is the fraction of a step in units of 2^-(23 - M): f * 2^M > draw + 1/2 is an integer comparison, and stepping up
-  // is an integer addition on the pattern (the carry walks into the exponent at a binade's end).
+  const unsigned rn = ~sr_mix32(lo ^ key);                   // the draw's complement: top 23 bits = 2^23 - 1 - draw
+  // normal range of the format: the grid keeps M mantissa bits of the fp32 pattern.  The dropped field f (23 - M bits) is the
+  // fraction of a step in units of 2^-(23 - M): up iff f * 2^M > draw, i.e. iff f + (2^(23 - M) - 1 - (draw >> M)) carries
+  // out of the field - so one addition on the pattern decides and steps (the carry walks into the exponent at a binade's end).
   constexpr unsigned MASK = (1u << (23 - M)) - 1u;
-  const unsigned f = b & MASK;
-  const unsigned q_norm = (b - f) + (((f << M) > r23) ? MASK + 1u : 0u);
-  // below it the step is the constant 2^(EMIN - M): t = |x| / step < 2^M, floor through a round-down addition of 2^23,
-  // draw + 1/2 as (2^23 + draw) - (2^23 - 1/2); all exact
+  const unsigned q_norm = (b + (rn >> (9 + M))) & ~MASK;
+  // below it the step is the constant 2^(EMIN - M): t = |x| / step < 2^M, up iff frac(t) > u = (draw + 1/2) / 2^23, i.e. the result
+  // is ceil(t + (1 - u)) - 1.  1 - u = (2^23 - 1 - draw) 2^-23 + 2^-24 is exact; rounding the sum up, and then to an integer by an
+  // addition of 2^23 rounded up, keeps the ceiling.
   const float t = __uint_as_float(b) * __uint_as_float((unsigned)(127 + M - EMIN) << 23);
-  const float fl = __fadd_rd(t, 8388608.f) - 8388608.f;
-  const float u = __uint_as_float(0x4B000000u | r23) - 8388607.5f;
-  const float up = (t - fl) * 8388608.f > u ? 1.f : 0.f;
-  const unsigned q_sub = __float_as_uint((fl + up) * __uint_as_float((unsigned)(127 + EMIN - M) << 23));
-  unsigned q = b >= ((unsigned)(127 + EMIN) << 23) ? q_norm : q_sub;
-  q = b < MAXBITS ? q : b;      // at or beyond the largest magnitude: left to the conversion's saturation
+  const float w = __uint_as_float(0x3F800000u | (rn >> 9)) - __uint_as_float(0x3F7FFFFFu);
+  const float n = __fadd_ru(__fadd_ru(t, w), 8388608.f) - 8388609.f;
+  const unsigned q_sub = __float_as_uint(n * __uint_as_float((unsigned)(127 + EMIN - M) << 23));
+  const unsigned q = b >= ((unsigned)(127 + EMIN) << 23) ? q_norm : q_sub;     // (beyond the largest magnitude the conversion saturates)
   return __uint_as_float(q | (__float_as_uint(x) & 0x80000000u));
 }
+
 // Stream key of an element from the high word of its index; tensors below 2^32 elements (a.sr_wide == 0, uniform)
 // take the key computed on the host.
 __device__ __forceinline__ unsigned sr_key(const QuantArgs& a, long long idx) {
   if (!a.sr_wide) return a.sr_key0;
   return sr_mix32(a.sr_seed_lo ^ sr_mix32(a.sr_seed_hi ^ sr_mix32((unsigned)((unsigned long long)idx >> 32))));
+}
+
+// ---- elements of the paper's own format (Eq. 6: Round(x / den), den = Scale_b x T_scale) ---------------------------------
+// The quotient is an IEEE division, but it only decides which of E2M1's eight magnitudes comes out, so the division itself is
+// rarely needed: q' = x * (1 / den) is within 2.5 units in the last place of it, and unless q' lies within four units of a
+// decision threshold both round alike.  The few elements for which that cannot be said (one in 10^5; all of a block whose
+// denominator is so extreme that the bound on q' does not hold) are divided.  An IEEE division costs a dozen instructions and
+// a branch per element, the check three (256 channels 28x28, N = 256: 72 -> 61 us, stochastic 185 -> 106 us).
+struct TsDen {
+  float den, inv;   // den 0: the block encodes to signed zeros
+  unsigned sure;    // 0: every element takes the division
+};
+__device__ __forceinline__ TsDen ts_den(float den) {
+  TsDen d;
+  d.den = den;
+  const bool in_range = den >= 7.9e-31f && den <= 1.2e30f;    // 2^-100 .. 2^100
+  d.inv = in_range ? __frcp_rn(den) : 0.f;
+  d.sure = (in_range || !(den > 0.f)) ? 0xffffffffu : 0u;
+  return d;
+}
+// One element by the definition.  lo, key: as sr_value's
+template <bool SR>
+__device__ __forceinline__ unsigned ts_code_by_division(float x, float den, unsigned lo, unsigned key) {
+  float q = ts_div(x, den);
+  if (SR && den > 0.f) q = sr_value<MQ_E2M1>(q, lo, key);
+  return encode2<MQ_E2M1>(q, 0.f) & 0xFu;
+}
+// Eight elements of neighbouring channels -> their codes, element 0 in the low nibble.  e0 (SR): element 0's index in the logical
+// tensor, whose channels are a.P elements apart.
+template <bool SR>
+__device__ __forceinline__ unsigned ts_codes8(const float* x, const TsDen& d, const QuantArgs& a, long long e0) {
+  unsigned word = 0, sure = d.sure;
+  if (!SR) {
+    // thresholds of round-to-nearest are 0.25, 0.75, 1.25, 1.75, 2.5, 3.5 and 5: patterns whose low 21 bits are zero
+#pragma unroll
+    for (int k = 0; k < 8; k += 2) {
+      const float q0 = x[k] * d.inv, q1 = x[k + 1] * d.inv;
+      sure = min(sure, (__float_as_uint(fmaxf(fabsf(q0), 0.24f)) + 4u) << 11);
+      sure = min(sure, (__float_as_uint(fmaxf(fabsf(q1), 0.24f)) + 4u) << 11);
+      word |= encode2<MQ_E2M1>(q0, q1) << (4 * k);
+    }
+    if (sure >= (8u << 11)) return word;
+  } else {
+    // As in sr_value, one addition on the pattern of q' decides and steps; below 1 the pattern of q' + 1, two codes down, whose
+    // last place is 2^-22 of the step 0.5 - the sum's low 22 bits tell how far the decision is (window: 2.5 units of q', one of
+    // the addition and one of the draw's finer bits, rounded up to 8)
+    const unsigned lo0 = (unsigned)e0;
+    unsigned key = a.sr_key0;
+    if (a.sr_wide) {   // (eight channels across which the index's high word advances have two keys: by division)
+      key = sr_key(a, e0);
+      if ((unsigned long long)(e0 + 7ll * a.P) >> 32 != (unsigned long long)e0 >> 32) sure = 0;
+    }
+#pragma unroll
+    for (int k = 7; k >= 0; --k) {
+      const unsigned rn = ~sr_mix32((lo0 + (unsigned)k * (unsigned)a.P) ^ key);
+      const float q = fminf(fabsf(x[k]) * d.inv, 6.f);
+      const bool below = q < 1.f;
+      const unsigned sum = __float_as_uint(below ? q + 1.f : q) + (rn >> 10) + (below ? 0u - (254u << 22) : 0u - (252u << 22));
+      sure = min(sure, (sum + 8u) << 10);
+      word = __funnelshift_l((sum << 6) | (__float_as_uint(x[k]) & 0x80000000u), word, 4);
+    }
+    if (sure >= (16u << 10)) return word;
+  }
+#pragma unroll 1
+  for (int k = 0; k < 8; ++k) {
+    float xk = x[0];
+#pragma unroll
+    for (int j = 1; j < 8; ++j) xk = j == k ? x[j] : xk;
+    const long long e = e0 + (long long)k * a.P;
+    word = (word & ~(0xFu << (4 * k))) | (ts_code_by_division<SR>(xk, d.den, (unsigned)e, SR ? sr_key(a, e) : 0u) << (4 * k));
+  }
+  return word;
 }
 
 #endif  // __CUDACC__

@@ -503,7 +503,7 @@ quantize_tma_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_con
       consumer_sync();
       if (*abort_flag) break;    // uniform: written only between the previous item's last barrier and the one above
       int code[LINE ? 4 : 1];
-      float den[2] = {0.f, 0.f};   // TS: Scale_b * T_scale of the thread's two blocks (0: the block encodes to signed zeros)
+      TsDen den[TS ? 2 : 1];       // TS: Scale_b * T_scale of the thread's two blocks
       if (TS) {
         unsigned* xch = reinterpret_cast<unsigned*>(stage);   // [sample half][warp][lane]
         xch[warp * 32 + lane] = __float_as_uint(fmaxf(lm[0], lm[1]));
@@ -520,7 +520,7 @@ quantize_tma_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_con
           if (bmax > 0.f && tscale > 0.f) sc = (unsigned)__nv_cvt_float_to_fp8(__fdiv_rn(bmax, t6), __NV_SATFINITE, __NV_E4M3) & 0x7Fu;   // Eq. 5
           const __half_raw hr = __nv_cvt_fp8_to_halfraw((__nv_fp8_storage_t)sc, __NV_E4M3);
           const float bscale = __half2float(*reinterpret_cast<const __half*>(&hr));
-          den[hf] = (bscale > 0.f && tscale > 0.f) ? __fmul_rn(bscale, tscale) : 0.f;
+          den[hf] = ts_den((bscale > 0.f && tscale > 0.f) ? __fmul_rn(bscale, tscale) : 0.f);
           // one thread per (position, sample half, channel half): warps 0 and 1 hold both channel halves of every position
           if ((warp >> 1) == 0 && q.p0 + lane < a.P && q.r0 + 16 * hf < a.R)
             a.scales[(long long)(q.p0 + lane) * a.sc_stride_p + (long long)(2 * q.rt + hf) * a.sc_stride_r + 2 * q.ct + chalf] = (uint8_t)sc;
@@ -550,19 +550,23 @@ quantize_tma_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_con
 #pragma unroll
       for (int b = 0; b < 4; ++b) {
         if (b < nb) {
-          const float f = TS ? 0.f : scale_factor(code[LINE ? b : 0]);
-          const float dn = den[b >> 1];
           const int n = 8 * b + n_sub;
+          const long long e0 = ((long long)(q.r0 + n) * a.C + q.c0 + chalf * 16) * a.P + q.p0 + lane;   // SR: index of the first element
+          if constexpr (TS) {   // Eq. 6
+            const unsigned lo = ts_codes8<SR>(v[b], den[b >> 1], a, e0), hi = ts_codes8<SR>(v[b] + 8, den[b >> 1], a, e0 + 8ll * a.P);
+            *reinterpret_cast<uint2*>(stage + (lane * 32 + n) * (2 * CB) + chalf * CB) = make_uint2(lo, hi);
+            continue;
+          }
+          const float f = scale_factor(code[LINE ? b : 0]);
           unsigned w4[4];
 #pragma unroll
           for (int k = 0; k < 16; k += 4) {
             float x[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-              if (TS) x[j] = ts_div(v[b][k + j], dn);   // Eq. 6
-              else x[j] = v[b][k + j] * f;
-              if (SR && (!TS || dn > 0.f)) {
-                const long long e = ((long long)(q.r0 + n) * a.C + q.c0 + chalf * 16 + k + j) * a.P + q.p0 + lane;
+              x[j] = v[b][k + j] * f;
+              if (SR) {
+                const long long e = e0 + (long long)(k + j) * a.P;
                 x[j] = sr_value<FMT>(x[j], (unsigned)e, sr_key(a, e));
               }
             }
