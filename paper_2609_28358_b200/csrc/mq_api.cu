@@ -572,12 +572,13 @@ WgradPlan wgrad_plan(const Geom& g, int fmt_x, int fmt_g, bool ts16 = false) {
   w.P_a = p.stages_total * p.KPX;
   w.P_b = (w.P_a + (g.Kh - 1) * p.Wp + g.Kw - 1 + 7) / 8 * 8;
   size_t o = up256((size_t)splits * g.Cout * g.Kh * g.Kw * g.Cp * sizeof(float));
-  w.off_sfa = o; o += up256((size_t)p.m_tiles128 * p.stages_total * 512 * spa);
+  w.off_sfa = o; if (!fp8 || p.cta2) o += up256((size_t)p.m_tiles128 * p.stages_total * 512 * spa);
   // flat mode with whole 128-channel tap panels: the X-side scale chunks once per padded start pixel (Kh Kw / KPX times fewer)
   p.sfb_S = (flat && p.b_rows == 128 && !MQ_ENV("MQ_WGRAD_NO_SFB_DEDUP", 0)) ? w.P_b : 0;
-  w.off_sfb = o; o += up256(fp8 ? (size_t)p.cb_tiles * p.Hp * p.Wp * p.nchunks * p.NB * 512
-                                : p.sfb_S > 0 ? ((size_t)p.cb_tiles * p.sfb_S + p.NB) * 512 * spa
-                                              : (size_t)p.cb_tiles * (g.Kh * g.Kw / p.TG) * p.stages_total * p.NB * 512 * spa);
+  w.off_sfb = o;
+  if (p.cta2) o += up256((size_t)p.cb_tiles * p.Hp * p.Wp * p.nchunks * p.NB * 512);
+  else if (!fp8) o += up256(p.sfb_S > 0 ? ((size_t)p.cb_tiles * p.sfb_S + p.NB) * 512 * spa
+                                   : (size_t)p.cb_tiles * (g.Kh * g.Kw / p.TG) * p.stages_total * p.NB * 512 * spa);
   w.off_xt = o;
   if (flat) { p.xt_block_bytes = (long long)w.P_b * p.b_rows * p.KBn; o += up256((size_t)p.cb_tiles * p.xt_block_bytes); }
   else if (fp4) o += up256((size_t)g.Cp * g.H * g.W * w.Npad / 2);
@@ -664,7 +665,7 @@ mq_status run_wgrad_tc(const Geom& g, WgradPlan& w, const mq_qtensor* qx, const 
   if (p.mode == MQ_WG_FP4_FLAT) {
     if (launch_wgrad_flat_prep(p, static_cast<const uint8_t*>(qx->codes), xt, w.P_b, static_cast<const uint8_t*>(qg->codes), gt, w.P_a, stream) != cudaSuccess)
       return MQ_ERR_CUDA;
-  } else if (launch_expand_wgrad_scales(p, stream) != cudaSuccess) return MQ_ERR_CUDA;
+  } else if ((p.mode == MQ_WG_FP4_PIXEL || p.cta2) && launch_expand_wgrad_scales(p, stream) != cudaSuccess) return MQ_ERR_CUDA;
   CUtensorMap map_p{};
   {
     const uint64_t J = (uint64_t)g.Kh * g.Kw * g.Cp;
@@ -675,11 +676,10 @@ mq_status run_wgrad_tc(const Geom& g, WgradPlan& w, const mq_qtensor* qx, const 
   }
   CUtensorMap map_sfa{}, map_sfb{};
   if (p.cta2) {   // a pair's scale chunks travel as tiled copies too (rows of 256 bytes), so that they can count on the leader's barrier
-    const int spa = 1;   // 8-bit operands only
-    const uint64_t rows_a = (uint64_t)p.m_tiles128 * p.stages_total * 2 * spa;
-    const uint64_t rows_b = (uint64_t)p.cb_tiles * p.Hp * p.Wp * p.nchunks * p.NB * 2 * spa;
+    const uint64_t rows_a = (uint64_t)p.m_tiles128 * p.stages_total * 2;
+    const uint64_t rows_b = (uint64_t)p.cb_tiles * p.Hp * p.Wp * p.nchunks * p.NB * 2;
     const uint64_t da[2] = {256, rows_a}, db[2] = {256, rows_b}, st[1] = {256};
-    const uint32_t ba[2] = {256u, (uint32_t)(2 * spa)}, bb[2] = {256u, (uint32_t)(2 * spa * p.NB)};
+    const uint32_t ba[2] = {256u, 2u}, bb[2] = {256u, (uint32_t)(2 * p.NB)};
     if (!encode_tensor_map_u8(&map_sfa, p.sfa_img, 2, da, st, ba, nullptr, 0)) return MQ_ERR_CUDA;
     if (!encode_tensor_map_u8(&map_sfb, p.sfb_img, 2, db, st, bb, nullptr, 0)) return MQ_ERR_CUDA;
   }

@@ -158,14 +158,16 @@ struct WgradTcParams {
   const uint8_t* gt;        // flat: [co block][padded pixel][128][KBn]
   const uint8_t* xt;        // flat: [ci block][padded pixel][b_rows][KBn]
   long long gt_block_bytes, xt_block_bytes;
-  uint8_t* sfa_img;         // [m tile][stage][512 * SPA]
-  uint8_t* sfb_img;         // E2M1: [ci block][tap group][stage][NB][512 * SPA]; 8-bit: [ci block][Hp][Wp][sample chunk][NB][512]
+  uint8_t* sfa_img;         // (E2M1 and pairs of blocks) [m tile][stage][512 * SPA]
+  uint8_t* sfb_img;         // pairs: [ci block][Hp][Wp][sample chunk][NB][512]; E2M1: [ci block][tap group][stage][NB][512 * SPA], or [ci block][padded start pixel][512 * SPA]
   float* partial;           // [splits][Cout][taps * Cp]
   unsigned int* status;
 };
 // map_p: the partial sums as an fp32 tensor (taps * Cp columns, C_out rows, splits), box 32 x 32 x 1, 128-byte swizzle
+// (map_sfa, map_sfb: pairs of blocks only - the scale images as rows of 256 bytes)
 cudaError_t launch_wgrad_tc(const WgradTcParams& p, const CUtensorMap& map_a, const CUtensorMap& map_b, const CUtensorMap& map_p, const CUtensorMap& map_sfa,
                             const CUtensorMap& map_sfb, cudaStream_t s);
+// The scale chunks of every stage: E2M1 modes and pairs of blocks (else 8-bit operands' blocks build their own)
 cudaError_t launch_expand_wgrad_scales(const WgradTcParams& p, cudaStream_t s);
 // E2M1 codes [P][N][Cp] -> [P][Cp][Npad] (n fastest, zero-padded): a permutation of nibbles, no requantization.
 cudaError_t launch_fp4_to_n_major(const uint8_t* in, uint8_t* out, int P, int N, int Cp, int Npad, cudaStream_t s);

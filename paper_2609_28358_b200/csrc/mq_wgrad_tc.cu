@@ -14,10 +14,11 @@
 //                    the input pixel of output pixel q at tap (kh, kw) is q + kh*Wp + kw, so a stage of
 //                    consecutive pixels is ONE contiguous, already swizzled run for each operand (bulk copy).
 //
-// A small kernel first expands the compact tile scales into the per-stage scale-vector chunks in scratch.
+// Scales: 8-bit operands, one block per tile - two warps of the block build each stage's scale-vector chunks from the compact
+// tile scales (build_stage_scales); pairs of blocks and E2M1 - a small kernel first expands them into per-stage chunks in scratch.
 // One thread block per work item (128 output channels x one tap's block of input channels x a slice of
 // the K range); partial sums go to scratch and are added in a fixed order by bwd_weight_reduce.
-// Warps: 0 producer (TMA / bulk copies), 1 MMA issuer, 2 scale copier (smem -> TMEM), 4-7 epilogue.
+// Warps: 1 MMA issuer, 2 scale copier (E2M1; smem -> TMEM), the others loaders (8-bit, one block per tile: two of them scale builders), 4-7 then epilogue.
 #include <cstdlib>
 #include "mq_conv_tc.cuh"
 #include "mq_tcgen05.cuh"
@@ -143,10 +144,10 @@ __device__ __forceinline__ void expand_wgrad_scales_body(const WgradTcParams& p,
   const int taps = p.Kh * p.Kw;
   const long long nA = (long long)p.m_tiles128 * p.stages_total;
   const int groups = taps / p.TG;
-  // B-side chunks: E2M1 modes one per (channel block, tap group, stage); 8-bit mode one per (channel block, padded X
-  // pixel, sample chunk) - a stage's chunk depends only on where its taps' pixels start, so the taps share them
-  const long long nB = (FP4 && p.sfb_S > 0) ? (long long)p.cb_tiles * p.sfb_S
-                     : FP4 ? (long long)p.cb_tiles * groups * p.stages_total * p.NB : (long long)p.cb_tiles * p.Hp * p.Wp * p.nchunks * p.NB;
+  // B-side chunks: E2M1 modes one per (channel block, tap group, stage), or per (channel block, padded start pixel); 8-bit pairs
+  // of blocks one per (channel block, padded X pixel, sample chunk) - a stage's chunk depends only on where its tap's pixels
+  // start, so the taps share them
+  const long long nB = !FP4 ? (long long)p.cb_tiles * p.Hp * p.Wp * p.nchunks * p.NB : p.sfb_S > 0 ? (long long)p.cb_tiles * p.sfb_S : (long long)p.cb_tiles * groups * p.stages_total * p.NB;
   if (wid >= nA + nB) return;
   // this lane's byte: 32-row group j of the 128-row chunk, K-block b of the stage
   const int j = lane >> 3, b = lane & 7;
@@ -169,14 +170,10 @@ __device__ __forceinline__ void expand_wgrad_scales_body(const WgradTcParams& p,
       const int nc = (int)(idx % p.nchunks); idx /= p.nchunks;
       const int wp = (int)(idx % p.Wp); idx /= p.Wp;
       const int hp = (int)(idx % p.Hp); const int cb = (int)(idx / p.Hp);
-      // rows of the chunk: input channels of one tap, or (grouped thin mode) tap-in-row major, input channel minor - tap tj
-      // reads the pixel tj further along the row
-      const int row0 = c * 128 + 32 * j;
-      const int tj = p.grp8 ? row0 / p.b_rows : 0;
-      const int cib = p.grp8 ? (row0 - tj * p.b_rows) / 32 : (cb * p.b_rows + row0) / 32;
-      if (b < NBS && cib < p.Ct && tj < p.TG) {
+      const int cib = (cb * p.b_rows + c * 128 + 32 * j) / 32;
+      if (b < NBS && cib < p.Ct) {
         const int px = b / p.BPP, nb = nc * p.BPP + (b - px * p.BPP);
-        const int h = hp - p.ph, w = wp - p.pw + px * p.sw + tj;
+        const int h = hp - p.ph, w = wp - p.pw + px * p.sw;
         if (nb < p.Nt && h >= 0 && h < p.H && w >= 0 && w < p.W) v = __ldg(p.x_scales + (((long long)h * p.W + w) * p.Nt + nb) * p.Ct + cib);
       }
     } else if (p.sfb_S > 0) {
@@ -231,6 +228,90 @@ __device__ __forceinline__ void expand_wgrad_scales_body(const WgradTcParams& p,
 template <bool FP4>
 __global__ void __launch_bounds__(256) expand_wgrad_scales_kernel(const WgradTcParams p) { pdl_wait(); expand_wgrad_scales_body<FP4>(p, blockIdx.x); }
 __global__ void __launch_bounds__(256) expand_wgrad_scales_nv_kernel(const WgradTcParams p) { pdl_wait(); expand_wgrad_scales_nv_body(p, blockIdx.x); }
+
+// ---- scale chunks of a stage, built where they are used (8-bit operands, one block per tile) ------------------------
+// A stage has four K-blocks (32 samples at one output pixel each), a 128-row chunk four 32-row groups: sixteen scale bytes,
+// each lane row repeating the same four words ([row % 32][row / 32] words of four K-blocks).  One warp gathers the bytes of
+// the G_Y chunk (lanes 0-15) and of the one or two X chunks (lanes 16-31; a second byte of lanes 0-15), assembles the words by
+// shuffles and writes the chunks.  The bytes are asked for four of the warp's own stages (two warps take even and odd ones) ahead,
+// so their latency is not in the pipeline.  A separate kernel that expanded every chunk into scratch (512 bytes per padded input
+// pixel) took 38 of 100 us of a 16 -> 32 channel layer at 320x320 (N = 16; now 64), 2-4 us of small layers, and a launch.
+// Pairs of blocks keep that kernel (4.8 of 89 us, 256 channels 28x28): the peer's builder would have to arrive on the leader's
+// barrier with a cluster-scope release of what it wrote, about a microsecond per stage (measured: 178 us).
+__device__ __forceinline__ void build_stage_scales(const WgradTcParams& p, uint8_t* smem, int sf_off, uint64_t* full, uint64_t* empty, volatile int* abort_flag,
+                                                   int lane, int half, int mt, int cb, int kh, int kw, int st_begin, int nst) {
+  constexpr int AHEAD = 4;
+  const int b = lane & 3, j = (lane >> 2) & 3, px = b / p.BPP, sub = b - px * p.BPP;
+  const bool is_a = lane < 16;
+  const int cob = mt * 4 + j;
+  // X chunk c of this lane's bytes: rows 128 c + 32 j .., input channels of one tap, or (grouped thin mode) tap-in-row major
+  int cib[2], tj[2];
+  bool x_ok[2];
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    const int row0 = c * 128 + 32 * j;
+    tj[c] = p.grp8 ? row0 / p.b_rows : 0;
+    cib[c] = p.grp8 ? (row0 - tj[c] * p.b_rows) / 32 : (cb * p.b_rows + row0) / 32;
+    x_ok[c] = c < p.NB && cib[c] < p.Ct && tj[c] < p.TG;
+  }
+  int nc, wg, ho;      // of the stage asked for next
+  {
+    const int st = st_begin + half;
+    nc = st % p.nchunks; const int t = st / p.nchunks;
+    wg = t % p.groups_w; ho = t / p.groups_w;
+  }
+  auto ask = [&](uint32_t& v0, uint32_t& v1) {
+    const int nb = nc * p.BPP + sub, wo = wg * p.KPX + px;
+    const int h = ho * p.sh + kh - p.ph, w = wo * p.sw + kw - p.pw;
+    auto x_byte = [&](int c) -> uint32_t {
+      const int wc = w + tj[c];
+      if (!(x_ok[c] && nb < p.Nt && h >= 0 && h < p.H && wc >= 0 && wc < p.W)) return 0u;
+      return __ldg(p.x_scales + (((long long)h * p.W + wc) * p.Nt + nb) * p.Ct + cib[c]);
+    };
+    v0 = v1 = 0u;
+    if (is_a) {
+      if (cob < p.Cot && wo < p.Wo && nb < p.Nt) v0 = __ldg(p.g_scales + (((long long)ho * p.Wo + wo) * p.Nt + nb) * p.Cot + cob);
+      v1 = x_byte(1);
+    } else v0 = x_byte(0);
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+      if (++nc == p.nchunks) { nc = 0; if (++wg == p.groups_w) { wg = 0; ++ho; } }
+  };
+  const int n_own = (nst - half + 1) >> 1;
+  uint32_t q0[AHEAD], q1[AHEAD];
+#pragma unroll
+  for (int u = 0; u < AHEAD; ++u) { q0[u] = q1[u] = 0u; if (u < n_own) ask(q0[u], q1[u]); }
+  uint32_t s = (uint32_t)half % (uint32_t)p.stages, phase = 0;   // stages >= 2
+#pragma unroll 1
+  for (int i = 0; i < n_own; i += AHEAD) {
+#pragma unroll
+    for (int u = 0; u < AHEAD; ++u) {
+      if (i + u < n_own) {
+        uint32_t w0 = q0[u] << (8 * b), w1 = q1[u] << (8 * b);
+        w0 |= __shfl_xor_sync(0xffffffffu, w0, 1); w0 |= __shfl_xor_sync(0xffffffffu, w0, 2);
+        w1 |= __shfl_xor_sync(0xffffffffu, w1, 1); w1 |= __shfl_xor_sync(0xffffffffu, w1, 2);
+        uint32_t a4[4], b4[4], c4[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          a4[k] = __shfl_sync(0xffffffffu, w0, 4 * k);
+          b4[k] = __shfl_sync(0xffffffffu, w0, 16 + 4 * k);
+          c4[k] = __shfl_sync(0xffffffffu, w1, 4 * k);
+        }
+        if (i + u + AHEAD < n_own) ask(q0[u], q1[u]);
+        if (*abort_flag) return;
+        if (!mbar_wait(&empty[s], phase ^ 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; return; }
+        uint8_t* dst = smem + (size_t)s * p.stage_bytes + sf_off + lane * 16;
+        *reinterpret_cast<uint4*>(dst) = make_uint4(a4[0], a4[1], a4[2], a4[3]);
+        *reinterpret_cast<uint4*>(dst + 1024) = make_uint4(b4[0], b4[1], b4[2], b4[3]);
+        if (p.NB > 1) *reinterpret_cast<uint4*>(dst + 1536) = make_uint4(c4[0], c4[1], c4[2], c4[3]);
+        fence_proxy_async_smem();      // the scale copies read these through the async proxy
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&full[s]);
+        s += 2; if (s >= (uint32_t)p.stages) { s -= (uint32_t)p.stages; phase ^= 1; }
+      }
+    }
+  }
+}
 
 //
 // CTA2 (8-bit operands, C_out and C_in >= 256): the two blocks of a cluster compute a 256 x 256 tile with
@@ -287,7 +368,7 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
 
   if (threadIdx.x == 0) {
 #pragma unroll 1
-    // full: one arrival per kind of copy
+    // full: one arrival per kind of copy, or of the scale builder
     for (int s = 0; s < p.stages; ++s) { mbar_init(&full[s], has_b1 ? 4 : 3); mbar_init(&empty[s], 1); mbar_init(&sffull[s], 1); mbar_init(&pfull[s], 1); }
     mbar_init(tfull, 1);
     *abort_flag = 0;
@@ -321,6 +402,8 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     const int kidx = lslot >> 1, half = lslot & 1;
     const int kind = kidx == 0 ? 0 : (kidx == 1 ? 1 : ((kidx == 2 && has_b1) ? 2 : 3));   // 0 G_Y, 1 X, 2 second X panel, 3 scales
     const int taps = p.Kh * p.Kw;
+    if (!FP4 && !CTA2 && kind == 3) build_stage_scales(p, smem, sf_off, full, empty, abort_flag, lane, half, mt, cb, kh, kw, st_begin, nst);
+    else {
     const uint8_t* sfa_src = p.sfa_img + ((size_t)mt * p.stages_total + st_begin) * (512 * SPA);
     const uint32_t sfb_bytes = (uint32_t)p.NB * 512 * SPA;
     // X-side scale chunks: per (tap group, stage), NB chunks each; or (sfb_S) per padded start pixel - the NB taps of the
@@ -359,18 +442,17 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       if (!mbar_wait(&empty[s], phase ^ 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
       if (elect_one()) {
         if (rank == 0) mbar_arrive_expect_tx(bar, my_bytes);
-        // 8-bit mode: the X-side chunk of (padded pixel, sample chunk); E2M1: of (tap group, stage)
-        const long long xchunk = !FP4 ? ((((long long)cb * p.Hp + (xh + p.ph)) * p.Wp + (xw + p.pw)) * p.nchunks + nc) : 0;
         if (CTA2) {
           if (kind == 0) tma_load_4d_pair(sa, &map_a, lbar, co0, nrow, wo0, ho);
           else if (kind == 1) tma_load_4d_pair(sb, &map_b, lbar, ci_ld, nrow, xw, xh);
-          else {
+          else {   // the X-side chunk of (padded pixel, sample chunk)
+            const long long xchunk = (((long long)cb * p.Hp + (xh + p.ph)) * p.Wp + (xw + p.pw)) * p.nchunks + nc;
             tma_load_2d_pair(ssf, &map_sfa, lbar, 0, sfa_row0 + i * (2 * SPA));
             tma_load_2d_pair(ssf + SFC_BYTES, &map_sfb, lbar, 0, (int)(xchunk * (2 * SPA * p.NB)));
           }
         } else if (kind == 3) {
           bulk_load(ssf, sfa_src + (size_t)i * (512 * SPA), 512 * SPA, bar);
-          bulk_load(ssf + SFC_BYTES, FP4 ? sfb_src + (size_t)i * sfb_step : p.sfb_img + (size_t)xchunk * sfb_bytes, sfb_bytes, bar);
+          bulk_load(ssf + SFC_BYTES, sfb_src + (size_t)i * sfb_step, sfb_bytes, bar);
         } else if (p.mode == MQ_WG_FP4_FLAT) {
           if (kind == 0) bulk_load(sa, ga + (size_t)i * a_bytes, a_bytes, bar);
           else bulk_load(sb, gb + (size_t)i * b_step, b_bytes, bar);          // KPX + TG - 1 consecutive pixels
@@ -393,6 +475,7 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
 #pragma unroll
       for (int r = 0; r < 2; ++r)
         if (++nc == p.nchunks) { nc = 0; if (++wg == p.groups_w) { wg = 0; ++ho; } }
+    }
     }
   }
   __syncwarp();
@@ -548,9 +631,6 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         const uint32_t sf_t = sf_base + ss * sf_cols;
         if (++ss == (uint32_t)p.sf_slots) ss = 0;
         if (elect_one()) {
-#ifdef MQ_WG_SKIPCP
-          if (i < p.stages)
-#endif
           {
 #pragma unroll
           for (int g = 0; g < SPA; ++g) {
@@ -820,9 +900,8 @@ cudaError_t launch_expand_wgrad_scales(const WgradTcParams& p, cudaStream_t s) {
   const long long warps = (long long)p.m_tiles128 * p.stages_total + nb;
   const unsigned blocks = (unsigned)((warps + 7) / 8);
   count_launches(1);
-  if (p.mode == MQ_WG_FP8) return launch_pdl(expand_wgrad_scales_kernel<false>, dim3(blocks), dim3(256), 0, s, p);
-  if (p.kind == 2) return launch_pdl(expand_wgrad_scales_nv_kernel, dim3(blocks), dim3(256), 0, s, p);
-  return launch_pdl(expand_wgrad_scales_kernel<true>, dim3(blocks), dim3(256), 0, s, p);
+  auto kernel = p.mode == MQ_WG_FP8 ? expand_wgrad_scales_kernel<false> : p.kind == 2 ? expand_wgrad_scales_nv_kernel : expand_wgrad_scales_kernel<true>;
+  return launch_pdl(kernel, dim3(blocks), dim3(256), 0, s, p);
 }
 
 cudaError_t launch_fp4_to_n_major(const uint8_t* in, uint8_t* out, int P, int N, int Cp, int Npad, cudaStream_t s) {
