@@ -14,11 +14,11 @@
 //                    the input pixel of output pixel q at tap (kh, kw) is q + kh*Wp + kw, so a stage of
 //                    consecutive pixels is ONE contiguous, already swizzled run for each operand (bulk copy).
 //
-// Scales: 8-bit operands, one block per tile - two warps of the block build each stage's scale-vector chunks from the compact
+// Scales: 8-bit operands, one block per tile - four warps of the block build each stage's scale-vector chunks from the compact
 // tile scales (build_stage_scales); pairs of blocks and E2M1 - a small kernel first expands them into per-stage chunks in scratch.
 // One thread block per work item (128 output channels x one tap's block of input channels x a slice of
 // the K range); partial sums go to scratch and are added in a fixed order by bwd_weight_reduce.
-// Warps: 1 MMA issuer, 2 scale copier (E2M1; smem -> TMEM), the others loaders (8-bit, one block per tile: two of them scale builders), 4-7 then epilogue.
+// Warps: 1 MMA issuer, 2 scale copier (E2M1; smem -> TMEM), the others loaders (8-bit, one block per tile: four of them scale builders), 4-7 then epilogue.
 #include <cstdlib>
 #include "mq_conv_tc.cuh"
 #include "mq_tcgen05.cuh"
@@ -27,7 +27,8 @@ namespace mq {
 namespace {
 using namespace tc;
 
-constexpr int WG_THREADS = 320;   // MMA warp, scale copier / loader, eight more loader warps (four of them the epilogue)
+constexpr int WG_THREADS = 384;   // MMA warp, scale copier / loader, ten more loader warps (four of them the epilogue)
+constexpr int BUILDERS = 4;       // warps that build scale chunks (8-bit operands, one block per tile)
 
 // K-block b of stage st: output pixel and 32-sample block
 __device__ __forceinline__ void stage_block(const WgradTcParams& p, int st, int b, int& ho, int& wo, int& nb) {
@@ -233,16 +234,20 @@ __global__ void __launch_bounds__(256) expand_wgrad_scales_nv_kernel(const Wgrad
 // A stage has four K-blocks (32 samples at one output pixel each), a 128-row chunk four 32-row groups: sixteen scale bytes,
 // each lane row repeating the same four words ([row % 32][row / 32] words of four K-blocks).  One warp gathers the bytes of
 // the G_Y chunk (lanes 0-15) and of the one or two X chunks (lanes 16-31; a second byte of lanes 0-15), assembles the words by
-// shuffles and writes the chunks.  The bytes are asked for four of the warp's own stages (two warps take even and odd ones) ahead,
-// so their latency is not in the pipeline.  A separate kernel that expanded every chunk into scratch (512 bytes per padded input
-// pixel) took 38 of 100 us of a 16 -> 32 channel layer at 320x320 (N = 16; now 64), 2-4 us of small layers, and a launch.
+// shuffles and writes the chunks; four warps take every fourth stage each (a stage takes one some 700 clocks; two were the bound of
+// 128-channel layers).  The bytes are asked for two of the warp's own stages ahead, so their latency is not in the pipeline.  A
+// separate kernel that expanded every chunk into scratch (512 bytes per padded input pixel) took 38 of 100 us of a 16 -> 32
+// channel layer at 320x320 (N = 16; now 64), 2-4 us of small layers, and a launch.
 // Pairs of blocks keep that kernel (4.8 of 89 us, 256 channels 28x28): the peer's builder would have to arrive on the leader's
 // barrier with a cluster-scope release of what it wrote, about a microsecond per stage (measured: 178 us).
+// Scale arrays are indexed in 32 bits (a byte stands for 1024 elements).
 __device__ __forceinline__ void build_stage_scales(const WgradTcParams& p, uint8_t* smem, int sf_off, uint64_t* full, uint64_t* empty, volatile int* abort_flag,
-                                                   int lane, int half, int mt, int cb, int kh, int kw, int st_begin, int nst) {
-  constexpr int AHEAD = 4;
+                                                   int lane, int first, int mt, int cb, int kh, int kw, int st_begin, int nst) {
+  // a warp's next stage must lie at most one round of the ring ahead (the barriers' parity tells no more): two warps for short rings
+  const int step = p.stages >= BUILDERS ? BUILDERS : 2;
+  if (first >= step) return;
   const int b = lane & 3, j = (lane >> 2) & 3, px = b / p.BPP, sub = b - px * p.BPP;
-  const bool is_a = lane < 16;
+  const bool is_a = lane < 16, two = p.NB > 1;
   const int cob = mt * 4 + j;
   // X chunk c of this lane's bytes: rows 128 c + 32 j .., input channels of one tap, or (grouped thin mode) tap-in-row major
   int cib[2], tj[2];
@@ -254,62 +259,56 @@ __device__ __forceinline__ void build_stage_scales(const WgradTcParams& p, uint8
     cib[c] = p.grp8 ? (row0 - tj[c] * p.b_rows) / 32 : (cb * p.b_rows + row0) / 32;
     x_ok[c] = c < p.NB && cib[c] < p.Ct && tj[c] < p.TG;
   }
-  int nc, wg, ho;      // of the stage asked for next
-  {
-    const int st = st_begin + half;
-    nc = st % p.nchunks; const int t = st / p.nchunks;
-    wg = t % p.groups_w; ho = t / p.groups_w;
-  }
+  // of the stage asked for next: sample chunk, pixel group, row; and `step` stages in that mixed radix
+  int nc = (st_begin + first) % p.nchunks, wg = (st_begin + first) / p.nchunks, ho = wg / p.groups_w;
+  wg -= ho * p.groups_w;
+  const int d_nc = step % p.nchunks, d_g = step / p.nchunks, d_ho = d_g / p.groups_w, d_wg = d_g - d_ho * p.groups_w;
+  const int dh = kh - p.ph, dw = kw - p.pw + px * p.sw;
   auto ask = [&](uint32_t& v0, uint32_t& v1) {
     const int nb = nc * p.BPP + sub, wo = wg * p.KPX + px;
-    const int h = ho * p.sh + kh - p.ph, w = wo * p.sw + kw - p.pw;
-    auto x_byte = [&](int c) -> uint32_t {
-      const int wc = w + tj[c];
-      if (!(x_ok[c] && nb < p.Nt && h >= 0 && h < p.H && wc >= 0 && wc < p.W)) return 0u;
-      return __ldg(p.x_scales + (((long long)h * p.W + wc) * p.Nt + nb) * p.Ct + cib[c]);
-    };
+    const int h = ho * p.sh + dh, w = wg * p.KPX * p.sw + dw;
+    const bool row_ok = nb < p.Nt && h >= 0 && h < p.H;
+    const int x_row = (h * p.W + w) * p.Nt + nb;
     v0 = v1 = 0u;
     if (is_a) {
-      if (cob < p.Cot && wo < p.Wo && nb < p.Nt) v0 = __ldg(p.g_scales + (((long long)ho * p.Wo + wo) * p.Nt + nb) * p.Cot + cob);
-      v1 = x_byte(1);
-    } else v0 = x_byte(0);
-#pragma unroll
-    for (int r = 0; r < 2; ++r)
-      if (++nc == p.nchunks) { nc = 0; if (++wg == p.groups_w) { wg = 0; ++ho; } }
+      if (cob < p.Cot && wo < p.Wo && nb < p.Nt) v0 = __ldg(p.g_scales + (uint32_t)(((ho * p.Wo + wo) * p.Nt + nb) * p.Cot + cob));
+    } else if (x_ok[0] && row_ok && w + tj[0] >= 0 && w + tj[0] < p.W) v0 = __ldg(p.x_scales + (uint32_t)((x_row + tj[0] * p.Nt) * p.Ct + cib[0]));
+    if (two && x_ok[1] && row_ok && w + tj[1] >= 0 && w + tj[1] < p.W) v1 = __ldg(p.x_scales + (uint32_t)((x_row + tj[1] * p.Nt) * p.Ct + cib[1]));
+    nc += d_nc; wg += d_wg; ho += d_ho;
+    if (nc >= p.nchunks) { nc -= p.nchunks; ++wg; }
+    if (wg >= p.groups_w) { wg -= p.groups_w; ++ho; }
   };
-  const int n_own = (nst - half + 1) >> 1;
-  uint32_t q0[AHEAD], q1[AHEAD];
-#pragma unroll
-  for (int u = 0; u < AHEAD; ++u) { q0[u] = q1[u] = 0u; if (u < n_own) ask(q0[u], q1[u]); }
-  uint32_t s = (uint32_t)half % (uint32_t)p.stages, phase = 0;   // stages >= 2
+  uint32_t q0[2], q1[2];
+  q0[0] = q1[0] = q0[1] = q1[1] = 0u;
+  if (first < nst) ask(q0[0], q1[0]);
+  if (first + step < nst) ask(q0[1], q1[1]);
+  uint32_t s = (uint32_t)first, phase = 0;
+  while (s >= (uint32_t)p.stages) { s -= (uint32_t)p.stages; phase ^= 1; }
 #pragma unroll 1
-  for (int i = 0; i < n_own; i += AHEAD) {
+  for (int i = first; i < nst; i += step) {
+    uint32_t w0 = q0[0] << (8 * b), w1 = q1[0] << (8 * b);
+    q0[0] = q0[1]; q1[0] = q1[1];
+    if (i + 2 * step < nst) ask(q0[1], q1[1]);
+    w0 |= __shfl_xor_sync(0xffffffffu, w0, 1); w0 |= __shfl_xor_sync(0xffffffffu, w0, 2);
+    uint32_t a4[4], b4[4], c4[4];
 #pragma unroll
-    for (int u = 0; u < AHEAD; ++u) {
-      if (i + u < n_own) {
-        uint32_t w0 = q0[u] << (8 * b), w1 = q1[u] << (8 * b);
-        w0 |= __shfl_xor_sync(0xffffffffu, w0, 1); w0 |= __shfl_xor_sync(0xffffffffu, w0, 2);
-        w1 |= __shfl_xor_sync(0xffffffffu, w1, 1); w1 |= __shfl_xor_sync(0xffffffffu, w1, 2);
-        uint32_t a4[4], b4[4], c4[4];
+    for (int k = 0; k < 4; ++k) { a4[k] = __shfl_sync(0xffffffffu, w0, 4 * k); b4[k] = __shfl_sync(0xffffffffu, w0, 16 + 4 * k); c4[k] = 0u; }
+    if (two) {
+      w1 |= __shfl_xor_sync(0xffffffffu, w1, 1); w1 |= __shfl_xor_sync(0xffffffffu, w1, 2);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          a4[k] = __shfl_sync(0xffffffffu, w0, 4 * k);
-          b4[k] = __shfl_sync(0xffffffffu, w0, 16 + 4 * k);
-          c4[k] = __shfl_sync(0xffffffffu, w1, 4 * k);
-        }
-        if (i + u + AHEAD < n_own) ask(q0[u], q1[u]);
-        if (*abort_flag) return;
-        if (!mbar_wait(&empty[s], phase ^ 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; return; }
-        uint8_t* dst = smem + (size_t)s * p.stage_bytes + sf_off + lane * 16;
-        *reinterpret_cast<uint4*>(dst) = make_uint4(a4[0], a4[1], a4[2], a4[3]);
-        *reinterpret_cast<uint4*>(dst + 1024) = make_uint4(b4[0], b4[1], b4[2], b4[3]);
-        if (p.NB > 1) *reinterpret_cast<uint4*>(dst + 1536) = make_uint4(c4[0], c4[1], c4[2], c4[3]);
-        fence_proxy_async_smem();      // the scale copies read these through the async proxy
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&full[s]);
-        s += 2; if (s >= (uint32_t)p.stages) { s -= (uint32_t)p.stages; phase ^= 1; }
-      }
+      for (int k = 0; k < 4; ++k) c4[k] = __shfl_sync(0xffffffffu, w1, 4 * k);
     }
+    if (*abort_flag) return;
+    if (!mbar_wait(&empty[s], phase ^ 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; return; }
+    uint8_t* dst = smem + (size_t)s * p.stage_bytes + sf_off + lane * 16;
+    *reinterpret_cast<uint4*>(dst) = make_uint4(a4[0], a4[1], a4[2], a4[3]);
+    *reinterpret_cast<uint4*>(dst + 1024) = make_uint4(b4[0], b4[1], b4[2], b4[3]);
+    if (two) *reinterpret_cast<uint4*>(dst + 1536) = make_uint4(c4[0], c4[1], c4[2], c4[3]);
+    fence_proxy_async_smem();      // the scale copies read these through the async proxy
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&full[s]);
+    s += (uint32_t)step;
+    while (s >= (uint32_t)p.stages) { s -= (uint32_t)p.stages; phase ^= 1; }
   }
 }
 
@@ -398,12 +397,13 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   const int nkinds = has_b1 ? 4 : 3;
   const int lslot = FP4 ? (warp == 0 ? 0 : (warp >= 3 ? warp - 2 : -1))          // E2M1: warp 2 is the scale copier
                         : (warp == 0 ? 0 : (warp == 2 ? 1 : (warp >= 3 ? warp - 1 : -1)));
-  if (lslot >= 0 && lslot < 2 * nkinds) {
+  const bool builds = !FP4 && !CTA2;                    // the last kind is not copied but built, by BUILDERS warps
+  if (builds && lslot >= 2 * nkinds - 2 && lslot < 2 * nkinds - 2 + BUILDERS) {
+    build_stage_scales(p, smem, sf_off, full, empty, abort_flag, lane, lslot - (2 * nkinds - 2), mt, cb, kh, kw, st_begin, nst);
+  } else if (lslot >= 0 && lslot < 2 * nkinds - (builds ? 2 : 0)) {
     const int kidx = lslot >> 1, half = lslot & 1;
     const int kind = kidx == 0 ? 0 : (kidx == 1 ? 1 : ((kidx == 2 && has_b1) ? 2 : 3));   // 0 G_Y, 1 X, 2 second X panel, 3 scales
     const int taps = p.Kh * p.Kw;
-    if (!FP4 && !CTA2 && kind == 3) build_stage_scales(p, smem, sf_off, full, empty, abort_flag, lane, half, mt, cb, kh, kw, st_begin, nst);
-    else {
     const uint8_t* sfa_src = p.sfa_img + ((size_t)mt * p.stages_total + st_begin) * (512 * SPA);
     const uint32_t sfb_bytes = (uint32_t)p.NB * 512 * SPA;
     // X-side scale chunks: per (tap group, stage), NB chunks each; or (sfb_S) per padded start pixel - the NB taps of the
@@ -475,7 +475,6 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
 #pragma unroll
       for (int r = 0; r < 2; ++r)
         if (++nc == p.nchunks) { nc = 0; if (++wg == p.groups_w) { wg = 0; ++ho; } }
-    }
     }
   }
   __syncwarp();
