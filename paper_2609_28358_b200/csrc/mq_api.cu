@@ -105,29 +105,73 @@ size_t wt_codes_bytes(const Geom& g, int fmt_w) {
 }
 size_t up256(size_t v) { return (v + 255) / 256 * 256; }
 
-// Output columns per tile.  Rows of a tile are TW consecutive output columns x TN = 128/TW samples with the
-// column index fastest.  An NCHW store writes runs of TW floats and the store path is bound by the NUMBER of
-// runs (about 2.2 cycles each per SM, measured), so the choice weighs the tile's MMA time against its store time
-// and both against the padding the tile shape wastes at the edges.
-//   k_bytes: bytes of K per tile row (taps x channel bytes); bn: output channels per tile.
-//   serial: the tile's store is not overlapped with the next tile's MMAs (a single 256-column accumulator).
-//   pair: the tiles of the even and the odd output columns are stored together (stride-2 input gradient): runs of
-//   2 tw floats, and the two accumulators belong to one pair, so the store is not overlapped either.
-int choose_tw(int w_eff, int N, int layout, double k_bytes, int bn, bool thin, bool serial, bool pair) {
-  const int forced = MQ_ENV("MQ_TC_TW", 0);
-  if (forced > 0) return forced;
-  if (thin) return 8;   // the whole-tile kernel (8-column tiles): its per-tile loads beat any per-tap shape on thin layers
+// Shape of the per-tap kernel's tiles with direct NCHW stores: TW output columns x TN samples, column index fastest.  Three things
+// weigh: rows of the 128 that are no positions (TW beyond the image's edge, TW * TN below 128, the batch's last samples)
+// cost what a full one costs; a store instruction's 32 lanes are runs of columns, and a run that ends inside a 32-byte sector
+// leaves a sector that two instructions write in part - twice the requests, and, where the output does not fit L2, a sector
+// read back from memory; a run below a sector costs a sector.  So: whole rows where they fit (any width, not a power of two), a
+// power of two above the width where that loses nothing (no run is then cut between two warps), splits at multiples of a
+// sector, other splits last.  Measured (N = 256 unless said, us): 512 channels 14x14 E4M3, widths 14 / 16 / 8 / 7: 111 / 119 / 130 /
+// 130; 256 channels 28x28 E2M1, 32 / 28 / 16 / 14: 85 / 89 / 117 / 160; 128 channels 42x42 N = 128, 42 / 32 / 16 / 14: 54 / 86 / 59 / 60;
+// 128 -> 256 channels 19x19 N = 64, 19 / 32 / 16 / 8: 20 / 26 / 27 / 24; 128 channels 56x56 E2M1, 8 / 56 / 32 / 14: 98 / 181 / 193 / 399;
+// stride-2 input gradient 256 channels 28x28 E4M3 (205 MB of output), 16 / 14: 86 / 100; 128 channels (103 MB): 43 / 41.
+struct TileRows { int tw, tn; };
+TileRows choose_rows(int w_eff, int N, int Wd, int max_tw, bool pair, bool big_output) {
+  TileRows best{1, 128};
+  double best_score = -1.0;
+  auto consider = [&](int tw, int k) {
+    if (tw < 1 || tw > max_tw) return;
+    const bool pow2 = (tw & (tw - 1)) == 0;
+    int tn = 128 / tw;
+    if (!pow2 && tn > N) tn = N;
+    const double tiles = (double)((w_eff + tw - 1) / tw) * ((N + tn - 1) / tn);
+    double score = (double)w_eff * N / (tiles * 128.0);
+    const int run = pair ? 2 * tw : tw;
+    if (tw >= w_eff) { if (!pow2) score *= big_output ? 0.87 : 0.99; }
+    else if (Wd % 8 != 0 || run % 8 != 0) score *= (big_output ? 0.6 : 0.86 - 0.01 * k) * (run < 8 ? run / 8.0 : 1.0);
+    if (score > best_score * (1.0 + 1e-9)) { best_score = score; best = TileRows{tw, tn}; }
+  };
+  int up = 8;
+  while (up < w_eff) up *= 2;
+  for (int tw = up > 128 ? 128 : up; tw >= 8; tw /= 2) consider(tw, (w_eff + tw - 1) / tw);
+  for (int k = 1; k <= 4; ++k) consider((w_eff + k - 1) / k, k);
+  return best;
+}
+// The same for staged TMA stores and for [H][W][N][C] output, whose tiles are powers of two: the tile's MMA time (107 clocks per 32
+// bytes of K and 128 columns) against its store time (about 2.2 clocks per run of TW floats, [H][W][N][C]: per line), both against
+// the padding at the edges.  serial: the store is not overlapped with the next tile's MMAs (a single 256-column accumulator).
+TileRows choose_rows_pow2(int w_eff, int N, int layout, double k_bytes, int bn, bool serial, int max_tw) {
   const double t_mma = k_bytes / 32.0 * 107.0 * (bn / 128.0 < 0.5 ? 0.5 : bn / 128.0);
-  int best = 1;
+  TileRows best{1, 128};
   double best_cost = 1e30;
-  for (int tw = 1; tw <= 32; tw *= 2) {
+  for (int tw = 1; tw <= 32 && tw <= max_tw; tw *= 2) {
     const int tn = 128 / tw;
     const double waste = (double)((w_eff + tw - 1) / tw * tw) / w_eff * (double)((N + tn - 1) / tn * tn) / N;
-    double t_store = 128.0 * (bn * 4.0 / 128.0) * 2.2;          // [H][W][N][C] output: whole lines
-    const int run = pair ? 2 * tw : tw;
-    if (layout == MQ_NCHW) t_store = 128.0 * bn / run * 2.2 * (run < 8 ? 8.0 / run : 1.0);   // runs below a 32-byte sector cost a sector each
-    double cost = waste * ((serial || pair) ? t_mma + t_store : (t_mma > t_store ? t_mma : t_store));
-    if (cost < best_cost * (1.0 - 1e-9)) { best_cost = cost; best = tw; }
+    double t_store = 128.0 * (bn * 4.0 / 128.0) * 2.2;
+    if (layout == MQ_NCHW) t_store = 128.0 * bn / tw * 2.2 * (tw < 8 ? 8.0 / tw : 1.0);   // runs below a 32-byte sector cost a sector each
+    const double cost = waste * (serial ? t_mma + t_store : (t_mma > t_store ? t_mma : t_store));
+    if (cost < best_cost * (1.0 - 1e-9)) { best_cost = cost; best = TileRows{tw, tn}; }
+  }
+  return best;
+}
+// Output channels per tile.  `rule` is the choice for layers that fill the chip; channel counts between its multiples (160, 208, 320
+// ...) are covered by fewer or narrower tiles that waste fewer columns, and a layer whose tiles leave SMs idle by more of them, where
+// the rounds over the chip's SMs, times a stage's clocks - about 107 per 32 bytes of K and 128 columns, 350 and a little per
+// column however narrow (the loaders' and the issuing warp's own instructions) - say so clearly.  Measured: 96 -> 208 channels 28x28 5x5, N = 99, one
+// tile of 208 against two of 128: E4M3 105 -> 85 us, E2M1 132 -> 103; 512 channels 7x7, N = 16, 64 against 256: 23.1 -> 18.8 us;
+// 320 -> 256 channels 12x12 stride 2, N = 15: 21.8 -> 13.9 us.
+int choose_columns(int Cd, int rule, int unit, int most, long long row_tiles, double stages, int sms) {
+  auto cost = [&](int bn) {
+    const long long tiles = row_tiles * ((Cd + bn - 1) / bn);
+    return (double)((tiles + sms - 1) / sms) * (stages * (bn < 165 ? 350.0 + 1.2 * bn : 428.0 * bn / 128.0) + 400.0);
+  };
+  int best = rule;
+  double best_cost = 0.9 * cost(rule);
+  for (int c = 1; c <= (Cd + unit - 1) / unit && c <= 16; ++c) {
+    int bn = ((Cd + c - 1) / c + unit - 1) / unit * unit;
+    if (bn > most) continue;
+    const double u = cost(bn);
+    if (u < best_cost * (1.0 - 1e-9)) { best_cost = u; best = bn; }
   }
   return best;
 }
@@ -176,7 +220,13 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
   p.last_atoms = atoms - (p.cpt - 1) * (p.KB / 32);
   const int w_eff = op == MQ_OP_FWD ? g.Wo : (g.W + g.sw - 1) / g.sw;
   // line blocks (one scale per row): the per-tap kernel, whose preparation launch lays out the scale vectors row by row
-  const bool thin = !line && !mx && !ts16 && g.sh == 1 && g.sw == 1 && p.cpt == 1 && p.KB <= 64 && !MQ_ENV("MQ_TC_NO_HALO", 0);
+  // ... and the whole-tile kernel's 8-column tiles only where they fit: with 25 taps of 64 bytes its resident weights leave two
+  // stages (E2M1 128 channels 28x28 5x5, N = 99: 51 us against 42 per tap), and NCHW rows that 8 columns cut inside a sector cost
+  // twice where the output does not fit L2 (E2M1 128 channels 42x42, N = 128: 80 against 54; 64 -> 448 channels 60x60: 682 against
+  // 264; below that size it wins: N = 64 27 against 32)
+  const bool big_output = (double)g.N * p.Cd * p.Hd * p.Wd * 4.0 > 110e6;
+  const bool thin = !line && !mx && !ts16 && g.sh == 1 && g.sw == 1 && p.cpt == 1 && p.KB <= 64 && !(p.KB == 64 && taps > 9) &&
+                    !(layout == MQ_NCHW && p.Wd % 8 != 0 && big_output) && !MQ_ENV("MQ_TC_NO_HALO", 0);
   p.line = line ? 1 : 0;
   const int cd16 = mx ? (p.Cd + 31) / 32 * 32 : (p.Cd + 15) / 16 * 16;
   p.BN = cd16 <= 128 ? cd16 : 128;
@@ -194,15 +244,20 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
   // 56x56 -10 %)
   const double act_bytes = (double)p.Hs * p.Ws * g.N * rowbytes;
   if (fp4 && p.Cd >= 256 && (double)taps * rowbytes >= 1024.0 && (op == MQ_OP_FWD || (g.sh == 1 && g.sw == 1)) && !MQ_ENV("MQ_TC_FP4_BN128", 0)) p.BN = 256;
+  const int forced_bn = MQ_ENV("MQ_TC_BN", 0);
+  if (forced_bn >= 32 && forced_bn <= 256 && forced_bn % 32 == 0) p.BN = forced_bn < cd16 ? forced_bn : cd16;
+  // staged TMA stores are wanted (see p.tma_store below; there the tile's width has the last word)
+  const bool strided_out = op == MQ_OP_BWD_DATA && (g.sh != 1 || g.sw != 1);
+  const bool s2_tma_ok = strided_out && layout == MQ_HWNC && g.sw <= 8 && !MQ_ENV("MQ_TC_NO_S2_TMA", 0);
+  const bool want_tma = !mx && (!strided_out || s2_tma_ok) && (layout == MQ_NCHW ? p.Wd % 4 == 0 : p.Cd % 4 == 0 && p.BN % 64 == 0) &&
+                        (MQ_ENV("MQ_TC_TMA_STORE", 0) || ((taps == 1 || layout == MQ_HWNC || strided_out) && !MQ_ENV("MQ_TC_NO_TMA_STORE", 0)));
   {
-    const int forced_bn_ = MQ_ENV("MQ_TC_BN", 0);
-    const int bn_ = (forced_bn_ >= 32 && forced_bn_ <= 256 && forced_bn_ % 32 == 0) ? (forced_bn_ < cd16 ? forced_bn_ : cd16) : p.BN;
-    const int nkh_ = op == MQ_OP_FWD ? g.Kh : (g.Kh + g.sh - 1) / g.sh, nkw_ = op == MQ_OP_FWD ? g.Kw : (g.Kw + g.sw - 1) / g.sw;
-    // with a single accumulator the store time adds to the tile's time instead of hiding behind the next tile: wider
-    // tiles (longer store runs) then win - as long as the activations stay in L2 (measured: 28x28 -11 %, 56x56 +11 %)
-    const bool serial = bn_ > 128 && act_bytes <= 110e6;
-    const bool pair_hint = !mx && op == MQ_OP_BWD_DATA && g.sw == 2 && layout == MQ_NCHW && p.Wd % 2 == 0 && bn_ <= 128 && !MQ_ENV("MQ_TC_NO_PAIR", 0);
-    p.TW = choose_tw(w_eff, g.N, layout, (double)nkh_ * nkw_ * rowbytes, bn_ < 128 ? bn_ : (serial ? bn_ : 128), thin, serial, pair_hint);
+    const int forced_tw = MQ_ENV("MQ_TC_TW", 0);
+    const bool pair_hint = !mx && op == MQ_OP_BWD_DATA && g.sw == 2 && layout == MQ_NCHW && p.Wd % 2 == 0 && !MQ_ENV("MQ_TC_NO_PAIR", 0);
+    const int wst = op == MQ_OP_FWD ? g.sw : 1;
+    int max_tw = 128;
+    while ((max_tw - 1) * wst + 1 > 256) --max_tw;    // columns of a copy's box
+    TileRows t{1, 128};
     if (mx) {   // a sample tile (32 samples) must lie inside a GEMM tile: 1, 2 or 4 columns; the least edge padding wins, then the
                 // narrowest: with one column a warp's 32 rows ARE a sample tile, and the epilogue needs no exchange between warps
                 // (measured, N = 256, 4 -> 1 columns: 1x1 512 channels 56x56 417 -> 368 us, 3x3 stride 2 input gradient 267 -> 234 us)
@@ -210,25 +265,37 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
       for (int tw = 1; tw <= (ts16 ? 2 : 4); tw <<= 1) {   // emitting 16-sample blocks: a warp's rows must hold whole blocks (1 or 2 columns)
         const int tn = 128 / tw;
         const double waste = (double)((w_eff + tw - 1) / tw * tw) / w_eff * (double)((g.N + tn - 1) / tn * tn) / g.N;
-        if (waste < best * (1.0 - 1e-9)) { best = waste; p.TW = tw; }
+        if (waste < best * (1.0 - 1e-9)) { best = waste; t = TileRows{tw, tn}; }
       }
       const int ftw = MQ_ENV("MQ_TC_MX_TW", 0);
-      if (ftw == 1 || ftw == 2 || (ftw == 4 && !ts16)) p.TW = ftw;
+      if (ftw == 1 || ftw == 2 || (ftw == 4 && !ts16)) t = TileRows{ftw, 128 / ftw};
+    } else if (forced_tw > 0) t = TileRows{forced_tw, 128 / forced_tw};
+    else if (thin) t = TileRows{8, 16};   // the whole-tile kernel (8-column tiles): its per-tile loads beat any per-tap shape on thin layers
+    else if (want_tma || layout != MQ_NCHW) {
+      const int nkh = op == MQ_OP_FWD ? g.Kh : (g.Kh + g.sh - 1) / g.sh, nkw = op == MQ_OP_FWD ? g.Kw : (g.Kw + g.sw - 1) / g.sw;
+      const bool serial = p.BN > 128 && act_bytes <= 110e6;
+      t = choose_rows_pow2(w_eff, g.N, layout, (double)nkh * nkw * rowbytes, serial || p.BN < 128 ? p.BN : 128, serial, max_tw);
+    }
+    else t = choose_rows(w_eff, g.N, p.Wd, max_tw, pair_hint, big_output);
+    p.TW = t.tw; p.TN = t.tn;
+    if (!thin && !(forced_bn >= 32 && forced_bn <= 256 && forced_bn % 32 == 0)) {
+      const long long row_tiles = (long long)((w_eff + t.tw - 1) / t.tw) * ((g.N + t.tn - 1) / t.tn) * p.tiles_h * p.classes;
+      p.BN = choose_columns(p.Cd, p.BN, want_tma && layout == MQ_HWNC ? 64 : 32,
+                            pair_hint || want_tma ? 128 : 256, row_tiles,
+                            ((double)taps / p.classes * p.cpt + p.G - 1) / p.G, sm_count());
     }
   }
-  if (p.TW < 1 || p.TW > 32 || (p.TW & (p.TW - 1))) return false;
-  p.TN = 128 / p.TW;
+  if (p.TW < 1 || p.TW > 128 || p.TN < 1) return false;
+  const bool pow2_tw = p.TW <= 32 && (p.TW & (p.TW - 1)) == 0 && p.TW * p.TN == 128;
+  p.m_TW = (uint32_t)((65536 + p.TW - 1) / p.TW);
   p.lgTW = 0;
   while ((1 << p.lgTW) < p.TW) ++p.lgTW;
-  const int forced_bn = MQ_ENV("MQ_TC_BN", 0);
-  if (forced_bn >= 32 && forced_bn <= 256 && forced_bn % 32 == 0) p.BN = forced_bn < cd16 ? forced_bn : cd16;
   if (mx && (p.BN % 32 != 0 || p.TW > (ts16 ? 2 : 4))) return false;
   p.tiles_c = (p.Cd + p.BN - 1) / p.BN;
   p.tiles_w = (w_eff + p.TW - 1) / p.TW;
   p.tiles_n = (g.N + p.TN - 1) / p.TN;
   p.total_tiles = (long long)p.tiles_c * p.tiles_w * p.tiles_n * p.tiles_h * p.classes;
   if (p.total_tiles > 0x7fffffffLL) return false;
-  p.lgTN = 7 - p.lgTW;
   {
     // multiply-high reciprocals for the per-tile index arithmetic: exact while numerator * divisor < 2^32
     bool exact = true;
@@ -248,9 +315,7 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
   // Strided input gradient, channel-fastest output: the staged epilogue writes a parity class through a tensor map that steps sw
   // pixels along W.  Not for NCHW: there W is the innermost axis and a class's first column (x = 1 for the odd one) would be
   // a TMA coordinate that is not on a 16-byte boundary, which the hardware refuses; NCHW keeps the paired direct stores.
-  const bool strided_out = op == MQ_OP_BWD_DATA && (g.sh != 1 || g.sw != 1);
-  const bool s2_tma_ok = strided_out && layout == MQ_HWNC && g.sw <= 8 && !MQ_ENV("MQ_TC_NO_S2_TMA", 0);
-  const bool tma_store_ok = (!strided_out || s2_tma_ok) && p.TW <= 32 &&
+  const bool tma_store_ok = (!strided_out || s2_tma_ok) && pow2_tw &&
                             (layout == MQ_NCHW ? (p.TW >= 4 && p.Wd % 4 == 0) : (p.Cd % 4 == 0 && p.BN % 64 == 0));
   // ... and for 1x1 layers, whose main loop is a handful of stages: the tile's time is its store (measured 4-12 % faster, 28x28 and
   // 56x56 images, 256 and 512 channels)
@@ -277,7 +342,7 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
   // one 256-column accumulator: the epilogue copies it into registers and frees it before storing (with the staged TMA
   // stores only when a tile has at least MQ_TC_SNAP_MIN_STAGES pipeline stages of MMAs to overlap: E2M1 1x1 512 channels, two
   // stages per tile, measured 384-407 us without and 517-601 us with it; E4M3, four stages, 562-567 against 521 us)
-  p.snap = (!mx && ((p.BN == 256 && p.n_acc == 1 && !p.pair) || (p.pair && p.BN == 128)) && !MQ_ENV("MQ_TC_NO_SNAP", 0) &&
+  p.snap = (!mx && ((p.BN > 128 && p.n_acc == 1 && !p.pair) || (p.pair && p.BN == 128)) && !MQ_ENV("MQ_TC_NO_SNAP", 0) &&
             (!p.tma_store || p.max_stages >= MQ_ENV("MQ_TC_SNAP_MIN_STAGES", 4))) ? 1 : 0;
   const uint32_t fa = fp4 ? 1u : fmt_mma_code(fmt_x_like);   // kind::mxf4: 1 = E2M1; kind::mxf8f6f4: E4M3 0, E5M2 1, E2M3 3, E3M2 4
   const uint32_t fb = fp4 ? 1u : fmt_mma_code(fmt_w);
@@ -296,9 +361,9 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
   // whole-tile-per-stage variant: stride 1, one chunk per tap (<= 64 bytes of channels).  One box with the column
   // halo needs 8-column tiles; one box per column shift takes 8, 16 or 32 columns (longer NCHW store runs).
   p.halo = 0;
-  if (!line && !mx && !ts16 && g.sh == 1 && g.sw == 1 && p.cpt == 1 && p.KB <= 64 && taps <= 64 && !MQ_ENV("MQ_TC_NO_HALO", 0)) {
+  if (thin && taps <= 64) {
     const int spa = fp4 ? 2 : 1, atoms_b = (p.BN + 127) / 128;
-    if (p.TW == 8) {
+    if (p.TW == 8 && p.TN == 16) {
       p.WH = p.TW + g.Kw - 1;
       p.halo_box_bytes = g.Kh * p.WH * p.TN * p.KB;
       p.halo_a_bytes = (p.halo_box_bytes + 1023) / 1024 * 1024;

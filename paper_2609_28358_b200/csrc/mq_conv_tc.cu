@@ -49,7 +49,13 @@ constexpr int SFA_BYTES_NV = 2048, SFB_BYTES_NV = 4096, SF_COLS_NV = 48;
 __host__ __device__ constexpr int spa_of_kind(int kind) { return kind == 2 ? 4 : (kind == 1 ? 2 : 1); }
 
 
-struct Tile { int c0, w0, n0, h, cls, ct; };
+struct Tile { int c0, w0, n0, h, cls, ct, wt, nt; };   // first channel, column, sample; row; stride class; tile indices along c, w, n
+// Row r of a tile: column tw, sample tn (TW need not divide 128: the last rows may belong to no position - tn is then beyond any batch)
+__device__ __forceinline__ void tile_row(const ConvTcParams& p, int r, int& tw, int& tn) {
+  tn = (int)(((uint32_t)r * p.m_TW) >> 16);
+  tw = r - tn * p.TW;
+  if (tn >= p.TN) tn = 1 << 28;
+}
 
 // Tile order: stride class fastest (the classes of an input gradient interleave inside the same 32-byte
 // sectors), then output column tile, output row, channel tile, sample tile.  Tiles that run at the same time
@@ -63,10 +69,10 @@ __device__ __forceinline__ Tile decode_tile(const ConvTcParams& p, unsigned t) {
   Tile q;
   unsigned u = fdiv(t, p.classes, p.m_classes);
   q.cls = (int)(t - u * p.classes); t = u;
-  u = fdiv(t, p.tiles_w, p.m_tiles_w); q.w0 = (int)(t - u * p.tiles_w) * p.TW; t = u;
+  u = fdiv(t, p.tiles_w, p.m_tiles_w); q.wt = (int)(t - u * p.tiles_w); q.w0 = q.wt * p.TW; t = u;
   u = fdiv(t, p.tiles_h, p.m_tiles_h); q.h = (int)(t - u * p.tiles_h); t = u;
   u = fdiv(t, p.tiles_c, p.m_tiles_c); q.ct = (int)(t - u * p.tiles_c); q.c0 = q.ct * p.BN;
-  q.n0 = (int)u * p.TN;
+  q.nt = (int)u; q.n0 = q.nt * p.TN;
   return q;
 }
 // number of A-side scale chunks of a launch
@@ -77,15 +83,15 @@ __host__ __device__ __forceinline__ unsigned conv_tc_sfa_chunks(const ConvTcPara
 }
 // index of a tile among the tiles that differ in anything but the channel tile (A-side scale chunks)
 __device__ __forceinline__ unsigned tile_m_index(const ConvTcParams& p, const Tile& q) {
-  return (((unsigned)(q.n0 >> p.lgTN) * p.tiles_h + q.h) * p.tiles_w + (q.w0 >> p.lgTW)) * p.classes + q.cls;
+  return (((unsigned)q.nt * p.tiles_h + q.h) * p.tiles_w + q.wt) * p.classes + q.cls;
 }
 __device__ __forceinline__ Tile tile_of_m_index(const ConvTcParams& p, unsigned tm) {
   Tile q;
   unsigned u = fdiv(tm, p.classes, p.m_classes);
   q.cls = (int)(tm - u * p.classes); tm = u;
-  u = fdiv(tm, p.tiles_w, p.m_tiles_w); q.w0 = (int)(tm - u * p.tiles_w) * p.TW; tm = u;
+  u = fdiv(tm, p.tiles_w, p.m_tiles_w); q.wt = (int)(tm - u * p.tiles_w); q.w0 = q.wt * p.TW; tm = u;
   u = fdiv(tm, p.tiles_h, p.m_tiles_h); q.h = (int)(tm - u * p.tiles_h);
-  q.n0 = (int)u * p.TN; q.c0 = 0; q.ct = 0;
+  q.nt = (int)u; q.n0 = q.nt * p.TN; q.c0 = 0; q.ct = 0;
   return q;
 }
 
@@ -164,7 +170,8 @@ __device__ __forceinline__ void epilogue_role(const ConvTcParams& p, uint32_t tm
     const int quad = warp & 3;           // TMEM lane quadrant this warp may read
     const int half = (warp - 4) >> 2;    // warps 4-7 take the first half of the tile's columns, 8-11 the second
     const int r = 32 * quad + lane;
-    const int tw_ = r & (p.TW - 1), tn = r >> p.lgTW;
+    int tw_, tn;
+    tile_row(p, r, tw_, tn);
     const int cbeg = half == 0 ? 0 : ((p.BN / 2 + 15) & ~15);
     const int cend = half == 0 ? ((p.BN / 2 + 15) & ~15) : p.BN;
     const long long cs = (long long)p.Hd * p.Wd;
@@ -231,8 +238,8 @@ __device__ __forceinline__ void epilogue_role(const ConvTcParams& p, uint32_t tm
     }
 }
 
-// Epilogue role for 256-column tiles (ONE accumulator: the MMA lane cannot start the next tile before this one has left
-// tensor memory).  Each of the eight warps copies its 32 rows x 128 columns into REGISTERS, hands the accumulator back at
+// Epilogue role for tiles of more than 128 columns with ONE accumulator (where two do not fit, the MMA lane cannot start the next
+// tile before this one has left tensor memory).  Each of the eight warps copies its 32 rows x 128 columns into REGISTERS, hands the accumulator back at
 // once and only then stores - so the stores of a tile (request-bound: 128 KB through 4-byte rows) overlap the next tile's
 // MMAs instead of holding them up.  The registers come from the loader / MMA warpgroups (warpgroup_regs_inc / _dec).
 template <int MODE>
@@ -241,7 +248,8 @@ __device__ __forceinline__ void epilogue_snap_role(const ConvTcParams& p, uint32
     const int quad = warp & 3;
     const int half = (warp - 4) >> 2;
     const int r = 32 * quad + lane;
-    const int tw_ = r & (p.TW - 1), tn = r >> p.lgTW;
+    int tw_, tn;
+    tile_row(p, r, tw_, tn);
     const int cbeg = 128 * half;
     const long long cs = (long long)p.Hd * p.Wd;
     const float os = out_scale_of(p);
@@ -278,7 +286,7 @@ __device__ __forceinline__ void epilogue_snap_role(const ConvTcParams& p, uint32
       }
       const int n = tile.n0 + tn;
       if (!(yo < p.Hd && xo < p.Wd && n < p.N)) continue;
-      const int ncols = min(128, p.Cd - tile.c0 - cbeg);     // columns of this half inside the tensor (may be <= 0)
+      const int ncols = min(min(128, p.BN - cbeg), p.Cd - tile.c0 - cbeg);     // columns of this half inside the tile and the tensor (may be <= 0)
       if (p.kind_fp4 == 2) {
 #pragma unroll
         for (int j = 0; j < 128; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) * os);
@@ -310,7 +318,8 @@ __device__ __forceinline__ void epilogue_pair_role(const ConvTcParams& p, uint32
     const int quad = warp & 3;
     const int half = (warp - 4) >> 2;
     const int r = 32 * quad + lane;
-    const int tw_ = r & (p.TW - 1), tn = r >> p.lgTW;
+    int tw_, tn;
+    tile_row(p, r, tw_, tn);
     const int cbeg = half == 0 ? 0 : ((p.BN / 2 + 15) & ~15);
     const int cend = half == 0 ? ((p.BN / 2 + 15) & ~15) : p.BN;
     const long long cs = (long long)p.Hd * p.Wd;
@@ -371,7 +380,8 @@ __device__ __forceinline__ void epilogue_pair_snap_role(const ConvTcParams& p, u
     const int quad = warp & 3;
     const int half = (warp - 4) >> 2;
     const int r = 32 * quad + lane;
-    const int tw_ = r & (p.TW - 1), tn = r >> p.lgTW;
+    int tw_, tn;
+    tile_row(p, r, tw_, tn);
     const int cbeg = 64 * half;
     const long long cs = (long long)p.Hd * p.Wd;
     const float os = out_scale_of(p);
@@ -618,7 +628,8 @@ __device__ __forceinline__ void epilogue_mx_role(const ConvTcParams& p, unsigned
     const int quad = warp & 3;
     const int half = warp < 12 ? (warp - 4) >> 2 : 2 + ((warp - 16) >> 2);   // column group 0..3 of this warp (four warps each, one per lane quadrant)
     const int r = 32 * quad + lane;
-    const int tw_ = r & (p.TW - 1), tn = r >> p.lgTW;
+    int tw_, tn;
+    tile_row(p, r, tw_, tn);
     const int nblk = p.BN >> 5;                         // 32-channel blocks of a tile
     constexpr int NG = FMT == 5 ? 4 : 2;                // column groups: 16 epilogue warps for the paper's format, else 8
     const int per = (nblk + NG - 1) / NG;
@@ -968,9 +979,9 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     if (EPI >= 0) epilogue_mx_role<MODE, EPI < 0 ? 0 : EPI>(p, mx_red, tmem, tfull, tempty, abort_flag, warp, lane, total);
     else if (p.pair && p.BN == 128 && p.snap) epilogue_pair_snap_role<MODE>(p, tmem, tfull, tempty, abort_flag, warp, lane, total);
     else if (p.pair) epilogue_pair_role<MODE>(p, tmem, tfull, tempty, abort_flag, warp, lane, total);
-    else if (p.tma_store && p.BN == 256 && p.snap) epilogue_tma_snap_role<MODE>(p, &map_out, staging, tmem, tfull, tempty, abort_flag, warp, lane, total, DUO && rank != 0);
+    else if (p.tma_store && p.snap) epilogue_tma_snap_role<MODE>(p, &map_out, staging, tmem, tfull, tempty, abort_flag, warp, lane, total, DUO && rank != 0);
     else if (p.tma_store) epilogue_tma_role<MODE>(p, &map_out, staging, tmem, tfull, tempty, abort_flag, warp, lane, total);
-    else if (p.BN == 256 && p.snap) epilogue_snap_role<MODE>(p, tmem, tfull, tempty, abort_flag, warp, lane, total, DUO && rank != 0);
+    else if (p.snap) epilogue_snap_role<MODE>(p, tmem, tfull, tempty, abort_flag, warp, lane, total, DUO && rank != 0);
     else epilogue_role<MODE>(p, tmem, tfull, tempty, abort_flag, warp, lane, total);
   } else {
   if (EPI < 0) warpgroup_regs_dec<OTHER_REGS>();
@@ -979,41 +990,52 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     // A warp gets one bulk copy accepted per ~170 cycles whatever its size, and the loop around it is a chain of
     // dependent instructions, so a stage's copies are spread over warps: one KIND of copy (activation boxes, weight
     // boxes, the two scale chunks) per pair of warps, which take even and odd stages.  Every warp walks all stages
-    // (the walk is a few additions) but waits and issues only for its own; each kind arrives once per stage on the
-    // stage's barrier with its own byte count.
+    // but computes, waits and issues only for its own; what changes from stage to stage is kept running (a column, a row, a
+    // tap, a pointer) and moved by additions.  Each kind arrives once per stage on the stage's barrier with its own byte count.
     {
-      uint32_t s = 0, phase = 0, gi = 0;
-      const uint32_t row_bytes = lkind == 1 ? (uint32_t)(DUO ? p.BN / 2 : p.BN) * KB : (p.a_tx34 ? 96u * KB : 128u * KB);
+      uint32_t s = 0, phase = 0;
+      bool mine = lhalf == 0;
+      const uint32_t row_bytes = lkind == 1 ? (uint32_t)(DUO ? p.BN / 2 : p.BN) * KB : (uint32_t)(p.TW * p.TN) * (p.a_tx34 ? KB / 4u * 3u : (uint32_t)KB);
+      constexpr int SFA_STEP = 512 * SPA;
+      const int sfb_step = SFA_STEP * atoms_b;
       for (unsigned i = 0, t; (t = tile_of_iter(p, i)) < total && !*abort_flag; ++i) {
         const Tile tile = decode_tile(p, t);
         TapWalk<MODE> tw;
         tw.init(p, tile);
         const int Q = tw.chunks(p);
-        ChunkPos pos;
-        pos.reset();
-        const uint8_t* sfa_src = p.sfa_img + (size_t)tile_m_index(p, tile) * p.max_stages * (512 * SPA);
-        const uint8_t* sfb_src = p.sfb_img + ((size_t)tile.cls * p.tiles_c + tile.ct) * p.max_stages * (512 * SPA * atoms_b);
-        // shared A-side chunks: keyed by the source row (output row + kh, or + Kh-1-kh for the input gradient)
-        const int dd_row = p.tiles_w * tw.nkw * p.cpt;
-        const uint8_t* sfa_dd = p.sfa_img + ((size_t)(((tile.n0 >> p.lgTN) * p.sfa_hk + tile.h + (MODE == MQ_OP_FWD ? 0 : p.Kh - 1)) * p.tiles_w +
-                                                      (tile.w0 >> p.lgTW)) * (tw.nkw * p.cpt)) * (512 * SPA);
-        for (int q0 = 0; q0 < Q; q0 += G, ++gi) {
-          const int nch = min(G, Q - q0);
-          const bool mine = (gi & 1u) == (uint32_t)lhalf;
-          if (G == 1 && p.sfa_dedup)
-            sfa_src = sfa_dd + (long long)((MODE == MQ_OP_FWD ? pos.ia : -pos.ia) * dd_row + pos.ib * p.cpt + pos.cc) * (512 * SPA);
-          // coordinates of the stage's boxes, before the wait
-          int c0[G], c1[G], c2[G];
-#pragma unroll
-          for (int c = 0; c < G; ++c) {
-            if (c < nch) {
-              c0[c] = pos.cc * KB;
-              c1[c] = lkind == 1 ? tap_index(tw, pos) : src_w0(tw, pos);
-              c2[c] = src_h(tw, pos);
-              pos.advance(tw, p.cpt);
+        // running position: chunk cc of the tap's row, taps left in the kernel row, source column / row (or weight tap / first tap of the kernel row)
+        constexpr int DIR = MODE == MQ_OP_FWD ? 1 : -1;
+        int cc = 0, ib = 0;
+        int x = lkind == 1 ? tw.tap0 : tw.ws0, y = lkind == 1 ? tw.tap0 : tw.hs0;
+        const int dx = lkind == 1 ? tw.tap_dw : DIR, dy = lkind == 1 ? tw.tap_dh : DIR, x0 = x;
+        // A-side scale chunks: in the tile's order, or (shared) keyed by the source row - output row + kh, or + Kh-1-kh for the input gradient
+        const bool dedup = G == 1 && p.sfa_dedup;
+        const long long dd_row = dedup ? (long long)DIR * (p.tiles_w * tw.nkw * p.cpt) * SFA_STEP : 0;
+        const uint8_t* sfa_row = dedup ? p.sfa_img + ((size_t)((tile.nt * p.sfa_hk + tile.h + (MODE == MQ_OP_FWD ? 0 : p.Kh - 1)) * p.tiles_w + tile.wt) *
+                                                      (tw.nkw * p.cpt)) * SFA_STEP
+                                       : p.sfa_img + (size_t)tile_m_index(p, tile) * p.max_stages * SFA_STEP;
+        const uint8_t* sfa_src = sfa_row;
+        const uint8_t* sfb_src = p.sfb_img + ((size_t)tile.cls * p.tiles_c + tile.ct) * p.max_stages * sfb_step;
+        auto advance = [&]() {      // to the next chunk
+          if (++cc == p.cpt) {
+            cc = 0; x += dx;
+            if (++ib == tw.nkw) {
+              ib = 0; y += dy; x = lkind == 1 ? y : x0;
+              if (dedup) { sfa_row += dd_row; sfa_src = sfa_row - SFA_STEP; }     // (one step is added below)
             }
           }
+        };
+        for (int q0 = 0; q0 < Q; q0 += G, mine = !mine) {
+          const int nch = G == 1 ? 1 : min(G, Q - q0);
           if (mine) {
+            // coordinates of the stage's boxes, before the wait
+            int c0[G], c1[G], c2[G];
+            if (G == 1) { c0[0] = cc * KB; c1[0] = x; c2[0] = y; }
+            else {
+#pragma unroll
+              for (int c = 0; c < G; ++c)
+                if (c < nch) { c0[c] = cc * KB; c1[c] = x; c2[c] = y; advance(); }
+            }
             uint8_t* sa = smem + (size_t)s * stage_bytes;
             uint8_t* sb = sa + A_STAGE_BYTES;
             if (!mbar_wait(&empty[s], phase ^ 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
@@ -1035,8 +1057,8 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             if (elect_one()) {
               if (lkind == 2) {
                 mbar_arrive_expect_tx(&full[s], 512u * SPA * (1 + atoms_b));
-                bulk_load(sb + b_stage_bytes, sfa_src, 512 * SPA, &full[s]);
-                bulk_load(sb + b_stage_bytes + SFA_B, sfb_src, 512 * SPA * atoms_b, &full[s]);
+                bulk_load(sb + b_stage_bytes, sfa_src, SFA_STEP, &full[s]);
+                bulk_load(sb + b_stage_bytes + SFA_B, sfb_src, sfb_step, &full[s]);
               } else {
                 mbar_arrive_expect_tx(&full[s], (uint32_t)nch * row_bytes);
 #pragma unroll
@@ -1050,8 +1072,13 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             }
             __syncwarp();
           }
-          sfa_src += 512 * SPA;
-          sfb_src += 512 * SPA * atoms_b;
+          if (G == 1) advance();
+          else if (!mine) {
+#pragma unroll 1
+            for (int c = 0; c < nch; ++c) advance();
+          }
+          sfa_src += SFA_STEP;
+          sfb_src += sfb_step;
           if (++s == (uint32_t)p.stages) { s = 0; phase ^= 1; }
         }
       }
@@ -1651,7 +1678,8 @@ __global__ void __launch_bounds__(256) expand_conv_scales_kernel(const ConvTcPar
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int r = 32 * j + lane;
-        const int tw_ = r & (p.TW - 1), tn = r >> p.lgTW;
+        int tw_, tn;
+        tile_row(p, r, tw_, tn);
         const int n = tile.n0 + tn, ws = ws0 + tw_;
         const bool ok = n < p.N && hs >= 0 && hs < p.Hs && ws >= 0 && ws < p.Ws;
         const uint8_t* rowp = p.a_scales + (((long long)hs * p.Ws + ws) * Nt16 + (n >> 4)) * Kb16;
@@ -1689,7 +1717,8 @@ __global__ void __launch_bounds__(256) expand_conv_scales_kernel(const ConvTcPar
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             const int r = 32 * j + lane;
-            const int tw_ = r & (p.TW - 1), tn = r >> p.lgTW;
+            int tw_, tn;
+            tile_row(p, r, tw_, tn);
             const int n = tile.n0 + tn, ws = ws0 + tw_ * wstep;
             if (n < p.N && hs >= 0 && hs < p.Hs && ws >= 0 && ws < p.Ws) {
               const uint8_t* rowp = p.a_scales + (((long long)hs * p.Ws + ws) * Nt16 + (n >> 4)) * Kb16;
@@ -1800,7 +1829,8 @@ __global__ void __launch_bounds__(256) expand_conv_scales_kernel(const ConvTcPar
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int r = 32 * j + lane;
-      const int tw_ = r & (p.TW - 1), tn = r >> p.lgTW;
+      int tw_, tn;
+      tile_row(p, r, tw_, tn);
       const int n = tile.n0 + tn, ws = ws0 + tw_;
       if (n < p.N && hs >= 0 && hs < p.Hs && ws >= 0 && ws < p.Ws)
         acc[j] = load_scale_bytes<BPC, WHOLE>(p.a_scales + (((long long)hs * p.Ws + ws) * (p.line ? p.N : p.Nt) + (p.line ? n : (n >> 5))) * p.Kblocks, pos.cc, p.Kblocks);
@@ -1834,7 +1864,8 @@ __global__ void __launch_bounds__(256) expand_conv_scales_kernel(const ConvTcPar
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           const int r = 32 * j + lane;
-          const int tw_ = r & (p.TW - 1), tn = r >> p.lgTW;
+          int tw_, tn;
+          tile_row(p, r, tw_, tn);
           const int n = tile.n0 + tn, ws = ws0 + tw_ * wstep;
           if (n < p.N && hs >= 0 && hs < p.Hs && ws >= 0 && ws < p.Ws)
             acc[j] |= load_scale_bytes<BPC, WHOLE>(p.a_scales + (((long long)hs * p.Ws + ws) * (p.line ? p.N : p.Nt) + (p.line ? n : (n >> 5))) * p.Kblocks, pos.cc, p.Kblocks) << (8 * c * BPC);

@@ -28,7 +28,9 @@ struct ConvTcParams {
   int BN;               // output channels per tile (multiple of 16, <= 256)
   int stages;
   int n_acc;            // accumulator buffers in TMEM (1 or 2)
-  int TW, TN, lgTW, lgTN;  // tile = TW output columns x TN samples (TW * TN = 128), TW fastest among rows
+  int TW, TN;           // tile = TW output columns x TN samples (TW * TN <= 128; rows beyond are not stored), TW fastest among rows
+  uint32_t m_TW;        // ceil(2^16 / TW)
+  int lgTW;             // log2 TW where it is a power of two (staged stores, quantizing epilogue, whole-tile kernel)
   // geometry
   int N, Nt;
   int Hs, Ws;           // spatial extent of the gathered source (fwd: H, W; bwd_data: Ho, Wo)

@@ -12,7 +12,7 @@
 // tile (per-thread max, one redux.sync per position, one shared-memory exchange), E8M0 code from the exponent field,
 // hardware RNE+saturate conversion; a thread owns 4 adjacent channels so codes leave as 32-bit (FP8) or
 // 16-bit (FP4) shared-memory stores, and each [n][c] slab is written with 16-byte global stores.
-// Fallback kernel (any P, e.g. the 3x3 = 9 positions of a weight tensor): scalar loads, same arithmetic.
+// Any other P: quantize_few_kernel (at most 25 positions, e.g. the nine taps of a weight tensor) and quantize_odd_kernel.
 #include <cstdlib>
 
 #include "mq_internal.cuh"
@@ -226,134 +226,102 @@ __global__ void __launch_bounds__(NT) quantize_pipe_kernel(QuantArgs a, int n_ps
   }
 }
 
-// Fallback for sources whose position axis is not a multiple of 4 elements (no 16-byte rows): one block per item.
-// LINE: line blocks - one scale per (position, row, 32 channels) instead of one per tile; the 32 channels of a line sit in
-// 16 lanes of each of two neighbouring warps (shuffles, then one exchange through shared memory).
+// Sources whose position axis is no multiple of 4 elements (images of odd size): no 16-byte row starts anywhere, so neither TMA nor
+// 16-byte copies apply.  One block per item of 32 rows x 32 channels x 16 positions; a warp's lanes are 16 positions x 2 channel
+// halves, so a load instruction reads two runs of 64 bytes, and a thread's 64 values (4 rows x 16 channels) are 64 loads in
+// flight - two blocks per SM keep 128 KB asked for.  A position's maximum is one shuffle and an exchange between the eight warps.
+// The codes are turned in shared memory (16-byte pieces, their index XORed with the position: a store's lanes are positions) and
+// leave as 16-byte stores.  E2M1, N = 50, 96 / 160 channels, 27x27: 8.8 / 13.3 -> 4.3 / 7.7 us against one 4-byte load per lane at
+// stride P, 8 positions at a time.  LINE: line blocks - one scale per (position, row, 32 channels), two lanes of a warp.
+constexpr int OD_P = 16;        // positions per item
 template <int FMT, bool SR, bool LINE = false>
-__global__ void __launch_bounds__(QT_THREADS) quantize_simple_kernel(QuantArgs a, int n_pstrips, int Ct) {
-  __shared__ __align__(16) unsigned red[8][2][4];
-  __shared__ unsigned lred[LINE ? 8 : 1][2][8][4];
-  __shared__ __align__(16) uint8_t stage[PS][32][32];   // one code per byte
+__global__ void __launch_bounds__(QT_THREADS, 2) quantize_odd_kernel(QuantArgs a, int n_pstrips, int Ct) {
+  constexpr int CB = FMT == MQ_E2M1 ? 8 : 16;      // bytes of 16 codes
+  constexpr int XM = FMT == MQ_E2M1 ? 15 : 7;      // pieces that the lanes of one shared-memory phase spread over
+  __shared__ unsigned red[8][OD_P];
+  __shared__ __align__(16) uint8_t stage[OD_P * 64 * CB];   // [position][piece = 2 row + channel half]
   pdl_wait();
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const Item q = item_of(blockIdx.x, n_pstrips, Ct);
-  const int quad = t & 1, c = (t >> 1) & 31, rsub = t >> 6;
-  const int pq = q.p0 + 4 * quad;
-  float v[8][4];
-  const bool c_ok = (q.c0 + c) < a.C;
+  const Item q = item_of(blockIdx.x, n_pstrips, Ct, OD_P);
+  const int pl = lane & (OD_P - 1), h = lane >> 4;
+  const bool p_ok = q.p0 + pl < a.P;
+  const int r0 = q.r0 + 4 * warp, c0 = q.c0 + 16 * h;
+  const long long e0 = ((long long)r0 * a.C + c0) * a.P + q.p0 + pl;      // index of this thread's first element
+  float v[4][16];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int r = q.r0 + 4 * i + rsub;
-    const bool ok = c_ok && r < a.R;
-    const float* row = a.src + ((long long)r * a.C + (q.c0 + c)) * a.P;
+  for (int i = 0; i < 4; ++i) {
+    const float* src = a.src + e0 + (long long)i * a.C * a.P;
+    const bool ok = p_ok && r0 + i < a.R;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) v[i][j] = (ok && pq + j < a.P) ? __ldg(row + pq + j) : 0.f;
+    for (int k = 0; k < 16; ++k) v[i][k] = (ok && c0 + k < a.C) ? __ldg(src + (long long)k * a.P) : 0.f;
   }
-  int code[LINE ? 8 : 1][4];
+  float m[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    m[i] = 0.f;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) m[i] = fmaxf(m[i], fabsf(v[i][k]));
+    if (LINE) m[i] = fmaxf(m[i], __shfl_xor_sync(0xffffffffu, m[i], 16));
+  }
+  int code[LINE ? 4 : 1];
   if (LINE) {
-    unsigned lm[8][4];
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        unsigned mm = __float_as_uint(v[i][j]) & 0x7fffffffu;
-#pragma unroll
-        for (int off = 2; off < 32; off <<= 1) mm = max(mm, __shfl_xor_sync(0xffffffffu, mm, off));
-        lm[i][j] = mm;
-      }
-    if (lane < 2) {
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) lred[warp][lane][i][j] = lm[i][j];
+    for (int i = 0; i < 4; ++i) {
+      code[i] = scale_code_of(__float_as_uint(m[i]), fmt_emax(FMT));
+      if (h == 0 && p_ok && r0 + i < a.R) a.scales[(long long)(q.p0 + pl) * a.sc_stride_p + (long long)(r0 + i) * a.sc_stride_r + q.ct] = (uint8_t)code[i];
     }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        code[i][j] = scale_code_of(max(lm[i][j], lred[warp ^ 1][quad][i][j]), fmt_emax(FMT));
-        // the line's first channel sits in an even warp, lanes 0 (quad 0) and 1 (quad 1)
-        if (c == 0 && q.p0 + 4 * quad + j < a.P && q.r0 + 4 * i + rsub < a.R)
-          a.scales[(long long)(q.p0 + 4 * quad + j) * a.sc_stride_p + (long long)(q.r0 + 4 * i + rsub) * a.sc_stride_r + q.ct] = (uint8_t)code[i][j];
-      }
   } else {
-    unsigned m[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      unsigned mm = 0;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) mm = max(mm, __float_as_uint(v[i][j]) & 0x7fffffffu);
-#pragma unroll
-      for (int off = 2; off < 32; off <<= 1) mm = max(mm, __shfl_xor_sync(0xffffffffu, mm, off));
-      m[j] = mm;
-    }
-    if (lane < 2) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) red[warp][lane][j] = m[j];
-    }
+    float mm = fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
+    mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, 16));
+    if (h == 0) red[warp][pl] = __float_as_uint(mm);
     __syncthreads();
+    unsigned mx = 0;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      unsigned mm = 0;
-#pragma unroll
-      for (int w = 0; w < 8; ++w) mm = max(mm, red[w][quad][j]);
-      code[0][j] = scale_code_of(mm, fmt_emax(FMT));
-    }
-    if (t < PS) {
-      unsigned mm = 0;
-#pragma unroll
-      for (int w = 0; w < 8; ++w) mm = max(mm, red[w][t >> 2][t & 3]);
-      if (q.p0 + t < a.P)
-        a.scales[(long long)(q.p0 + t) * a.sc_stride_p + (long long)q.rt * a.sc_stride_r + q.ct] = (uint8_t)scale_code_of(mm, fmt_emax(FMT));
-    }
+    for (int w = 0; w < 8; ++w) mx = max(mx, red[w][pl]);
+    code[0] = scale_code_of(mx, fmt_emax(FMT));
+    if (t < OD_P && p_ok) a.scales[(long long)(q.p0 + t) * a.sc_stride_p + (long long)q.rt * a.sc_stride_r + q.ct] = (uint8_t)code[0];
   }
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
+  for (int i = 0; i < 4; ++i) {
+    const float f = scale_factor(code[LINE ? i : 0]);
+    unsigned w4[4];
 #pragma unroll
-    for (int i = 0; i < 8; i += 2) {
-      float x0 = v[i][j] * scale_factor(code[LINE ? i : 0][j]), x1 = v[i + 1][j] * scale_factor(code[LINE ? i + 1 : 0][j]);
-      if (SR) {
-        const long long e0 = ((long long)(q.r0 + 4 * i + rsub) * a.C + (q.c0 + c)) * a.P + pq + j;
-        const long long e1 = e0 + 4ll * a.C * a.P;
-        x0 = sr_value<FMT>(x0, (unsigned)e0, sr_key(a, e0));
-        x1 = sr_value<FMT>(x1, (unsigned)e1, sr_key(a, e1));
+    for (int k = 0; k < 16; k += 4) {
+      float x[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        x[j] = v[i][k + j] * f;
+        if (SR) {
+          const long long e = e0 + ((long long)i * a.C + k + j) * a.P;
+          x[j] = sr_value<FMT>(x[j], (unsigned)e, sr_key(a, e));
+        }
       }
-      const unsigned two = encode2<FMT>(x0, x1);
-      unsigned lo, hi;
-      if (FMT == MQ_E2M1) { lo = two & 0xF; hi = (two >> 4) & 0xF; }
-      else { lo = two & 0xFF; hi = (two >> 8) & 0xFF; }
-      stage[4 * quad + j][4 * i + rsub][c] = (uint8_t)lo;
-      stage[4 * quad + j][4 * (i + 1) + rsub][c] = (uint8_t)hi;
+      const unsigned lo = encode2<FMT>(x[0], x[1]), hi = encode2<FMT>(x[2], x[3]);
+      w4[k >> 2] = FMT == MQ_E2M1 ? (lo | (hi << 8)) : (lo | (hi << 16));
     }
+    uint8_t* dst = stage + (pl * 64 + ((2 * (4 * warp + i) + h) ^ (pl & XM))) * CB;
+    if (FMT == MQ_E2M1) *reinterpret_cast<uint2*>(dst) = make_uint2(w4[0] | (w4[1] << 16), w4[2] | (w4[3] << 16));
+    else *reinterpret_cast<uint4*>(dst) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
   }
   __syncthreads();
   if (FMT == MQ_E2M1) {
-    const int p = t >> 5, r = t & 31;
-    if (q.p0 + p < a.P && q.r0 + r < a.R) {
-      const uint4* srcw = reinterpret_cast<const uint4*>(&stage[p][r][0]);
-      const uint4 lo = srcw[0], hi = srcw[1];
-      const uint32_t in[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
-      uint32_t outw[4];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        // 8 one-byte codes (two words) -> one word of 8 nibbles, lower index in the lower nibble
-        const uint32_t w0 = in[2 * k], w1 = in[2 * k + 1];
-        const uint32_t b0 = (w0 & 0xF) | ((w0 >> 4) & 0xF0) | ((w0 >> 8) & 0xF00) | ((w0 >> 12) & 0xF000);
-        const uint32_t b1 = (w1 & 0xF) | ((w1 >> 4) & 0xF0) | ((w1 >> 8) & 0xF00) | ((w1 >> 12) & 0xF000);
-        outw[k] = b0 | (b1 << 16);
+    for (int k = 0; k < OD_P * 32 / QT_THREADS; ++k) {    // rows of 16 bytes: [position][row]
+      const int id = t + QT_THREADS * k, p = id >> 5, r = id & 31;
+      if (q.p0 + p < a.P && q.r0 + r < a.R) {
+        const uint2* row = reinterpret_cast<const uint2*>(stage) + p * 64;
+        const uint2 lo = row[(2 * r) ^ (p & XM)], hi = row[(2 * r + 1) ^ (p & XM)];
+        const long long e = (long long)(q.p0 + p) * a.out_stride_p + (long long)(q.r0 + r) * a.out_stride_r + q.c0;
+        *reinterpret_cast<uint4*>(a.codes + (e >> 1)) = make_uint4(lo.x, lo.y, hi.x, hi.y);
       }
-      const long long e = (long long)(q.p0 + p) * a.out_stride_p + (long long)(q.r0 + r) * a.out_stride_r + q.c0;
-      *reinterpret_cast<uint4*>(a.codes + (e >> 1)) = make_uint4(outw[0], outw[1], outw[2], outw[3]);
     }
   } else {
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int id = t + QT_THREADS * k;
-      const int p = id >> 6, r = (id >> 1) & 31, half = id & 1;
+    for (int k = 0; k < OD_P * 64 / QT_THREADS; ++k) {    // pieces of 16 bytes: [position][row][half]
+      const int id = t + QT_THREADS * k, p = id >> 6, piece = id & 63, r = piece >> 1;
       if (q.p0 + p < a.P && q.r0 + r < a.R) {
-        const uint4 val = *reinterpret_cast<const uint4*>(&stage[p][r][16 * half]);
-        const long long e = (long long)(q.p0 + p) * a.out_stride_p + (long long)(q.r0 + r) * a.out_stride_r + q.c0 + 16 * half;
+        const uint4 val = *(reinterpret_cast<const uint4*>(stage) + p * 64 + (piece ^ (p & XM)));
+        const long long e = (long long)(q.p0 + p) * a.out_stride_p + (long long)(q.r0 + r) * a.out_stride_r + q.c0 + 16 * (piece & 1);
         store_codes16(a, e, val);
       }
     }
@@ -619,6 +587,105 @@ quantize_tma_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_con
   __syncthreads();
 }
 
+// One 32 x 32 tile at one position held by a warp, lane (cq, rq) = (lane & 7, lane >> 3) with 4 adjacent channels of rows
+// rq, rq + 4, ...: scale(s), codes, stores.  LINE: one scale per row (line blocks), reduced over the 8 lanes of a row.
+template <int FMT, bool SR, bool LINE>
+__device__ __forceinline__ void finish_tile(const QuantArgs& a, const float4 (&v)[8], int pos, int rt, int ct, int lane) {
+  const int cq = lane & 7, rq = lane >> 3;
+  const int r0 = rt * 32 + rq, c0 = ct * 32 + 4 * cq;
+      int code[LINE ? 8 : 1];
+      if (LINE) {
+  #pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          unsigned mm = __float_as_uint(fmaxf(fmaxf(fabsf(v[i].x), fabsf(v[i].y)), fmaxf(fabsf(v[i].z), fabsf(v[i].w))));
+          mm = max(mm, __shfl_xor_sync(0xffffffffu, mm, 1));
+          mm = max(mm, __shfl_xor_sync(0xffffffffu, mm, 2));
+          mm = max(mm, __shfl_xor_sync(0xffffffffu, mm, 4));
+          code[i] = scale_code_of(mm, fmt_emax(FMT));
+          if (cq == 0 && r0 + 4 * i < a.R) a.scales[(long long)pos * a.sc_stride_p + (long long)(r0 + 4 * i) * a.sc_stride_r + ct] = (uint8_t)code[i];
+        }
+      } else {
+        float m = 0.f;
+  #pragma unroll
+        for (int i = 0; i < 8; ++i) m = fmaxf(fmaxf(m, fmaxf(fabsf(v[i].x), fabsf(v[i].y))), fmaxf(fabsf(v[i].z), fabsf(v[i].w)));
+        code[0] = scale_code_of(__reduce_max_sync(0xffffffffu, __float_as_uint(m)), fmt_emax(FMT));
+        if (lane == 0) a.scales[(long long)pos * a.sc_stride_p + (long long)rt * a.sc_stride_r + ct] = (uint8_t)code[0];
+      }
+      const long long pbase = (long long)pos * a.out_stride_p + c0;
+  #pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int r = r0 + 4 * i;
+        const float f = scale_factor(code[LINE ? i : 0]);
+        float x[4] = {v[i].x * f, v[i].y * f, v[i].z * f, v[i].w * f};
+        if (SR) {
+          const long long e0 = ((long long)r * a.C + c0) * a.P + pos;    // index in the logical tensor, whatever the source order
+  #pragma unroll
+          for (int k = 0; k < 4; ++k) x[k] = sr_value<FMT>(x[k], (unsigned)e0 + (unsigned)k * (unsigned)a.P, sr_key(a, e0 + (long long)k * a.P));
+        }
+        const unsigned lo = encode2<FMT>(x[0], x[1]), hi = encode2<FMT>(x[2], x[3]);
+        const long long e = pbase + (long long)r * a.out_stride_r;
+        if (FMT == MQ_E2M1) {
+          const unsigned mine = lo | (hi << 8);                       // 4 codes; the odd lane's go above the even lane's
+          const unsigned other = __shfl_xor_sync(0xffffffffu, mine, 1);
+          if ((lane & 1) == 0 && r < a.R) *reinterpret_cast<unsigned*>(a.codes + (e >> 1)) = mine | (other << 16);
+        } else if ((FMT == MQ_E3M2 || FMT == MQ_E2M3) && a.packed6) {
+          // packed 6-bit storage: a lane's four codes are 24 bits; lanes 4j .. 4j+3 hold a 12-byte group, its word k written by
+          // lane 4j + k from its own bits and the next lane's
+          const unsigned w = lo | (hi << 16);
+          const unsigned t24 = (w & 0x3Fu) | ((w >> 2) & 0xFC0u) | ((w >> 4) & 0x3F000u) | ((w >> 6) & 0xFC0000u);
+          const unsigned nxt = __shfl_down_sync(0xffffffffu, t24, 1);
+          const int k = lane & 3;
+          if (k < 3 && r < a.R) {
+            const long long e16 = (e - 4 * k) >> 4;    // the group's index
+            *reinterpret_cast<unsigned*>(a.codes + e16 * 12 + 4 * k) = (t24 >> (8 * k)) | (nxt << (24 - 8 * k));
+          }
+        } else {
+          if (r < a.R) *reinterpret_cast<unsigned*>(a.codes + e) = lo | (hi << 16);
+        }
+      }
+}
+
+// Few positions (at most FEW_P, no multiple of 4: the taps of a weight tensor, tiny images): the 32 channels x P positions of a row
+// are ONE run of 32 P floats.  A block copies the 32 runs of a tile into shared memory (asynchronous 4-byte copies, a warp's lanes
+// side by side: whole lines, all in flight at once; rows of 32 P + 1 floats, so that the reads below meet no bank twice), and
+// each warp then quantizes a position at a time.  512 -> 512 channels, 3x3: 5.6 -> 4.3 us against one 4-byte load per lane at stride P (32 -> 64 channels: 2.4 -> 2.8 us, where one
+// round of loads is all there is; quantize_odd_kernel 3.3).
+constexpr int FEW_P = 25;
+__device__ __forceinline__ void cp_async4(void* dst, const void* src, bool valid) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "r"(valid ? 4 : 0) : "memory");
+}
+template <int FMT, bool SR, bool LINE = false>
+__global__ void __launch_bounds__(512) quantize_few_kernel(QuantArgs a, int Ct) {
+  extern __shared__ float runs[];
+  pdl_wait();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = (int)blockDim.x >> 5;   // at least 8
+  const int rt = (int)(blockIdx.x / (unsigned)Ct), ct = (int)(blockIdx.x - (unsigned)rt * (unsigned)Ct);
+  const int run = 32 * a.P, stride = run + 1, valid = min(32, a.C - ct * 32) * a.P;
+#pragma unroll 1
+  for (int row = warp; row < 32; row += nwarps) {
+    const int r = rt * 32 + row;
+    const float* src = a.src + ((long long)r * a.C + ct * 32) * a.P;
+    for (int k = lane; k < run; k += 32) {
+      const bool ok = r < a.R && k < valid;
+      cp_async4(runs + row * stride + k, ok ? src + k : a.src, ok);
+    }
+  }
+  cp_async_commit();
+  cp_async_wait<0>();
+  __syncthreads();
+  const int cq = lane & 7, rq = lane >> 3;
+#pragma unroll 1
+  for (int p = warp; p < a.P; p += nwarps) {
+    float4 v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float* src = runs + (rq + 4 * i) * stride + 4 * cq * a.P + p;
+      v[i] = make_float4(src[0], src[a.P], src[2 * a.P], src[3 * a.P]);
+    }
+    finish_tile<FMT, SR, LINE>(a, v, p, rt, ct, lane);
+  }
+}
+
 // ---- channel-fastest source ([H][W][N][C] activations / gradients, [Cout][Kh][Kw][Cin] weights) ------------------
 // No re-layout is needed: a tile's 32 rows are runs of 32 consecutive floats.  One warp per (position, tile): lane
 // (cq, rq) = (lane & 7, lane >> 3) loads 4 adjacent channels of rows rq, rq + 4, ... as one 128-bit load each (8 in
@@ -656,56 +723,7 @@ __global__ void __launch_bounds__(256) quantize_cfast_kernel(QuantArgs a, unsign
       for (int i = 0; i < 8; ++i)
         v[i] = make_float4(mx_activation(v[i].x, a.act), mx_activation(v[i].y, a.act), mx_activation(v[i].z, a.act), mx_activation(v[i].w, a.act));
     }
-    int code[LINE ? 8 : 1];
-    if (LINE) {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        unsigned mm = __float_as_uint(fmaxf(fmaxf(fabsf(v[i].x), fabsf(v[i].y)), fmaxf(fabsf(v[i].z), fabsf(v[i].w))));
-        mm = max(mm, __shfl_xor_sync(0xffffffffu, mm, 1));
-        mm = max(mm, __shfl_xor_sync(0xffffffffu, mm, 2));
-        mm = max(mm, __shfl_xor_sync(0xffffffffu, mm, 4));
-        code[i] = scale_code_of(mm, fmt_emax(FMT));
-        if (cq == 0 && r0 + 4 * i < a.R) a.scales[(long long)pos * a.sc_stride_p + (long long)(r0 + 4 * i) * a.sc_stride_r + ct] = (uint8_t)code[i];
-      }
-    } else {
-      float m = 0.f;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) m = fmaxf(fmaxf(m, fmaxf(fabsf(v[i].x), fabsf(v[i].y))), fmaxf(fabsf(v[i].z), fabsf(v[i].w)));
-      code[0] = scale_code_of(__reduce_max_sync(0xffffffffu, __float_as_uint(m)), fmt_emax(FMT));
-      if (lane == 0) a.scales[(long long)pos * a.sc_stride_p + (long long)rt * a.sc_stride_r + ct] = (uint8_t)code[0];
-    }
-    const long long pbase = (long long)pos * a.out_stride_p + c0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int r = r0 + 4 * i;
-      const float f = scale_factor(code[LINE ? i : 0]);
-      float x[4] = {v[i].x * f, v[i].y * f, v[i].z * f, v[i].w * f};
-      if (SR) {
-        const long long e0 = ((long long)r * a.C + c0) * a.P + pos;    // index in the logical tensor, whatever the source order
-#pragma unroll
-        for (int k = 0; k < 4; ++k) x[k] = sr_value<FMT>(x[k], (unsigned)e0 + (unsigned)k * (unsigned)a.P, sr_key(a, e0 + (long long)k * a.P));
-      }
-      const unsigned lo = encode2<FMT>(x[0], x[1]), hi = encode2<FMT>(x[2], x[3]);
-      const long long e = pbase + (long long)r * a.out_stride_r;
-      if (FMT == MQ_E2M1) {
-        const unsigned mine = lo | (hi << 8);                       // 4 codes; the odd lane's go above the even lane's
-        const unsigned other = __shfl_xor_sync(0xffffffffu, mine, 1);
-        if ((lane & 1) == 0 && r < a.R) *reinterpret_cast<unsigned*>(a.codes + (e >> 1)) = mine | (other << 16);
-      } else if ((FMT == MQ_E3M2 || FMT == MQ_E2M3) && a.packed6) {
-        // packed 6-bit storage: a lane's four codes are 24 bits; lanes 4j .. 4j+3 hold a 12-byte group, its word k written by
-        // lane 4j + k from its own bits and the next lane's
-        const unsigned w = lo | (hi << 16);
-        const unsigned t24 = (w & 0x3Fu) | ((w >> 2) & 0xFC0u) | ((w >> 4) & 0x3F000u) | ((w >> 6) & 0xFC0000u);
-        const unsigned nxt = __shfl_down_sync(0xffffffffu, t24, 1);
-        const int k = lane & 3;
-        if (k < 3 && r < a.R) {
-          const long long e16 = (e - 4 * k) >> 4;    // the group's index
-          *reinterpret_cast<unsigned*>(a.codes + e16 * 12 + 4 * k) = (t24 >> (8 * k)) | (nxt << (24 - 8 * k));
-        }
-      } else {
-        if (r < a.R) *reinterpret_cast<unsigned*>(a.codes + e) = lo | (hi << 16);
-      }
-    }
+    finish_tile<FMT, SR, LINE>(a, v, (int)pos, (int)rt, (int)ct, lane);
   }
 }
 
@@ -780,13 +798,23 @@ constexpr size_t QPIPE_SMEM = 2 * QBUF_BYTES + PS * 32 * 32 + 16 * 2 * 4 * sizeo
 
 template <int FMT>
 cudaError_t launch_q(const QuantArgs& a, int n_pstrips, int Ct, long long n_items, bool vec, bool r16, cudaStream_t s) {
-  if (a.line) {   // line blocks without 16-byte rows (large aligned tensors take the whole-line kernel): the one-block-per-item kernel
-    if (a.sr) return launch_pdl(quantize_simple_kernel<FMT, true, true>, dim3((unsigned)n_items), dim3(QT_THREADS), 0, s, a, n_pstrips, Ct);
-    return launch_pdl(quantize_simple_kernel<FMT, false, true>, dim3((unsigned)n_items), dim3(QT_THREADS), 0, s, a, n_pstrips, Ct);
-  }
-  if (!vec) {
-    if (a.sr) return launch_pdl(quantize_simple_kernel<FMT, true>, dim3((unsigned)n_items), dim3(QT_THREADS), 0, s, a, n_pstrips, Ct);
-    return launch_pdl(quantize_simple_kernel<FMT, false>, dim3((unsigned)n_items), dim3(QT_THREADS), 0, s, a, n_pstrips, Ct);
+  if (a.line || !vec) {   // (line blocks with 16-byte rows get here only as small tensors: large ones take the whole-line kernel)
+    if (a.P <= FEW_P && a.P % 4 != 0) {
+      auto kernel = a.line ? (a.sr ? quantize_few_kernel<FMT, true, true> : quantize_few_kernel<FMT, false, true>)
+                           : (a.sr ? quantize_few_kernel<FMT, true> : quantize_few_kernel<FMT, false>);
+      const size_t smem = (size_t)32 * (32 * a.P + 1) * sizeof(float);
+      if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 32 * (32 * FEW_P + 1) * (int)sizeof(float));
+        if (e != cudaSuccess) return e;
+      }
+      const int rounds = (a.P + 15) / 16, warps = (a.P + rounds - 1) / rounds;      // as few positions per warp as 16 warps allow: nine taps, nine warps
+      return launch_pdl(kernel, dim3((unsigned)(n_items / n_pstrips)), dim3((unsigned)(warps < 8 ? 8 : warps) * 32), smem, s, a, Ct);
+    }
+    const int strips = (a.P + OD_P - 1) / OD_P;
+    const long long items = n_items / n_pstrips * strips;
+    auto kernel = a.line ? (a.sr ? quantize_odd_kernel<FMT, true, true> : quantize_odd_kernel<FMT, false, true>)
+                         : (a.sr ? quantize_odd_kernel<FMT, true> : quantize_odd_kernel<FMT, false>);
+    return launch_pdl(kernel, dim3((unsigned)items), dim3(QT_THREADS), 0, s, a, strips, Ct);
   }
   static bool attr_set = false;
   const int ctas_per_sm = 2;   // 80 KB of shared memory per block; 256 threads (512-thread blocks measured slower: bound by instruction issue)

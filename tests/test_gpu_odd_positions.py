@@ -1,0 +1,48 @@
+"""Quantizer of sources whose positions are no multiple of four (needs a B200): the staged-run kernel (at most 25 positions) and the
+odd-size kernel at the edges of their ranges and of their items (16 positions, 32 rows, 32 channels), every element format, both
+block shapes, stochastic rounding.  Codes and scales are the oracle's bit for bit."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2609_28358_b200 import inputs, mq
+from parity_util import assert_same_bytes, dev
+
+pytestmark = pytest.mark.gpu
+
+FMTS = [mq.E4M3, mq.E5M2, mq.E2M1, mq.E3M2, mq.E2M3, mq.E3M2_P6]
+# weights [C_out][C_in][Kh][Kw]: one tap, two, 3x3, 5x5 (the most staged), and 3x9 = 27 and 7x7 (odd-size kernel)
+W_SHAPES = [(3, 40, 1, 1), (33, 32, 1, 2), (70, 37, 3, 3), (32, 64, 5, 5), (31, 35, 3, 9), (16, 48, 7, 7)]
+# activations N, C, H, W: 30, 31, 33 and 47 positions; ragged rows and channels
+X_SHAPES = [(40, 48, 5, 6), (33, 35, 1, 31), (5, 96, 3, 11), (64, 20, 1, 47)]
+
+
+def _case(kind, shape):
+    rng = np.random.default_rng(11)
+    if kind == "W":
+        co, ci, kh, kw = shape
+        d, role = inputs.ConvDesc(2, ci, kh + 1, kw + 1, co, kh, kw, 1, 1, 0, 0), mq.ROLE_W
+    else:
+        n, c, h, w = shape
+        d, role = inputs.ConvDesc(n, c, h, w, 32, 1, 1, 1, 1, 0, 0), mq.ROLE_X
+    x = rng.standard_normal(shape).astype(np.float32)
+    x[0] = 0.0
+    return d, role, x
+
+
+@pytest.mark.parametrize("fmt", FMTS)
+@pytest.mark.parametrize("kind,shape", [("W", s) for s in W_SHAPES] + [("X", s) for s in X_SHAPES], ids=str)
+def test_codes_and_scales(kind, shape, fmt):
+    d, role, x = _case(kind, shape)
+    base, packed = (mq.E3M2, True) if fmt == mq.E3M2_P6 else (fmt, False)
+    pack = oracle.pack6 if packed else (lambda c: c)
+    blocks = [(mq.TILE32, (32, 32))] + ([] if packed else [(mq.LINE32, (1, 32))])
+    for block, shape_b in blocks:
+        codes, scales = oracle.quantize(d, role, base, x, shape_b)
+        q = mq.quantize(d, role, fmt, dev(x), block=block)
+        assert_same_bytes(q.scales, scales, f"scales {block}")
+        assert_same_bytes(q.codes, pack(codes), f"codes {block}")
+    codes, scales = oracle.quantize_sr(d, role, base, x, 99)
+    q = mq.quantize_sr(d, role, fmt, dev(x), 99)
+    assert_same_bytes(q.scales, scales, "stochastic scales")
+    assert_same_bytes(q.codes, pack(codes), "stochastic codes")
