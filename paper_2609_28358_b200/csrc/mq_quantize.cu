@@ -12,7 +12,7 @@
 // tile (per-thread max, one redux.sync per position, one shared-memory exchange), E8M0 code from the exponent field,
 // hardware RNE+saturate conversion; a thread owns 4 adjacent channels so codes leave as 32-bit (FP8) or
 // 16-bit (FP4) shared-memory stores, and each [n][c] slab is written with 16-byte global stores.
-// Any other P: quantize_few_kernel (at most 25 positions, e.g. the nine taps of a weight tensor) and quantize_odd_kernel.
+// Any other P: quantize_odd_kernel, or quantize_few_kernel where there are many tiles of at most 25 positions (weights).
 #include <cstdlib>
 
 #include "mq_internal.cuh"
@@ -232,36 +232,43 @@ __global__ void __launch_bounds__(NT) quantize_pipe_kernel(QuantArgs a, int n_ps
 // flight - two blocks per SM keep 128 KB asked for.  A position's maximum is one shuffle and an exchange between the eight warps.
 // The codes are turned in shared memory (16-byte pieces, their index XORed with the position: a store's lanes are positions) and
 // leave as 16-byte stores.  E2M1, N = 50, 96 / 160 channels, 27x27: 8.8 / 13.3 -> 4.3 / 7.7 us against one 4-byte load per lane at
-// stride P, 8 positions at a time.  LINE: line blocks - one scale per (position, row, 32 channels), two lanes of a warp.
-constexpr int OD_P = 16;        // positions per item
-template <int FMT, bool SR, bool LINE = false>
+// stride P.  PI = 8 (half the loads per thread, twice the blocks) where the whole grid runs at once, us, PI = 16 / 8: 64 channels
+// 13x13, N = 20: 3.4 / 2.6; 512 channels 7x7, N = 64 (224 blocks): 3.7 / 3.6; 96 channels 27x27, N = 50 (552 blocks): 4.3 / 5.1;
+// weights against quantize_few_kernel / PI = 8: 128 -> 128 3x3 3.1 / 2.6, 288 -> 78 5x5 4.8 / 2.7, 512 -> 512 3x3 (512 blocks)
+// 4.2 / 5.0.  LINE: line blocks - one scale per (position, row, 32 channels).
+template <int FMT, bool SR, bool LINE, int PI>   // PI: positions per item, 16 or 8
 __global__ void __launch_bounds__(QT_THREADS, 2) quantize_odd_kernel(QuantArgs a, int n_pstrips, int Ct) {
-  constexpr int CB = FMT == MQ_E2M1 ? 8 : 16;      // bytes of 16 codes
-  constexpr int XM = FMT == MQ_E2M1 ? 15 : 7;      // pieces that the lanes of one shared-memory phase spread over
-  __shared__ unsigned red[8][OD_P];
-  __shared__ __align__(16) uint8_t stage[OD_P * 64 * CB];   // [position][piece = 2 row + channel half]
+  constexpr int CG = PI, HN = 32 / PI;             // a thread's channels, a row's channel groups
+  constexpr int CB = FMT == MQ_E2M1 ? CG / 2 : CG; // bytes of a piece: CG codes
+  constexpr int XM = FMT == MQ_E2M1 && PI == 16 ? 15 : 7;    // XOR of a position's pieces, in units of XU pieces (16 bytes where
+  constexpr int XU = PI == 16 ? 1 : (FMT == MQ_E2M1 ? 4 : 2);   // a piece is smaller and the stores below read 16 at once)
+  __shared__ unsigned red[8][PI];
+  __shared__ __align__(16) uint8_t stage[PI * 32 * HN * CB];   // [position][piece = HN row + channel group]
   pdl_wait();
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const Item q = item_of(blockIdx.x, n_pstrips, Ct, OD_P);
-  const int pl = lane & (OD_P - 1), h = lane >> 4;
+  const Item q = item_of(blockIdx.x, n_pstrips, Ct, PI);
+  const int pl = lane & (PI - 1), h = lane / PI;
   const bool p_ok = q.p0 + pl < a.P;
-  const int r0 = q.r0 + 4 * warp, c0 = q.c0 + 16 * h;
+  const int r0 = q.r0 + 4 * warp, c0 = q.c0 + CG * h;
   const long long e0 = ((long long)r0 * a.C + c0) * a.P + q.p0 + pl;      // index of this thread's first element
-  float v[4][16];
+  float v[4][CG];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const float* src = a.src + e0 + (long long)i * a.C * a.P;
     const bool ok = p_ok && r0 + i < a.R;
 #pragma unroll
-    for (int k = 0; k < 16; ++k) v[i][k] = (ok && c0 + k < a.C) ? __ldg(src + (long long)k * a.P) : 0.f;
+    for (int k = 0; k < CG; ++k) v[i][k] = (ok && c0 + k < a.C) ? __ldg(src + (long long)k * a.P) : 0.f;
   }
   float m[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     m[i] = 0.f;
 #pragma unroll
-    for (int k = 0; k < 16; ++k) m[i] = fmaxf(m[i], fabsf(v[i][k]));
-    if (LINE) m[i] = fmaxf(m[i], __shfl_xor_sync(0xffffffffu, m[i], 16));
+    for (int k = 0; k < CG; ++k) m[i] = fmaxf(m[i], fabsf(v[i][k]));
+    if (LINE) {
+#pragma unroll
+      for (int off = PI; off < 32; off <<= 1) m[i] = fmaxf(m[i], __shfl_xor_sync(0xffffffffu, m[i], off));
+    }
   }
   int code[LINE ? 4 : 1];
   if (LINE) {
@@ -272,21 +279,22 @@ __global__ void __launch_bounds__(QT_THREADS, 2) quantize_odd_kernel(QuantArgs a
     }
   } else {
     float mm = fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
-    mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, 16));
+#pragma unroll
+    for (int off = PI; off < 32; off <<= 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, off));
     if (h == 0) red[warp][pl] = __float_as_uint(mm);
     __syncthreads();
     unsigned mx = 0;
 #pragma unroll
     for (int w = 0; w < 8; ++w) mx = max(mx, red[w][pl]);
     code[0] = scale_code_of(mx, fmt_emax(FMT));
-    if (t < OD_P && p_ok) a.scales[(long long)(q.p0 + t) * a.sc_stride_p + (long long)q.rt * a.sc_stride_r + q.ct] = (uint8_t)code[0];
+    if (t < PI && p_ok) a.scales[(long long)(q.p0 + t) * a.sc_stride_p + (long long)q.rt * a.sc_stride_r + q.ct] = (uint8_t)code[0];
   }
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const float f = scale_factor(code[LINE ? i : 0]);
-    unsigned w4[4];
+    unsigned w4[CG / 4];
 #pragma unroll
-    for (int k = 0; k < 16; k += 4) {
+    for (int k = 0; k < CG; k += 4) {
       float x[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
@@ -299,25 +307,33 @@ __global__ void __launch_bounds__(QT_THREADS, 2) quantize_odd_kernel(QuantArgs a
       const unsigned lo = encode2<FMT>(x[0], x[1]), hi = encode2<FMT>(x[2], x[3]);
       w4[k >> 2] = FMT == MQ_E2M1 ? (lo | (hi << 8)) : (lo | (hi << 16));
     }
-    uint8_t* dst = stage + (pl * 64 + ((2 * (4 * warp + i) + h) ^ (pl & XM))) * CB;
-    if (FMT == MQ_E2M1) *reinterpret_cast<uint2*>(dst) = make_uint2(w4[0] | (w4[1] << 16), w4[2] | (w4[3] << 16));
-    else *reinterpret_cast<uint4*>(dst) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+    uint8_t* dst = stage + (pl * 32 * HN + ((HN * (4 * warp + i) + h) ^ ((pl & XM) * XU))) * CB;
+    if constexpr (FMT == MQ_E2M1 && PI == 16) *reinterpret_cast<uint2*>(dst) = make_uint2(w4[0] | (w4[1] << 16), w4[2] | (w4[3] << 16));
+    else if constexpr (FMT == MQ_E2M1) *reinterpret_cast<unsigned*>(dst) = w4[0] | (w4[1] << 16);
+    else if constexpr (PI == 16) *reinterpret_cast<uint4*>(dst) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+    else *reinterpret_cast<uint2*>(dst) = make_uint2(w4[0], w4[1]);
   }
   __syncthreads();
   if (FMT == MQ_E2M1) {
 #pragma unroll
-    for (int k = 0; k < OD_P * 32 / QT_THREADS; ++k) {    // rows of 16 bytes: [position][row]
+    for (int k = 0; k < PI * 32 / QT_THREADS; ++k) {    // rows of 16 bytes: [position][row]
       const int id = t + QT_THREADS * k, p = id >> 5, r = id & 31;
       if (q.p0 + p < a.P && q.r0 + r < a.R) {
-        const uint2* row = reinterpret_cast<const uint2*>(stage) + p * 64;
-        const uint2 lo = row[(2 * r) ^ (p & XM)], hi = row[(2 * r + 1) ^ (p & XM)];
+        uint4 val;
+        if constexpr (PI == 16) {
+          const uint2* row = reinterpret_cast<const uint2*>(stage) + p * 64;
+          const uint2 lo = row[(2 * r) ^ (p & XM)], hi = row[(2 * r + 1) ^ (p & XM)];
+          val = make_uint4(lo.x, lo.y, hi.x, hi.y);
+        } else {
+          val = *(reinterpret_cast<const uint4*>(stage) + p * 32 + (r ^ (p & XM)));
+        }
         const long long e = (long long)(q.p0 + p) * a.out_stride_p + (long long)(q.r0 + r) * a.out_stride_r + q.c0;
-        *reinterpret_cast<uint4*>(a.codes + (e >> 1)) = make_uint4(lo.x, lo.y, hi.x, hi.y);
+        *reinterpret_cast<uint4*>(a.codes + (e >> 1)) = val;
       }
     }
   } else {
 #pragma unroll
-    for (int k = 0; k < OD_P * 64 / QT_THREADS; ++k) {    // pieces of 16 bytes: [position][row][half]
+    for (int k = 0; k < PI * 64 / QT_THREADS; ++k) {    // pieces of 16 bytes: [position][row][half]
       const int id = t + QT_THREADS * k, p = id >> 6, piece = id & 63, r = piece >> 1;
       if (q.p0 + p < a.P && q.r0 + r < a.R) {
         const uint4 val = *(reinterpret_cast<const uint4*>(stage) + p * 64 + (piece ^ (p & XM)));
@@ -648,8 +664,8 @@ __device__ __forceinline__ void finish_tile(const QuantArgs& a, const float4 (&v
 // Few positions (at most FEW_P, no multiple of 4: the taps of a weight tensor, tiny images): the 32 channels x P positions of a row
 // are ONE run of 32 P floats.  A block copies the 32 runs of a tile into shared memory (asynchronous 4-byte copies, a warp's lanes
 // side by side: whole lines, all in flight at once; rows of 32 P + 1 floats, so that the reads below meet no bank twice), and
-// each warp then quantizes a position at a time.  512 -> 512 channels, 3x3: 5.6 -> 4.3 us against one 4-byte load per lane at stride P (32 -> 64 channels: 2.4 -> 2.8 us, where one
-// round of loads is all there is; quantize_odd_kernel 3.3).
+// each warp then quantizes a position at a time.  512 -> 512 channels, 3x3: 5.6 -> 4.3 us against one 4-byte load per lane at
+// stride P.  (Rows fetched by cp.async.bulk instead: 5.4 us, 4.0 instead of 3.0 where one round of loads is all there is.)
 constexpr int FEW_P = 25;
 __device__ __forceinline__ void cp_async4(void* dst, const void* src, bool valid) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "r"(valid ? 4 : 0) : "memory");
@@ -799,7 +815,10 @@ constexpr size_t QPIPE_SMEM = 2 * QBUF_BYTES + PS * 32 * 32 + 16 * 2 * 4 * sizeo
 template <int FMT>
 cudaError_t launch_q(const QuantArgs& a, int n_pstrips, int Ct, long long n_items, bool vec, bool r16, cudaStream_t s) {
   if (a.line || !vec) {   // (line blocks with 16-byte rows get here only as small tensors: large ones take the whole-line kernel)
-    if (a.P <= FEW_P && a.P % 4 != 0) {
+    const long long tiles = n_items / n_pstrips;
+    // 8-position items while they all run at once (two blocks per SM): see quantize_odd_kernel
+    const bool small = a.P > 2 && tiles * ((a.P + 7) / 8) <= 2 * sm_count();
+    if (!small && a.P <= FEW_P && a.P % 4 != 0) {
       auto kernel = a.line ? (a.sr ? quantize_few_kernel<FMT, true, true> : quantize_few_kernel<FMT, false, true>)
                            : (a.sr ? quantize_few_kernel<FMT, true> : quantize_few_kernel<FMT, false>);
       const size_t smem = (size_t)32 * (32 * a.P + 1) * sizeof(float);
@@ -808,12 +827,14 @@ cudaError_t launch_q(const QuantArgs& a, int n_pstrips, int Ct, long long n_item
         if (e != cudaSuccess) return e;
       }
       const int rounds = (a.P + 15) / 16, warps = (a.P + rounds - 1) / rounds;      // as few positions per warp as 16 warps allow: nine taps, nine warps
-      return launch_pdl(kernel, dim3((unsigned)(n_items / n_pstrips)), dim3((unsigned)(warps < 8 ? 8 : warps) * 32), smem, s, a, Ct);
+      return launch_pdl(kernel, dim3((unsigned)tiles), dim3((unsigned)(warps < 8 ? 8 : warps) * 32), smem, s, a, Ct);
     }
-    const int strips = (a.P + OD_P - 1) / OD_P;
-    const long long items = n_items / n_pstrips * strips;
-    auto kernel = a.line ? (a.sr ? quantize_odd_kernel<FMT, true, true> : quantize_odd_kernel<FMT, false, true>)
-                         : (a.sr ? quantize_odd_kernel<FMT, true> : quantize_odd_kernel<FMT, false>);
+    const int strips = (a.P + (small ? 7 : 15)) / (small ? 8 : 16);
+    const long long items = tiles * strips;
+    auto kernel = small ? (a.line ? (a.sr ? quantize_odd_kernel<FMT, true, true, 8> : quantize_odd_kernel<FMT, false, true, 8>)
+                                  : (a.sr ? quantize_odd_kernel<FMT, true, false, 8> : quantize_odd_kernel<FMT, false, false, 8>))
+                        : (a.line ? (a.sr ? quantize_odd_kernel<FMT, true, true, 16> : quantize_odd_kernel<FMT, false, true, 16>)
+                                  : (a.sr ? quantize_odd_kernel<FMT, true, false, 16> : quantize_odd_kernel<FMT, false, false, 16>));
     return launch_pdl(kernel, dim3((unsigned)items), dim3(QT_THREADS), 0, s, a, strips, Ct);
   }
   static bool attr_set = false;

@@ -1,6 +1,6 @@
 """Quantizer of sources whose positions are no multiple of four (needs a B200): the staged-run kernel (at most 25 positions) and the
-odd-size kernel at the edges of their ranges and of their items (16 positions, 32 rows, 32 channels), every element format, both
-block shapes, stochastic rounding.  Codes and scales are the oracle's bit for bit."""
+odd-size kernel at the edges of their ranges and of their items (8 or 16 positions, 32 rows, 32 channels), every element format,
+both block shapes, stochastic rounding.  Codes and scales are the oracle's bit for bit."""
 import numpy as np
 import pytest
 
@@ -11,10 +11,12 @@ from parity_util import assert_same_bytes, dev
 pytestmark = pytest.mark.gpu
 
 FMTS = [mq.E4M3, mq.E5M2, mq.E2M1, mq.E3M2, mq.E2M3, mq.E3M2_P6]
-# weights [C_out][C_in][Kh][Kw]: one tap, two, 3x3, 5x5 (the most staged), and 3x9 = 27 and 7x7 (odd-size kernel)
-W_SHAPES = [(3, 40, 1, 1), (33, 32, 1, 2), (70, 37, 3, 3), (32, 64, 5, 5), (31, 35, 3, 9), (16, 48, 7, 7)]
-# activations N, C, H, W: 30, 31, 33 and 47 positions; ragged rows and channels
-X_SHAPES = [(40, 48, 5, 6), (33, 35, 1, 31), (5, 96, 3, 11), (64, 20, 1, 47)]
+# weights [C_out][C_in][Kh][Kw]: one tap and two (staged runs), 3x3, 5x5, 27 and 49 taps (items of 8 positions); then enough tiles to
+# leave the 8-position items: staged runs of 9 and 25 taps, items of 16
+W_SHAPES = [(3, 40, 1, 1), (33, 32, 1, 2), (70, 37, 3, 3), (32, 64, 5, 5), (31, 35, 3, 9), (16, 48, 7, 7),
+            (3, 9573, 3, 3), (35, 2400, 5, 5), (5, 1500, 7, 7)]
+# activations N, C, H, W: 15, 30, 31, 33 and 47 positions, ragged rows and channels; then items of 16 positions
+X_SHAPES = [(70, 36, 3, 5), (40, 48, 5, 6), (33, 35, 1, 31), (5, 96, 3, 11), (64, 20, 1, 47), (3, 2380, 1, 31), (33, 1000, 3, 11)]
 
 
 def _case(kind, shape):
