@@ -965,7 +965,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   __syncthreads();
   if (DUO) cluster_sync_all();   // both blocks' barriers and tensor memory exist before anything crosses over
   tc_fence_after_sync();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
   pdl_wait();   // set-up above touched only shared memory, tensor memory and the kernel parameters
 
   // loader warps: (kind, parity of the stages it serves)
@@ -998,7 +998,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       const uint32_t row_bytes = lkind == 1 ? (uint32_t)(DUO ? p.BN / 2 : p.BN) * KB : (uint32_t)(p.TW * p.TN) * (p.a_tx34 ? KB / 4u * 3u : (uint32_t)KB);
       constexpr int SFA_STEP = 512 * SPA;
       const int sfb_step = SFA_STEP * atoms_b;
-      for (unsigned i = 0, t; (t = tile_of_iter(p, i)) < total && !*abort_flag; ++i) {
+      for (unsigned i = 0, t; (t = tile_of_iter(p, i)) < total && !warp_flag(abort_flag); ++i) {
         const Tile tile = decode_tile(p, t);
         TapWalk<MODE> tw;
         tw.init(p, tile);
@@ -1038,7 +1038,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             }
             uint8_t* sa = smem + (size_t)s * stage_bytes;
             uint8_t* sb = sa + A_STAGE_BYTES;
-            if (!mbar_wait(&empty[s], phase ^ 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
+            if (!mbar_wait_warp(&empty[s], phase ^ 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
             if (DUO) {
               // both blocks' copies count on the leader's barrier; its loaders announce the bytes of both
               if (elect_one()) {
@@ -1100,13 +1100,13 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       for (int i = 0; i < 4; ++i) idesc_id[i] = idesc_with_sf_ids(p.idesc, i, i);
       const bool self_cp = !FP4 || p.mma_cp;
       uint32_t s = 0, phase = 0, tcount = 0;
-      for (unsigned t; (t = tile_of_iter(p, tcount)) < total && !*abort_flag; ++tcount) {
+      for (unsigned t; (t = tile_of_iter(p, tcount)) < total && !warp_flag(abort_flag); ++tcount) {
         const Tile tile = decode_tile(p, t);
         TapWalk<MODE> tw;
         tw.init(p, tile);
         const int Q = tw.chunks(p);
         const int acc = acc_index(p, tcount);
-        if (!mbar_wait(&tempty[acc], acc_phase(p, tcount) ^ 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
+        if (!mbar_wait_warp(&tempty[acc], acc_phase(p, tcount) ^ 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
         tc_fence_after_sync();
         const uint32_t d_tmem = tmem + acc * p.BN;
         uint32_t accumulate = 0;
@@ -1116,7 +1116,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           // E2M1: the scale copier signals sffull[s] once the stage's scale vectors are in TMEM.  8-bit operands: this
           // warp waits for the stage itself and its lane issues the (three) scale copies right before the MMAs that
           // read them - same thread, so the tensor pipe keeps the order, and no copy queues behind MMAs issued earlier.
-          if (!mbar_wait(self_cp ? &full[s] : &sffull[s], phase, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
+          if (!mbar_wait_warp(self_cp ? &full[s] : &sffull[s], phase, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
           tc_fence_after_sync();
           const uint32_t so = s * stage16;
           const uint32_t sfa_t = sf_base + s * SFC, sfb_t = sfa_t + SFB_OFF;
@@ -1182,13 +1182,13 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       const uint64_t sfb_desc0 = smem_desc(sf_desc, smem_u32(smem + A_STAGE_BYTES + b_stage_bytes + SFA_B));
       uint32_t s = 0, phase = 0;
       bool alive = true;
-      for (unsigned i = 0, t; (t = tile_of_iter(p, i)) < total && alive && !*abort_flag; ++i) {
+      for (unsigned i = 0, t; (t = tile_of_iter(p, i)) < total && alive && !warp_flag(abort_flag); ++i) {
         const Tile tile = decode_tile(p, t);
         TapWalk<MODE> tw;
         tw.init(p, tile);
         const int Q = tw.chunks(p);
         for (int q0 = 0; q0 < Q; q0 += G) {
-          if (!mbar_wait(&full[s], phase, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; alive = false; break; }
+          if (!mbar_wait_warp(&full[s], phase, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; alive = false; break; }
           tc_fence_after_sync();
           const uint32_t so = s * stage16;
           const uint32_t sfa_t = sf_base + s * SFC, sfb_t = sfa_t + SFB_OFF;
@@ -1362,7 +1362,7 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
   // TMEM columns: accumulators, the resident weight scale vectors (16 per chunk), then 8 per chunk per stage
   const uint32_t sfb_base = tmem + p.n_acc * p.BN;
   const uint32_t sfa_base = sfb_base + (uint32_t)nsf * 16;
@@ -1373,12 +1373,12 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     {
       uint32_t s = 0, phase = 0, bcount = 0;
       int cur_ct = -1;
-      for (unsigned t = blockIdx.x; t < total && !*abort_flag; t += gridDim.x) {
+      for (unsigned t = blockIdx.x; t < total && !warp_flag(abort_flag); t += gridDim.x) {
         const Tile tile = decode_tile(p, t);
         const int ct = tile.ct;
         if (!p.fused && ct != cur_ct) {
           // new weight tile: wait until the MMAs of the previous one have retired, then one copy of image + scales
-          if (bcount > 0 && !mbar_wait(bempty, (bcount - 1) & 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
+          if (bcount > 0 && !mbar_wait_warp(bempty, (bcount - 1) & 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
           if (elect_one()) {
             mbar_arrive_expect_tx(bfull, (uint32_t)(b_bytes + sfb_bytes));
             bulk_load(smem, p.b_img + (size_t)ct * b_bytes, b_bytes, bfull);
@@ -1387,7 +1387,7 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
           __syncwarp();
           cur_ct = ct; ++bcount;
         }
-        if (!mbar_wait(&empty[s], phase ^ 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
+        if (!mbar_wait_warp(&empty[s], phase ^ 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
         uint8_t* sa = stage0 + (size_t)s * stage_bytes;
         // first source pixel of the halo: forward (h - ph, w0 - pw); input gradient (h + ph - (Kh-1), w0 + pw - (Kw-1))
         const int hs = MODE == MQ_OP_FWD ? tile.h - p.ph : tile.h + p.ph - (p.Kh - 1);
@@ -1417,16 +1417,16 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
 #pragma unroll
       for (int q = 0; q < TU; ++q) { ta[q] = tap_a[q]; tb[q] = tap_b[q]; }
       const uint32_t acc_mask = (uint32_t)p.n_acc - 1, acc_shift = (uint32_t)p.n_acc - 1;   // n_acc is 1 or 2
-      for (unsigned t = blockIdx.x; t < total && !*abort_flag; t += gridDim.x, ++tcount) {
+      for (unsigned t = blockIdx.x; t < total && !warp_flag(abort_flag); t += gridDim.x, ++tcount) {
         const int ct = p.tiles_c == 1 ? 0 : (int)((t / tiles_per_c) % (unsigned)p.tiles_c);
         const bool new_b = ct != cur_ct;
         if (new_b) {
-          if (!mbar_wait(bfull, bcount & 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
+          if (!mbar_wait_warp(bfull, bcount & 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
           cur_ct = ct; ++bcount;
         }
         const int acc = (int)(tcount & acc_mask);
-        if (!mbar_wait(&tempty[acc], ((tcount >> acc_shift) & 1) ^ 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
-        if (!mbar_wait(p.mma_cp ? &full[s] : &sffull[s], phase, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
+        if (!mbar_wait_warp(&tempty[acc], ((tcount >> acc_shift) & 1) ^ 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
+        if (!mbar_wait_warp(p.mma_cp ? &full[s] : &sffull[s], phase, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
         tc_fence_after_sync();
         const uint32_t d_tmem = tmem + acc * p.BN;
         const uint32_t sa16 = smem_u32(stage0 + (size_t)s * stage_bytes) >> 4;
@@ -1490,14 +1490,14 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       const uint64_t sf_desc = smem_desc_base(0, 128, 0);
       uint32_t s = 0, phase = 0, bcount = 0;
       int cur_ct = -1;
-      for (unsigned t = blockIdx.x; t < total && !*abort_flag; t += gridDim.x) {
+      for (unsigned t = blockIdx.x; t < total && !warp_flag(abort_flag); t += gridDim.x) {
         const int ct = p.tiles_c == 1 ? 0 : (int)((t / tiles_per_c) % (unsigned)p.tiles_c);
         const bool new_b = ct != cur_ct;
         if (new_b) {
-          if (!p.fused && !mbar_wait(bfull, bcount & 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
+          if (!p.fused && !mbar_wait_warp(bfull, bcount & 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
           cur_ct = ct; ++bcount;
         }
-        if (!mbar_wait(&full[s], phase, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
+        if (!mbar_wait_warp(&full[s], phase, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
         tc_fence_after_sync();
         if (elect_one()) {
         if (new_b) {

@@ -298,8 +298,8 @@ __device__ __forceinline__ void build_stage_scales(const WgradTcParams& p, uint8
 #pragma unroll
       for (int k = 0; k < 4; ++k) c4[k] = __shfl_sync(0xffffffffu, w1, 4 * k);
     }
-    if (*abort_flag) return;
-    if (!mbar_wait(&empty[s], phase ^ 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; return; }
+    if (warp_flag(abort_flag)) return;
+    if (!mbar_wait_warp(&empty[s], phase ^ 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; return; }
     uint8_t* dst = smem + (size_t)s * p.stage_bytes + sf_off + lane * 16;
     *reinterpret_cast<uint4*>(dst) = make_uint4(a4[0], a4[1], a4[2], a4[3]);
     *reinterpret_cast<uint4*>(dst + 1024) = make_uint4(b4[0], b4[1], b4[2], b4[3]);
@@ -383,7 +383,7 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   __syncthreads();
   if (CTA2) cluster_sync_all();   // both blocks' barriers and tensor memory exist before anything crosses over
   tc_fence_after_sync();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
   pdl_wait();   // set-up above touched only shared memory, tensor memory and the kernel parameters
 
   // ------------------------------------------------------------------ loaders
@@ -438,8 +438,8 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       const int wo0 = wg * p.KPX;
       const int xw = wo0 * p.sw + kw - p.pw, xh = ho * p.sh + kh - p.ph;
       const int nrow = nc * p.BPP * 32;
-      if (*abort_flag) break;
-      if (!mbar_wait(&empty[s], phase ^ 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
+      if (warp_flag(abort_flag)) break;
+      if (!mbar_wait_warp(&empty[s], phase ^ 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
       if (elect_one()) {
         if (rank == 0) mbar_arrive_expect_tx(bar, my_bytes);
         if (CTA2) {
@@ -534,9 +534,9 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       uint32_t ss = 0, es = 0, ephase = 0;   // scale slot of this stage; stage (and its parity) whose MMAs used that slot last
 #pragma unroll 1
       for (int i = 0; i < nst; ++i) {   // another role's abort shows here as this thread's own bounded wait running out
-        if (!mbar_wait((FP4 && !p.mma_cp) ? &sffull[s] : &full[s], phase, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
+        if (!mbar_wait_warp((FP4 && !p.mma_cp) ? &sffull[s] : &full[s], phase, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
         if (FP4 && p.mma_cp && p.sf_slots < p.stages && i >= p.sf_slots) {
-          if (!mbar_wait(&empty[es], ephase, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
+          if (!mbar_wait_warp(&empty[es], ephase, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
           if (++es == (uint32_t)p.stages) { es = 0; ephase ^= 1; }
         }
         tc_fence_after_sync();
@@ -619,10 +619,10 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       uint32_t s = 0, phase = 0;
       uint32_t ss = 0, es = 0, ephase = 0;   // see the MMA issuer
 #pragma unroll 1
-      for (int i = 0; i < nst && !*abort_flag; ++i) {
-        if (!mbar_wait(&full[s], phase, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
+      for (int i = 0; i < nst && !warp_flag(abort_flag); ++i) {
+        if (!mbar_wait_warp(&full[s], phase, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
         if (p.sf_slots < p.stages && i >= p.sf_slots) {
-          if (!mbar_wait(&empty[es], ephase, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
+          if (!mbar_wait_warp(&empty[es], ephase, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
           if (++es == (uint32_t)p.stages) { es = 0; ephase ^= 1; }
         }
         tc_fence_after_sync();
