@@ -233,8 +233,8 @@ mq_status mq_conv_bwd_data_static(const mq_conv_desc* desc, const mq_qtensor* wq
  *                      layouts of N x C_in x H x W (codes [H][W][N][C_in_p], scales [H][W][ceil(N/32)][C_in_p/32]).
  * Arithmetic of the emitted tensor: exactly mq_quantize's (tile amax over valid elements of the fp32 result, E8M0 floor
  * rule, round-to-nearest-even, saturating, padded channels code 0) applied to the fp32-accumulated GEMM result.
- * Square blocks only.  Layers the tensor-core kernels do not take (a tap's channel row not a multiple of 32 bytes, an
- * E2M1 operand mixed with a one-byte format) give the same result in two launches inside the call: the CUDA-core GEMM
+ * Square blocks only.  Layers the tensor-core kernels do not take (an E2M1 operand mixed with a one-byte format; the paper's
+ * format with a channel count that is no multiple of 64) give the same result in two launches inside the call: the CUDA-core GEMM
  * writes fp32 into the workspace and the quantizer, applying the activation, reads it back.
  * workspace: ws_bytes >= mq_conv_mx_workspace_size(desc, op, fmt of the first operand, fmt of the second). */
 mq_status mq_conv_mx_workspace_size(const mq_conv_desc* desc, int op, int fmt_a, int fmt_b, size_t* bytes);
