@@ -177,16 +177,13 @@ __device__ __forceinline__ void epilogue_role(const ConvTcParams& p, uint32_t tm
     const long long cs = (long long)p.Hd * p.Wd;
     const float os = out_scale_of(p);
     uint32_t tcount = 0;
-    for (unsigned t = blockIdx.x; t < total && !*abort_flag; t += gridDim.x, ++tcount) {
+    for (unsigned t = blockIdx.x; t < total && !warp_flag(abort_flag); t += gridDim.x, ++tcount) {
       const Tile tile = decode_tile(p, t);
       TapWalk<MODE> tw;
       tw.init(p, tile);
       const int Q = tw.chunks(p);
       const int acc = acc_index(p, tcount);
-      bool ok = true;
-      if (lane == 0) ok = mbar_wait(&tfull[acc], acc_phase(p, tcount), p.status, MQ_ERR_TIMEOUT);
-      ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-      if (!ok) { *abort_flag = 1; break; }
+      if (!mbar_wait_warp(&tfull[acc], acc_phase(p, tcount), p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
       tc_fence_after_sync();
       int yo, xo;
       if (MODE == MQ_OP_FWD) { yo = tile.h; xo = tile.w0 + tw_; }
@@ -254,16 +251,13 @@ __device__ __forceinline__ void epilogue_snap_role(const ConvTcParams& p, uint32
     const long long cs = (long long)p.Hd * p.Wd;
     const float os = out_scale_of(p);
     uint32_t tcount = 0;
-    for (unsigned t = blockIdx.x; t < total && !*abort_flag; t += gridDim.x, ++tcount) {
+    for (unsigned t = blockIdx.x; t < total && !warp_flag(abort_flag); t += gridDim.x, ++tcount) {
       const Tile tile = decode_tile(p, t);
       TapWalk<MODE> tw;
       tw.init(p, tile);
       const int Q = tw.chunks(p);
       const int acc = acc_index(p, tcount);
-      bool ok = true;
-      if (lane == 0) ok = mbar_wait(&tfull[acc], acc_phase(p, tcount), p.status, MQ_ERR_TIMEOUT);
-      ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-      if (!ok) { *abort_flag = 1; break; }
+      if (!mbar_wait_warp(&tfull[acc], acc_phase(p, tcount), p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
       tc_fence_after_sync();
       uint32_t v[128];
       if (Q > 0) {
@@ -325,15 +319,12 @@ __device__ __forceinline__ void epilogue_pair_role(const ConvTcParams& p, uint32
     const long long cs = (long long)p.Hd * p.Wd;
     const float os = out_scale_of(p);
 #pragma unroll 1
-    for (unsigned j = 0, t; (t = tile_of_iter(p, 2 * j)) < total && !*abort_flag; ++j) {
+    for (unsigned j = 0, t; (t = tile_of_iter(p, 2 * j)) < total && !warp_flag(abort_flag); ++j) {
       const Tile t0 = decode_tile(p, t), t1 = decode_tile(p, t + 1);
       TapWalk<MODE> w0, w1;
       w0.init(p, t0); w1.init(p, t1);
       const int Q0 = w0.chunks(p), Q1 = w1.chunks(p);
-      bool ok = true;
-      if (lane == 0) ok = mbar_wait(&tfull[0], j & 1, p.status, MQ_ERR_TIMEOUT) && mbar_wait(&tfull[1], j & 1, p.status, MQ_ERR_TIMEOUT);
-      ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-      if (!ok) { *abort_flag = 1; break; }
+      if (!mbar_wait_warp(&tfull[0], j & 1, p.status, MQ_ERR_TIMEOUT) || !mbar_wait_warp(&tfull[1], j & 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
       tc_fence_after_sync();
       const int ch = (int)fdiv((unsigned)t0.cls, p.sw, p.m_sw);
       const int yo = ch + p.sh * t0.h, xo = p.sw * (t0.w0 + tw_);     // even column; the odd class writes xo + 1
@@ -386,15 +377,12 @@ __device__ __forceinline__ void epilogue_pair_snap_role(const ConvTcParams& p, u
     const long long cs = (long long)p.Hd * p.Wd;
     const float os = out_scale_of(p);
 #pragma unroll 1
-    for (unsigned j = 0, t; (t = tile_of_iter(p, 2 * j)) < total && !*abort_flag; ++j) {
+    for (unsigned j = 0, t; (t = tile_of_iter(p, 2 * j)) < total && !warp_flag(abort_flag); ++j) {
       const Tile t0 = decode_tile(p, t), t1 = decode_tile(p, t + 1);
       TapWalk<MODE> w0, w1;
       w0.init(p, t0); w1.init(p, t1);
       const int Q0 = w0.chunks(p), Q1 = w1.chunks(p);
-      bool ok = true;
-      if (lane == 0) ok = mbar_wait(&tfull[0], j & 1, p.status, MQ_ERR_TIMEOUT) && mbar_wait(&tfull[1], j & 1, p.status, MQ_ERR_TIMEOUT);
-      ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-      if (!ok) { *abort_flag = 1; break; }
+      if (!mbar_wait_warp(&tfull[0], j & 1, p.status, MQ_ERR_TIMEOUT) || !mbar_wait_warp(&tfull[1], j & 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
       tc_fence_after_sync();
       uint32_t v0[64], v1[64];
       const uint32_t taddr = tmem + ((uint32_t)(32 * quad) << 16) + cbeg;
@@ -657,11 +645,10 @@ __device__ __forceinline__ void epilogue_mx_role(const ConvTcParams& p, unsigned
       tw.init(p, tile);
       const int Q = tw.chunks(p);
       const int acc = acc_index(p, tcount);
-      bool ok = true;
-      if (lane == 0) ok = !*abort_flag && mbar_wait(&tfull[acc], acc_phase(p, tcount), p.status, MQ_ERR_TIMEOUT);
+      const bool ok = !warp_flag(abort_flag) && mbar_wait_warp(&tfull[acc], acc_phase(p, tcount), p.status, MQ_ERR_TIMEOUT);
       // the four warps of a half leave together or not at all: they meet at barriers inside the tile
       // (one-column tiles have no barriers inside: each warp decides for itself)
-      if (p.TW > 1 ? half_any(half, !ok) : __shfl_sync(0xffffffffu, ok ? 0 : 1, 0) != 0) { *abort_flag = 1; break; }
+      if (p.TW > 1 ? half_any(half, !ok) : !ok) { *abort_flag = 1; break; }
       tc_fence_after_sync();
       int yo, xo;
       if (MODE == MQ_OP_FWD) { yo = tile.h; xo = tile.w0 + tw_; }
@@ -744,16 +731,13 @@ __device__ __forceinline__ void epilogue_tma_role(const ConvTcParams& p, const C
     const int hrow = lane;   // the [H][W][N][C] store's box walks (sample, column) in the rows' own order
     const float os = out_scale_of(p);
     uint32_t tcount = 0;
-    for (unsigned t = blockIdx.x; t < total && !*abort_flag; t += gridDim.x, ++tcount) {
+    for (unsigned t = blockIdx.x; t < total && !warp_flag(abort_flag); t += gridDim.x, ++tcount) {
       const Tile tile = decode_tile(p, t);
       TapWalk<MODE> tw;
       tw.init(p, tile);
       const int Q = tw.chunks(p);
       const int acc = acc_index(p, tcount);
-      bool ok = true;
-      if (lane == 0) ok = mbar_wait(&tfull[acc], acc_phase(p, tcount), p.status, MQ_ERR_TIMEOUT);
-      ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-      if (!ok) { *abort_flag = 1; break; }
+      if (!mbar_wait_warp(&tfull[acc], acc_phase(p, tcount), p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
       tc_fence_after_sync();
       const int cls_h = MODE == MQ_OP_FWD ? 0 : (int)fdiv((unsigned)tile.cls, p.sw, p.m_sw);
       const int yo = MODE == MQ_OP_FWD ? tile.h : cls_h + p.sh * tile.h;
@@ -829,16 +813,13 @@ __device__ __forceinline__ void epilogue_tma_snap_role(const ConvTcParams& p, co
     const int hrow = lane;
     const float os = out_scale_of(p);
     uint32_t tcount = 0;
-    for (unsigned t = blockIdx.x; t < total && !*abort_flag; t += gridDim.x, ++tcount) {
+    for (unsigned t = blockIdx.x; t < total && !warp_flag(abort_flag); t += gridDim.x, ++tcount) {
       const Tile tile = decode_tile(p, t);
       TapWalk<MODE> tw;
       tw.init(p, tile);
       const int Q = tw.chunks(p);
       const int acc = acc_index(p, tcount);
-      bool ok = true;
-      if (lane == 0) ok = mbar_wait(&tfull[acc], acc_phase(p, tcount), p.status, MQ_ERR_TIMEOUT);
-      ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-      if (!ok) { *abort_flag = 1; break; }
+      if (!mbar_wait_warp(&tfull[acc], acc_phase(p, tcount), p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
       tc_fence_after_sync();
       uint32_t v[128];
       if (Q > 0) {

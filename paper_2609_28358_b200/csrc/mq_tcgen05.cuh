@@ -57,7 +57,8 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, unsign
 // keeps the loops around it - and the operands of the copy and MMA instructions inside - in the uniform datapath.  (One pipeline
 // stage of the conv GEMMs is ~520 cycles of MMAs, but 590-850 cycles of the issuing warp's own dependent instructions; with
 // these waits, us, before / after: E2M1 512 channels 14x14 N = 256: fwd 71 / 67, dW 90 / 86; 3x3 stride 2, 16 channels at
-// 320x320, input gradient 90 / 79; 256 channels 28x28 E4M3 105.5 / 104.)
+// 320x320, input gradient 90 / 79; 256 channels 28x28 E4M3 105.5 / 104.  In the epilogue roles too: that input gradient 79 / 74,
+// 256 channels 28x28 stride 2 E2M1 79 / 71.)
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, unsigned int* status, unsigned int tag) {
 #pragma unroll 1
   for (uint32_t i = 0; i < kWaitLimit; ++i) {
