@@ -131,14 +131,7 @@ struct TapWalk {
   __device__ __forceinline__ int chunks(const ConvTcParams& p) const { return nkh * nkw * p.cpt; }
 };
 // position inside a TapWalk: (ia, ib, cc) with cc the chunk of the tap's channel row
-struct ChunkPos {
-  int ia, ib, cc;
-  __device__ __forceinline__ void reset() { ia = 0; ib = 0; cc = 0; }
-  template <int MODE>
-  __device__ __forceinline__ void advance(const TapWalk<MODE>& w, int cpt) {
-    if (++cc == cpt) { cc = 0; if (++ib == w.nkw) { ib = 0; ++ia; } }
-  }
-};
+struct ChunkPos { int ia, ib, cc; };
 template <int MODE>
 __device__ __forceinline__ int src_h(const TapWalk<MODE>& w, const ChunkPos& c) { return MODE == MQ_OP_FWD ? w.hs0 + c.ia : w.hs0 - c.ia; }
 template <int MODE>
