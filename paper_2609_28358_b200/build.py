@@ -5,7 +5,7 @@
 Each ``csrc/*.cu`` is compiled to an object under ``csrc/build/`` (skipped when up to date) and the
 objects are linked into ``paper_2609_28358_b200/libmq.so``.  nvcc cross-compiles: no GPU is needed.
 ``csrc/mq_torch.cpp`` (host code only: the Python binding's marshalling) becomes ``_mq_torch.so`` beside it, linked to
-``libmq.so`` and PyTorch's libraries.
+``libmq.so`` and PyTorch's libraries; without PyTorch the library is built alone.
 """
 from __future__ import annotations
 
@@ -37,38 +37,45 @@ def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(OBJ, exist_ok=True)
     srcs = sorted(glob.glob(os.path.join(CSRC, "*.cu")))
     hdr = _newest_header()
-    cmd, binding_obj = _compile_binding(force)
-    jobs = [] if cmd is None else [cmd]
-    objs = []
+    jobs, objs = [], []
     for s in srcs:
         o = os.path.join(OBJ, os.path.basename(s)[:-3] + ".o")
         objs.append(o)
         if force or not os.path.exists(o) or os.path.getmtime(o) < max(os.path.getmtime(s), hdr):
             cmd = [NVCC] + FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-c", s, "-o", o]
             jobs.append(cmd)
+    cmd, binding_obj = _compile_binding(force)
 
     def run(cmd):
         r = subprocess.run(cmd, capture_output=True, text=True)
-        return cmd, r
+        if verbose or r.returncode != 0:
+            sys.stderr.write(" ".join(cmd) + "\n" + r.stdout + r.stderr)
+        if r.returncode != 0:
+            raise RuntimeError("compilation failed for " + cmd[-3])
 
-    with ThreadPoolExecutor(max_workers=min(8, max(1, len(jobs)))) as ex:
-        for cmd, r in ex.map(run, jobs):
-            if verbose or r.returncode != 0:
-                sys.stderr.write(" ".join(cmd) + "\n" + r.stdout + r.stderr)
-            if r.returncode != 0:
-                raise RuntimeError("compilation failed for " + cmd[-3])
+    with ThreadPoolExecutor(max_workers=min(9, len(jobs) + 1)) as ex:
+        binding = ex.submit(run, cmd) if cmd else None      # its outcome is asked for after the library has been linked
+        list(ex.map(run, jobs))
     if jobs or not os.path.exists(LIB) or any(os.path.getmtime(o) > os.path.getmtime(LIB) for o in objs):
         tmp = LIB + ".tmp.%d" % os.getpid()
         subprocess.check_call([NVCC, "-shared", "-o", tmp] + objs + ["-lcudart"])
         os.replace(tmp, LIB)
+    if binding_obj is None:
+        sys.stderr.write("PyTorch is not installed: its binding (_mq_torch.so) is not built\n")
+        return LIB
+    if binding:
+        binding.result()
     if not os.path.exists(BINDING) or os.path.getmtime(binding_obj) > os.path.getmtime(BINDING):
         _link_binding(binding_obj)
     return LIB
 
 
 def _compile_binding(force: bool):
-    """(command, object) of the binding's compilation; the command is None when the object is up to date."""
-    import torch
+    """(command, object) of the binding's compilation; the command is None when the object is up to date, both without PyTorch."""
+    try:
+        import torch
+    except ImportError:
+        return None, None
 
     src, obj = os.path.join(CSRC, "mq_torch.cpp"), os.path.join(OBJ, "mq_torch.o")
     newest = max(os.path.getmtime(p) for p in (src, os.path.join(ROOT, "include", "mq.h"), os.path.abspath(__file__)))
