@@ -65,9 +65,18 @@ def build(force: bool = False, verbose: bool = False) -> str:
         return LIB
     if binding:
         binding.result()
+        with open(binding_obj + ".of", "w") as f:
+            f.write(_binding_of())
     if not os.path.exists(BINDING) or os.path.getmtime(binding_obj) > os.path.getmtime(BINDING):
         _link_binding(binding_obj)
     return LIB
+
+
+def _binding_of() -> str:
+    """What a compiled binding belongs to, kept beside its object: it works with this build of PyTorch and this Python only."""
+    import torch
+
+    return " ".join(str(v) for v in (torch.__version__, torch.version.git_version, os.path.abspath(torch.__file__), sysconfig.get_config_var("SOABI"), CXX))
 
 
 def _compile_binding(force: bool):
@@ -79,7 +88,8 @@ def _compile_binding(force: bool):
 
     src, obj = os.path.join(CSRC, "mq_torch.cpp"), os.path.join(OBJ, "mq_torch.o")
     newest = max(os.path.getmtime(p) for p in (src, os.path.join(ROOT, "include", "mq.h"), os.path.abspath(__file__)))
-    if not force and os.path.exists(obj) and os.path.getmtime(obj) >= newest:
+    made_for = open(obj + ".of").read() if os.path.exists(obj + ".of") else ""
+    if not force and os.path.exists(obj) and os.path.getmtime(obj) >= newest and made_for == _binding_of():
         return None, obj
     t = os.path.join(os.path.dirname(os.path.abspath(torch.__file__)), "include")
     cuda = os.path.dirname(os.path.dirname(os.path.abspath(NVCC)))

@@ -41,3 +41,13 @@ def test_the_library_needs_no_pytorch(made, monkeypatch):
 def test_the_binding_is_built_where_pytorch_is(made):
     assert {"libmq.so", "mq_torch.o", "_mq_torch.so"} <= made()
     assert made() == set()                               # up to date
+
+
+def test_the_binding_follows_its_pytorch_and_python(made, monkeypatch):
+    import torch
+
+    made()
+    monkeypatch.setattr(torch, "__version__", "0.0.0+other")
+    assert made() == {"mq_torch.o", "_mq_torch.so"} and made() == set()
+    monkeypatch.setattr(build.sysconfig, "get_config_var", lambda name: "cpython-other")
+    assert made() == {"mq_torch.o", "_mq_torch.so"} and made() == set()
