@@ -3,12 +3,14 @@
 // A small layer's call is two or three launches of a few microseconds of GPU work, so what it costs is the host: marshalled in
 // Python through ctypes (argument structures, size queries, two to three torch.empty, the stream object) a quantizer call took
 // 17.1 us and a weight gradient 26.8 us of host time, 4.3 and 8.8 us of them in the library.  Here the same steps run natively:
-// sizes come from the library, buffers from at::empty on the operands' device, the stream is PyTorch's current one, and the
-// interpreter lock is released around the library call (as ctypes does).  Nothing is kept between calls.
+// sizes come from the library, buffers from at::empty on the operands' device and the call's stream (see Launch), and the
+// interpreter lock is released around the allocations and the library call.  Nothing is kept between calls.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
 #include <ATen/ops/empty.h>
+#include <c10/cuda/CUDACachingAllocator.h>
+#include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Dtype.h>
 #include <torch/csrc/Exceptions.h>
@@ -81,16 +83,57 @@ int dtype_code(at::ScalarType t) {
   PyErr_SetString(PyExc_KeyError, "element type of an unquantized tensor: torch.float32 or torch.bfloat16");
   throw PyFail{};
 }
-void* stream_of(PyObject* o) {
-  if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
+cudaStream_t stream_of(PyObject* o) {
   PyObject* v = PyObject_GetAttr(o, s_stream);
   if (!v) throw PyFail{};
   const unsigned long long p = PyLong_AsUnsignedLongLong(v);
   Py_DECREF(v);
   if (p == (unsigned long long)-1 && PyErr_Occurred()) throw PyFail{};
-  return reinterpret_cast<void*>(p);
+  const auto s = reinterpret_cast<cudaStream_t>(p);
+  return s == cudaStreamLegacy ? nullptr : s;
 }
+// the interpreter lock is not held while one of these lives
+class Unlocked {
+ public:
+  Unlocked() : state_(PyEval_SaveThread()) {}
+  ~Unlocked() { PyEval_RestoreThread(state_); }
+  Unlocked(const Unlocked&) = delete;
+  Unlocked& operator=(const Unlocked&) = delete;
+
+ private:
+  PyThreadState* state_;
+};
+// Where a call runs: the operands' device, and PyTorch's current stream there or the one the caller names.  What the call
+// allocates comes from the pool of ITS stream, for PyTorch's allocator orders a block's uses by the stream it was given out
+// for: a block of another stream's pool might still be in use there when the kernels write it, and a workspace dropped at the
+// end of the call be given out there while they run.
+class Launch {
+ public:
+  void* stream = nullptr;
+  Launch(PyObject* given, const at::Device& dev) {
+    if (dev.is_cuda()) device_.emplace(dev);
+    if (given == Py_None) { stream = c10::cuda::getCurrentCUDAStream().stream(); return; }
+    const cudaStream_t s = stream_of(given);
+    stream = s;
+    if (!dev.is_cuda()) return;
+    const c10::cuda::CUDAStream current = c10::cuda::getCurrentCUDAStream();
+    if (current.stream() == s) return;
+    pool_.emplace(c10::cuda::getStreamFromExternal(s, dev.index()));
+    callers_ = current;
+  }
+  // A result leaves with the caller, who may read it on the current stream (ordered after the call's) and drop it: its block
+  // then waits for that stream too before it is given out again.
+  void hand_out(const at::Tensor& t) const {
+    if (callers_ && t.defined() && t.is_cuda()) c10::cuda::CUDACachingAllocator::recordStream(t.storage().data_ptr(), *callers_);
+  }
+
+ private:
+  std::optional<c10::cuda::CUDAGuard> device_;
+  std::optional<c10::cuda::CUDAStreamGuard> pool_;
+  std::optional<c10::cuda::CUDAStream> callers_;
+};
 at::Tensor fresh(at::IntArrayRef shape, at::ScalarType t, const at::Device& dev, bool fill) {
+  Unlocked u;
   at::Tensor r = at::empty(shape, at::TensorOptions().dtype(t).device(dev));
   if (fill) {
     if (at::isFloatingType(t)) r.fill_(std::numeric_limits<double>::quiet_NaN()); else r.fill_(0xA5);
@@ -145,7 +188,8 @@ struct Created {
     q.scales = scales.data_ptr<uint8_t>(); q.scales_bytes = sb;
     q.fmt = fmt; q.role = role; q.block = block;
   }
-  PyObject* to_python() {   // (codes, scales, tensor scale or None)
+  PyObject* to_python(const Launch& l) {   // (codes, scales, tensor scale or None)
+    l.hand_out(codes); l.hand_out(scales); l.hand_out(tscale);
     PyObject* t = Py_None;
     if (tscale.defined()) t = THPVariable_Wrap(tscale); else Py_INCREF(t);
     return Py_BuildValue("(NNN)", THPVariable_Wrap(codes), THPVariable_Wrap(scales), t);
@@ -170,11 +214,8 @@ struct Workspace {
 
 template <typename F>
 mq_status unlocked(F&& f) {
-  mq_status st;
-  Py_BEGIN_ALLOW_THREADS
-  st = f();
-  Py_END_ALLOW_THREADS
-  return st;
+  Unlocked u;
+  return f();
 }
 
 template <typename F>
@@ -201,6 +242,7 @@ PyObject* py_quantize(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
     require(src.is_cuda(), "src is a CUDA tensor");
     require(src.scalar_type() == at::kFloat || src.scalar_type() == at::kBFloat16, "src is float32 or bfloat16");
     require(src.is_contiguous(), "src is contiguous");
+    const Launch launch(a[10], src.device());
     std::optional<Stored> given;
     std::optional<Created> made;
     if (a[7] != Py_None) given.emplace(a[7]);
@@ -220,14 +262,14 @@ PyObject* py_quantize(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
     }
     const float* amax = a[9] != Py_None ? static_cast<const float*>(tensor_of(a[9]).data_ptr()) : nullptr;
     const bool sr = a[8] != Py_None;
-    void* s = stream_of(a[10]);
+    void* s = launch.stream;
     const void* p = src.data_ptr();
     const int dt = dtype_code(src.scalar_type());
     if (kind == 2) check("mq_quantize_ts", unlocked([&] { return mq_quantize_ts(&d, p, dt, layout, q, amax, sr ? &seed : nullptr, s); }));
     else if (kind == 1) check("mq_quantize_sr", unlocked([&] { return mq_quantize_sr(&d, p, dt, layout, q, seed, s); }));
     else check("mq_quantize", unlocked([&] { return mq_quantize(&d, p, dt, layout, q, s); }));
     if (given) Py_RETURN_NONE;
-    return made->to_python();
+    return made->to_python(launch);
   });
 }
 
@@ -237,12 +279,14 @@ PyObject* py_im2col(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
     const mq_conv_desc d = desc_of(a[0]);
     Stored x(a[1]);
     const bool fill = PyObject_IsTrue(a[5]) == 1;
+    const Launch launch(a[4], *x.device);
     size_t cb = 0, sb = 0;
     check("mq_im2col_sizes", mq_im2col_sizes(&d, x.q.fmt, x.q.block, &cb, &sb));
     at::Tensor codes = a[2] != Py_None ? tensor_of(a[2]) : fresh({(int64_t)cb}, at::kByte, *x.device, fill);
     at::Tensor scales = a[3] != Py_None ? tensor_of(a[3]) : fresh({(int64_t)sb}, at::kByte, *x.device, fill);
-    void* s = stream_of(a[4]);
-    check("mq_cbf_im2col", unlocked([&] { return mq_cbf_im2col(&d, &x.q, codes.data_ptr(), static_cast<uint8_t*>(scales.data_ptr()), s); }));
+    check("mq_cbf_im2col", unlocked([&] { return mq_cbf_im2col(&d, &x.q, codes.data_ptr(), static_cast<uint8_t*>(scales.data_ptr()), launch.stream); }));
+    if (a[2] == Py_None) launch.hand_out(codes);
+    if (a[3] == Py_None) launch.hand_out(scales);
     return Py_BuildValue("(NN)", THPVariable_Wrap(codes), THPVariable_Wrap(scales));
   });
 }
@@ -254,6 +298,7 @@ PyObject* py_conv(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
     const mq_conv_desc d = desc_of(a[1]);
     Stored qa(a[2]), qb(a[3]);
     const bool fill = PyObject_IsTrue(a[9]) == 1;
+    const Launch launch(a[7], *qa.device);
     at::Tensor out;
     if (a[4] != Py_None) out = tensor_of(a[4]);
     else {
@@ -271,11 +316,12 @@ PyObject* py_conv(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
     check("mq_workspace_size", mq_workspace_size(&d, op, qa.q.fmt, qb.q.fmt, qa.q.block, &need));
     Workspace ws(a[6], need, *qa.device, fill);
     const int dt = dtype_code(out.scalar_type());
-    void* s = stream_of(a[7]);
+    void* s = launch.stream;
     void* o = out.data_ptr();
     if (op == MQ_OP_FWD) check("mq_conv_fwd", unlocked([&] { return mq_conv_fwd(&d, &qa.q, &qb.q, o, dt, layout, ws.ptr, ws.bytes, s); }));
     else if (op == MQ_OP_BWD_DATA) check("mq_conv_bwd_data", unlocked([&] { return mq_conv_bwd_data(&d, &qa.q, &qb.q, o, dt, layout, ws.ptr, ws.bytes, s); }));
     else check("mq_conv_bwd_weight", unlocked([&] { return mq_conv_bwd_weight(&d, &qa.q, &qb.q, o, dt, layout, ws.ptr, ws.bytes, s); }));
+    if (a[4] == Py_None) launch.hand_out(out);
     return THPVariable_Wrap(out);
   });
 }
@@ -294,6 +340,7 @@ PyObject* py_conv_emit(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
       amax = t.data_ptr<float>();
     }
     Stored qa(a[2]), qb(a[3]);
+    const Launch launch(a[9], *qa.device);
     std::optional<Stored> given;
     std::optional<Created> made;
     if (a[7] != Py_None) given.emplace(a[7]);
@@ -311,13 +358,13 @@ PyObject* py_conv_emit(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
     if (ts) check("mq_conv_ts_workspace_size", mq_conv_ts_workspace_size(&d, op, &need));
     else check("mq_conv_mx_workspace_size", mq_conv_mx_workspace_size(&d, op, qa.q.fmt, qb.q.fmt, &need));
     Workspace ws(a[8], need, *qa.device, fill);
-    void* s = stream_of(a[9]);
+    void* s = launch.stream;
     if (ts && op == MQ_OP_FWD) check("mq_conv_fwd_ts", unlocked([&] { return mq_conv_fwd_ts(&d, &qa.q, &qb.q, act, amax, q, ws.ptr, ws.bytes, s); }));
     else if (ts) check("mq_conv_bwd_data_ts", unlocked([&] { return mq_conv_bwd_data_ts(&d, &qa.q, &qb.q, amax, q, ws.ptr, ws.bytes, s); }));
     else if (op == MQ_OP_FWD) check("mq_conv_fwd_mx", unlocked([&] { return mq_conv_fwd_mx(&d, &qa.q, &qb.q, act, q, ws.ptr, ws.bytes, s); }));
     else check("mq_conv_bwd_data_mx", unlocked([&] { return mq_conv_bwd_data_mx(&d, &qa.q, &qb.q, q, ws.ptr, ws.bytes, s); }));
     if (given) Py_RETURN_NONE;
-    return made->to_python();
+    return made->to_python(launch);
   });
 }
 

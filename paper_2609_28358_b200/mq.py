@@ -114,6 +114,19 @@ def _new(shape, dtype, device):
     return t
 
 
+def _result(shape, dtype, device, stream):
+    """A result's buffer from the pool of the stream that will write it (as the native calls do); the current stream, on which it
+    leaves with the caller, is noted as another user of its memory."""
+    if stream is None:
+        return _new(shape, dtype, device)
+    current = torch.cuda.current_stream(device)
+    with torch.cuda.stream(torch.cuda.ExternalStream(stream.cuda_stream, device)):
+        t = _new(shape, dtype, device)
+    if stream.cuda_stream != current.cuda_stream:
+        t.record_stream(current)
+    return t
+
+
 def qtensor_sizes(desc, role, fmt, block=TILE32):
     cb, sb = ctypes.c_size_t(), ctypes.c_size_t()
     _check("mq_qtensor_sizes", lib().mq_qtensor_sizes(ctypes.byref(_d(desc)), role, fmt, block, ctypes.byref(cb), ctypes.byref(sb)))
@@ -241,7 +254,7 @@ def conv_bwd_data_static(desc, wq, dyq, dx=None, layout=NCHW, stream=None):
     `dx` should be passed in by such callers; it is only created here for convenience when omitted."""
     d = ConvDesc(*desc)
     if dx is None:
-        dx = _new((d.N, d.C_in, d.H, d.W) if layout == NCHW else (d.H, d.W, d.N, d.C_in), torch.float32, wq.codes.device)
+        dx = _result((d.N, d.C_in, d.H, d.W) if layout == NCHW else (d.H, d.W, d.N, d.C_in), torch.float32, wq.codes.device, stream)
     a, b = wq._c(), dyq._c()
     _check("mq_conv_bwd_data_static", lib().mq_conv_bwd_data_static(ctypes.byref(_d(desc)), ctypes.byref(a), ctypes.byref(b),
                                                                   ctypes.c_void_p(dx.data_ptr()), _DTYPES[dx.dtype], layout, _stream(stream)))

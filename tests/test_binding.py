@@ -67,3 +67,49 @@ def test_caller_owned_buffers_streams_and_threads():
     with ThreadPoolExecutor(4) as ex:
         assert all(ex.map(work, range(8)))
     assert mq.last_device_status() == 0
+
+
+@pytest.mark.gpu
+def test_a_stream_that_is_not_the_current_one():
+    """Calls given a stream while another is current: neither stream's work reaches memory that the other still uses."""
+    d = inputs.conv_desc(64, 128, 28, 28, 128, 3, 1, 1)
+    x, x2, w, dy = [torch.from_numpy(f(d, s)).cuda() for f, s in ((inputs.make_x, 5), (inputs.make_x, 6), (inputs.make_w, 5), (inputs.make_dy, 5))]
+    qs = [mq.quantize(d, r, mq.E4M3, t) for r, t in enumerate((x, w, dy))]
+    q2 = mq.quantize(d, mq.ROLE_X, mq.E4M3, x2)
+    calls = [lambda **kw: mq.conv_fwd(d, qs[0], qs[1], **kw), lambda **kw: mq.conv_bwd_data(d, qs[1], qs[2], **kw), lambda **kw: mq.conv_bwd_weight(d, qs[0], qs[2], **kw),
+             lambda **kw: mq.conv_fwd_mx(d, qs[0], qs[1], mq.E4M3, **kw).codes, lambda **kw: mq.quantize(d, mq.ROLE_X, mq.E4M3, x, **kw).codes,
+             lambda **kw: mq.cbf_im2col(d, qs[0], **kw)[0], lambda **kw: mq.conv_bwd_data_static(d, qs[1], qs[2], **kw)]
+    ops = [(mq.OP_FWD, 0, 0), (mq.OP_BWD_DATA, 0, 0), (mq.OP_BWD_WEIGHT, 0, 0)]
+    sizes = [mq.workspace_size(d, *o) for o in ops] + [mq.conv_mx_workspace_size(d, mq.OP_FWD, 0, 0)]
+    want = [c() for c in calls]
+    want2 = mq.conv_fwd(d, q2, qs[1])
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for call, ref in zip(calls, want):
+        nbytes = sizes + [ref.numel() * ref.element_size()]
+        # the current stream is about to overwrite blocks of the call's sizes that were dropped just before the call
+        torch.cuda._sleep(20_000_000)
+        for n in nbytes:
+            torch.empty(n, dtype=torch.uint8, device="cuda").fill_(0xA5)
+        got = call(stream=side)
+        side.synchronize()
+        torch.cuda.synchronize()
+        assert torch.equal(got, ref)
+        # ... and blocks given out right after it, before its kernels have started
+        with torch.cuda.stream(side):
+            torch.cuda._sleep(20_000_000)
+        got = call(stream=side)
+        for n in nbytes:
+            torch.empty(n, dtype=torch.uint8, device="cuda").fill_(0xA5)
+        torch.cuda.synchronize()
+        assert torch.equal(got, ref)
+    # a result read on the current stream and dropped while that read is waiting
+    y = mq.conv_fwd(d, qs[0], qs[1], stream=side)
+    torch.cuda.current_stream().wait_stream(side)
+    torch.cuda._sleep(20_000_000)
+    z = y + 0.0
+    del y
+    y2 = mq.conv_fwd(d, q2, qs[1], stream=side)
+    torch.cuda.synchronize()
+    assert torch.equal(z, want[0]) and torch.equal(y2, want2)
+    assert mq.last_device_status() == 0
