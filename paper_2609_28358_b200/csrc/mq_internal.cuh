@@ -283,7 +283,9 @@ __device__ __forceinline__ float sr_value(float x, unsigned lo, unsigned key) {
   const float w = __uint_as_float(0x3F800000u | (rn >> 9)) - __uint_as_float(0x3F7FFFFFu);
   const float n = __fadd_ru(__fadd_ru(t, w), 8388608.f) - 8388609.f;
   const unsigned q_sub = __float_as_uint(n * __uint_as_float((unsigned)(127 + EMIN - M) << 23));
-  const unsigned q = b >= ((unsigned)(127 + EMIN) << 23) ? q_norm : q_sub;     // (beyond the largest magnitude the conversion saturates)
+  // Beyond the largest magnitude the conversion saturates.  The comparison is one of floats because a NaN has to take the second
+  // branch, whose arithmetic keeps it one: the addition above would carry its pattern into the sign, that is to -0.
+  const unsigned q = __uint_as_float(b) >= __uint_as_float((unsigned)(127 + EMIN) << 23) ? q_norm : q_sub;
   return __uint_as_float(q | (__float_as_uint(x) & 0x80000000u));
 }
 
