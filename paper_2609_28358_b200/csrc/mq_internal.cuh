@@ -314,6 +314,9 @@ __device__ __forceinline__ TsDen ts_den(float den) {
   d.sure = (in_range || !(den > 0.f)) ? 0xffffffffu : 0u;
   return d;
 }
+// fmaxf / fminf that keep a NaN
+__device__ __forceinline__ float max_nan(float a, float b) { float r; asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b)); return r; }
+__device__ __forceinline__ float min_nan(float a, float b) { float r; asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b)); return r; }
 // One element by the definition.  lo, key: as sr_value's
 template <bool SR>
 __device__ __forceinline__ unsigned ts_code_by_division(float x, float den, unsigned lo, unsigned key) {
@@ -322,17 +325,19 @@ __device__ __forceinline__ unsigned ts_code_by_division(float x, float den, unsi
   return encode2<MQ_E2M1>(q, 0.f) & 0xFu;
 }
 // Eight elements of neighbouring channels -> their codes, element 0 in the low nibble.  e0 (SR): element 0's index in the logical
-// tensor, whose channels are a.P elements apart.
+// tensor, whose channels are a.P elements apart.  A NaN product - of a NaN, or of an infinity and the 0 of a block that encodes to
+// zeros - says nothing either: the window tests let it through to the division.
 template <bool SR>
 __device__ __forceinline__ unsigned ts_codes8(const float* x, const TsDen& d, const QuantArgs& a, long long e0) {
   unsigned word = 0, sure = d.sure;
   if (!SR) {
-    // thresholds of round-to-nearest are 0.25, 0.75, 1.25, 1.75, 2.5, 3.5 and 5: patterns whose low 21 bits are zero
+    // thresholds of round-to-nearest are 0.25, 0.75, 1.25, 1.75, 2.5, 3.5 and 5: patterns whose low 21 bits are zero (and a
+    // NaN's, all ones, is one short of it)
 #pragma unroll
     for (int k = 0; k < 8; k += 2) {
       const float q0 = x[k] * d.inv, q1 = x[k + 1] * d.inv;
-      sure = min(sure, (__float_as_uint(fmaxf(fabsf(q0), 0.24f)) + 4u) << 11);
-      sure = min(sure, (__float_as_uint(fmaxf(fabsf(q1), 0.24f)) + 4u) << 11);
+      sure = min(sure, (__float_as_uint(max_nan(fabsf(q0), 0.24f)) + 4u) << 11);
+      sure = min(sure, (__float_as_uint(max_nan(fabsf(q1), 0.24f)) + 4u) << 11);
       word |= encode2<MQ_E2M1>(q0, q1) << (4 * k);
     }
     if (sure >= (8u << 11)) return word;
@@ -346,16 +351,18 @@ __device__ __forceinline__ unsigned ts_codes8(const float* x, const TsDen& d, co
       key = sr_key(a, e0);
       if ((unsigned long long)(e0 + 7ll * a.P) >> 32 != (unsigned long long)e0 >> 32) sure = 0;
     }
+    float total = 0.f;     // NaN if any product is (a float addition, on a pipe that this loop leaves idle)
 #pragma unroll
     for (int k = 7; k >= 0; --k) {
       const unsigned rn = ~sr_mix32((lo0 + (unsigned)k * (unsigned)a.P) ^ key);
-      const float q = fminf(fabsf(x[k]) * d.inv, 6.f);
+      const float q = min_nan(fabsf(x[k]) * d.inv, 6.f);
+      total += q;
       const bool below = q < 1.f;
       const unsigned sum = __float_as_uint(below ? q + 1.f : q) + (rn >> 10) + (below ? 0u - (254u << 22) : 0u - (252u << 22));
       sure = min(sure, (sum + 8u) << 10);
       word = __funnelshift_l((sum << 6) | (__float_as_uint(x[k]) & 0x80000000u), word, 4);
     }
-    if (sure >= (16u << 10)) return word;
+    if (sure >= (16u << 10) && total == total) return word;
   }
 #pragma unroll 1
   for (int k = 0; k < 8; ++k) {

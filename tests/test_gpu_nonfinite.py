@@ -52,3 +52,29 @@ def test_nan_elements(name, fmt, layout):
             assert (codes[np.isnan(x)] == NAN_CODE[fmt]).all(), np.unique(codes[np.isnan(x)])
             assert (codes[np.isposinf(x)] == top).all() and (codes[np.isneginf(x)] == top | sign).all()
     assert mq.last_device_status() == 0
+
+
+@pytest.mark.parametrize("seed", [None, 5], ids=["nearest", "stochastic"])
+@pytest.mark.parametrize("layout", [mq.NCHW, mq.HWNC], ids=["nchw", "hwnc"])
+@pytest.mark.parametrize("name", SHAPES)
+def test_paper_format(name, layout, seed):
+    """Eq. 6 of a NaN, in a block that is not zero, is the largest magnitude; in a block that encodes to zeros, as with T_scale 0 or
+    infinite, it and an infinity are zeros with their sign.  The other elements are the oracle's."""
+    import torch
+
+    b16 = (16, 16)
+    amax = lambda v: torch.tensor([v], dtype=torch.float32, device="cuda")
+    d, x = tensor(name, PATTERNS)
+    q = mq.quantize_ts(d, mq.ROLE_X, source(x, layout), src_layout=layout, amax_in=amax(3.0), seed=seed)
+    codes, scales = oracle.quantize_ts(d, mq.ROLE_X, np.nan_to_num(x, nan=0.0), b16, amax=3.0, seed=seed)[:2]
+    want = logical(mq.QTensor(torch.from_numpy(codes), None, mq.E2M1, mq.ROLE_X), x, mq.E2M1)
+    assert np.array_equal(host(q.scales), scales) and host(q.tensor_scale)[1] == np.nanmax(np.abs(x))
+    assert np.array_equal(logical(q, x, mq.E2M1), np.where(np.isnan(x), 7, want))
+    d, x = tensor(name, np.concatenate([PATTERNS, np.array([np.inf, -np.inf], np.float32).view(np.uint32)]))
+    sign = np.where(np.signbit(x), 8, 0)
+    for am in (None, 0.0, np.inf, np.nan):        # None: the tensor's own maximum, which is infinite
+        q = mq.quantize_ts(d, mq.ROLE_X, source(x, layout), src_layout=layout, amax_in=None if am is None else amax(am), seed=seed)
+        assert np.array_equal(logical(q, x, mq.E2M1), sign), am
+    q = mq.quantize_ts(d, mq.ROLE_X, source(x, layout), src_layout=layout, amax_in=amax(3.0), seed=seed)
+    got = logical(q, x, mq.E2M1)
+    assert (got[np.isnan(x)] == 7).all() and (got[np.isinf(x)] == 7 + sign[np.isinf(x)]).all()
