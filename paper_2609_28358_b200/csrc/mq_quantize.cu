@@ -235,7 +235,8 @@ __global__ void __launch_bounds__(NT) quantize_pipe_kernel(QuantArgs a, int n_ps
 // stride P.  PI = 8 (half the loads per thread, twice the blocks) where the whole grid runs at once, us, PI = 16 / 8: 64 channels
 // 13x13, N = 20: 3.4 / 2.6; 512 channels 7x7, N = 64 (224 blocks): 3.7 / 3.6; 96 channels 27x27, N = 50 (552 blocks): 4.3 / 5.1;
 // weights against quantize_few_kernel / PI = 8: 128 -> 128 3x3 3.1 / 2.6, 288 -> 78 5x5 4.8 / 2.7, 512 -> 512 3x3 (512 blocks)
-// 4.2 / 5.0.  LINE: line blocks - one scale per (position, row, 32 channels).
+// 4.2 / 5.0.  LINE: line blocks - one scale per (position, row, 32 channels).  A block that holds a NaN gets the scale of an
+// infinite maximum, here and in quantize_few_kernel; the other kernels' maxima pass over it.
 template <int FMT, bool SR, bool LINE, int PI>   // PI: positions per item, 16 or 8
 __global__ void __launch_bounds__(QT_THREADS, 2) quantize_odd_kernel(QuantArgs a, int n_pstrips, int Ct) {
   constexpr int CG = PI, HN = 32 / PI;             // a thread's channels, a row's channel groups
@@ -264,10 +265,10 @@ __global__ void __launch_bounds__(QT_THREADS, 2) quantize_odd_kernel(QuantArgs a
   for (int i = 0; i < 4; ++i) {
     m[i] = 0.f;
 #pragma unroll
-    for (int k = 0; k < CG; ++k) m[i] = fmaxf(m[i], fabsf(v[i][k]));
+    for (int k = 0; k < CG; ++k) m[i] = max_nan(m[i], fabsf(v[i][k]));
     if (LINE) {
 #pragma unroll
-      for (int off = PI; off < 32; off <<= 1) m[i] = fmaxf(m[i], __shfl_xor_sync(0xffffffffu, m[i], off));
+      for (int off = PI; off < 32; off <<= 1) m[i] = max_nan(m[i], __shfl_xor_sync(0xffffffffu, m[i], off));
     }
   }
   int code[LINE ? 4 : 1];
@@ -278,9 +279,9 @@ __global__ void __launch_bounds__(QT_THREADS, 2) quantize_odd_kernel(QuantArgs a
       if (h == 0 && p_ok && r0 + i < a.R) a.scales[(long long)(q.p0 + pl) * a.sc_stride_p + (long long)(r0 + i) * a.sc_stride_r + q.ct] = (uint8_t)code[i];
     }
   } else {
-    float mm = fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
+    float mm = max_nan(max_nan(m[0], m[1]), max_nan(m[2], m[3]));
 #pragma unroll
-    for (int off = PI; off < 32; off <<= 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, off));
+    for (int off = PI; off < 32; off <<= 1) mm = max_nan(mm, __shfl_xor_sync(0xffffffffu, mm, off));
     if (h == 0) red[warp][pl] = __float_as_uint(mm);
     __syncthreads();
     unsigned mx = 0;
@@ -604,8 +605,11 @@ quantize_tma_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_con
 }
 
 // One 32 x 32 tile at one position held by a warp, lane (cq, rq) = (lane & 7, lane >> 3) with 4 adjacent channels of rows
-// rq, rq + 4, ...: scale(s), codes, stores.  LINE: one scale per row (line blocks), reduced over the 8 lanes of a row.
-template <int FMT, bool SR, bool LINE>
+// rq, rq + 4, ...: scale(s), codes, stores.  LINE: one scale per row (line blocks), reduced over the 8 lanes of a row.  KEEP_NAN: the
+// maximum of a block that holds a NaN is one (see quantize_odd_kernel).
+template <bool KEEP_NAN>
+__device__ __forceinline__ float max_of(float a, float b) { return KEEP_NAN ? max_nan(a, b) : fmaxf(a, b); }
+template <int FMT, bool SR, bool LINE, bool KEEP_NAN>
 __device__ __forceinline__ void finish_tile(const QuantArgs& a, const float4 (&v)[8], int pos, int rt, int ct, int lane) {
   const int cq = lane & 7, rq = lane >> 3;
   const int r0 = rt * 32 + rq, c0 = ct * 32 + 4 * cq;
@@ -613,7 +617,7 @@ __device__ __forceinline__ void finish_tile(const QuantArgs& a, const float4 (&v
       if (LINE) {
   #pragma unroll
         for (int i = 0; i < 8; ++i) {
-          unsigned mm = __float_as_uint(fmaxf(fmaxf(fabsf(v[i].x), fabsf(v[i].y)), fmaxf(fabsf(v[i].z), fabsf(v[i].w))));
+          unsigned mm = __float_as_uint(max_of<KEEP_NAN>(max_of<KEEP_NAN>(fabsf(v[i].x), fabsf(v[i].y)), max_of<KEEP_NAN>(fabsf(v[i].z), fabsf(v[i].w))));
           mm = max(mm, __shfl_xor_sync(0xffffffffu, mm, 1));
           mm = max(mm, __shfl_xor_sync(0xffffffffu, mm, 2));
           mm = max(mm, __shfl_xor_sync(0xffffffffu, mm, 4));
@@ -623,7 +627,7 @@ __device__ __forceinline__ void finish_tile(const QuantArgs& a, const float4 (&v
       } else {
         float m = 0.f;
   #pragma unroll
-        for (int i = 0; i < 8; ++i) m = fmaxf(fmaxf(m, fmaxf(fabsf(v[i].x), fabsf(v[i].y))), fmaxf(fabsf(v[i].z), fabsf(v[i].w)));
+        for (int i = 0; i < 8; ++i) m = max_of<KEEP_NAN>(max_of<KEEP_NAN>(m, max_of<KEEP_NAN>(fabsf(v[i].x), fabsf(v[i].y))), max_of<KEEP_NAN>(fabsf(v[i].z), fabsf(v[i].w)));
         code[0] = scale_code_of(__reduce_max_sync(0xffffffffu, __float_as_uint(m)), fmt_emax(FMT));
         if (lane == 0) a.scales[(long long)pos * a.sc_stride_p + (long long)rt * a.sc_stride_r + ct] = (uint8_t)code[0];
       }
@@ -698,7 +702,7 @@ __global__ void __launch_bounds__(512) quantize_few_kernel(QuantArgs a, int Ct) 
       const float* src = runs + (rq + 4 * i) * stride + 4 * cq * a.P + p;
       v[i] = make_float4(src[0], src[a.P], src[2 * a.P], src[3 * a.P]);
     }
-    finish_tile<FMT, SR, LINE>(a, v, p, rt, ct, lane);
+    finish_tile<FMT, SR, LINE, true>(a, v, p, rt, ct, lane);
   }
 }
 
@@ -739,7 +743,7 @@ __global__ void __launch_bounds__(256) quantize_cfast_kernel(QuantArgs a, unsign
       for (int i = 0; i < 8; ++i)
         v[i] = make_float4(mx_activation(v[i].x, a.act), mx_activation(v[i].y, a.act), mx_activation(v[i].z, a.act), mx_activation(v[i].w, a.act));
     }
-    finish_tile<FMT, SR, LINE>(a, v, (int)pos, (int)rt, (int)ct, lane);
+    finish_tile<FMT, SR, LINE, false>(a, v, (int)pos, (int)rt, (int)ct, lane);
   }
 }
 

@@ -2,6 +2,7 @@
 the block's other elements, on every kernel.  Codes and scales are compared byte for byte."""
 import numpy as np
 import pytest
+import torch
 
 import oracle
 from paper_2609_28358_b200 import inputs, mq
@@ -60,8 +61,6 @@ def test_nan_elements(name, fmt, layout):
 def test_paper_format(name, layout, seed):
     """Eq. 6 of a NaN, in a block that is not zero, is the largest magnitude; in a block that encodes to zeros, as with T_scale 0 or
     infinite, it and an infinity are zeros with their sign.  The other elements are the oracle's."""
-    import torch
-
     b16 = (16, 16)
     amax = lambda v: torch.tensor([v], dtype=torch.float32, device="cuda")
     d, x = tensor(name, PATTERNS)
@@ -78,3 +77,29 @@ def test_paper_format(name, layout, seed):
     q = mq.quantize_ts(d, mq.ROLE_X, source(x, layout), src_layout=layout, amax_in=amax(3.0), seed=seed)
     got = logical(q, x, mq.E2M1)
     assert (got[np.isnan(x)] == 7).all() and (got[np.isinf(x)] == 7 + sign[np.isinf(x)]).all()
+
+
+@pytest.mark.parametrize("fmt", sorted(NAN_CODE))
+@pytest.mark.parametrize("name", SHAPES)
+def test_scales_of_blocks_with_a_nan(name, fmt):
+    """Where the positions are no multiple of four, and in small tensors of line blocks, a block with a NaN has the scale of an infinite maximum, under which its finite
+    elements are zeros with their sign; elsewhere the maximum passes over the NaN.  All other bytes are the oracle's."""
+    d, x = tensor(name, PATTERNS, 0.0005)
+    n, c, h, w = x.shape
+    infinite = min(255 - {mq.E4M3: 8, mq.E5M2: 15, mq.E3M2: 4}.get(fmt, 2), 254)
+    sign = {mq.E2M1: 8, mq.E3M2: 0x20, mq.E2M3: 0x20}.get(fmt, 0x80)
+    for block, side in ((mq.TILE32, 32), (mq.LINE32, 1)):
+        codes, scales = oracle.quantize(d, mq.ROLE_X, fmt, np.nan_to_num(x, nan=0.0), (side, 32))
+        want = logical(mq.QTensor(torch.from_numpy(codes), None, fmt, mq.ROLE_X), x, fmt)
+        scales = scales.reshape(h * w, (n + side - 1) // side, -1)
+        if (h * w) % 4 != 0 or (block == mq.LINE32 and x.size < 1 << 18):
+            rows, chans, ys, xs = np.nonzero(np.isnan(x))
+            marked = np.zeros(scales.shape, bool)
+            marked[ys * w + xs, rows // side, chans // 32] = True
+            scales = np.where(marked, infinite, scales)
+            of = np.repeat(np.repeat(marked, side, 1)[:, :n], 32, 2)[:, :, :c].transpose(1, 2, 0).reshape(x.shape)
+            want = np.where(of, np.where(np.signbit(x), sign, 0), want)
+        want = np.where(np.isnan(x), NAN_CODE[fmt], want)
+        q = mq.quantize(d, mq.ROLE_X, fmt, source(x, mq.NCHW), block=block)
+        assert np.array_equal(host(q.scales), scales.reshape(-1))
+        assert np.array_equal(logical(q, x, fmt), want)
