@@ -190,6 +190,7 @@ struct ConvTcPlan {
 bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, ConvTcPlan* out, bool line = false, bool mx = false, bool ts16 = false) {
   const bool fp4 = fmt_w == MQ_E2M1;
   if (ts16 && (!fp4 || fmt_x_like != MQ_E2M1 || line)) return false;
+  if (op == MQ_OP_FWD && g.sw > 8) return false;   // the copy engine steps over at most eight columns
   const int bits = fp4 ? 4 : 8;
   const int taps = g.Kh * g.Kw;
   ConvTcParams p{};
