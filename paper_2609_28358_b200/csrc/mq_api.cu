@@ -602,6 +602,7 @@ WgradPlan wgrad_plan(const Geom& g, int fmt_x, int fmt_g, bool ts16 = false) {
   // (With a column stride the strip is the contiguous run of (KPX - 1) sw + Kw input pixels: output pixel a's tap kw is
   // input pixel a sw + kw of the strip, so panels stay one pixel apart and K slices sw pixels apart.)
   p.grp8 = (fp8 && !p.cta2 && g.Kw > 1 && (g.Cp == 32 || g.Cp == 64) && g.Kw * g.Cp <= 256 && !MQ_ENV("MQ_WGRAD_NO_GROUP8", 0)) ? 1 : 0;
+  if (fp8 && !p.grp8 && g.sw > 8) return w;   // the copy engine steps over at most eight columns
   if (p.grp8) p.b_rows = g.Cp;
   p.cb_tiles = (g.Cp + p.b_rows - 1) / p.b_rows;
   // taps per block: a whole kernel row in the flat mode when its accumulators fit in tensor memory
