@@ -205,8 +205,9 @@ mq_status mq_conv_bwd_data(const mq_conv_desc* desc, const mq_qtensor* wq, const
  * input-gradient GEMM, and the per-stage scale-vector chunks expanded from the tile scales) lives here in a
  * static array inside the library's device image, MQ_STATIC_SCRATCH_BYTES (16 MiB) long; every GPU that
  * loads the library keeps that much memory reserved until the process exits.  A layer whose
- * mq_workspace_size(desc, MQ_OP_BWD_DATA, ...) exceeds it is rejected with MQ_ERR_STATIC_SCRATCH and nothing
- * is launched (for scale: N=32, 128->64 channels, 80x80, 3x3 needs about 6 MB).
+ * mq_workspace_size(desc, MQ_OP_BWD_DATA, ...) exceeds it runs on tiles that need less scratch where those fit, or,
+ * E2M1 with C_out (rounded up to 32) no multiple of 64, on the CUDA-core kernels, which need none; any other is
+ * rejected with MQ_ERR_STATIC_SCRATCH and nothing is launched (for scale: N=32, 128->64 channels, 80x80, 3x3 needs about 6 MB).
  * The call performs no cudaMalloc / cudaFree and calls no allocating library routine.
  *
  * Arguments are checked exactly as by mq_conv_bwd_data (same codes), then the size limit.

@@ -187,7 +187,9 @@ struct ConvTcPlan {
 // line: line-block operands (forward only).  mx: the quantizing epilogue (tiles of at most 4 output columns, channel tiles
 // of whole 32-channel blocks, per-tap kernel).
 // ts16: the paper's own format (E2M1 elements, one E4M3 scale per 16 x 16 block, an fp32 scale per tensor): kind::mxf4nvf4, per-tap kernel.
-bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, ConvTcPlan* out, bool line = false, bool mx = false, bool ts16 = false) {
+// compact: the shapes with the least scratch rather than the fastest (the allocation-free input gradient, where the others' does not fit).
+bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, ConvTcPlan* out, bool line = false, bool mx = false, bool ts16 = false,
+                  bool compact = false) {
   const bool fp4 = fmt_w == MQ_E2M1;
   if (ts16 && (!fp4 || fmt_x_like != MQ_E2M1 || line)) return false;
   if (op == MQ_OP_FWD && g.sw > 8) return false;   // the copy engine steps over at most eight columns
@@ -216,6 +218,7 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
   // cost three times as many of them for 96-byte rows (E4M3 129 -> 186 channels, N = 23, 45x56, forward: 74 -> 60 us).
   const int atoms = (rowbytes + 31) / 32;
   p.KB = atoms == 1 ? 32 : (atoms == 2 || (rowbytes % 64 == 0 && rowbytes % 128 != 0) ? 64 : 128);
+  if (compact && rowbytes % 32 == 0) p.KB = rowbytes % 128 == 0 ? 128 : (rowbytes % 64 == 0 ? 64 : 32);   // no short boxes: full stages, fewest scale chunks
   p.G = 128 / p.KB;
   p.cpt = (rowbytes + p.KB - 1) / p.KB;
   p.last_atoms = atoms - (p.cpt - 1) * (p.KB / 32);
@@ -271,6 +274,13 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
       const int ftw = MQ_ENV("MQ_TC_MX_TW", 0);
       if (ftw == 1 || ftw == 2 || (ftw == 4 && !ts16)) t = TileRows{ftw, 128 / ftw};
     } else if (forced_tw > 0) t = TileRows{forced_tw, 128 / forced_tw};
+    else if (compact) {   // a scale chunk per tile and stage: the fewest tiles
+      double fewest = 1e30;
+      for (int tw = 1; tw <= 32 && tw <= max_tw; tw <<= 1) {
+        const double tiles = (double)((w_eff + tw - 1) / tw) * ((g.N + 128 / tw - 1) / (128 / tw));
+        if (tiles < fewest) { fewest = tiles; t = TileRows{tw, 128 / tw}; }
+      }
+    }
     else if (thin) t = TileRows{8, 16};   // the whole-tile kernel (8-column tiles): its per-tile loads beat any per-tap shape on thin layers
     else if (want_tma || layout != MQ_NCHW) {
       const int nkh = op == MQ_OP_FWD ? g.Kh : (g.Kh + g.sh - 1) / g.sh, nkw = op == MQ_OP_FWD ? g.Kw : (g.Kw + g.sw - 1) / g.sw;
@@ -279,7 +289,7 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
     }
     else t = choose_rows(w_eff, g.N, p.Wd, max_tw, pair_hint, big_output);
     p.TW = t.tw; p.TN = t.tn;
-    if (!thin && !(forced_bn >= 32 && forced_bn <= 256 && forced_bn % 32 == 0)) {
+    if (!thin && !compact && !(forced_bn >= 32 && forced_bn <= 256 && forced_bn % 32 == 0)) {
       const long long row_tiles = (long long)((w_eff + t.tw - 1) / t.tw) * ((g.N + t.tn - 1) / t.tn) * p.tiles_h * p.classes;
       p.BN = choose_columns(p.Cd, p.BN, want_tma && layout == MQ_HWNC ? 64 : 32,
                             pair_hint || want_tma ? 128 : 256, row_tiles,
@@ -406,11 +416,11 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
 
 // Scratch of a forward / input-gradient call: the tensor-core plan's where one exists (it depends on the output layout: the
 // larger of the two), never less than what the CUDA-core kernels need, which take the layers a plan refuses.
-size_t conv_tc_workspace(int op, const Geom& g, int fmt_x_like, int fmt_w, bool line, bool ts16 = false) {
+size_t conv_tc_workspace(int op, const Geom& g, int fmt_x_like, int fmt_w, bool line, bool ts16, bool compact) {
   size_t need = conv_generic_workspace(op, g);
   for (int layout = 0; layout < 2; ++layout) {   // the tile shape, hence the scratch, depends on the output layout
     ConvTcPlan pl;
-    if (conv_tc_plan(op, g, fmt_x_like, fmt_w, layout, &pl, line, false, ts16) && pl.total > need) need = pl.total;
+    if (conv_tc_plan(op, g, fmt_x_like, fmt_w, layout, &pl, line, false, ts16, compact) && pl.total > need) need = pl.total;
   }
   return need;
 }
@@ -783,10 +793,13 @@ mq_status check_conv_args(int op, const mq_conv_desc* desc, const mq_qtensor* qa
   return MQ_OK;
 }
 
+// How a call's kernels are chosen: by the rules, or - the allocation-free input gradient - for what they need of scratch
+enum class Route { RULES, COMPACT, CUDA_CORES };
+
 // Does a forward / input-gradient call of this layer, formats and output layout run on the tensor cores?  (formats: one code per byte)
-bool conv_takes_tc(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, bool line, bool ts16, ConvTcPlan* pl) {
-  return (!ts16 || !MQ_ENV("MQ_TC_NO_TS16", 0)) && (op == MQ_OP_FWD || op == MQ_OP_BWD_DATA) && conv_tc_eligible(op, g, fmt_x_like, fmt_w) &&
-         conv_tc_plan(op, g, fmt_x_like, fmt_w, layout, pl, line, false, ts16);
+bool conv_takes_tc(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, bool line, bool ts16, ConvTcPlan* pl, Route route) {
+  return route != Route::CUDA_CORES && (!ts16 || !MQ_ENV("MQ_TC_NO_TS16", 0)) && (op == MQ_OP_FWD || op == MQ_OP_BWD_DATA) && conv_tc_eligible(op, g, fmt_x_like, fmt_w) &&
+         conv_tc_plan(op, g, fmt_x_like, fmt_w, layout, pl, line, false, ts16, route == Route::COMPACT);
 }
 
 // Operands in packed 6-bit storage: scratch, behind the call's own, for the one-code-per-byte copies of the operands no
@@ -799,7 +812,7 @@ int operand_role(int op, int which) {
   if (op == MQ_OP_BWD_DATA) return which == 0 ? MQ_ROLE_W : MQ_ROLE_DY;
   return which == 0 ? MQ_ROLE_X : MQ_ROLE_DY;
 }
-PackedExtra packed_extra(int op, const Geom& g, int fmt_a, int fmt_b, int block) {
+PackedExtra packed_extra(int op, const Geom& g, int fmt_a, int fmt_b, int block, Route route) {
   PackedExtra e{false, false, 0, 0};
   const bool pa = fmt_is_packed6(fmt_a), pb = fmt_is_packed6(fmt_b);
   if (!pa && !pb) return e;
@@ -808,7 +821,7 @@ PackedExtra packed_extra(int op, const Geom& g, int fmt_a, int fmt_b, int block)
   bool tc = true;    // on the tensor cores whatever the output layout
   ConvTcPlan pl;
   if (op == MQ_OP_BWD_WEIGHT) tc = wgrad_plan(g, fa, fb, ts16).ok;
-  else for (int layout = 0; layout < 2; ++layout) tc = tc && conv_takes_tc(op, g, op == MQ_OP_FWD ? fa : fb, op == MQ_OP_FWD ? fb : fa, layout, line, ts16, &pl);
+  else for (int layout = 0; layout < 2; ++layout) tc = tc && conv_takes_tc(op, g, op == MQ_OP_FWD ? fa : fb, op == MQ_OP_FWD ? fb : fa, layout, line, ts16, &pl, route);
   e.keep_a = pa && (!tc || op == MQ_OP_BWD_DATA);
   e.keep_b = pb && !tc;
   const View va = view_of(g, operand_role(op, 0)), vb = view_of(g, operand_role(op, 1));
@@ -816,11 +829,12 @@ PackedExtra packed_extra(int op, const Geom& g, int fmt_a, int fmt_b, int block)
   e.bytes_b = e.keep_b ? ((size_t)(vb.P * vb.R * vb.Cp) + 255) / 256 * 256 : 0;
   return e;
 }
-size_t conv_workspace_unpacked(int op, const Geom& g, int fa, int fb, int block) {
+size_t conv_workspace_unpacked(int op, const Geom& g, int fa, int fb, int block, Route route) {
   const bool line = block == MQ_BLOCK_LINE32, ts16 = block == MQ_BLOCK_TS16;
   size_t bytes = conv_generic_workspace(op, g);
-  if (op == MQ_OP_FWD && conv_tc_eligible(op, g, fa, fb)) bytes = conv_tc_workspace(op, g, fa, fb, line, ts16);
-  if (op == MQ_OP_BWD_DATA && conv_tc_eligible(op, g, fb, fa)) bytes = conv_tc_workspace(op, g, fb, fa, false, ts16);
+  if (route == Route::CUDA_CORES) return bytes;
+  if (op == MQ_OP_FWD && conv_tc_eligible(op, g, fa, fb)) bytes = conv_tc_workspace(op, g, fa, fb, line, ts16, route == Route::COMPACT);
+  if (op == MQ_OP_BWD_DATA && conv_tc_eligible(op, g, fb, fa)) bytes = conv_tc_workspace(op, g, fb, fa, false, ts16, route == Route::COMPACT);
   if (op == MQ_OP_BWD_WEIGHT) {
     const WgradPlan w = wgrad_plan(g, fa, fb, ts16);
     if (w.ok) bytes = w.total;
@@ -828,14 +842,21 @@ size_t conv_workspace_unpacked(int op, const Geom& g, int fa, int fb, int block)
   return bytes;
 }
 
+// scratch of a call on a route
+size_t conv_workspace(int op, const Geom& g, int fmt_a, int fmt_b, int block, Route route) {
+  const size_t bytes = conv_workspace_unpacked(op, g, fmt_base(fmt_a), fmt_base(fmt_b), block, route);
+  if (!fmt_is_packed6(fmt_a) && !fmt_is_packed6(fmt_b)) return bytes;
+  const PackedExtra pe = packed_extra(op, g, fmt_a, fmt_b, block, route);
+  return (bytes + 255) / 256 * 256 + pe.bytes_a + pe.bytes_b;
+}
+
 mq_status run_conv(int op, const mq_conv_desc* desc, const mq_qtensor* qa_in, int role_a, const mq_qtensor* qb_in, int role_b,
-                   void* out, int dtype, int layout, void* ws, size_t ws_bytes, void* stream) {
+                   void* out, int dtype, int layout, void* ws, size_t ws_bytes, void* stream, Route route = Route::RULES) {
   mq_status st = check_conv_args(op, desc, qa_in, role_a, qb_in, role_b, out, dtype, layout);
   if (st != MQ_OK) return st;
   Geom g = make_geom(*desc);
   if (ws && !aligned16(ws)) return MQ_ERR_ALIGNMENT;
-  size_t need = 0;
-  mq_workspace_size(desc, op, qa_in->fmt, qb_in->fmt, qa_in->block, &need);
+  const size_t need = conv_workspace(op, g, qa_in->fmt, qb_in->fmt, qa_in->block, route);
   if (need > 0 && (!ws || ws_bytes < need)) return MQ_ERR_BUFFER_TOO_SMALL;
   const int fa = fmt_base(qa_in->fmt), fb = fmt_base(qb_in->fmt);
   const bool ts16 = qa_in->block == MQ_BLOCK_TS16, line = qa_in->block == MQ_BLOCK_LINE32;
@@ -843,14 +864,14 @@ mq_status run_conv(int op, const mq_conv_desc* desc, const mq_qtensor* qa_in, in
   ConvTcPlan pl;
   WgradPlan wp;
   wp.ok = false;
-  const bool conv_tc = op != MQ_OP_BWD_WEIGHT && conv_takes_tc(op, g, op == MQ_OP_FWD ? fa : fb, op == MQ_OP_FWD ? fb : fa, layout, line, ts16, &pl);
+  const bool conv_tc = op != MQ_OP_BWD_WEIGHT && conv_takes_tc(op, g, op == MQ_OP_FWD ? fa : fb, op == MQ_OP_FWD ? fb : fa, layout, line, ts16, &pl, route);
   if (op == MQ_OP_BWD_WEIGHT) wp = wgrad_plan(g, fa, fb, ts16);
   const bool tc = conv_tc || wp.ok;
   // operands in packed 6-bit storage that this route reads one code per byte: copies behind the call's own scratch
   mq_qtensor qa_v = *qa_in, qb_v = *qb_in;
   if (fmt_is_packed6(qa_in->fmt) || fmt_is_packed6(qb_in->fmt)) {
-    const PackedExtra pe = packed_extra(op, g, qa_in->fmt, qb_in->fmt, qa_in->block);
-    uint8_t* extra = static_cast<uint8_t*>(ws) + (conv_workspace_unpacked(op, g, fa, fb, qa_in->block) + 255) / 256 * 256;
+    const PackedExtra pe = packed_extra(op, g, qa_in->fmt, qb_in->fmt, qa_in->block, route);
+    uint8_t* extra = static_cast<uint8_t*>(ws) + (conv_workspace_unpacked(op, g, fa, fb, qa_in->block, route) + 255) / 256 * 256;
     if (fmt_is_packed6(qa_in->fmt) && (!tc || op == MQ_OP_BWD_DATA)) {
       const View v = view_of(g, role_a);
       if (launch_unpack6(static_cast<const uint8_t*>(qa_in->codes), extra, (size_t)(v.P * v.R * v.Cp), 1, fa, static_cast<cudaStream_t>(stream)) != cudaSuccess) return MQ_ERR_CUDA;
@@ -919,11 +940,7 @@ mq_status mq_workspace_size(const mq_conv_desc* desc, int op, int fmt_a, int fmt
   if (block == MQ_BLOCK_LINE32 && op != MQ_OP_FWD) return MQ_ERR_UNSUPPORTED;
   const Geom g = make_geom(*desc);
   if (block == MQ_BLOCK_TS16 && (fmt_a != MQ_E2M1 || fmt_b != MQ_E2M1)) return MQ_ERR_INVALID_ARG;
-  *bytes = conv_workspace_unpacked(op, g, fmt_base(fmt_a), fmt_base(fmt_b), block);
-  if (fmt_is_packed6(fmt_a) || fmt_is_packed6(fmt_b)) {
-    const PackedExtra pe = packed_extra(op, g, fmt_a, fmt_b, block);
-    *bytes = (*bytes + 255) / 256 * 256 + pe.bytes_a + pe.bytes_b;
-  }
+  *bytes = conv_workspace(op, g, fmt_a, fmt_b, block, Route::RULES);
   return MQ_OK;
 }
 
@@ -1172,12 +1189,20 @@ mq_status mq_conv_bwd_data_static(const mq_conv_desc* desc, const mq_qtensor* wq
   // the ordinary call's argument checks first, so that a bad argument is reported as such whatever the layer's size
   mq_status st = check_conv_args(MQ_OP_BWD_DATA, desc, wq, MQ_ROLE_W, dyq, MQ_ROLE_DY, dx, dx_dtype, dx_layout);
   if (st != MQ_OK) return st;
-  size_t need = 0;
-  if ((st = mq_workspace_size(desc, MQ_OP_BWD_DATA, wq->fmt, dyq->fmt, wq->block, &need)) != MQ_OK) return st;
-  if (need > MQ_STATIC_SCRATCH_BYTES) return MQ_ERR_STATIC_SCRATCH;
+  const Geom g = make_geom(*desc);
+  // The first route whose scratch fits.  CUDA cores (which need none) only for 4-bit rows that end inside an MMA's K-atom: other
+  // layers that do not fit are the caller's to give a workspace to, not to be run at a tenth of the speed.
+  const bool short_rows = wq->fmt == MQ_E2M1 && dyq->fmt == MQ_E2M1 && g.Cop % 64 != 0;
+  auto fits = [&](Route r) { return conv_workspace(MQ_OP_BWD_DATA, g, wq->fmt, dyq->fmt, wq->block, r) <= MQ_STATIC_SCRATCH_BYTES; };
+  Route route = Route::RULES;
+  if (!fits(route)) {
+    if (fits(Route::COMPACT)) route = Route::COMPACT;
+    else if (short_rows && fits(Route::CUDA_CORES)) route = Route::CUDA_CORES;
+    else return MQ_ERR_STATIC_SCRATCH;
+  }
   void* addr = nullptr;
   if (cudaGetSymbolAddress(&addr, g_static_scratch) != cudaSuccess || !addr) return MQ_ERR_CUDA;
-  return run_conv(MQ_OP_BWD_DATA, desc, wq, MQ_ROLE_W, dyq, MQ_ROLE_DY, dx, dx_dtype, dx_layout, addr, MQ_STATIC_SCRATCH_BYTES, stream);
+  return run_conv(MQ_OP_BWD_DATA, desc, wq, MQ_ROLE_W, dyq, MQ_ROLE_DY, dx, dx_dtype, dx_layout, addr, MQ_STATIC_SCRATCH_BYTES, stream, route);
 }
 
 namespace {

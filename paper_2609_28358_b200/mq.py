@@ -250,7 +250,7 @@ STATIC_SCRATCH_BYTES = 16 << 20
 def conv_bwd_data_static(desc, wq, dyq, dx=None, layout=NCHW, stream=None):
     """mq_conv_bwd_data_static: the input gradient for callers that cannot allocate device memory (a plug-in
     inside an application that owns the allocator, a frozen memory pool).  The library's own static device
-    array serves as scratch; layers needing more than STATIC_SCRATCH_BYTES raise MqError(MQ_ERR_STATIC_SCRATCH).
+    array serves as scratch; layers that cannot do with STATIC_SCRATCH_BYTES raise MqError(MQ_ERR_STATIC_SCRATCH).
     `dx` should be passed in by such callers; it is only created here for convenience when omitted."""
     d = ConvDesc(*desc)
     if dx is None:
