@@ -321,13 +321,14 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
   }
   // NCHW output through TMA stores (unit-stride output columns, rows of 16-byte multiples): worth its 64 KB of
   // staging only in the whole-tile kernel, whose pipeline is short; the per-tap kernel keeps its stages
-  // (NCHW: rows of TW floats, at least 16 bytes; [H][W][N][C]: rows of 32 channels whatever the tile's width, whole 32-channel
-  // groups per column half)
+  // (NCHW: rows of TW floats, at least 16 bytes, and boxes of 64 channels, so a column half is at most one box or whole boxes - a
+  // box that reached into the next half would race with its store; [H][W][N][C]: rows of 32 channels whatever the tile's width,
+  // whole 32-channel groups per column half)
   // Strided input gradient, channel-fastest output: the staged epilogue writes a parity class through a tensor map that steps sw
   // pixels along W.  Not for NCHW: there W is the innermost axis and a class's first column (x = 1 for the odd one) would be
   // a TMA coordinate that is not on a 16-byte boundary, which the hardware refuses; NCHW keeps the paired direct stores.
   const bool tma_store_ok = (!strided_out || s2_tma_ok) && pow2_tw &&
-                            (layout == MQ_NCHW ? (p.TW >= 4 && p.Wd % 4 == 0) : (p.Cd % 4 == 0 && p.BN % 64 == 0));
+                            (layout == MQ_NCHW ? (p.TW >= 4 && p.Wd % 4 == 0 && (p.BN <= 128 || p.BN == 256)) : (p.Cd % 4 == 0 && p.BN % 64 == 0));
   // ... and for 1x1 layers, whose main loop is a handful of stages: the tile's time is its store (measured 4-12 % faster, 28x28 and
   // 56x56 images, 256 and 512 channels)
   // ... and for the channel-fastest output order, where a direct store is one 16-byte request per row and instruction - the request
@@ -352,9 +353,10 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
   p.max_stages = (nkh * nkw * p.cpt + p.G - 1) / p.G;
   // one 256-column accumulator: the epilogue copies it into registers and frees it before storing (with the staged TMA
   // stores only when a tile has at least MQ_TC_SNAP_MIN_STAGES pipeline stages of MMAs to overlap: E2M1 1x1 512 channels, two
-  // stages per tile, measured 384-407 us without and 517-601 us with it; E4M3, four stages, 562-567 against 521 us)
+  // stages per tile, measured 384-407 us without and 517-601 us with it; E4M3, four stages, 562-567 against 521 us; and only of 256
+  // columns: that role stores two whole 64-column slices per half)
   p.snap = (!mx && ((p.BN > 128 && p.n_acc == 1 && !p.pair) || (p.pair && p.BN == 128)) && !MQ_ENV("MQ_TC_NO_SNAP", 0) &&
-            (!p.tma_store || p.max_stages >= MQ_ENV("MQ_TC_SNAP_MIN_STAGES", 4))) ? 1 : 0;
+            (!p.tma_store || (p.BN == 256 && p.max_stages >= MQ_ENV("MQ_TC_SNAP_MIN_STAGES", 4)))) ? 1 : 0;
   const uint32_t fa = fp4 ? 1u : fmt_mma_code(fmt_x_like);   // kind::mxf4: 1 = E2M1; kind::mxf8f6f4: E4M3 0, E5M2 1, E2M3 3, E3M2 4
   const uint32_t fb = fp4 ? 1u : fmt_mma_code(fmt_w);
   // pairs of blocks on 256 x 256 tiles (see conv_tc_kernel's DUO): tiles 2k and 2k + 1 must exist and share the channel tile

@@ -21,6 +21,10 @@ CASES = [
     ("bn160", (9, 128, 4, 14, 160, 3, 1, 1), {"MQ_TC_BN": "160"}),  # one accumulator copied into registers, 80 columns a half
     ("bn192", (9, 128, 4, 14, 192, 3, 1, 1), {"MQ_TC_BN": "192"}),
     ("bn224_tail", (9, 128, 4, 14, 250, 3, 1, 1), {"MQ_TC_BN": "224"}),
+    ("k1_bn160", (9, 512, 4, 16, 250, 1, 1, 0), {"MQ_TC_BN": "160"}),   # 1x1: staged stores where the halves are whole boxes, else direct ones
+    ("k1_bn192", (9, 512, 4, 16, 250, 1, 1, 0), {"MQ_TC_BN": "192"}),
+    ("k1_bn224", (9, 512, 4, 16, 250, 1, 1, 0), {"MQ_TC_BN": "224"}),
+    ("k1_bn256", (9, 512, 4, 16, 600, 1, 1, 0), {"MQ_TC_BN": "256"}),
     ("pairs_14", (9, 256, 4, 14, 256, 3, 1, 1), {"MQ_TC_BN": "256"}),   # four tiles of 126 rows: block pairs, E4M3 and E2M1
 ]
 
