@@ -39,12 +39,18 @@ void check(const char* call, mq_status st) {
 void require(bool ok, const char* what) {
   if (!ok) { PyErr_SetString(PyExc_AssertionError, what); throw PyFail{}; }
 }
+// an integer argument: an int, or an object that stands for one; no float and no text
 long to_long(PyObject* o) {
-  if (PyLong_CheckExact(o)) {
-    const long v = PyLong_AsLong(o);
-    if (v == -1 && PyErr_Occurred()) throw PyFail{};
-    return v;
-  }
+  PyObject* n = PyNumber_Index(o);
+  if (!n) throw PyFail{};
+  const long v = PyLong_AsLong(n);
+  Py_DECREF(n);
+  if (v == -1 && PyErr_Occurred()) throw PyFail{};
+  return v;
+}
+// an extent of the layer: whatever int() takes
+long extent_of(PyObject* o) {
+  if (PyLong_CheckExact(o)) return to_long(o);
   PyObject* n = PyNumber_Long(o);
   if (!n) throw PyFail{};
   const long v = PyLong_AsLong(n);
@@ -65,7 +71,7 @@ mq_conv_desc desc_of(PyObject* o) {
   bool ok = n == 11;
   if (!ok) PyErr_SetString(PyExc_TypeError, "the layer descriptor is a sequence of eleven integers");
   try {
-    for (Py_ssize_t i = 0; ok && i < n; ++i) f[i] = (int)to_long(PySequence_Fast_GET_ITEM(seq, i));
+    for (Py_ssize_t i = 0; ok && i < n; ++i) f[i] = (int)extent_of(PySequence_Fast_GET_ITEM(seq, i));
   } catch (PyFail&) { ok = false; }
   Py_DECREF(seq);
   if (!ok) throw PyFail{};
@@ -302,8 +308,8 @@ PyObject* py_conv(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
     at::Tensor out;
     if (a[4] != Py_None) out = tensor_of(a[4]);
     else {
-      if (!THPDtype_Check(a[8])) { PyErr_SetString(PyExc_TypeError, "dtype is a torch.dtype"); throw PyFail{}; }
-      const at::ScalarType t = reinterpret_cast<THPDtype*>(a[8])->scalar_type;
+      if (a[8] != Py_None && !THPDtype_Check(a[8])) { PyErr_SetString(PyExc_TypeError, "dtype is a torch.dtype"); throw PyFail{}; }
+      const at::ScalarType t = a[8] != Py_None ? reinterpret_cast<THPDtype*>(a[8])->scalar_type : c10::get_default_dtype_as_scalartype();
       int64_t n, c, h, w;   // logical NCHW (weight gradient: OIHW) extents
       if (op == MQ_OP_BWD_WEIGHT) { n = d.C_out; c = d.C_in; h = d.Kh; w = d.Kw; }
       else if (op == MQ_OP_BWD_DATA) { n = d.N; c = d.C_in; h = d.H; w = d.W; }

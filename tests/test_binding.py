@@ -34,6 +34,20 @@ def test_argument_errors_are_python_exceptions():
         mq.conv_fwd(D, _small(mq.ROLE_X), _small(mq.ROLE_W), dtype=torch.float16, stream=_NullStream())
 
 
+def test_arguments_are_taken_as_they_were_through_ctypes():
+    q = _small(mq.ROLE_X), _small(mq.ROLE_W)
+    call = lambda d=D, **kw: mq.conv_fwd(d, *q, stream=_NullStream(), **kw)
+    for bad in (dict(layout=0.0), dict(layout="0")):                            # neither floats nor text are integers
+        with pytest.raises(TypeError):
+            call(**bad)
+    with pytest.raises(TypeError):
+        mq.conv_fwd(D, mq.QTensor(q[0].codes, q[0].scales, 0.0, mq.ROLE_X), q[1], stream=_NullStream())
+    for good in (dict(dtype=None), dict(layout=True), dict(d=[float(v) for v in D])):   # PyTorch's default type; int()'s arguments as extents
+        with pytest.raises(mq.MqError) as e:
+            call(**good)
+        assert e.value.status == 4
+
+
 def _pass(x, w, dy, **kw):
     qs = [mq.quantize(D, r, mq.E4M3, t, **kw) for r, t in enumerate((x, w, dy))]
     return [mq.conv_fwd(D, qs[0], qs[1], **kw), mq.conv_bwd_data(D, qs[1], qs[2], **kw), mq.conv_bwd_weight(D, qs[0], qs[2], **kw)]
