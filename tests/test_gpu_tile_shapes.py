@@ -38,3 +38,13 @@ def test_gemms(name, shape, env, fmts, knobs):
     knobs(**env)
     check_convs(ol, qs, layouts=(mq.NCHW, mq.HWNC))
     assert mq.last_device_status() == 0
+
+
+@pytest.mark.parametrize("cout", [64, 96])
+def test_outputs_beyond_l2(cout):
+    """More than 110 MB of output in NCHW rows that 8 columns cut inside a sector: the whole-tile kernel up to 64 output channels,
+    per-tap tiles of whole rows above.  Sampled outputs, the borders among them."""
+    d = inputs.conv_desc(340 * 64 // cout, 32, 36, 36, cout, 3, 1, 1)
+    ol = OracleLayer(inputs.Layer("beyond l2", d, mq.E4M3, mq.E4M3, mq.E5M2, "relu", "kaiming", "gauss", 48))
+    check_convs(ol, check_quantize(ol), samples=3000, ops=("fwd",))
+    assert mq.last_device_status() == 0
