@@ -224,13 +224,18 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
   p.last_atoms = atoms - (p.cpt - 1) * (p.KB / 32);
   const int w_eff = op == MQ_OP_FWD ? g.Wo : (g.W + g.sw - 1) / g.sw;
   // line blocks (one scale per row): the per-tap kernel, whose preparation launch lays out the scale vectors row by row
-  // ... and the whole-tile kernel's 8-column tiles only where they fit: with 25 taps of 64 bytes its resident weights leave two
-  // stages (E2M1 128 channels 28x28 5x5, N = 99: 51 us against 42 per tap), and NCHW rows that 8 columns cut inside a sector cost
-  // twice where the output does not fit L2 (E2M1 128 channels 42x42, N = 128: 80 against 54; 64 -> 448 channels 60x60: 682 against
-  // 264; below that size it wins: N = 64 27 against 32)
+  // ... and the whole-tile kernel's 8-column tiles only where they pay.  With 25 taps of 64 bytes its resident weights leave two
+  // stages and per-tap tiles win (E2M1 128 channels 28x28 5x5, N = 99: 51 us against 42), but for channel-fastest output of at most 32
+  // channels, whose weights are small (58 -> 6 channels 36x36, N = 208, input gradient: 47 against 73; 32 channels: 58 against 79; 64:
+  // 90 against 88).  NCHW rows that 8 columns cut inside a sector cost twice where the output does not fit L2: there per-tap tiles
+  // win above 64 output channels (E2M1 128 channels 42x42, N = 128: 80 against 54; 64 -> 448 channels 60x60: 682 against 264) and for
+  // 1x1 (32 -> 64 channels 42x42, N = 333: 114 against 70); up to 64, where a tap's stage is mostly the per-tap loaders' own time,
+  // they do not (3x3, 150 MB of output, E4M3 32 -> 64 channels, W = 36 / 50 / 74: 58 / 76 / 76 against 115 / 121 / 149; 64 -> 64: 61 / 78 /
+  // 78 against 85 / 91 / 112)
   const bool big_output = (double)g.N * p.Cd * p.Hd * p.Wd * 4.0 > 110e6;
-  const bool thin = !line && !mx && !ts16 && g.sh == 1 && g.sw == 1 && p.cpt == 1 && p.KB <= 64 && !(p.KB == 64 && taps > 9) &&
-                    !(layout == MQ_NCHW && p.Wd % 8 != 0 && big_output) && !MQ_ENV("MQ_TC_NO_HALO", 0);
+  const bool thin = !line && !mx && !ts16 && g.sh == 1 && g.sw == 1 && p.cpt == 1 && p.KB <= 64 &&
+                    !(p.KB == 64 && taps > 9 && (layout == MQ_NCHW || p.Cd > 32)) &&
+                    !(layout == MQ_NCHW && p.Wd % 8 != 0 && big_output && (taps == 1 || p.Cd > 64)) && !MQ_ENV("MQ_TC_NO_HALO", 0);
   p.line = line ? 1 : 0;
   const int cd16 = mx ? (p.Cd + 31) / 32 * 32 : (p.Cd + 15) / 16 * 16;
   p.BN = cd16 <= 128 ? cd16 : 128;
