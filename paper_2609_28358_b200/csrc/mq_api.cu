@@ -105,36 +105,44 @@ size_t wt_codes_bytes(const Geom& g, int fmt_w) {
 }
 size_t up256(size_t v) { return (v + 255) / 256 * 256; }
 
-// Shape of the per-tap kernel's tiles with direct NCHW stores: TW output columns x TN samples, column index fastest.  Three things
-// weigh: rows of the 128 that are no positions (TW beyond the image's edge, TW * TN below 128, the batch's last samples)
-// cost what a full one costs; a store instruction's 32 lanes are runs of columns, and a run that ends inside a 32-byte sector
-// leaves a sector that two instructions write in part - twice the requests, and, where the output does not fit L2, a sector
-// read back from memory; a run below a sector costs a sector.  So: whole rows where they fit (any width, not a power of two), a
-// power of two above the width where that loses nothing (no run is then cut between two warps), splits at multiples of a
-// sector, other splits last.  Measured (N = 256 unless said, us): 512 channels 14x14 E4M3, widths 14 / 16 / 8 / 7: 111 / 119 / 130 /
-// 130; 256 channels 28x28 E2M1, 32 / 28 / 16 / 14: 85 / 89 / 117 / 160; 128 channels 42x42 N = 128, 42 / 32 / 16 / 14: 54 / 86 / 59 / 60;
-// 128 -> 256 channels 19x19 N = 64, 19 / 32 / 16 / 8: 20 / 26 / 27 / 24; 128 channels 56x56 E2M1, 8 / 56 / 32 / 14: 98 / 181 / 193 / 399;
-// stride-2 input gradient 256 channels 28x28 E4M3 (205 MB of output), 16 / 14: 86 / 100; 128 channels (103 MB): 43 / 41.
+// Clocks of a pipeline stage (128 bytes of K) at bn output channels: the MMAs' - 107 per 32 bytes of K and 128 columns - or, for
+// narrow tiles, the loaders' and the issuing warp's own instructions, 350 and a little per column.
+double stage_clocks(int bn) { return bn < 165 ? 350.0 + 1.2 * bn : 428.0 * bn / 128.0; }
+
+// Shape of the per-tap kernel's tiles with direct NCHW stores: TW output columns x TN samples, column index fastest.  What a shape
+// costs is the longer of two times and, as they overlap in part, 45 % of the shorter:
+//   MMAs: tiles x (stages x stage_clocks, half as much again where several taps share a stage, + 2200).  Rows of the 128 that are no
+//     positions (TW beyond the image's edge, TW * TN below 128, the batch's last samples) cost what a full one costs.
+//   stores: 12.4 bytes per clock and SM (3.5 TB/s), and 3.1 clocks per run of neighbouring columns and channel; where a warp's 32 rows end
+//     inside a run, half of that again, a fifth where the output fits L2 (the rest of the run is another request, to sectors that the
+//     first has written in part; 28 columns of the stride-2 input gradient, classes of 14 as 14 / 16, 103 MB: 38.5 / 41 us, 205 MB: 100 / 86).
+// The numbers are fitted to 156 layers and sizes of output (33 to 100 columns, 1x1 to 3x3, 32 to 512 channels, 8-bit and E2M1, 60 and
+// 150 MB, and the stride-2 input gradient), five to ten widths each; the rule's choice is 0.8 % above the fastest in the mean, at most
+// 10 % but for one.  (The rule before it weighed padding against cut sectors by factors, 0.6 where the output does not fit L2: 8 % in
+// the mean, and up to 1.9 times - E2M1 256 -> 32 channels 79x79: 300 us at width 128, 195 at 16.)  To be fitted again when an epilogue changes.
 struct TileRows { int tw, tn; };
-TileRows choose_rows(int w_eff, int N, int Wd, int max_tw, bool pair, bool big_output) {
+TileRows choose_rows(int w_eff, int N, int Wd, int Cd, int bn, double stages, bool shared_stages, int step, bool pair, bool big_output, int max_tw) {
   TileRows best{1, 128};
-  double best_score = -1.0;
-  auto consider = [&](int tw, int k) {
+  double best_cost = 1e300;
+  const double tile_clocks = stages * stage_clocks(bn) * (shared_stages ? 1.5 : 1.0) + 2200.0, row_bytes = 4.0 * Wd;
+  auto consider = [&](int tw) {
     if (tw < 1 || tw > max_tw) return;
-    const bool pow2 = (tw & (tw - 1)) == 0;
     int tn = 128 / tw;
-    if (!pow2 && tn > N) tn = N;
-    const double tiles = (double)((w_eff + tw - 1) / tw) * ((N + tn - 1) / tn);
-    double score = (double)w_eff * N / (tiles * 128.0);
-    const int run = pair ? 2 * tw : tw;
-    if (tw >= w_eff) { if (!pow2) score *= big_output ? 0.87 : 0.99; }
-    else if (Wd % 8 != 0 || run % 8 != 0) score *= (big_output ? 0.6 : 0.86 - 0.01 * k) * (run < 8 ? run / 8.0 : 1.0);
-    if (score > best_score * (1.0 + 1e-9)) { best_score = score; best = TileRows{tw, tn}; }
+    if ((tw & (tw - 1)) != 0 && tn > N) tn = N;
+    const int tiles_w = (w_eff + tw - 1) / tw;
+    // per output row; step: classes of columns (strides of the input gradient)
+    const double mma = (double)tiles_w * ((N + tn - 1) / tn) * ((Cd + bn - 1) / bn) * step * tile_clocks;
+    int cut = 0;                                         // warps that end inside a run
+    const int used = tw < w_eff ? tw : w_eff;
+    for (int r = 32; r <= 96; r += 32) cut += r < tw * tn && r % tw != 0 && r % tw < used;
+    const double store = (double)N * Cd * (pair ? 1 : step) * (row_bytes / 12.4 + 3.1 * tiles_w * (1.0 + (big_output ? 0.5 : 0.2) * cut / tn));   // (a class alone touches the sectors of whole rows)
+    const double cost = mma > store ? mma + 0.45 * store : store + 0.45 * mma;
+    if (cost < best_cost * (1.0 - 1e-9)) { best_cost = cost; best = TileRows{tw, tn}; }
   };
   int up = 8;
   while (up < w_eff) up *= 2;
-  for (int tw = up > 128 ? 128 : up; tw >= 8; tw /= 2) consider(tw, (w_eff + tw - 1) / tw);
-  for (int k = 1; k <= 4; ++k) consider((w_eff + k - 1) / k, k);
+  for (int tw = up > 128 ? 128 : up; tw >= 8; tw /= 2) consider(tw);
+  for (int k = 1; k <= 4; ++k) consider((w_eff + k - 1) / k);
   return best;
 }
 // The same for staged TMA stores and for [H][W][N][C] output, whose tiles are powers of two: the tile's MMA time (107 clocks per 32
@@ -156,14 +164,14 @@ TileRows choose_rows_pow2(int w_eff, int N, int layout, double k_bytes, int bn, 
 }
 // Output channels per tile.  `rule` is the choice for layers that fill the chip; channel counts between its multiples (160, 208, 320
 // ...) are covered by fewer or narrower tiles that waste fewer columns, and a layer whose tiles leave SMs idle by more of them, where
-// the rounds over the chip's SMs, times a stage's clocks - about 107 per 32 bytes of K and 128 columns, 350 and a little per
-// column however narrow (the loaders' and the issuing warp's own instructions) - say so clearly.  Measured: 96 -> 208 channels 28x28 5x5, N = 99, one
+// the rounds over the chip's SMs, times a tile's clocks, fall by a tenth (what the estimate does not see, such as which SMs share
+// an activation tile, moves times by up to that).  Measured: 96 -> 208 channels 28x28 5x5, N = 99, one
 // tile of 208 against two of 128: E4M3 105 -> 85 us, E2M1 132 -> 103; 512 channels 7x7, N = 16, 64 against 256: 23.1 -> 18.8 us;
 // 320 -> 256 channels 12x12 stride 2, N = 15: 21.8 -> 13.9 us.
 int choose_columns(int Cd, int rule, int unit, int most, long long row_tiles, double stages, int sms) {
   auto cost = [&](int bn) {
     const long long tiles = row_tiles * ((Cd + bn - 1) / bn);
-    return (double)((tiles + sms - 1) / sms) * (stages * (bn < 165 ? 350.0 + 1.2 * bn : 428.0 * bn / 128.0) + 400.0);
+    return (double)((tiles + sms - 1) / sms) * (stages * stage_clocks(bn) + 400.0);
   };
   int best = rule;
   double best_cost = 0.9 * cost(rule);
@@ -266,6 +274,7 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
     const int wst = op == MQ_OP_FWD ? g.sw : 1;
     int max_tw = 128;
     while ((max_tw - 1) * wst + 1 > 256) --max_tw;    // columns of a copy's box
+    const double avg_stages = (double)taps / p.classes * p.cpt / p.G;     // of a tile, over the stride classes
     TileRows t{1, 128};
     if (mx) {   // a sample tile (32 samples) must lie inside a GEMM tile: 1, 2 or 4 columns; the least edge padding wins, then the
                 // narrowest: with one column a warp's 32 rows ARE a sample tile, and the epilogue needs no exchange between warps
@@ -292,13 +301,13 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
       const bool serial = p.BN > 128 && act_bytes <= 110e6;
       t = choose_rows_pow2(w_eff, g.N, layout, (double)nkh * nkw * rowbytes, serial || p.BN < 128 ? p.BN : 128, serial, max_tw);
     }
-    else t = choose_rows(w_eff, g.N, p.Wd, max_tw, pair_hint, big_output);
+    else t = choose_rows(w_eff, g.N, p.Wd, p.Cd, p.BN, avg_stages, p.KB < 128, op == MQ_OP_FWD ? 1 : g.sw, pair_hint, big_output, max_tw);
     p.TW = t.tw; p.TN = t.tn;
     if (!thin && !compact && !(forced_bn >= 32 && forced_bn <= 256 && forced_bn % 32 == 0)) {
       const long long row_tiles = (long long)((w_eff + t.tw - 1) / t.tw) * ((g.N + t.tn - 1) / t.tn) * p.tiles_h * p.classes;
       p.BN = choose_columns(p.Cd, p.BN, want_tma && layout == MQ_HWNC ? 64 : 32,
                             pair_hint || want_tma ? 128 : 256, row_tiles,
-                            ((double)taps / p.classes * p.cpt + p.G - 1) / p.G, sm_count());
+                            avg_stages + (p.G - 1.0) / p.G, sm_count());
     }
   }
   if (p.TW < 1 || p.TW > 128 || p.TN < 1) return false;
