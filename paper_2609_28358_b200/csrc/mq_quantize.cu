@@ -235,7 +235,8 @@ __global__ void __launch_bounds__(NT) quantize_pipe_kernel(QuantArgs a, int n_ps
 // stride P.  PI = 8 (half the loads per thread, twice the blocks) where the whole grid runs at once, us, PI = 16 / 8: 64 channels
 // 13x13, N = 20: 3.4 / 2.6; 512 channels 7x7, N = 64 (224 blocks): 3.7 / 3.6; 96 channels 27x27, N = 50 (552 blocks): 4.3 / 5.1;
 // weights against quantize_few_kernel / PI = 8: 128 -> 128 3x3 3.1 / 2.6, 288 -> 78 5x5 4.8 / 2.7, 512 -> 512 3x3 (512 blocks)
-// 4.2 / 5.0.  LINE: line blocks - one scale per (position, row, 32 channels).  A block that holds a NaN gets the scale of an
+// 4.2 / 5.0; at most 8 rows, of which one or two of the eight warps hold all, 2 x 416 channels 19x19 6.9 / 5.4, 64 channels 49x49 6.1 / 4.9.
+// LINE: line blocks - one scale per (position, row, 32 channels).  A block that holds a NaN gets the scale of an
 // infinite maximum, here and in quantize_few_kernel; the other kernels' maxima pass over it.
 template <int FMT, bool SR, bool LINE, int PI>   // PI: positions per item, 16 or 8
 __global__ void __launch_bounds__(QT_THREADS, 2) quantize_odd_kernel(QuantArgs a, int n_pstrips, int Ct) {
@@ -824,7 +825,7 @@ cudaError_t launch_q(const QuantArgs& a, int n_pstrips, int Ct, long long n_item
   if (a.line || !vec) {   // (line blocks with 16-byte rows get here only as small tensors: large ones take the whole-line kernel)
     const long long tiles = n_items / n_pstrips;
     // 8-position items while they all run at once (two blocks per SM): see quantize_odd_kernel
-    const bool small = a.P > 2 && tiles * ((a.P + 7) / 8) <= 2 * sm_count();
+    const bool small = (a.P > 2 && tiles * ((a.P + 7) / 8) <= 2 * sm_count()) || (a.P > FEW_P && a.R <= 8);
     if (!small && a.P <= FEW_P && a.P % 4 != 0) {
       auto kernel = a.line ? (a.sr ? quantize_few_kernel<FMT, true, true> : quantize_few_kernel<FMT, false, true>)
                            : (a.sr ? quantize_few_kernel<FMT, true> : quantize_few_kernel<FMT, false>);

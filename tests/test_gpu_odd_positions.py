@@ -16,7 +16,8 @@ FMTS = [mq.E4M3, mq.E5M2, mq.E2M1, mq.E3M2, mq.E2M3, mq.E3M2_P6]
 W_SHAPES = [(3, 40, 1, 1), (33, 32, 1, 2), (70, 37, 3, 3), (32, 64, 5, 5), (31, 35, 3, 9), (16, 48, 7, 7),
             (3, 9573, 3, 3), (35, 2400, 5, 5), (5, 1500, 7, 7)]
 # activations N, C, H, W: 15, 30, 31, 33 and 47 positions, ragged rows and channels; then items of 16 positions
-X_SHAPES = [(70, 36, 3, 5), (40, 48, 5, 6), (33, 35, 1, 31), (5, 96, 3, 11), (64, 20, 1, 47), (3, 2380, 1, 31), (33, 1000, 3, 11)]
+X_SHAPES = [(70, 36, 3, 5), (40, 48, 5, 6), (33, 35, 1, 31), (5, 96, 3, 11), (64, 20, 1, 47), (3, 2380, 1, 31), (33, 1000, 3, 11),
+            (8, 640, 5, 9), (1, 3000, 1, 27)]          # at most 8 rows: items of 8 whatever the number of tiles
 
 
 def _case(kind, shape):
