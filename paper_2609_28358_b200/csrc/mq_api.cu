@@ -809,13 +809,30 @@ mq_status check_conv_args(int op, const mq_conv_desc* desc, const mq_qtensor* qa
   return MQ_OK;
 }
 
+// Is a 4-bit layer whose rows end inside an MMA's K-atom faster on the CUDA cores?  These have no preparation launch and no tiles to
+// fill, but a thread adds its products one after the other, so it takes sums of few products.  fp32 output, 1x1 with at most 32
+// channels: up to 20 million products, where the tensor-core call is two launches (us, tensor / CUDA cores: 32 -> 160 channels 56x56,
+// N = 1, 14.8 / 7.0; N = 2, 32 million, 15.1 / 9.7, but 28x28, N = 8, 10.7 / 12.7; paper's format 32 -> 32 7x7 8.2 / 6.6; in one launch, 32 ->
+// 32, 5.4 / 6.6).  Quantizing epilogue, whose tiles hold 32 samples even of a batch of one: by the time of each in us - rounds of tiles over
+// the SMs, by stages and blocks of 64 channels, against the chain of a sum, its products and the fp32 result between the two kernels
+// (us, tensor / CUDA cores: 32 -> 160 channels 56x56, N = 1, 30 / 14; 32 -> 224 channels 63x63 3x3, N = 1, 66 / 44; 32 -> 32 56x56 3x3,
+// N = 2, 31 / 23; N = 4, 33 / 34; 96 -> 160 channels 56x56, N = 4, 27 / 28).
+bool cuda_cores_faster(const Geom& g, const ConvTcPlan& pl) {
+  if (pl.p.kind_fp4 == 0 || pl.rowbytes % 32 == 0) return false;
+  const double terms = (double)g.Kh * g.Kw * 2.0 * pl.rowbytes, products = (double)g.N * g.Ho * g.Wo * g.Kh * g.Kw * g.Cin * g.Cout;
+  if (!pl.p.mx_out) return terms <= 32.0 && products <= 20e6 && !(pl.p.halo && pl.p.fused);
+  const double rounds = (double)((pl.p.total_tiles + sm_count() - 1) / sm_count()), outputs = (double)g.N * pl.p.Hd * pl.p.Wd * pl.p.Cd;
+  const double tc = 6.0 + rounds * (1.2 * pl.p.max_stages + 1.2 * ((pl.p.BN + 63) / 64) - 0.6), cc = 6.0 + 0.05 * terms + products / 16e6 + outputs / 0.3e6;
+  return cc < 0.92 * tc;
+}
+
 // How a call's kernels are chosen: by the rules, or - the allocation-free input gradient - for what they need of scratch
 enum class Route { RULES, COMPACT, CUDA_CORES };
 
 // Does a forward / input-gradient call of this layer, formats and output layout run on the tensor cores?  (formats: one code per byte)
 bool conv_takes_tc(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, bool line, bool ts16, ConvTcPlan* pl, Route route) {
   return route != Route::CUDA_CORES && (!ts16 || !MQ_ENV("MQ_TC_NO_TS16", 0)) && (op == MQ_OP_FWD || op == MQ_OP_BWD_DATA) && conv_tc_eligible(op, g, fmt_x_like, fmt_w) &&
-         conv_tc_plan(op, g, fmt_x_like, fmt_w, layout, pl, line, false, ts16, route == Route::COMPACT);
+         conv_tc_plan(op, g, fmt_x_like, fmt_w, layout, pl, line, false, ts16, route == Route::COMPACT) && !cuda_cores_faster(g, *pl);
 }
 
 // Operands in packed 6-bit storage: scratch, behind the call's own, for the one-code-per-byte copies of the operands no
@@ -1112,7 +1129,7 @@ mq_status run_conv_mx(int op, const mq_conv_desc* desc, const mq_qtensor* qa, in
   ConvTcPlan pl;
   // the paper's own format with rows that end inside an MMA's K-atom keeps the CUDA-core route (as its tests fix)
   const bool ts_short = ts && (op == MQ_OP_FWD ? g.Cp : g.Cop) % 64 != 0;
-  if (ts_short || !conv_tc_eligible(op, g, fmt_x_like, fmt_w) || !conv_tc_plan(op, g, fmt_x_like, fmt_w, MQ_HWNC, &pl, false, true, ts)) {
+  if (ts_short || !conv_tc_eligible(op, g, fmt_x_like, fmt_w) || !conv_tc_plan(op, g, fmt_x_like, fmt_w, MQ_HWNC, &pl, false, true, ts) || cuda_cores_faster(g, pl)) {
     // layers the tensor-core kernels do not take: the same result in two launches - the CUDA-core GEMM writes fp32
     // [pixel][sample][channel] into scratch and the channel-fastest quantizer, which applies the activation, reads it back
     const long long P = op == MQ_OP_FWD ? (long long)g.Ho * g.Wo : (long long)g.H * g.W;

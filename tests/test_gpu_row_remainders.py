@@ -15,6 +15,8 @@ SHAPES = [
     ("rows48_80", (40, 96, 5, 7, 160, 3, 1, 1)),
     ("rows112_144_s2", (33, 224, 7, 8, 288, 3, 2, 1)),  # stride 2: parity classes of the input gradient
     ("rows96_k1", (36, 192, 6, 6, 96, 1, 1, 0)),
+    ("rows16_k1", (3, 32, 6, 9, 160, 1, 1, 0)),        # E2M1: sums of 32 products, few of them - on the CUDA cores
+    ("rows16_k1_one", (1, 32, 40, 44, 160, 1, 1, 0)),  # ... and the quantizing epilogue of one sample
     ("rows16_k5", (9, 16, 9, 8, 352, 5, 1, 2)),        # three channel tiles on a thin contraction (weight tile reloaded)
 ]
 
