@@ -102,7 +102,7 @@ SHAPES = [
     ("k1_wide", (32, 256, 4, 8, 288, 1, 1, 0)),         # 256-channel tiles and a remainder tile
     ("deep_batch", (250, 128, 3, 4, 160, 3, 1, 1)),     # 8 sample tiles, the last ragged
     ("w14", (64, 64, 14, 14, 64, 3, 1, 1)),             # 14 columns: two-column tiles
-    ("odd_channels", (36, 40, 6, 6, 72, 3, 1, 1)),      # 40 -> 72 channels (E2M1: 16-byte rows): not a tensor-core layer, the two-launch route
+    ("odd_channels", (36, 40, 6, 6, 72, 3, 1, 1)),      # 40 -> 72 channels (E2M1: rows of 32 and 48 bytes, the second ending inside a K-atom)
 ]
 
 
@@ -251,6 +251,32 @@ def test_paper_format_in_and_out(name, shape, act):
         assert mq.kernel_launch_count() - n0 == (3 if name == "odd_channels" else 2)
         d_prev = inputs.conv_desc(d.N, 32, d.H, d.W, d.C_in, 1, 1, 0)
         check_emitted_ts(f"{name} bwd_data", d_prev, oracle.ROLE_DY, gx64, GEMM_TOL * ab, mq.ACT_NONE, amax, dxq)
+
+
+@pytest.mark.parametrize("fmts,env", [((E2M1, E4M3, E2M1), {}), ((E4M3, E4M3, E5M2), {"MQ_DISABLE_TC": "1"})], ids=["mixed", "forced"])
+def test_two_launch_route(fmts, env, knobs):
+    """Layers that no tensor-core kernel takes (E2M1 with an 8-bit format; forced): the CUDA-core GEMM and the quantizer that applies the
+    activation, two launches of one call."""
+    name, shape = SHAPES[1]
+    d = inputs.conv_desc(*shape)
+    src = (inputs.make_x(d, 65, "gauss"), inputs.make_w(d, 65), inputs.make_dy(d, 65, "gauss"))
+    roles = (mq.ROLE_X, mq.ROLE_W, mq.ROLE_DY)
+    hat = [oracle.dequant(d, r, f, *oracle.quantize(d, r, f, t)) for r, f, t in zip(roles, fmts, src)]
+    q = [mq.quantize(d, r, f, dev(t)) for r, f, t in zip(roles, fmts, src)]
+    knobs(**env)
+    ho, wo = inputs.out_hw(d)
+    y64, ab = oracle.conv_fwd(d, hat[0], hat[1])
+    for act in (mq.ACT_NONE, mq.ACT_RELU, mq.ACT_SILU):
+        n0 = mq.kernel_launch_count()
+        yq = mq.conv_fwd_mx(d, q[0], q[1], fmts[0], act)
+        assert mq.kernel_launch_count() - n0 == 2
+        check_emitted(f"{name} fwd", d._replace(C_in=d.C_out, H=ho, W=wo), oracle.ROLE_X, fmts[0], y64, GEMM_TOL * ab, act, yq)
+    gx64, ab = oracle.conv_bwd_data(d, hat[1], hat[2])
+    n0 = mq.kernel_launch_count()
+    dxq = mq.conv_bwd_data_mx(d, q[1], q[2], fmts[2])
+    assert mq.kernel_launch_count() - n0 == 2
+    check_emitted(f"{name} bwd_data", inputs.conv_desc(d.N, 32, d.H, d.W, d.C_in, 1, 1, 0), oracle.ROLE_DY, fmts[2], gx64, GEMM_TOL * ab, mq.ACT_NONE, dxq)
+    assert mq.last_device_status() == 0
 
 
 def _tiles_of_slab(rng, n_pix, n_cb, border, count):

@@ -1,11 +1,12 @@
 """GEMM tiles whose width is no power of two and whose channels lie between the multiples of 128 (needs a B200): whole rows of 13, 14, 19
-and 42 columns (117, 126, 114 and 126 rows of the MMA used), sector-aligned splits of a row, parity classes of 14 columns, one
-accumulator of 160 to 256 channels, narrow channel tiles where SMs are idle, block pairs on short tiles.  fp32 outputs against
-the CPU oracle within the bound of the other GEMM tests."""
+and 42 columns (117, 126, 114 and 126 rows of the MMA used), splits of a row, parity classes of 14 columns, channel tiles of 160 to
+256 channels with two accumulators and with one, narrow ones where SMs are idle, block pairs on short tiles and of every such
+width.  fp32 outputs against the CPU oracle within the bound of the other GEMM tests."""
 import pytest
 
+import oracle
 from paper_2609_28358_b200 import inputs, mq
-from parity_util import OracleLayer, check_convs, check_quantize
+from parity_util import OracleLayer, assert_gemm_close, check_convs, check_quantize, dev
 
 pytestmark = pytest.mark.gpu
 
@@ -18,9 +19,9 @@ CASES = [
     ("w60_split", (3, 64, 3, 60, 64, 5, 1, 2), {}),                 # more taps than the whole-tile kernel takes
     ("s2_28", (11, 64, 6, 28, 128, 3, 2, 1), {}),                   # 14 output columns; input gradient: classes of 14, pairs of columns
     ("s2_38", (6, 64, 5, 38, 128, 3, 2, 1), {}),                    # 19 columns
-    ("bn160", (9, 128, 4, 14, 160, 3, 1, 1), {"MQ_TC_BN": "160"}),  # one accumulator copied into registers, 80 columns a half
+    ("bn160", (9, 128, 4, 14, 160, 3, 1, 1), {"MQ_TC_BN": "160"}),  # two accumulators (2 x 160 + 5 x 24 of 512 columns), 80 columns a half
     ("bn192", (9, 128, 4, 14, 192, 3, 1, 1), {"MQ_TC_BN": "192"}),
-    ("bn224_tail", (9, 128, 4, 14, 250, 3, 1, 1), {"MQ_TC_BN": "224"}),
+    ("bn224_tail", (9, 128, 4, 14, 250, 3, 1, 1), {"MQ_TC_BN": "224"}),   # one, copied into registers
     ("k1_bn160", (9, 512, 4, 16, 250, 1, 1, 0), {"MQ_TC_BN": "160"}),   # 1x1: staged stores where the halves are whole boxes, else direct ones
     ("k1_bn192", (9, 512, 4, 16, 250, 1, 1, 0), {"MQ_TC_BN": "192"}),
     ("k1_bn224", (9, 512, 4, 16, 250, 1, 1, 0), {"MQ_TC_BN": "224"}),
@@ -47,4 +48,34 @@ def test_outputs_beyond_l2(cout):
     d = inputs.conv_desc(340 * 64 // cout, 32, 36, 36, cout, 3, 1, 1)
     ol = OracleLayer(inputs.Layer("beyond l2", d, mq.E4M3, mq.E4M3, mq.E5M2, "relu", "kaiming", "gauss", 48))
     check_convs(ol, check_quantize(ol), samples=3000, ops=("fwd",))
+    assert mq.last_device_status() == 0
+
+
+@pytest.mark.parametrize("bn", [160, 192, 224])
+def test_one_accumulator_in_the_papers_format(bn, knobs):
+    """Scale buffers of 48 columns leave one accumulator at any width above 128: the register copy, and - four tiles of 126 rows, 9
+    stages of 128-byte chunks - pairs of blocks, each with a half weight tile of 80, 96 or 112 rows.  Forward to `bn` channels and
+    back to `bn`; then with an odd number of tiles, that is without pairs."""
+    for h in (4, 3):
+        for op, cin, cout in (("fwd", 256, bn), ("dx", bn, 256)):
+            d = inputs.conv_desc(9, cin, h, 14, cout, 3, 1, 1)
+            src = (inputs.make_x(d, 51, "relu"), inputs.make_w(d, 51), inputs.make_dy(d, 51, "gauss"))
+            use = (0, 1) if op == "fwd" else (1, 2)
+            hat = [oracle.dequant_ts(d, r, *oracle.quantize_ts(d, r, src[r], (16, 16))[:3], (16, 16)) for r in use]
+            ref, ab = oracle.conv_fwd(d, *hat) if op == "fwd" else oracle.conv_bwd_data(d, *hat)
+            knobs(MQ_TC_BN=bn)
+            q = [mq.quantize_ts(d, r, dev(src[r])) for r in use]
+            for layout in (mq.NCHW, mq.HWNC):
+                got = (mq.conv_fwd if op == "fwd" else mq.conv_bwd_data)(d, *q, layout=layout)
+                assert_gemm_close(got if layout == mq.NCHW else got.permute(2, 3, 0, 1), ref, ab, f"{op} {bn} h{h} layout {layout}")
+    assert mq.last_device_status() == 0
+
+
+def test_pairs_with_a_short_last_chunk(knobs):
+    """Pairs of blocks on rows of 288 bytes: three 128-byte chunks a tap, of the last of which one K-atom is multiplied."""
+    d = inputs.conv_desc(9, 288, 4, 14, 256, 3, 1, 1)
+    ol = OracleLayer(inputs.Layer("pairs_288", d, mq.E4M3, mq.E4M3, mq.E5M2, "relu", "kaiming", "gauss", 52))
+    qs = check_quantize(ol)
+    knobs(MQ_TC_BN="256")
+    check_convs(ol, qs, layouts=(mq.NCHW, mq.HWNC))
     assert mq.last_device_status() == 0
