@@ -4,7 +4,7 @@
 // Python through ctypes (argument structures, size queries, two to three torch.empty, the stream object) a quantizer call took
 // 17.1 us and a weight gradient 26.8 us of host time, 4.3 and 8.8 us of them in the library.  Here the same steps run natively:
 // sizes come from the library, buffers from at::empty on the operands' device and the call's stream (see Launch), and the
-// interpreter lock is released around the allocations and the library call.  Nothing is kept between calls.
+// interpreter lock is released around large allocations and the library call.  Nothing is kept between calls.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
@@ -117,7 +117,7 @@ class Launch {
  public:
   void* stream = nullptr;
   Launch(PyObject* given, const at::Device& dev) {
-    if (dev.is_cuda()) device_.emplace(dev);
+    if (dev.is_cuda() && dev.index() != c10::cuda::current_device()) device_.emplace(dev);
     if (given == Py_None) { stream = c10::cuda::getCurrentCUDAStream().stream(); return; }
     const cudaStream_t s = stream_of(given);
     stream = s;
@@ -139,7 +139,10 @@ class Launch {
   std::optional<c10::cuda::CUDAStream> callers_;
 };
 at::Tensor fresh(at::IntArrayRef shape, at::ScalarType t, const at::Device& dev, bool fill) {
-  Unlocked u;
+  int64_t n = (int64_t)c10::elementSize(t);
+  for (const int64_t v : shape) n *= v;
+  std::optional<Unlocked> u;
+  if (n >= 1 << 20 || fill) u.emplace();     // (large blocks may take a cudaMalloc, or a wait for one; small ones cost less than the lock)
   at::Tensor r = at::empty(shape, at::TensorOptions().dtype(t).device(dev));
   if (fill) {
     if (at::isFloatingType(t)) r.fill_(std::numeric_limits<double>::quiet_NaN()); else r.fill_(0xA5);
