@@ -1,4 +1,5 @@
 // extern "C" entry points: argument validation, size arithmetic, kernel selection.
+#include <cmath>
 #include <atomic>
 #include <cstdlib>
 #include <map>
@@ -87,7 +88,7 @@ mq_status check_qtensor(const Geom& g, const mq_qtensor* q, int role) {
 
 // fwd / bwd_data run on the tcgen05 kernel when both operands are 8-bit formats or both are E2M1, at any channel count: a row
 // that ends inside an MMA's 32-byte K-atom is completed by the copy engine's zero fill (E2M1, 96 -> 160 channels, N = 50,
-// 27x27: the CUDA-core kernels, which took these layers before, 410 / 445 us forward / input gradient; here 30 / 30 us).
+// 27x27: the CUDA-core kernels, which took these layers before, 410 / 445 us forward / input gradient; here 30 / 30 us; small ones: cuda_cores_faster).
 bool conv_tc_eligible(int op, const Geom& g, int fmt_x_like, int fmt_w) {
   if (op != MQ_OP_FWD && op != MQ_OP_BWD_DATA) return false;
   if (MQ_ENV("MQ_DISABLE_TC", 0)) return false;
@@ -111,7 +112,7 @@ double stage_clocks(int bn) { return bn < 165 ? 350.0 + 1.2 * bn : 428.0 * bn / 
 
 // Shape of the per-tap kernel's tiles with direct NCHW stores: TW output columns x TN samples, column index fastest.  What a shape
 // costs is the longer of two times and, as they overlap in part, 45 % of the shorter:
-//   MMAs: tiles x (stages x stage_clocks, half as much again where several taps share a stage, + 2200).  Rows of the 128 that are no
+//   MMAs: rounds of tiles over the SMs x (stages x stage_clocks, half as much again where several taps share a stage, + 2200).  Rows of the 128 that are no
 //     positions (TW beyond the image's edge, TW * TN below 128, the batch's last samples) cost what a full one costs.
 //   stores: 12.4 bytes per clock and SM (3.5 TB/s), and 3.1 clocks per run of neighbouring columns and channel; where a warp's 32 rows end
 //     inside a run, half of that again, a fifth where the output fits L2 (the rest of the run is another request, to sectors that the
@@ -120,8 +121,12 @@ double stage_clocks(int bn) { return bn < 165 ? 350.0 + 1.2 * bn : 428.0 * bn / 
 // 150 MB, and the stride-2 input gradient), five to ten widths each; the rule's choice is 0.8 % above the fastest in the mean, at most
 // 10 % but for one.  (The rule before it weighed padding against cut sectors by factors, 0.6 where the output does not fit L2: 8 % in
 // the mean, and up to 1.9 times - E2M1 256 -> 32 channels 79x79: 300 us at width 128, 195 at 16.)  To be fitted again when an epilogue changes.
+// Rows that begin on a sector (multiples of 8 columns) are cut at sectors only, and there the fewest tiles are the fastest: the time
+// model's choice was 1.1 % slower in the mean over 132 layers of 16 to 112 columns, up to 26 % (whole rows between the powers of two are
+// 1 % behind, 15 % where the output does not fit L2).
 struct TileRows { int tw, tn; };
-TileRows choose_rows(int w_eff, int N, int Wd, int Cd, int bn, double stages, bool shared_stages, int step, bool pair, bool big_output, int max_tw) {
+TileRows choose_rows(int w_eff, int N, int Wd, int Cd, int bn, double stages, bool shared_stages, int step, bool pair, bool big_output, int max_tw, int Hd,
+                     int sms) {
   TileRows best{1, 128};
   double best_cost = 1e300;
   const double tile_clocks = stages * stage_clocks(bn) * (shared_stages ? 1.5 : 1.0) + 2200.0, row_bytes = 4.0 * Wd;
@@ -131,12 +136,18 @@ TileRows choose_rows(int w_eff, int N, int Wd, int Cd, int bn, double stages, bo
     if ((tw & (tw - 1)) != 0 && tn > N) tn = N;
     const int tiles_w = (w_eff + tw - 1) / tw;
     // per output row; step: classes of columns (strides of the input gradient)
-    const double mma = (double)tiles_w * ((N + tn - 1) / tn) * ((Cd + bn - 1) / bn) * step * tile_clocks;
+    const double tiles = (double)tiles_w * ((N + tn - 1) / tn) * ((Cd + bn - 1) / bn) * step;
+    const double mma = std::ceil(tiles * Hd / sms) * sms / Hd * tile_clocks;
     int cut = 0;                                         // warps that end inside a run
     const int used = tw < w_eff ? tw : w_eff;
     for (int r = 32; r <= 96; r += 32) cut += r < tw * tn && r % tw != 0 && r % tw < used;
     const double store = (double)N * Cd * (pair ? 1 : step) * (row_bytes / 12.4 + 3.1 * tiles_w * (1.0 + (big_output ? 0.5 : 0.2) * cut / tn));   // (a class alone touches the sectors of whole rows)
-    const double cost = mma > store ? mma + 0.45 * store : store + 0.45 * mma;
+    double cost = mma > store ? mma + 0.45 * store : store + 0.45 * mma;
+    if (Wd % 8 == 0) {
+      if (tw < w_eff && (pair ? 2 * tw : tw) % 8 != 0) return;
+      cost = tiles;
+      if (tw >= w_eff && (tw & (tw - 1)) != 0) cost *= big_output ? 1.15 : 1.01;
+    }
     if (cost < best_cost * (1.0 - 1e-9)) { best_cost = cost; best = TileRows{tw, tn}; }
   };
   int up = 8;
@@ -166,8 +177,8 @@ TileRows choose_rows_pow2(int w_eff, int N, int layout, double k_bytes, int bn, 
 // ...) are covered by fewer or narrower tiles that waste fewer columns, and a layer whose tiles leave SMs idle by more of them, where
 // the rounds over the chip's SMs, times a tile's clocks, fall by a tenth (what the estimate does not see, such as which SMs share
 // an activation tile, moves times by up to that).  Measured: 96 -> 208 channels 28x28 5x5, N = 99, one
-// tile of 208 against two of 128: E4M3 105 -> 85 us, E2M1 132 -> 103; 512 channels 7x7, N = 16, 64 against 256: 23.1 -> 18.8 us;
-// 320 -> 256 channels 12x12 stride 2, N = 15: 21.8 -> 13.9 us.
+// tile of 224 columns against two of 128: E4M3 101 -> 72 us, E2M1 128 -> 101; 512 channels 7x7, N = 16, the rule's tiles against 256:
+// E4M3 21.5 -> 14.8, E2M1 16.4 -> 10.8; 320 -> 256 channels 12x12 stride 2, N = 15: E4M3 20.9 -> 11.3, E2M1 17.9 -> 10.7.
 int choose_columns(int Cd, int rule, int unit, int most, long long row_tiles, double stages, int sms) {
   auto cost = [&](int bn) {
     const long long tiles = row_tiles * ((Cd + bn - 1) / bn);
@@ -240,6 +251,7 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
   // 1x1 (32 -> 64 channels 42x42, N = 333: 114 against 70); up to 64, where a tap's stage is mostly the per-tap loaders' own time,
   // they do not (3x3, 150 MB of output, E4M3 32 -> 64 channels, W = 36 / 50 / 74: 58 / 76 / 76 against 115 / 121 / 149; 64 -> 64: 61 / 78 /
   // 78 against 85 / 91 / 112)
+  // (beyond what the 126 MB of L2 hold beside the operands: sectors written in part are read back)
   const bool big_output = (double)g.N * p.Cd * p.Hd * p.Wd * 4.0 > 110e6;
   const bool thin = !line && !mx && !ts16 && g.sh == 1 && g.sw == 1 && p.cpt == 1 && p.KB <= 64 &&
                     !(p.KB == 64 && taps > 9 && (layout == MQ_NCHW || p.Cd > 32)) &&
@@ -301,7 +313,8 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
       const bool serial = p.BN > 128 && act_bytes <= 110e6;
       t = choose_rows_pow2(w_eff, g.N, layout, (double)nkh * nkw * rowbytes, serial || p.BN < 128 ? p.BN : 128, serial, max_tw);
     }
-    else t = choose_rows(w_eff, g.N, p.Wd, p.Cd, p.BN, avg_stages, p.KB < 128, op == MQ_OP_FWD ? 1 : g.sw, pair_hint, big_output, max_tw);
+    else t = choose_rows(w_eff, g.N, p.Wd, p.Cd, p.BN, avg_stages, p.KB < 128, op == MQ_OP_FWD ? 1 : g.sw, pair_hint, big_output, max_tw,
+                         p.Hd, sm_count());
     p.TW = t.tw; p.TN = t.tn;
     if (!thin && !compact && !(forced_bn >= 32 && forced_bn <= 256 && forced_bn % 32 == 0)) {
       const long long row_tiles = (long long)((w_eff + t.tw - 1) / t.tw) * ((g.N + t.tn - 1) / t.tn) * p.tiles_h * p.classes;
@@ -1127,10 +1140,12 @@ mq_status run_conv_mx(int op, const mq_conv_desc* desc, const mq_qtensor* qa, in
     fmt_x_like = op == MQ_OP_FWD ? qa->fmt : qb->fmt; fmt_w = op == MQ_OP_FWD ? qb->fmt : qa->fmt;
   }
   ConvTcPlan pl;
-  // the paper's own format with rows that end inside an MMA's K-atom keeps the CUDA-core route (as its tests fix)
+  // The paper's own format with rows that end inside an MMA's K-atom takes the CUDA-core GEMM and the quantizer: three launches, which a
+  // test counts.  It is no limit of the tensor-core kernels, which take such rows with fp32 output, and it is slow (96 -> 160
+  // channels 27x27, N = 50: 421 us forward, 456 us input gradient; with fp32 output 29 and 31, 128 -> 192 channels emitted 30 and 29).
   const bool ts_short = ts && (op == MQ_OP_FWD ? g.Cp : g.Cop) % 64 != 0;
   if (ts_short || !conv_tc_eligible(op, g, fmt_x_like, fmt_w) || !conv_tc_plan(op, g, fmt_x_like, fmt_w, MQ_HWNC, &pl, false, true, ts) || cuda_cores_faster(g, pl)) {
-    // layers the tensor-core kernels do not take: the same result in two launches - the CUDA-core GEMM writes fp32
+    // layers the tensor-core kernels do not take, or are slower on: the same result in separate launches - the CUDA-core GEMM writes fp32
     // [pixel][sample][channel] into scratch and the channel-fastest quantizer, which applies the activation, reads it back
     const long long P = op == MQ_OP_FWD ? (long long)g.Ho * g.Wo : (long long)g.H * g.W;
     const int Cd = op == MQ_OP_FWD ? g.Cout : g.Cin, Cdp = op == MQ_OP_FWD ? g.Cop : g.Cp;
