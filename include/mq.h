@@ -234,8 +234,9 @@ mq_status mq_conv_bwd_data_static(const mq_conv_desc* desc, const mq_qtensor* wq
  *                      layouts of N x C_in x H x W (codes [H][W][N][C_in_p], scales [H][W][ceil(N/32)][C_in_p/32]).
  * Arithmetic of the emitted tensor: exactly mq_quantize's (tile amax over valid elements of the fp32 result, E8M0 floor
  * rule, round-to-nearest-even, saturating, padded channels code 0) applied to the fp32-accumulated GEMM result.
- * Square blocks only.  Layers the tensor-core kernels do not take (an E2M1 operand mixed with a one-byte format; the paper's
- * format with a channel count that is no multiple of 64) give the same result in two launches inside the call: the CUDA-core GEMM
+ * Square blocks only.  Layers the tensor-core kernels do not take (an E2M1 operand mixed with a one-byte format; a forward column
+ * stride above 8; the paper's format with a contraction over channels that, rounded up to 32, are no multiple of 64) and small
+ * E2M1 layers of the latter kind give the same result in separate launches inside the call: the CUDA-core GEMM
  * writes fp32 into the workspace and the quantizer, applying the activation, reads it back.
  * workspace: ws_bytes >= mq_conv_mx_workspace_size(desc, op, fmt of the first operand, fmt of the second). */
 mq_status mq_conv_mx_workspace_size(const mq_conv_desc* desc, int op, int fmt_a, int fmt_b, size_t* bytes);
@@ -255,7 +256,7 @@ mq_status mq_conv_bwd_data_mx(const mq_conv_desc* desc, const mq_qtensor* wq, co
  *            amax_in / (448 x 6) and tensor_scale[1] = the emitted tensor's own max|value| (for the next step).
  * Arithmetic: mq_quantize_ts's, one IEEE single-precision operation per written operation of Eq. 4-6, applied to the
  * fp32-accumulated GEMM result times the two operands' tensor scales, after the activation.  Round-to-nearest-even.
- * Layers the tensor-core kernels do not take run as two launches inside the call, as above.
+ * Layers the tensor-core kernels do not take run as separate launches inside the call, as above.
  * workspace: ws_bytes >= mq_conv_ts_workspace_size(desc, op).  Errors as mq_conv_fwd_mx; operands or output that are not
  * MQ_BLOCK_TS16 give MQ_ERR_UNSUPPORTED, a null amax_in MQ_ERR_INVALID_ARG. */
 mq_status mq_conv_ts_workspace_size(const mq_conv_desc* desc, int op, size_t* bytes);

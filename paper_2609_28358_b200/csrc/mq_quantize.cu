@@ -614,61 +614,62 @@ template <int FMT, bool SR, bool LINE, bool KEEP_NAN>
 __device__ __forceinline__ void finish_tile(const QuantArgs& a, const float4 (&v)[8], int pos, int rt, int ct, int lane) {
   const int cq = lane & 7, rq = lane >> 3;
   const int r0 = rt * 32 + rq, c0 = ct * 32 + 4 * cq;
-      int code[LINE ? 8 : 1];
-      if (LINE) {
-  #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          unsigned mm = __float_as_uint(max_of<KEEP_NAN>(max_of<KEEP_NAN>(fabsf(v[i].x), fabsf(v[i].y)), max_of<KEEP_NAN>(fabsf(v[i].z), fabsf(v[i].w))));
-          mm = max(mm, __shfl_xor_sync(0xffffffffu, mm, 1));
-          mm = max(mm, __shfl_xor_sync(0xffffffffu, mm, 2));
-          mm = max(mm, __shfl_xor_sync(0xffffffffu, mm, 4));
-          code[i] = scale_code_of(mm, fmt_emax(FMT));
-          if (cq == 0 && r0 + 4 * i < a.R) a.scales[(long long)pos * a.sc_stride_p + (long long)(r0 + 4 * i) * a.sc_stride_r + ct] = (uint8_t)code[i];
-        }
-      } else {
-        float m = 0.f;
-  #pragma unroll
-        for (int i = 0; i < 8; ++i) m = max_of<KEEP_NAN>(max_of<KEEP_NAN>(m, max_of<KEEP_NAN>(fabsf(v[i].x), fabsf(v[i].y))), max_of<KEEP_NAN>(fabsf(v[i].z), fabsf(v[i].w)));
-        code[0] = scale_code_of(__reduce_max_sync(0xffffffffu, __float_as_uint(m)), fmt_emax(FMT));
-        if (lane == 0) a.scales[(long long)pos * a.sc_stride_p + (long long)rt * a.sc_stride_r + ct] = (uint8_t)code[0];
+  int code[LINE ? 8 : 1];
+  if (LINE) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      unsigned mm = __float_as_uint(max_of<KEEP_NAN>(max_of<KEEP_NAN>(fabsf(v[i].x), fabsf(v[i].y)), max_of<KEEP_NAN>(fabsf(v[i].z), fabsf(v[i].w))));
+      mm = max(mm, __shfl_xor_sync(0xffffffffu, mm, 1));
+      mm = max(mm, __shfl_xor_sync(0xffffffffu, mm, 2));
+      mm = max(mm, __shfl_xor_sync(0xffffffffu, mm, 4));
+      code[i] = scale_code_of(mm, fmt_emax(FMT));
+      if (cq == 0 && r0 + 4 * i < a.R) a.scales[(long long)pos * a.sc_stride_p + (long long)(r0 + 4 * i) * a.sc_stride_r + ct] = (uint8_t)code[i];
+    }
+  } else {
+    float m = 0.f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) m = max_of<KEEP_NAN>(max_of<KEEP_NAN>(m, max_of<KEEP_NAN>(fabsf(v[i].x), fabsf(v[i].y))), max_of<KEEP_NAN>(fabsf(v[i].z), fabsf(v[i].w)));
+    code[0] = scale_code_of(__reduce_max_sync(0xffffffffu, __float_as_uint(m)), fmt_emax(FMT));
+    if (lane == 0) a.scales[(long long)pos * a.sc_stride_p + (long long)rt * a.sc_stride_r + ct] = (uint8_t)code[0];
+  }
+  const long long pbase = (long long)pos * a.out_stride_p + c0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int r = r0 + 4 * i;
+    const float f = scale_factor(code[LINE ? i : 0]);
+    float x[4] = {v[i].x * f, v[i].y * f, v[i].z * f, v[i].w * f};
+    if (SR) {
+      const long long e0 = ((long long)r * a.C + c0) * a.P + pos;    // index in the logical tensor, whatever the source order
+#pragma unroll
+      for (int k = 0; k < 4; ++k) x[k] = sr_value<FMT>(x[k], (unsigned)e0 + (unsigned)k * (unsigned)a.P, sr_key(a, e0 + (long long)k * a.P));
+    }
+    const unsigned lo = encode2<FMT>(x[0], x[1]), hi = encode2<FMT>(x[2], x[3]);
+    const long long e = pbase + (long long)r * a.out_stride_r;
+    if (FMT == MQ_E2M1) {
+      const unsigned mine = lo | (hi << 8);                       // 4 codes; the odd lane's go above the even lane's
+      const unsigned other = __shfl_xor_sync(0xffffffffu, mine, 1);
+      if ((lane & 1) == 0 && r < a.R) *reinterpret_cast<unsigned*>(a.codes + (e >> 1)) = mine | (other << 16);
+    } else if ((FMT == MQ_E3M2 || FMT == MQ_E2M3) && a.packed6) {
+      // packed 6-bit storage: a lane's four codes are 24 bits; lanes 4j .. 4j+3 hold a 12-byte group, its word k written by
+      // lane 4j + k from its own bits and the next lane's
+      const unsigned w = lo | (hi << 16);
+      const unsigned t24 = (w & 0x3Fu) | ((w >> 2) & 0xFC0u) | ((w >> 4) & 0x3F000u) | ((w >> 6) & 0xFC0000u);
+      const unsigned nxt = __shfl_down_sync(0xffffffffu, t24, 1);
+      const int k = lane & 3;
+      if (k < 3 && r < a.R) {
+        const long long e16 = (e - 4 * k) >> 4;    // the group's index
+        *reinterpret_cast<unsigned*>(a.codes + e16 * 12 + 4 * k) = (t24 >> (8 * k)) | (nxt << (24 - 8 * k));
       }
-      const long long pbase = (long long)pos * a.out_stride_p + c0;
-  #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int r = r0 + 4 * i;
-        const float f = scale_factor(code[LINE ? i : 0]);
-        float x[4] = {v[i].x * f, v[i].y * f, v[i].z * f, v[i].w * f};
-        if (SR) {
-          const long long e0 = ((long long)r * a.C + c0) * a.P + pos;    // index in the logical tensor, whatever the source order
-  #pragma unroll
-          for (int k = 0; k < 4; ++k) x[k] = sr_value<FMT>(x[k], (unsigned)e0 + (unsigned)k * (unsigned)a.P, sr_key(a, e0 + (long long)k * a.P));
-        }
-        const unsigned lo = encode2<FMT>(x[0], x[1]), hi = encode2<FMT>(x[2], x[3]);
-        const long long e = pbase + (long long)r * a.out_stride_r;
-        if (FMT == MQ_E2M1) {
-          const unsigned mine = lo | (hi << 8);                       // 4 codes; the odd lane's go above the even lane's
-          const unsigned other = __shfl_xor_sync(0xffffffffu, mine, 1);
-          if ((lane & 1) == 0 && r < a.R) *reinterpret_cast<unsigned*>(a.codes + (e >> 1)) = mine | (other << 16);
-        } else if ((FMT == MQ_E3M2 || FMT == MQ_E2M3) && a.packed6) {
-          // packed 6-bit storage: a lane's four codes are 24 bits; lanes 4j .. 4j+3 hold a 12-byte group, its word k written by
-          // lane 4j + k from its own bits and the next lane's
-          const unsigned w = lo | (hi << 16);
-          const unsigned t24 = (w & 0x3Fu) | ((w >> 2) & 0xFC0u) | ((w >> 4) & 0x3F000u) | ((w >> 6) & 0xFC0000u);
-          const unsigned nxt = __shfl_down_sync(0xffffffffu, t24, 1);
-          const int k = lane & 3;
-          if (k < 3 && r < a.R) {
-            const long long e16 = (e - 4 * k) >> 4;    // the group's index
-            *reinterpret_cast<unsigned*>(a.codes + e16 * 12 + 4 * k) = (t24 >> (8 * k)) | (nxt << (24 - 8 * k));
-          }
-        } else {
-          if (r < a.R) *reinterpret_cast<unsigned*>(a.codes + e) = lo | (hi << 16);
-        }
-      }
+    } else {
+      if (r < a.R) *reinterpret_cast<unsigned*>(a.codes + e) = lo | (hi << 16);
+    }
+  }
 }
 
 // Few positions (at most FEW_P, no multiple of 4: the taps of a weight tensor, tiny images): the 32 channels x P positions of a row
 // are ONE run of 32 P floats.  A block copies the 32 runs of a tile into shared memory (asynchronous 4-byte copies, a warp's lanes
-// side by side: whole lines, all in flight at once; rows of 32 P + 1 floats, so that the reads below meet no bank twice), and
+// side by side: whole lines, all in flight at once; rows of 32 P + 1 floats, so that the reads below meet no bank twice for an odd P,
+// two lanes in a bank for 2, 6, 10, ...), and
 // each warp then quantizes a position at a time.  512 -> 512 channels, 3x3: 5.6 -> 4.3 us against one 4-byte load per lane at
 // stride P.  (Rows fetched by cp.async.bulk instead: 5.4 us, 4.0 instead of 3.0 where one round of loads is all there is.)
 constexpr int FEW_P = 25;

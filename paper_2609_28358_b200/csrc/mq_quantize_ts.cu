@@ -9,7 +9,8 @@
 // that an atomic maximum starts from costs what the reduction does, keep the two launches).
 //
 // Every operation of Eq. 4-6 is one IEEE single-precision operation, in the order written (division = __fdiv_rn,
-// products = __fmul_rn): the roundings decide integer codes, so nothing here may be contracted or approximated.
+// products = __fmul_rn): the roundings decide integer codes, so nothing here may be contracted.  Eq. 6's quotient decides no more than
+// which of eight magnitudes comes out: ts_codes8 multiplies by the reciprocal and divides only where that product does not say.
 // CastE4M3 and Round(.) are the hardware's round-to-nearest-even, saturating conversions.
 //
 // quantize_ts_kernel: one warp per (16 x 16 block, 8 consecutive positions).  Lane (r, h) = (lane >> 1, lane & 1) owns
