@@ -248,51 +248,93 @@ __global__ void __launch_bounds__(GT) bwd_weight_generic(ConvArgs a, int splits)
   }
 }
 
-// Adds the split-K partial sums [split][Cout][taps][Cp] in a fixed order and writes G_W in its final layout.
-// The reads are `splits` times the writes, so threads follow the partials' own order (4 consecutive input
-// channels per thread, 16-byte loads); a block's four thread groups take every fourth split each and are
-// combined through shared memory in group order, so the result does not depend on scheduling.
+// ---- sums of the split-K partials [split][Cout][taps][Cp], added in a fixed order and written in G_W's final layout -----------------
+// Reads are 16 bytes per thread, consecutive threads along the partials' own order; `groups` neighbouring thread groups share a
+// block's sums (every groups-th split each, combined through shared memory in group order: independent of scheduling).
 // ta, tb: the two tensors' fp32 scales when the partial sums still lack them (tensor-core GEMM on E4M3-scaled blocks, Eq. 4), else null
-__global__ void __launch_bounds__(256) bwd_weight_reduce(const float* __restrict__ part, float* __restrict__ out, Geom g, int splits, int layout,
-                                                         const float* __restrict__ ta, const float* __restrict__ tb) {
+constexpr int RED_THREADS = 256, RED_RUNS_MAX = 512;
+template <int GROUPS>
+__device__ __forceinline__ float4 sum_of_splits(const float4* p, long long slab4, int grp, int splits) {
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+  for (int k = grp; k < splits; k += GROUPS) {
+    const float4 v = __ldg(p + (long long)k * slab4);
+    s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+  }
+  return s;
+}
+// adds the other groups' sums to group 0's (threads of group q hold theirs `per` threads apart)
+template <int GROUPS>
+__device__ __forceinline__ void sum_of_groups(float4& s, float4* sh, int grp, int per) {
+  if (GROUPS == 1) return;
+  if (grp > 0 && grp < GROUPS) sh[threadIdx.x] = s;
+  __syncthreads();
+  if (grp == 0) {
+#pragma unroll
+    for (int q = 1; q < GROUPS; ++q) { const float4 v = sh[threadIdx.x + q * per]; s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w; }
+  }
+}
+// Any layer: a block takes RED_THREADS / GROUPS consecutive float4s of the partials.
+template <int GROUPS>
+__global__ void __launch_bounds__(RED_THREADS) bwd_weight_reduce(const float* __restrict__ part, float* __restrict__ out, Geom g, int splits, int layout,
+                                                                 const float* __restrict__ ta, const float* __restrict__ tb) {
   pdl_wait();
+  __shared__ float4 sh[RED_THREADS];
+  constexpr int per = RED_THREADS / GROUPS;
   const float os = ta ? __ldg(ta) * __ldg(tb) : 1.f;
-  __shared__ float4 sh[3][64];
   const int taps = g.Kh * g.Kw;
   const int cq = g.Cp >> 2;                                   // float4 columns per (co, tap)
   const long long quads = (long long)g.Cout * taps * cq;
-  const long long slab = (long long)g.Cout * taps * g.Cp;     // floats per split
-  const int col = threadIdx.x & 63, grp = threadIdx.x >> 6;
-  for (long long base = (long long)blockIdx.x * 64; base < quads; base += (long long)gridDim.x * 64) {
+  const int grp = (int)threadIdx.x / per, col = (int)threadIdx.x % per;
+  for (long long base = (long long)blockIdx.x * per; base < quads; base += (long long)gridDim.x * per) {
     const long long qd = base + col;
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (qd < quads) {
-      const float4* p = reinterpret_cast<const float4*>(part) + qd;
-#pragma unroll 4
-      for (int k = grp; k < splits; k += 4) {
-        const float4 v = __ldg(p + (long long)k * (slab >> 2));
-        s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
-      }
-    }
-    if (grp > 0) sh[grp - 1][col] = s;
-    __syncthreads();
+    if (qd < quads) s = sum_of_splits<GROUPS>(reinterpret_cast<const float4*>(part) + qd, quads, grp, splits);
+    sum_of_groups<GROUPS>(s, sh, grp, per);
     if (grp == 0 && qd < quads) {
-#pragma unroll
-      for (int q = 0; q < 3; ++q) { const float4 v = sh[q][col]; s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w; }
       const int c4 = (int)(qd % cq); const long long r = qd / cq;
-      const int tap = (int)(r % taps), co = (int)(r / taps);
+      const int tap = (int)(r % taps), co = (int)(r / taps), ci0 = 4 * c4;
       const float vals[4] = {s.x * os, s.y * os, s.z * os, s.w * os};
+      const bool rows = layout != MQ_NCHW || taps == 1;       // channel-fastest
+      float* o = rows ? out + ((long long)co * taps + tap) * g.Cin + ci0 : out + ((long long)co * g.Cin + ci0) * taps + tap;
+      if (rows && (g.Cin & 3) == 0) { if (ci0 < g.Cin) *reinterpret_cast<float4*>(o) = make_float4(vals[0], vals[1], vals[2], vals[3]); }
+      else {
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int ci = 4 * c4 + e;
-        if (ci < g.Cin) {
-          if (layout == MQ_NCHW) out[((long long)co * g.Cin + ci) * taps + tap] = vals[e];
-          else out[((long long)co * taps + tap) * g.Cin + ci] = vals[e];
-        }
+        for (int e = 0; e < 4; ++e) if (ci0 + e < g.Cin) o[(long long)e * (rows ? 1 : taps)] = vals[e];
       }
     }
     __syncthreads();
   }
+}
+// [C_out][C_in][taps] results of layers with many channels.  There the four channels that a thread has added lie taps floats apart, a
+// sector each, and those stores take longer than the reads; so a block takes all taps of R channels of one output channel, which
+// G_W holds as one run, turns them in shared memory and stores whole lines.  (Whole call, before -> now: 512 -> 512 channels 14x14, E2M1,
+// N = 256, 3 splits 85.5 -> 75.7 us, N = 64 41.8 -> 31.8; 256 -> 256 14x14, N = 64, 12 splits 22.1 -> 19.4.)
+template <int GROUPS>
+__global__ void __launch_bounds__(RED_RUNS_MAX) bwd_weight_reduce_runs(const float* __restrict__ part, float* __restrict__ out, Geom g, int splits, int R, int nr,
+                                                                       int per, const float* __restrict__ ta, const float* __restrict__ tb) {
+  pdl_wait();
+  extern __shared__ __align__(16) float red_stage[];          // [R][taps]
+  __shared__ float4 sh[RED_RUNS_MAX];
+  const float os = ta ? __ldg(ta) * __ldg(tb) : 1.f;
+  const int taps = g.Kh * g.Kw;
+  const long long slab4 = (long long)g.Cout * taps * (g.Cp >> 2);     // float4s per split
+  const int co = (int)blockIdx.x / nr, ci0 = ((int)blockIdx.x - co * nr) * R;
+  const int rq = min(R, g.Cp - ci0) >> 2, nq = taps * rq;
+  const int grp = (int)threadIdx.x / per, i = (int)threadIdx.x - grp * per;
+  const int tap = i / rq, c = 4 * (i - tap * rq);
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (grp < GROUPS && i < nq)      // (the block's last warp may be only partly in use)
+    s = sum_of_splits<GROUPS>(reinterpret_cast<const float4*>(part + ((long long)co * taps + tap) * g.Cp + ci0 + c), slab4, grp, splits);
+  sum_of_groups<GROUPS>(s, sh, grp, per);
+  if (grp == 0 && i < nq) {
+    red_stage[c * taps + tap] = s.x * os; red_stage[(c + 1) * taps + tap] = s.y * os;
+    red_stage[(c + 2) * taps + tap] = s.z * os; red_stage[(c + 3) * taps + tap] = s.w * os;
+  }
+  __syncthreads();
+  const int n = min(R, g.Cin - ci0) * taps;       // (channels of the padding are left out)
+  float* o = out + ((long long)co * g.Cin + ci0) * taps;
+  for (int k = threadIdx.x; k < n; k += blockDim.x) o[k] = red_stage[k];
 }
 
 }  // namespace
@@ -315,11 +357,30 @@ size_t conv_generic_workspace(int op, const Geom& g) {
 
 cudaError_t launch_bwd_weight_reduce(const float* partial, float* out, const Geom& g, int splits, int layout, cudaStream_t s, const float* ta,
                                      const float* tb) {
-  const long long quads = (long long)g.Cout * g.Kh * g.Kw * (g.Cp / 4);
-  unsigned blocks = (unsigned)((quads + 63) / 64);
-  if (blocks > (unsigned)sm_count() * 16) blocks = (unsigned)sm_count() * 16;
+  const int taps = g.Kh * g.Kw, sms = sm_count();
   count_launches(1);
-  return launch_pdl(bwd_weight_reduce, dim3(blocks), dim3(256), 0, s, partial, out, g, splits, layout, ta, tb);
+  // Whole runs: blocks of 64 or 128 channels (two lines per read, at least) that give every SM two, and more with many splits, where the
+  // reads are what takes the time and the other kernel has more threads in flight (whole call, 96 -> 160 channels 27x27, 320 blocks, 24
+  // splits: 24.1 us as runs, 22.1; 64 -> 320 102x178 stride 2, 320, 16: 28.9 / 27.3; 256 -> 256 28x28, 512, 12: 87.6 / 91.8).
+  for (int R = 128; R >= 64 && layout == MQ_NCHW && taps > 1; R /= 2) {
+    const int nr = (g.Cp + R - 1) / R, per = taps * (R / 4);
+    const long long units = (long long)g.Cout * nr;
+    if (R > g.Cp || per > RED_RUNS_MAX || 4 * units < sms * (splits > 8 ? splits : 8) || units > 0x7fffffffLL) continue;
+    const bool two = 2 * per <= RED_RUNS_MAX && splits > 1;
+    const unsigned threads = (unsigned)((two ? 2 : 1) * per + 31) / 32 * 32;
+    return launch_pdl(two ? bwd_weight_reduce_runs<2> : bwd_weight_reduce_runs<1>, dim3((unsigned)units), dim3(threads), (size_t)R * taps * sizeof(float), s,
+                      partial, out, g, splits, R, nr, per, ta, tb);
+  }
+  // four groups, more where that leaves SMs idle and a group still has a few splits to add (32 -> 32 channels 32x32, 49 splits, the call:
+  // 9.9 us with four, 9.1 with sixteen)
+  const long long quads = (long long)g.Cout * taps * (g.Cp / 4);
+  int groups = 4;
+  while (groups < 16 && quads * groups < 512ll * sms && splits >= 4 * groups) groups *= 2;
+  const int per = RED_THREADS / groups;
+  unsigned blocks = (unsigned)((quads + per - 1) / per);
+  if (blocks > (unsigned)sms * 16) blocks = (unsigned)sms * 16;
+  auto kernel = groups == 4 ? bwd_weight_reduce<4> : groups == 8 ? bwd_weight_reduce<8> : bwd_weight_reduce<16>;
+  return launch_pdl(kernel, dim3(blocks), dim3(RED_THREADS), 0, s, partial, out, g, splits, layout, ta, tb);
 }
 
 // Two template classes per operand: packed E2M1 (2) or one byte per code (0; the format itself is read at run time)
@@ -349,11 +410,8 @@ cudaError_t launch_conv_generic(int op, const ConvArgs& a, cudaStream_t s) {
     MQ_DISPATCH2(a.fmt_a, a.fmt_b, (bwd_weight_generic<A_, B_><<<grid, GT, 0, s>>>(a, splits)));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const long long quads = (long long)g.Cout * g.Kh * g.Kw * (g.Cp / 4);
-    unsigned blocks = (unsigned)((quads + 63) / 64);
-    if (blocks > (unsigned)sm_count() * 16) blocks = (unsigned)sm_count() * 16;
-    bwd_weight_reduce<<<blocks, 256, 0, s>>>(reinterpret_cast<const float*>(a.workspace), a.out, g, splits, a.out_layout, nullptr, nullptr);
-    count_launches(1);
+    e = launch_bwd_weight_reduce(reinterpret_cast<const float*>(a.workspace), a.out, g, splits, a.out_layout, s, nullptr, nullptr);
+    if (e != cudaSuccess) return e;
   }
   count_launches(1);
   return cudaGetLastError();

@@ -1,0 +1,33 @@
+"""Sums of the weight gradient's split-K partials (needs a B200): blocks of whole runs of G_W with one and two thread groups, a run that
+ends in padding channels, kernels of 4 to 25 taps, and the kernel for every other layer with 4, 8 and 16 groups, in both layouts.  Against the CPU
+oracle within the bound of the other GEMM tests."""
+import pytest
+
+from paper_2609_28358_b200 import inputs, mq
+from parity_util import OracleLayer, check_convs, check_quantize
+
+pytestmark = pytest.mark.gpu
+
+# N, C_in, H, W, C_out, kernel, stride, padding; split-K slices (0: the plan's)
+CASES = [
+    ("runs128", (3, 128, 4, 4, 300, 3, 1, 1), 5),
+    ("runs128_tail", (3, 205, 4, 4, 160, 3, 1, 1), 3),     # 224 stored channels: the second run holds 96, 77 of them G_W's
+    ("runs64_two_groups", (3, 70, 5, 5, 160, 3, 1, 1), 5),   # 96 stored channels, 70 real ones
+    ("runs64_one_split", (3, 64, 4, 4, 300, 2, 1, 0), 1),
+    ("runs64_25_taps", (3, 64, 6, 6, 300, 5, 1, 2), 8),
+    ("groups4", (3, 33, 5, 5, 40, 3, 1, 1), 7),
+    ("groups8", (3, 33, 8, 8, 40, 3, 1, 1), 16),
+    ("groups16", (3, 32, 10, 10, 32, 3, 1, 1), 33),
+    ("pointwise_odd", (3, 30, 9, 9, 40, 1, 1, 0), 16),
+]
+
+
+@pytest.mark.parametrize("fmts", [(mq.E4M3, mq.E4M3, mq.E5M2), (mq.E2M1,) * 3], ids=["fp8", "fp4"])
+@pytest.mark.parametrize("name,shape,splits", CASES, ids=[c[0] for c in CASES])
+def test_weight_gradient(name, shape, splits, fmts, knobs):
+    d = inputs.conv_desc(*shape)
+    ol = OracleLayer(inputs.Layer(name, d, *fmts, "relu", "kaiming", "gauss", 51))
+    qs = check_quantize(ol)
+    knobs(MQ_WGRAD_SPLITS=str(splits))
+    check_convs(ol, qs, layouts=(mq.NCHW, mq.HWNC), ops=("dw",))
+    assert mq.last_device_status() == 0
