@@ -1354,6 +1354,7 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   const uint32_t sfb_base = tmem + p.n_acc * p.BN;
   const uint32_t sfa_base = sfb_base + (uint32_t)nsf * 16;
   const uint32_t sfa_cols_stage = (uint32_t)nsf * 8;
+  const bool two_issuers = p.fused && p.mma_cp && p.n_acc == 2;
 
   if (warp == 0) {
     // ------------------------------------------------------------------ producer
@@ -1388,27 +1389,30 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         if (++s == (uint32_t)p.stages) { s = 0; phase ^= 1; }
       }
     }
-  } else if (warp == 1) {
-    // ------------------------------------------------------------------ MMA issuer: all taps of a tile per stage
+  } else if (warp == 1 || (warp == 2 && two_issuers)) {
+    // ------------------------------------------------------------------ MMA issuers: all taps of a tile per stage
     {
+      const uint32_t first = two_issuers ? (uint32_t)warp - 1u : 0u, step = two_issuers ? 2u : 1u;
       const uint64_t a_desc_base = smem_desc_base(16, (uint32_t)(p.WH * KB), LAYOUT);   // 8-row groups one halo row apart
       const uint64_t b_desc_base = smem_desc_base(16, 8 * KB, LAYOUT);
       const uint32_t sb16 = smem_u32(smem) >> 4;
       uint32_t idesc_id[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) idesc_id[i] = idesc_with_sf_ids(p.idesc, i, i);
-      uint32_t s = 0, phase = 0, tcount = 0, bcount = 0;
+      uint32_t s = first, phase = 0, tcount = first, bcount = 0;
       int cur_ct = -1;
       constexpr int TU = TAPS > 0 ? TAPS : 1;
       uint32_t ta[TU], tb[TU];
 #pragma unroll
       for (int q = 0; q < TU; ++q) { ta[q] = tap_a[q]; tb[q] = tap_b[q]; }
       const uint32_t acc_mask = (uint32_t)p.n_acc - 1, acc_shift = (uint32_t)p.n_acc - 1;   // n_acc is 1 or 2
-      for (unsigned t = blockIdx.x; t < total && !warp_flag(abort_flag); t += gridDim.x, ++tcount) {
+      for (unsigned t = blockIdx.x + first * gridDim.x; t < total && !warp_flag(abort_flag); t += step * gridDim.x, tcount += step) {
         const int ct = p.tiles_c == 1 ? 0 : (int)((t / tiles_per_c) % (unsigned)p.tiles_c);
         const bool new_b = ct != cur_ct;
         if (new_b) {
           if (!mbar_wait_warp(bfull, bcount & 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
+          // the second issuer: the first one's copies of the resident scale vectors have arrived in tensor memory
+          if (first == 1u && !mbar_wait_warp(bempty, 0, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
           cur_ct = ct; ++bcount;
         }
         const int acc = (int)(tcount & acc_mask);
@@ -1421,7 +1425,7 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         if (elect_one()) {
         if (p.mma_cp) {   // this lane issues the scale copies itself, right before the MMAs that read them
           const uint64_t sf_desc = smem_desc_base(0, 128, 0);
-          if (new_b) {
+          if (new_b && first == 0u) {
             const uint32_t sfb_s = smem_u32(smem + b_bytes);
 #pragma unroll 1
             for (int st = 0; st < nsf; ++st)
@@ -1430,6 +1434,7 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
 #pragma unroll 1
                 for (int a2 = 0; a2 < atoms_b; ++a2)
                   tmem_cp_32x128b_warpx4(sfb_base + st * 16 + 4 * (g * atoms_b + a2), smem_desc(sf_desc, sfb_s + ((st * SPA + g) * atoms_b + a2) * 512));
+            if (two_issuers) tc_commit(bempty);
           }
           const uint32_t sfa_sm = smem_u32(stage0 + (size_t)s * stage_bytes + p.halo_a_bytes);
 #pragma unroll 1
@@ -1468,7 +1473,8 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         }
         }
         __syncwarp();
-        if (++s == (uint32_t)p.stages) { s = 0; phase ^= 1; }
+        s += step;
+        if (s >= (uint32_t)p.stages) { s -= (uint32_t)p.stages; phase ^= 1; }
       }
     }
   } else if (warp == 2) {
@@ -1510,9 +1516,11 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         if (++s == (uint32_t)p.stages) { s = 0; phase ^= 1; }
       }
     }
-  } else if (warp == 3) {
-    // ------------------------------------------------------------------ activation-scale expander (fused mode)
-    if (p.fused) {
+  } else if (warp == 3 || warp >= 12) {
+    // ------------------------------------------------------------------ activation-scale expanders (fused mode): a warp per stage
+    const int s = warp == 3 ? 0 : warp - 11;
+    if (p.fused && s < p.stages) {
+      uint8_t* tbl = sc_tbl + 128 * s;
       constexpr int BPC = APC * SPA;                       // scale bytes per tap per row = K-blocks of a tap
       const int WT = p.TW + p.Kw - 1, npix = p.Kh * WT;
       // this lane's patch entries e = lane + 32 i: (halo row, column, K-block), fixed for the whole kernel
@@ -1526,8 +1534,8 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       int twj[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) twj[j] = (32 * j + lane) & (p.TW - 1);
-      uint32_t s = 0, phase = 0;
-      for (unsigned t = blockIdx.x; t < total && !*abort_flag; t += gridDim.x) {
+      uint32_t phase = 0;
+      for (unsigned t = blockIdx.x + (unsigned)s * gridDim.x; t < total && !*abort_flag; t += (unsigned)p.stages * gridDim.x, phase ^= 1) {
         const Tile tile = decode_tile(p, t);
         const int hs = MODE == MQ_OP_FWD ? tile.h - p.ph : tile.h + p.ph - (p.Kh - 1);
         const int ws = MODE == MQ_OP_FWD ? tile.w0 - p.pw : tile.w0 + p.pw - (p.Kw - 1);
@@ -1546,7 +1554,7 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
         if (!ok) { *abort_flag = 1; break; }
 #pragma unroll
-        for (int i = 0; i < 4; ++i) sc_tbl[lane + 32 * i] = raw[i];
+        for (int i = 0; i < 4; ++i) tbl[lane + 32 * i] = raw[i];
         __syncwarp();
         uint8_t* dst = stage0 + (size_t)s * stage_bytes + p.halo_a_bytes + lane * 16;
 #pragma unroll 1
@@ -1559,7 +1567,7 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
               const uint32_t pb = tap_p[q];
 #pragma unroll
               for (int j = 0; j < 4; ++j) {
-                const uint8_t* src = sc_tbl + (pb + twj[j]) * BPC;
+                const uint8_t* src = tbl + (pb + twj[j]) * BPC;
                 unsigned long long v;
                 if (BPC == 1) v = *src;
                 else if (BPC == 2) v = *reinterpret_cast<const unsigned short*>(src);
@@ -1576,7 +1584,6 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) mbar_arrive(&full[s]);
-        if (++s == (uint32_t)p.stages) { s = 0; phase ^= 1; }
       }
     }
   } else if (warp >= 4 && warp < 12) {
