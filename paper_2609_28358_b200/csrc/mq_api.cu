@@ -745,8 +745,7 @@ mq_status run_wgrad_tc(const Geom& g, WgradPlan& w, const mq_qtensor* qx, const 
       g_codes = gt; fmt_g_eff = MQ_E4M3;
     }
     if (w.recode4) {
-      if (launch_recode4_e4m3(x_codes, xt, (size_t)g.H * g.W * g.N * g.Cp, stream) != cudaSuccess) return MQ_ERR_CUDA;
-      if (launch_recode4_e4m3(g_codes, gt, (size_t)g.Ho * g.Wo * g.N * g.Cop, stream) != cudaSuccess) return MQ_ERR_CUDA;
+      if (launch_wgrad_recode4(p, x_codes, xt, (size_t)g.H * g.W * g.N * g.Cp, g_codes, gt, (size_t)g.Ho * g.Wo * g.N * g.Cop, stream) != cudaSuccess) return MQ_ERR_CUDA;
       x_codes = xt; g_codes = gt; fmt_x_eff = MQ_E4M3; fmt_g_eff = MQ_E4M3;
     }
     const uint32_t fa = fmt_mma_code(fmt_g_eff), fb = fmt_mma_code(fmt_x_eff);
@@ -771,7 +770,7 @@ mq_status run_wgrad_tc(const Geom& g, WgradPlan& w, const mq_qtensor* qx, const 
   if (p.mode == MQ_WG_FP4_FLAT) {
     if (launch_wgrad_flat_prep(p, static_cast<const uint8_t*>(qx->codes), xt, w.P_b, static_cast<const uint8_t*>(qg->codes), gt, w.P_a, stream) != cudaSuccess)
       return MQ_ERR_CUDA;
-  } else if ((p.mode == MQ_WG_FP4_PIXEL || p.cta2) && launch_expand_wgrad_scales(p, stream) != cudaSuccess) return MQ_ERR_CUDA;
+  } else if ((p.mode == MQ_WG_FP4_PIXEL || (p.cta2 && !w.recode4)) && launch_expand_wgrad_scales(p, stream) != cudaSuccess) return MQ_ERR_CUDA;
   CUtensorMap map_p{};
   {
     const uint64_t J = (uint64_t)g.Kh * g.Kw * g.Cp;

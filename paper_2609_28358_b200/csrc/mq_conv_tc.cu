@@ -2141,14 +2141,27 @@ cudaError_t launch_pack6(const uint8_t* in, uint8_t* out, size_t nbytes, cudaStr
 
 // Packed 6-bit storage (16 codes in 12 bytes) -> what a kernel reads.  MODE 0: the MMA's container (the 12 bytes + 4 bytes of
 // padding); 1: one code per byte; 2: E4M3 bytes of the same values (the weight gradient's 8-bit path).
+// Bound by memory: a thread asks for its four groups before it converts the first (one group at a time, of a persistent grid,
+// left 24 KB per SM in flight).
+constexpr int UNPACK_PER_THREAD = 4;
 template <int MODE, bool IS_E3M2>
 __global__ void __launch_bounds__(256) unpack6_kernel(const uint32_t* __restrict__ in, uint4* __restrict__ out, size_t ngroups) {
   pdl_wait();
-  for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < ngroups; i += (size_t)gridDim.x * 256) {
-    const uint32_t f[3] = {__ldg(in + 3 * i), __ldg(in + 3 * i + 1), __ldg(in + 3 * i + 2)};
-    if (MODE == 0) { out[i] = make_uint4(f[0], f[1], f[2], 0u); continue; }
+  const size_t base = (size_t)blockIdx.x * (256 * UNPACK_PER_THREAD) + threadIdx.x;
+  uint32_t f[UNPACK_PER_THREAD][3];
+#pragma unroll
+  for (int k = 0; k < UNPACK_PER_THREAD; ++k) {
+    const size_t i = base + 256 * k;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) f[k][j] = i < ngroups ? __ldg(in + 3 * i + j) : 0u;
+  }
+#pragma unroll
+  for (int k = 0; k < UNPACK_PER_THREAD; ++k) {
+    const size_t i = base + 256 * k;
+    if (i >= ngroups) return;
+    if (MODE == 0) { out[i] = make_uint4(f[k][0], f[k][1], f[k][2], 0u); continue; }
     uint32_t w[4];
-    unpack6x16(f, w);
+    unpack6x16(f[k], w);
     if (MODE == 2) {
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
@@ -2168,8 +2181,7 @@ __global__ void __launch_bounds__(256) unpack6_kernel(const uint32_t* __restrict
 cudaError_t launch_unpack6(const uint8_t* in, uint8_t* out, size_t n_codes, int mode, int fmt6, cudaStream_t s) {
   const size_t ngroups = n_codes / 16;
   if (ngroups == 0) return cudaSuccess;
-  size_t blocks = (ngroups + 255) / 256;
-  if (blocks > sm_count() * 16) blocks = sm_count() * 16;
+  const size_t blocks = (ngroups + 256 * UNPACK_PER_THREAD - 1) / (256 * UNPACK_PER_THREAD);
   count_launches(1);
   const uint32_t* src = reinterpret_cast<const uint32_t*>(in);
   uint4* dst = reinterpret_cast<uint4*>(out);
@@ -2207,36 +2219,6 @@ cudaError_t launch_recode6_e4m3(const uint8_t* in, uint8_t* out, size_t nbytes, 
   count_launches(1);
   if (fmt6 == MQ_E3M2) return launch_pdl(recode6_kernel<true>, dim3((unsigned)blocks), dim3(256), 0, s, reinterpret_cast<const uint4*>(in), reinterpret_cast<uint4*>(out), nchunks);
   return launch_pdl(recode6_kernel<false>, dim3((unsigned)blocks), dim3(256), 0, s, reinterpret_cast<const uint4*>(in), reinterpret_cast<uint4*>(out), nchunks);
-}
-
-__global__ void __launch_bounds__(256) recode4_kernel(const uint2* __restrict__ in, uint4* __restrict__ out, size_t nchunks) {
-  pdl_wait();
-  // E2M1 magnitudes 0, .5, 1, 1.5, 2, 3, 4, 6 as E4M3 bytes; the sign moves from bit 3 of the nibble to bit 7 of the byte
-  const uint32_t lut_lo = 0x3C383000u, lut_hi = 0x4C484440u;
-  for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < nchunks; i += (size_t)gridDim.x * 256) {
-    const uint2 v = __ldg(in + i);
-    const uint32_t src[2] = {v.x, v.y};
-    uint32_t w[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      uint32_t r = 0;
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const uint32_t nib = (src[q >> 1] >> (16 * (q & 1) + 4 * b)) & 0xFu;
-        r |= (__byte_perm(lut_lo, lut_hi, nib & 7u) & 0xFFu | ((nib & 8u) << 4)) << (8 * b);
-      }
-      w[q] = r;
-    }
-    out[i] = make_uint4(w[0], w[1], w[2], w[3]);
-  }
-}
-cudaError_t launch_recode4_e4m3(const uint8_t* in, uint8_t* out, size_t n_out, cudaStream_t s) {
-  const size_t nchunks = n_out / 16;
-  if (nchunks == 0) return cudaSuccess;
-  size_t blocks = (nchunks + 255) / 256;
-  if (blocks > sm_count() * 16) blocks = sm_count() * 16;
-  count_launches(1);
-  return launch_pdl(recode4_kernel, dim3((unsigned)blocks), dim3(256), 0, s, reinterpret_cast<const uint2*>(in), reinterpret_cast<uint4*>(out), nchunks);
 }
 
 cudaError_t launch_conv_tc(const ConvTcParams& p, const CUtensorMap& map_a, const CUtensorMap& map_w, const CUtensorMap& map_out, cudaStream_t s,

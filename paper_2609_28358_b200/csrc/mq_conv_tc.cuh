@@ -104,7 +104,6 @@ cudaError_t launch_unpack6(const uint8_t* in, uint8_t* out, size_t n_codes, int 
 // one-code-per-byte E3M2 / E2M3 codes -> the E4M3 codes of the same values (every 6-bit value is an E4M3 value)
 cudaError_t launch_recode6_e4m3(const uint8_t* in, uint8_t* out, size_t nbytes, int fmt6, cudaStream_t s);
 // packed E2M1 codes (two per byte) -> the E4M3 codes of the same values, one per byte; n_out = elements = output bytes
-cudaError_t launch_recode4_e4m3(const uint8_t* in, uint8_t* out, size_t n_out, cudaStream_t s);
 // map_sfa, map_sfb: p.duo only - the two scale images as rows of 256 bytes (boxes of one stage's chunks)
 cudaError_t launch_conv_tc(const ConvTcParams& p, const CUtensorMap& map_a, const CUtensorMap& map_w, const CUtensorMap& map_out, cudaStream_t s,
                            const CUtensorMap* map_sfa = nullptr, const CUtensorMap* map_sfb = nullptr);
@@ -171,6 +170,9 @@ cudaError_t launch_wgrad_tc(const WgradTcParams& p, const CUtensorMap& map_a, co
                             const CUtensorMap& map_sfb, cudaStream_t s);
 // The scale chunks of every stage: E2M1 modes and pairs of blocks (else 8-bit operands' blocks build their own)
 cudaError_t launch_expand_wgrad_scales(const WgradTcParams& p, cudaStream_t s);
+// E2M1 codes of X (nx of them) and G_Y (ng; both multiples of 32) -> E4M3 bytes of the same values and, for pairs of blocks, the
+// scale chunks of expand_wgrad_scales: one launch.
+cudaError_t launch_wgrad_recode4(const WgradTcParams& p, const uint8_t* x, uint8_t* x_out, size_t nx, const uint8_t* gy, uint8_t* gy_out, size_t ng, cudaStream_t s);
 // E2M1 codes [P][N][Cp] -> [P][Cp][Npad] (n fastest, zero-padded): a permutation of nibbles, no requantization.
 cudaError_t launch_fp4_to_n_major(const uint8_t* in, uint8_t* out, int P, int N, int Cp, int Npad, cudaStream_t s);
 // Flat-mode preparation in one launch.  E2M1 codes [Hs][Ws][N][Cs_p] -> [channel block][q][rows][KBn] over the
