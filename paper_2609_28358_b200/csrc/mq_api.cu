@@ -232,11 +232,13 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
   out->rowbytes = rowbytes;
   // Box width.  Rows of up to 64 bytes go as one box per tap; multiples of 64 as 64-byte boxes, two of which fill a stage (192-byte
   // rows: 14 stages for nine taps instead of 18 half-empty ones; measured, quantizing forward of 183 -> 48 channels, N = 21,
-  // 19x14: 11.3 us against 12.5; 64 -> 320 channels stride 2, input gradient 43 against 47 us).  Every other row goes as 128-byte boxes,
+  // 19x14: 11.3 us against 12.5; 64 -> 320 channels stride 2, input gradient 43 against 47 us), up to 192-byte rows: from 320 on the half box that is wasted costs less than
+  // what 128-byte chunks save, an expansion of scale chunks per source row instead of per tile among it (us, 64 / 128: 448 -> 64 channels
+  // 60x75, N = 119, 360 / 292; 320 channels 28x28, N = 64, 77.5 / 71.8; stride 2 448 channels 42 / 35; 192 channels 28x28 39.9 / 40.9).  Every other row goes as 128-byte boxes,
   // the last one short: a box costs a request per row whatever its width, and 32-byte boxes (one per K-atom, the rule before)
   // cost three times as many of them for 96-byte rows (E4M3 129 -> 186 channels, N = 23, 45x56, forward: 74 -> 60 us).
   const int atoms = (rowbytes + 31) / 32;
-  p.KB = atoms == 1 ? 32 : (atoms == 2 || (rowbytes % 64 == 0 && rowbytes % 128 != 0) ? 64 : 128);
+  p.KB = atoms == 1 ? 32 : (atoms == 2 || (rowbytes % 64 == 0 && rowbytes % 128 != 0 && rowbytes < 320) ? 64 : 128);
   if (compact && rowbytes % 32 == 0) p.KB = rowbytes % 128 == 0 ? 128 : (rowbytes % 64 == 0 ? 64 : 32);   // no short boxes: full stages, fewest scale chunks
   p.G = 128 / p.KB;
   p.cpt = (rowbytes + p.KB - 1) / p.KB;
@@ -253,9 +255,34 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
   // 78 against 85 / 91 / 112)
   // (beyond what the 126 MB of L2 hold beside the operands: sectors written in part are read back)
   const bool big_output = (double)g.N * p.Cd * p.Hd * p.Wd * 4.0 > 110e6;
-  const bool thin = !line && !mx && !ts16 && g.sh == 1 && g.sw == 1 && p.cpt == 1 && p.KB <= 64 &&
+  bool thin = !line && !mx && !ts16 && g.sh == 1 && g.sw == 1 && p.cpt == 1 && p.KB <= 64 &&
                     !(p.KB == 64 && taps > 9 && (layout == MQ_NCHW || p.Cd > 32)) &&
                     !(layout == MQ_NCHW && p.Wd % 8 != 0 && big_output && (taps == 1 || p.Cd > 64)) && !MQ_ENV("MQ_TC_NO_HALO", 0);
+  // Strides of two, forward: the whole-tile kernel with a box per class of columns, where a channel tile is the whole output
+  // and two stages fit beside its resident weights (us, per-tap kernel with its preparation launch / this one: E4M3 16 -> 32 channels 320x320,
+  // N = 16, 53.2 / 27.8; 32 -> 64 75x75, N = 200, 45.1 / 30.3, 33x33, N = 8, 10.6 / 7.1; E2M1 64 -> 64 80x80, N = 64, 24.0 / 11.7; 100 channels
+  // 63x63, N = 200, 52.6 / 31.1; 25 taps of 64 bytes 21.8 / 22.3, the one shape of those measured that it is behind on).
+  const int spa_h = fp4 ? 2 : 1, halo_boxes = op == MQ_OP_FWD ? (g.sw < g.Kw ? g.sw : g.Kw) : 1;
+  const int halo_wh = op == MQ_OP_FWD ? 8 + (g.Kw + g.sw - 1) / g.sw - 1 : 8 + g.Kw - 1;
+  auto halo_stages = [&](int bn, bool staged, ConvTcParams* q) {   // stages of the whole-tile kernel (below two: it does not fit)
+    const int groups = (taps * p.cpt + p.G - 1) / p.G, atoms_b = (bn + 127) / 128;
+    q->WH = halo_wh; q->sw_halo = op == MQ_OP_FWD ? g.sw : 1; q->halo_boxes = halo_boxes;
+    q->halo_box_bytes = g.Kh * halo_wh * 16 * p.KB;
+    q->halo_a_bytes = (halo_boxes * q->halo_box_bytes + 1023) / 1024 * 1024;
+    q->halo_stage_bytes = (q->halo_a_bytes + groups * 512 * spa_h + 1023) / 1024 * 1024;
+    q->halo_b_bytes = (taps * bn * p.KB + groups * 512 * spa_h * atoms_b + 1023) / 1024 * 1024;
+    int hst = (227 * 1024 - 4096 - q->halo_b_bytes - (staged ? 65536 : 0)) / q->halo_stage_bytes;
+    if (hst > 4) hst = 4;
+    // TMEM: accumulator(s), 16 columns per chunk of resident weight scales, 8 per chunk per stage
+    while (hst >= 2 && bn + 16 * groups + 8 * groups * hst > 512) --hst;
+    return hst;
+  };
+  if (!line && !mx && !ts16 && op == MQ_OP_FWD && g.sw == 2 && g.sh <= 2 && taps <= 64 && p.cpt == 1 && p.KB <= 64 && p.Cd <= 128 &&
+      !(layout == MQ_NCHW && p.Wd % 8 != 0 && big_output && taps == 1) && !MQ_ENV("MQ_TC_NO_HALO", 0) && !MQ_ENV("MQ_TC_NO_HALO_S2", 0) &&
+      halo_boxes * g.Kh * halo_wh * (p.KB / 32) * spa_h <= (p.KB / 32 * spa_h == 1 ? 128 : 256)) {
+    ConvTcParams q{};
+    thin = halo_stages((p.Cd + 15) / 16 * 16, false, &q) >= 2;
+  }
   p.line = line ? 1 : 0;
   const int cd16 = mx ? (p.Cd + 31) / 32 * 32 : (p.Cd + 15) / 16 * 16;
   p.BN = cd16 <= 128 ? cd16 : 128;
@@ -402,22 +429,15 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
   // halo needs 8-column tiles; one box per column shift takes 8, 16 or 32 columns (longer NCHW store runs).
   p.halo = 0;
   if (thin && taps <= 64) {
-    const int spa = fp4 ? 2 : 1, atoms_b = (p.BN + 127) / 128;
     if (p.TW == 8 && p.TN == 16) {
-      p.WH = p.TW + g.Kw - 1;
-      p.halo_box_bytes = g.Kh * p.WH * p.TN * p.KB;
-      p.halo_a_bytes = (p.halo_box_bytes + 1023) / 1024 * 1024;
-      p.halo_stage_bytes = (p.halo_a_bytes + p.max_stages * 512 * spa + 1023) / 1024 * 1024;
-      p.halo_b_bytes = (taps * p.BN * p.KB + p.max_stages * 512 * spa * atoms_b + 1023) / 1024 * 1024;
-      const int halo_tma = tma_store_ok && !MQ_ENV("MQ_TC_NO_TMA_STORE", 0) ? 1 : 0;
-      int hst = (227 * 1024 - 4096 - p.halo_b_bytes - (halo_tma ? 65536 : 0)) / p.halo_stage_bytes;
-      if (hst > 4) hst = 4;
-      // TMEM: accumulator(s), 16 columns per chunk of resident weight scales, 8 per chunk per stage
-      while (hst >= 2 && p.BN + 16 * p.max_stages + 8 * p.max_stages * hst > 512) --hst;
+      int halo_tma = tma_store_ok && !MQ_ENV("MQ_TC_NO_TMA_STORE", 0) ? 1 : 0;
+      int hst = halo_stages(p.BN, halo_tma != 0, &p);
+      if (hst < 2 && g.sw == 2) { halo_tma = 0; hst = halo_stages(p.BN, false, &p); }   // (the staged stores' 64 KB or the halo: the halo)
       if (hst >= 2 && p.WH <= 256) {
         p.halo = 1;
         p.tma_store = halo_tma;
-        p.fused = p.tiles_c == 1 && p.TN <= 32 && g.Kh * (p.TW + g.Kw - 1) * (p.KB / 32) * spa <= 128 && !MQ_ENV("MQ_TC_NO_FUSED", 0);
+        p.fused = p.tiles_c == 1 && p.TN <= 32 && p.halo_boxes * g.Kh * p.WH * (p.KB / 32) * spa_h <= (p.KB / 32 * spa_h == 1 ? 128 : 256) &&
+                  !MQ_ENV("MQ_TC_NO_FUSED", 0);
         p.stages = hst;
         p.n_acc = (2 * p.BN + 16 * p.max_stages + 8 * p.max_stages * hst <= 512) ? 2 : 1;
       }
@@ -500,7 +520,7 @@ mq_status run_conv_tc(int op, const Geom& g, ConvTcPlan& pl, const mq_qtensor* q
     const uint64_t strides[3] = {(uint64_t)g.N * rb, rb, (uint64_t)p.Ws * g.N * rb};
     const uint32_t wst = op == MQ_OP_FWD ? (uint32_t)g.sw : 1u;
     uint32_t box[4] = {(uint32_t)p.KB, (uint32_t)((p.TW - 1) * wst + 1), (uint32_t)p.TN, 1u};
-    if (p.halo) { box[1] = (uint32_t)p.WH; box[3] = (uint32_t)g.Kh; }   // the whole halo of a tile in one box
+    if (p.halo) { box[1] = (uint32_t)((p.WH - 1) * wst + 1); box[3] = (uint32_t)g.Kh; }   // the whole halo of a tile (one class of its columns) in one box
     const uint32_t es[4] = {1u, wst, 1u, 1u};
     // a packed activation / gradient tensor with rows of whole 128-code boxes is read where it is stored (the copy engine pads
     // each 12-byte group on its way into shared memory): no scratch copy, no pass over the tensor before the GEMM

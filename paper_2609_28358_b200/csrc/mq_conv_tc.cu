@@ -1275,14 +1275,20 @@ __device__ __forceinline__ void halo_build_sfb(const ConvTcParams& p, uint8_t* s
 //  * a pipeline stage holds the whole K range of a tile's activations, every stored pixel once (the data reuse
 //    of Sec. IV-A): ONE TMA box [Kh rows][TN samples][TW + Kw - 1 columns][KB], and each tap's A operand is a
 //    view into it: tap (kh, kw) starts at (kh * TN * WH + kw) * KB with 8-row groups WH * KB bytes apart (TW = 8:
-//    one 8-row swizzle group per sample).
+//    one 8-row swizzle group per sample).  With a column stride (forward) the halo is one such box per class of columns that are
+//    sw apart (the copy engine steps over the others): tap kw lies in box kw % sw, kw / sw columns on.
 // Roles and barriers are those of conv_tc_kernel, plus bfull / bempty for the resident weight tile.
 // With a single channel tile (p.fused) no preparation kernel runs at all: every block builds the weight image and
-// its scale chunks in shared memory itself at start-up, and warp 3 expands each tile's activation scales (a
-// Kh x (TW + Kw - 1) patch of tile scales: all rows of a tile lie in one 32-sample block) into the scale-vector
-// chunks of the tile's stage, a few tiles ahead of the MMAs.
+// its scale chunks in shared memory itself at start-up, and warps 3, 12, 13 and 14 expand the tiles' activation scales (the
+// patch of tile scales under the halo: all rows of a tile lie in one 32-sample block) into the scale-vector chunks of the
+// tile's stage, each those of its own stage, a few tiles ahead of the MMAs; warps 1 and 2 issue the MMAs of every other tile, into an
+// accumulator each.  A tile is a chain of dependent instructions for either role - some 1000 clocks to expand (a load from
+// L2 among them), 700 to issue - against 300 of MMAs; with one warp for each role the chain was what a tile took (us, forward / input
+// gradient, one / several warps, E4M3 3x3: 16 channels 160x160, N = 16, 26.9 / 29.6 -> 16.8 / 20.7; 64 channels 56x56, N = 256,
+// 65.4 / 69.0 -> 53.5 / 58.1, where the fp32 output takes 51 at 4 TB/s; 5x5 32 channels 64x64, N = 64, 35.5 / 38.2 -> 25.6 / 28.6).
 // TAPS > 0 fixes the tap count at compile time (the MMA issue loop is then fully unrolled with the tap offsets in
 // registers: the single issuing thread is latency-bound, every instruction between two MMAs counts); 0 = any.
+__host__ __device__ constexpr int HALO_PATCH_BYTES(int bytes_per_pixel) { return bytes_per_pixel == 1 ? 128 : 256; }   // most scale bytes under a halo
 template <int MODE, int KB, bool FP4, int TAPS>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_w,
@@ -1311,7 +1317,7 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   uint32_t* tap_a = tmem_slot + 4;                     // per tap: offset of its A view / B rows, in 16-byte units
   uint32_t* tap_b = tap_a + 64;
   uint32_t* tap_p = tap_b + 64;                        // per tap: first pixel of its view in the tile's scale patch
-  uint8_t* sc_tbl = reinterpret_cast<uint8_t*>(tap_p + 64);   // the tile's patch of raw scale bytes (<= 512)
+  uint8_t* sc_tbl = reinterpret_cast<uint8_t*>(tap_p + 64);   // the patches of raw scale bytes, one per expander warp
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // warp-uniform, see conv_tc_kernel
   const unsigned total = (unsigned)p.total_tiles;
   const unsigned tiles_per_c = (unsigned)(p.classes * p.tiles_w * p.tiles_h);   // tile order: (class, w, h) below the channel tile
@@ -1335,10 +1341,11 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     // forward reads halo row kh, column shift kw; the input gradient walks the taps in the same order but its
     // source pixel moves the other way
     const int hrow = MODE == MQ_OP_FWD ? kh : p.Kh - 1 - kh, wsh = MODE == MQ_OP_FWD ? kw : p.Kw - 1 - kw;
-    const int aoff = (hrow * p.TN * p.WH + wsh) * KB;
+    const int par = wsh % p.sw_halo;         // column class of the tap's pixels: a box of its own
+    const int aoff = (((par * p.Kh) + hrow) * p.TN * p.WH + wsh / p.sw_halo) * KB;
     tap_a[threadIdx.x] = (uint32_t)aoff >> 4;
     tap_b[threadIdx.x] = (uint32_t)(threadIdx.x * p.BN * KB) >> 4;
-    tap_p[threadIdx.x] = (uint32_t)(hrow * (p.TW + p.Kw - 1) + wsh);
+    tap_p[threadIdx.x] = (uint32_t)((par * p.Kh + hrow) * p.WH + wsh / p.sw_halo);
   }
   if (warp == 1) { tmem_alloc(tmem_slot, 512); tmem_relinquish(); }
   pdl_wait();
@@ -1378,11 +1385,12 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         if (!mbar_wait_warp(&empty[s], phase ^ 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
         uint8_t* sa = stage0 + (size_t)s * stage_bytes;
         // first source pixel of the halo: forward (h - ph, w0 - pw); input gradient (h + ph - (Kh-1), w0 + pw - (Kw-1))
-        const int hs = MODE == MQ_OP_FWD ? tile.h - p.ph : tile.h + p.ph - (p.Kh - 1);
-        const int ws = MODE == MQ_OP_FWD ? tile.w0 - p.pw : tile.w0 + p.pw - (p.Kw - 1);
+        const int hs = MODE == MQ_OP_FWD ? tile.h * p.sh - p.ph : tile.h + p.ph - (p.Kh - 1);
+        const int ws = MODE == MQ_OP_FWD ? tile.w0 * p.sw - p.pw : tile.w0 + p.pw - (p.Kw - 1);
         if (elect_one()) {
-          mbar_arrive_expect_tx(&full[s], (uint32_t)(p.halo_box_bytes + (p.fused ? 0 : sfa_bytes)));
-          tma_load_4d(sa, &map_a, &full[s], 0, ws, tile.n0, hs);
+          mbar_arrive_expect_tx(&full[s], (uint32_t)(p.halo_boxes * p.halo_box_bytes + (p.fused ? 0 : sfa_bytes)));
+#pragma unroll 1
+          for (int q = 0; q < p.halo_boxes; ++q) tma_load_4d(sa + q * p.halo_box_bytes, &map_a, &full[s], 0, ws + q, tile.n0, hs);
           if (!p.fused) bulk_load(sa + p.halo_a_bytes, p.sfa_img + (size_t)tile_m_index(p, tile) * sfa_bytes, sfa_bytes, &full[s]);
         }
         __syncwarp();
@@ -1520,15 +1528,16 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     // ------------------------------------------------------------------ activation-scale expanders (fused mode): a warp per stage
     const int s = warp == 3 ? 0 : warp - 11;
     if (p.fused && s < p.stages) {
-      uint8_t* tbl = sc_tbl + 128 * s;
+      uint8_t* tbl = sc_tbl + 256 * s;
       constexpr int BPC = APC * SPA;                       // scale bytes per tap per row = K-blocks of a tap
-      const int WT = p.TW + p.Kw - 1, npix = p.Kh * WT;
-      // this lane's patch entries e = lane + 32 i: (halo row, column, K-block), fixed for the whole kernel
-      int e_h[4], e_w[4], e_k[4];
+      constexpr int NE = HALO_PATCH_BYTES(BPC) / 32;
+      const int npix = p.halo_boxes * p.Kh * p.WH;
+      // this lane's patch entries e = lane + 32 i: (column class, halo row, column, K-block), fixed for the whole kernel
+      int e_h[NE], e_w[NE], e_k[NE];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int e = lane + 32 * i, pe = e / BPC;
-        e_k[i] = e - pe * BPC; e_h[i] = pe / WT; e_w[i] = pe - e_h[i] * WT;
+      for (int i = 0; i < NE; ++i) {
+        const int e = lane + 32 * i, pe = e / BPC, row = pe / p.WH, par = row / p.Kh;
+        e_k[i] = e - pe * BPC; e_h[i] = row - par * p.Kh; e_w[i] = par + p.sw_halo * (pe - row * p.WH);
         if (pe >= npix) e_h[i] = -1;
       }
       int twj[4];
@@ -1537,13 +1546,13 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       uint32_t phase = 0;
       for (unsigned t = blockIdx.x + (unsigned)s * gridDim.x; t < total && !*abort_flag; t += (unsigned)p.stages * gridDim.x, phase ^= 1) {
         const Tile tile = decode_tile(p, t);
-        const int hs = MODE == MQ_OP_FWD ? tile.h - p.ph : tile.h + p.ph - (p.Kh - 1);
-        const int ws = MODE == MQ_OP_FWD ? tile.w0 - p.pw : tile.w0 + p.pw - (p.Kw - 1);
+        const int hs = MODE == MQ_OP_FWD ? tile.h * p.sh - p.ph : tile.h + p.ph - (p.Kh - 1);
+        const int ws = MODE == MQ_OP_FWD ? tile.w0 * p.sw - p.pw : tile.w0 + p.pw - (p.Kw - 1);
         const int nblk = tile.n0 >> 5;
         // raw tile scales of the patch (zero outside the image: those codes are zero-filled anyway)
-        uint8_t raw[4];
+        uint8_t raw[NE];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < NE; ++i) {
           const int hh = hs + e_h[i], ww = ws + e_w[i];
           raw[i] = 0;
           if (e_h[i] >= 0 && e_k[i] < p.Kblocks && hh >= 0 && hh < p.Hs && ww >= 0 && ww < p.Ws)
@@ -1554,7 +1563,7 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
         if (!ok) { *abort_flag = 1; break; }
 #pragma unroll
-        for (int i = 0; i < 4; ++i) tbl[lane + 32 * i] = raw[i];
+        for (int i = 0; i < NE; ++i) tbl[lane + 32 * i] = raw[i];
         __syncwarp();
         uint8_t* dst = stage0 + (size_t)s * stage_bytes + p.halo_a_bytes + lane * 16;
 #pragma unroll 1
@@ -2097,7 +2106,7 @@ template <int MODE, int KB, bool FP4, int TAPS>
 cudaError_t launch_conv_tc_halo_taps(const ConvTcParams& p, const CUtensorMap& map_a, const CUtensorMap& map_b, const CUtensorMap& map_w, cudaStream_t s) {
   static bool attr_set = false;
   const size_t smem = 1024 + (size_t)p.halo_b_bytes + (size_t)p.stages * p.halo_stage_bytes + (p.tma_store ? EPI_STAGING_BYTES : 0) +
-                      (3 * (size_t)p.stages + 6) * 8 + 16 + 3 * 64 * 4 + 512;
+                      (3 * (size_t)p.stages + 6) * 8 + 16 + 3 * 64 * 4 + 4 * 256;
   if (!attr_set) {
     cudaError_t e = cudaFuncSetAttribute(conv_tc_halo_kernel<MODE, KB, FP4, TAPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (e != cudaSuccess) return e;

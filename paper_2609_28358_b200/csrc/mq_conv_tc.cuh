@@ -54,11 +54,12 @@ struct ConvTcParams {
   int sfa_hk;               // source-row keys per sample tile = output rows + Kh - 1
   // whole-tile-per-stage variant (small channel counts, stride 1): see conv_tc_halo_kernel
   int halo;                 // 1: use it
-  int WH;                   // columns of the activation halo box = TW + Kw - 1
+  int WH;                   // columns of an activation halo box = TW + ceil(Kw / sw) - 1
+  int sw_halo, halo_boxes;  // column stride of the walk (forward: sw, else 1); boxes of a halo, one per class of columns = min(sw, Kw)
   int duo;                  // 1: clusters of two blocks on 256 x 256 tiles (cta_group::2), each loading half of the weight tile
   int snap;                 // 1: 256-column tiles, direct fp32 stores: the epilogue copies the accumulator into registers and frees it before storing
   int a_tx34;               // 1: the activation boxes come from packed 6-bit storage - a box counts 3/4 of its shared-memory bytes on the barrier
-  int halo_box_bytes;       // bytes of one activation box = Kh * TN * WH * KB
+  int halo_box_bytes;       // bytes of one activation box = Kh * TN * WH * KB (a multiple of 512)
   int halo_a_bytes;         // bytes of a tile's activation boxes (rounded up to 1024)
   int halo_stage_bytes;     // bytes of one pipeline stage (activation boxes + A-side scale chunks)
   int halo_b_bytes;         // bytes of the resident weight image + its scale chunks (rounded up to 1024)

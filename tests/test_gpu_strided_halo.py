@@ -1,0 +1,34 @@
+"""Forward of thin layers with a column stride of two on the whole-tile kernel (needs a B200): a halo box per class of columns, rows of 32
+and 64 bytes, kernels of 1 to 25 taps, weights that leave no room for the staged stores, ragged images, batches and channels, a row
+stride of its own.  Against the CPU oracle within the bound of the other GEMM tests; one launch says that the kernel is the one meant."""
+import pytest
+
+from paper_2609_28358_b200 import inputs, mq
+from parity_util import OracleLayer, check_convs, check_quantize
+
+pytestmark = pytest.mark.gpu
+
+# N, C_in (E2M1: twice as many), H, W, C_out, kernel, stride_h, stride_w, padding
+CASES = [
+    ("k3", 5, 32, 9, 11, 48, 3, 2, 2, 1),
+    ("k3_many_tiles", 40, 16, 21, 70, 32, 3, 2, 2, 1),      # more tiles than stages: every expander and both issuers go round
+    ("k3_no_staging", 17, 64, 10, 16, 128, 3, 2, 2, 1),
+    ("k3_staged", 18, 64, 6, 32, 64, 3, 2, 2, 1),
+    ("k5", 33, 20, 8, 9, 17, 5, 2, 2, 2),
+    ("k2", 6, 32, 16, 34, 32, 2, 2, 2, 0),
+    ("k1", 4, 64, 7, 7, 64, 1, 2, 2, 0),
+    ("rows_of_their_own", 6, 33, 7, 15, 40, 3, 1, 2, 1),
+]
+
+
+@pytest.mark.parametrize("fmts", [(mq.E4M3, mq.E4M3, mq.E5M2), (mq.E2M1,) * 3], ids=["fp8", "fp4"])
+@pytest.mark.parametrize("name,n,cin,h,w,cout,k,sh,sw,pad", CASES, ids=[c[0] for c in CASES])
+def test_forward(name, n, cin, h, w, cout, k, sh, sw, pad, fmts):
+    d = mq.ConvDesc(n, cin * (2 if fmts[0] == mq.E2M1 else 1), h, w, cout, k, k, sh, sw, pad, pad)
+    ol = OracleLayer(inputs.Layer(name, d, *fmts, "relu", "kaiming", "gauss", 53))
+    qs = check_quantize(ol)
+    before = mq.kernel_launch_count()
+    mq.conv_fwd(d, qs[0], qs[1])
+    assert mq.kernel_launch_count() - before == 1
+    check_convs(ol, qs, layouts=(mq.NCHW, mq.HWNC), ops=("fwd",))
+    assert mq.last_device_status() == 0
