@@ -238,32 +238,36 @@ __global__ void __launch_bounds__(NT) quantize_pipe_kernel(QuantArgs a, int n_ps
 // 4.2 / 5.0; at most 8 rows, of which one or two of the eight warps hold all, 2 x 416 channels 19x19 6.9 / 5.4, 64 channels 49x49 6.1 / 4.9.
 // LINE: line blocks - one scale per (position, row, 32 channels).  A block that holds a NaN gets the scale of an
 // infinite maximum, here and in quantize_few_kernel; the other kernels' maxima pass over it.
-template <int FMT, bool SR, bool LINE, int PI>   // PI: positions per item, 16 or 8
+// PI = 32 (tensors of at most 16 rows that fill the chip): two rows of 32 channels per thread, so that no warp is without rows, a load reads
+// one run of 128 bytes and a position's maximum needs no shuffle (us, items of 16 or 8 / 32: E4M3 16 channels 159x159, N = 16, 18.6 / 14.1;
+// 320 channels 51x89, N = 8, 28.7 / 24.8; E2M1 512 channels 31x31, N = 12, 12.5 / 10.6; 64 channels 75x75, N = 16, 9.4 / 8.5).
+template <int FMT, bool SR, bool LINE, int PI>   // PI: positions per item, 32, 16 or 8
 __global__ void __launch_bounds__(QT_THREADS, 2) quantize_odd_kernel(QuantArgs a, int n_pstrips, int Ct) {
   constexpr int CG = PI, HN = 32 / PI;             // a thread's channels, a row's channel groups
+  constexpr int RW = PI == 32 ? 2 : 4, TR = 8 * RW;  // a warp's rows, an item's
   constexpr int CB = FMT == MQ_E2M1 ? CG / 2 : CG; // bytes of a piece: CG codes
   constexpr int XM = FMT == MQ_E2M1 && PI == 16 ? 15 : 7;    // XOR of a position's pieces, in units of XU pieces (16 bytes where
   constexpr int XU = PI == 16 ? 1 : (FMT == MQ_E2M1 ? 4 : 2);   // a piece is smaller and the stores below read 16 at once)
   __shared__ unsigned red[8][PI];
-  __shared__ __align__(16) uint8_t stage[PI * 32 * HN * CB];   // [position][piece = HN row + channel group]
+  __shared__ __align__(16) uint8_t stage[PI * TR * HN * CB];   // [position][piece = HN row + channel group]
   pdl_wait();
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const Item q = item_of(blockIdx.x, n_pstrips, Ct, PI);
   const int pl = lane & (PI - 1), h = lane / PI;
   const bool p_ok = q.p0 + pl < a.P;
-  const int r0 = q.r0 + 4 * warp, c0 = q.c0 + CG * h;
+  const int r0 = q.r0 + RW * warp, c0 = q.c0 + CG * h;
   const long long e0 = ((long long)r0 * a.C + c0) * a.P + q.p0 + pl;      // index of this thread's first element
-  float v[4][CG];
+  float v[RW][CG];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < RW; ++i) {
     const float* src = a.src + e0 + (long long)i * a.C * a.P;
     const bool ok = p_ok && r0 + i < a.R;
 #pragma unroll
     for (int k = 0; k < CG; ++k) v[i][k] = (ok && c0 + k < a.C) ? __ldg(src + (long long)k * a.P) : 0.f;
   }
-  float m[4];
+  float m[RW];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < RW; ++i) {
     m[i] = 0.f;
 #pragma unroll
     for (int k = 0; k < CG; ++k) m[i] = max_nan(m[i], fabsf(v[i][k]));
@@ -272,15 +276,16 @@ __global__ void __launch_bounds__(QT_THREADS, 2) quantize_odd_kernel(QuantArgs a
       for (int off = PI; off < 32; off <<= 1) m[i] = max_nan(m[i], __shfl_xor_sync(0xffffffffu, m[i], off));
     }
   }
-  int code[LINE ? 4 : 1];
+  int code[LINE ? RW : 1];
   if (LINE) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < RW; ++i) {
       code[i] = scale_code_of(__float_as_uint(m[i]), fmt_emax(FMT));
       if (h == 0 && p_ok && r0 + i < a.R) a.scales[(long long)(q.p0 + pl) * a.sc_stride_p + (long long)(r0 + i) * a.sc_stride_r + q.ct] = (uint8_t)code[i];
     }
   } else {
-    float mm = max_nan(max_nan(m[0], m[1]), max_nan(m[2], m[3]));
+    float mm = max_nan(m[0], m[1]);
+    if constexpr (RW == 4) mm = max_nan(mm, max_nan(m[2], m[3]));
 #pragma unroll
     for (int off = PI; off < 32; off <<= 1) mm = max_nan(mm, __shfl_xor_sync(0xffffffffu, mm, off));
     if (h == 0) red[warp][pl] = __float_as_uint(mm);
@@ -292,7 +297,7 @@ __global__ void __launch_bounds__(QT_THREADS, 2) quantize_odd_kernel(QuantArgs a
     if (t < PI && p_ok) a.scales[(long long)(q.p0 + t) * a.sc_stride_p + (long long)q.rt * a.sc_stride_r + q.ct] = (uint8_t)code[0];
   }
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < RW; ++i) {
     const float f = scale_factor(code[LINE ? i : 0]);
     unsigned w4[CG / 4];
 #pragma unroll
@@ -309,17 +314,27 @@ __global__ void __launch_bounds__(QT_THREADS, 2) quantize_odd_kernel(QuantArgs a
       const unsigned lo = encode2<FMT>(x[0], x[1]), hi = encode2<FMT>(x[2], x[3]);
       w4[k >> 2] = FMT == MQ_E2M1 ? (lo | (hi << 8)) : (lo | (hi << 16));
     }
+    if constexpr (PI == 32) {     // pieces of 16 bytes: [position][row] or [position][row][half]
+      uint4* row = reinterpret_cast<uint4*>(stage) + pl * (TR * CB / 16);
+      if constexpr (FMT == MQ_E2M1) {
+        row[(RW * warp + i) ^ (pl & 7)] = make_uint4(w4[0] | (w4[1] << 16), w4[2] | (w4[3] << 16), w4[4] | (w4[5] << 16), w4[6] | (w4[7] << 16));
+      } else {
+        row[(2 * (RW * warp + i)) ^ (pl & 7)] = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+        row[(2 * (RW * warp + i) + 1) ^ (pl & 7)] = make_uint4(w4[4], w4[5], w4[6], w4[7]);
+      }
+      continue;
+    }
     uint8_t* dst = stage + (pl * 32 * HN + ((HN * (4 * warp + i) + h) ^ ((pl & XM) * XU))) * CB;
     if constexpr (FMT == MQ_E2M1 && PI == 16) *reinterpret_cast<uint2*>(dst) = make_uint2(w4[0] | (w4[1] << 16), w4[2] | (w4[3] << 16));
     else if constexpr (FMT == MQ_E2M1) *reinterpret_cast<unsigned*>(dst) = w4[0] | (w4[1] << 16);
-    else if constexpr (PI == 16) *reinterpret_cast<uint4*>(dst) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+    else if constexpr (PI == 16 || PI == 32) *reinterpret_cast<uint4*>(dst) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
     else *reinterpret_cast<uint2*>(dst) = make_uint2(w4[0], w4[1]);
   }
   __syncthreads();
   if (FMT == MQ_E2M1) {
 #pragma unroll
-    for (int k = 0; k < PI * 32 / QT_THREADS; ++k) {    // rows of 16 bytes: [position][row]
-      const int id = t + QT_THREADS * k, p = id >> 5, r = id & 31;
+    for (int k = 0; k < PI * TR / QT_THREADS; ++k) {    // rows of 16 bytes: [position][row]
+      const int id = t + QT_THREADS * k, p = id / TR, r = id % TR;
       if (q.p0 + p < a.P && q.r0 + r < a.R) {
         uint4 val;
         if constexpr (PI == 16) {
@@ -327,7 +342,7 @@ __global__ void __launch_bounds__(QT_THREADS, 2) quantize_odd_kernel(QuantArgs a
           const uint2 lo = row[(2 * r) ^ (p & XM)], hi = row[(2 * r + 1) ^ (p & XM)];
           val = make_uint4(lo.x, lo.y, hi.x, hi.y);
         } else {
-          val = *(reinterpret_cast<const uint4*>(stage) + p * 32 + (r ^ (p & XM)));
+          val = *(reinterpret_cast<const uint4*>(stage) + p * TR + (r ^ (p & XM)));
         }
         const long long e = (long long)(q.p0 + p) * a.out_stride_p + (long long)(q.r0 + r) * a.out_stride_r + q.c0;
         *reinterpret_cast<uint4*>(a.codes + (e >> 1)) = val;
@@ -335,10 +350,10 @@ __global__ void __launch_bounds__(QT_THREADS, 2) quantize_odd_kernel(QuantArgs a
     }
   } else {
 #pragma unroll
-    for (int k = 0; k < PI * 64 / QT_THREADS; ++k) {    // pieces of 16 bytes: [position][row][half]
-      const int id = t + QT_THREADS * k, p = id >> 6, piece = id & 63, r = piece >> 1;
+    for (int k = 0; k < PI * 2 * TR / QT_THREADS; ++k) {    // pieces of 16 bytes: [position][row][half]
+      const int id = t + QT_THREADS * k, p = id / (2 * TR), piece = id % (2 * TR), r = piece >> 1;
       if (q.p0 + p < a.P && q.r0 + r < a.R) {
-        const uint4 val = *(reinterpret_cast<const uint4*>(stage) + p * 64 + (piece ^ (p & XM)));
+        const uint4 val = *(reinterpret_cast<const uint4*>(stage) + p * (2 * TR) + (piece ^ (p & XM)));
         const long long e = (long long)(q.p0 + p) * a.out_stride_p + (long long)(q.r0 + r) * a.out_stride_r + q.c0 + 16 * (piece & 1);
         store_codes16(a, e, val);
       }
@@ -826,7 +841,9 @@ cudaError_t launch_q(const QuantArgs& a, int n_pstrips, int Ct, long long n_item
   if (a.line || !vec) {   // (line blocks with 16-byte rows get here only as small tensors: large ones take the whole-line kernel)
     const long long tiles = n_items / n_pstrips;
     // 8-position items while they all run at once (two blocks per SM): see quantize_odd_kernel
-    const bool small = (a.P > 2 && tiles * ((a.P + 7) / 8) <= 2 * sm_count()) || (a.P > FEW_P && a.R <= 8);
+    // ... of 32 where at most 16 rows leave half of the warps without any and the grid is still two blocks per SM
+    const bool thin = a.P > FEW_P && a.R <= 16 && tiles * ((a.P + 31) / 32) >= 2 * sm_count();
+    const bool small = !thin && ((a.P > 2 && tiles * ((a.P + 7) / 8) <= 2 * sm_count()) || (a.P > FEW_P && a.R <= 8));
     if (!small && a.P <= FEW_P && a.P % 4 != 0) {
       auto kernel = a.line ? (a.sr ? quantize_few_kernel<FMT, true, true> : quantize_few_kernel<FMT, false, true>)
                            : (a.sr ? quantize_few_kernel<FMT, true> : quantize_few_kernel<FMT, false>);
@@ -838,9 +855,11 @@ cudaError_t launch_q(const QuantArgs& a, int n_pstrips, int Ct, long long n_item
       const int rounds = (a.P + 15) / 16, warps = (a.P + rounds - 1) / rounds;      // as few positions per warp as 16 warps allow: nine taps, nine warps
       return launch_pdl(kernel, dim3((unsigned)tiles), dim3((unsigned)(warps < 8 ? 8 : warps) * 32), smem, s, a, Ct);
     }
-    const int strips = (a.P + (small ? 7 : 15)) / (small ? 8 : 16);
+    const int pi = thin ? 32 : (small ? 8 : 16), strips = (a.P + pi - 1) / pi;
     const long long items = tiles * strips;
-    auto kernel = small ? (a.line ? (a.sr ? quantize_odd_kernel<FMT, true, true, 8> : quantize_odd_kernel<FMT, false, true, 8>)
+    auto kernel = thin ? (a.line ? (a.sr ? quantize_odd_kernel<FMT, true, true, 32> : quantize_odd_kernel<FMT, false, true, 32>)
+                                 : (a.sr ? quantize_odd_kernel<FMT, true, false, 32> : quantize_odd_kernel<FMT, false, false, 32>))
+                : small ? (a.line ? (a.sr ? quantize_odd_kernel<FMT, true, true, 8> : quantize_odd_kernel<FMT, false, true, 8>)
                                   : (a.sr ? quantize_odd_kernel<FMT, true, false, 8> : quantize_odd_kernel<FMT, false, false, 8>))
                         : (a.line ? (a.sr ? quantize_odd_kernel<FMT, true, true, 16> : quantize_odd_kernel<FMT, false, true, 16>)
                                   : (a.sr ? quantize_odd_kernel<FMT, true, false, 16> : quantize_odd_kernel<FMT, false, false, 16>));
