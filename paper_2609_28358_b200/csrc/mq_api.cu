@@ -264,13 +264,15 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
   // 63x63, N = 200, 52.6 / 31.1; 25 taps of 64 bytes 21.8 / 22.3, the one shape of those measured that it is behind on).
   const int spa_h = fp4 ? 2 : 1, halo_boxes = op == MQ_OP_FWD ? (g.sw < g.Kw ? g.sw : g.Kw) : 1;
   const int halo_wh = op == MQ_OP_FWD ? 8 + (g.Kw + g.sw - 1) / g.sw - 1 : 8 + g.Kw - 1;
+  // (input gradient: 8-bit weights of a single channel tile are multiplied as they are stored)
+  const bool mn_weights = op == MQ_OP_BWD_DATA && !fp4 && !fmt_is_6bit(fmt_w) && !fmt_is_6bit(fmt_x_like) && p.Cd <= 128 && !MQ_ENV("MQ_TC_NO_MN_WEIGHTS", 0);
   auto halo_stages = [&](int bn, bool staged, ConvTcParams* q) {   // stages of the whole-tile kernel (below two: it does not fit)
     const int groups = (taps * p.cpt + p.G - 1) / p.G, atoms_b = (bn + 127) / 128;
     q->WH = halo_wh; q->sw_halo = op == MQ_OP_FWD ? g.sw : 1; q->halo_boxes = halo_boxes;
     q->halo_box_bytes = g.Kh * halo_wh * 16 * p.KB;
     q->halo_a_bytes = (halo_boxes * q->halo_box_bytes + 1023) / 1024 * 1024;
     q->halo_stage_bytes = (q->halo_a_bytes + groups * 512 * spa_h + 1023) / 1024 * 1024;
-    q->halo_b_bytes = (taps * bn * p.KB + groups * 512 * spa_h * atoms_b + 1023) / 1024 * 1024;
+    q->halo_b_bytes = (taps * (mn_weights && bn < g.Cp ? g.Cp : bn) * p.KB + groups * 512 * spa_h * atoms_b + 1023) / 1024 * 1024;
     int hst = (227 * 1024 - 4096 - q->halo_b_bytes - (staged ? 65536 : 0)) / q->halo_stage_bytes;
     if (hst > 4) hst = 4;
     // TMEM: accumulator(s), 16 columns per chunk of resident weight scales, 8 per chunk per stage
@@ -438,6 +440,7 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
         p.tma_store = halo_tma;
         p.fused = p.tiles_c == 1 && p.TN <= 32 && p.halo_boxes * g.Kh * p.WH * (p.KB / 32) * spa_h <= (p.KB / 32 * spa_h == 1 ? 128 : 256) &&
                   !MQ_ENV("MQ_TC_NO_FUSED", 0);
+        if (p.fused && mn_weights) p.b_mn = g.Cp % 128 == 0 ? 128 : (g.Cp % 64 == 0 ? 64 : 32);
         p.stages = hst;
         p.n_acc = (2 * p.BN + 16 * p.max_stages + 8 * p.max_stages * hst <= 512) ? 2 : 1;
       }
@@ -502,14 +505,15 @@ mq_status run_conv_tc(int op, const Geom& g, ConvTcPlan& pl, const mq_qtensor* q
     if (p.wt_fused) {
       p.wt_in = w_stored; p.wt_out = base; p.wt_sc_in = qw->scales;
       p.wt_Cout = g.Cout; p.wt_Cop = g.Cop; p.wt_Cp = g.Cp; p.wt_bx = g.Cp / 32; p.wt_by = g.Cop / 32;
-    } else separate_transpose = true;
-    p.b_scales = wt_scales;
+    } else separate_transpose = p.b_mn == 0;
+    p.b_scales = p.b_mn ? qw->scales : wt_scales;
   }
   p.a_scales = qx_like->scales;
   p.a_tscale = qx_like->tensor_scale; p.b_tscale = qw->tensor_scale;
   p.sfa_img = base + pl.off_sfa;
   p.sfb_img = base + pl.off_sfb;
-  p.b_codes = b_codes; p.b_rows_total = pl.rows_b; p.b_rowbytes = pl.rowbytes; p.b_img = base + pl.off_bimg;
+  p.b_codes = b_codes; p.b_rows_total = pl.rows_b; p.b_rowbytes = p.b_mn ? g.Cp : pl.rowbytes;
+  if (p.b_mn) p.idesc |= 1u << 16; p.b_img = base + pl.off_bimg;
   p.out = out; p.out_layout = layout; p.status = status;
 
   CUtensorMap map_a, map_w;
@@ -534,7 +538,13 @@ mq_status run_conv_tc(int op, const Geom& g, ConvTcPlan& pl, const mq_qtensor* q
   }
   map_w = map_a;
   if (p.halo) {
-    if (p.fused) {
+    if (p.fused && p.b_mn) {
+      // all taps of a panel of input channels, as stored: dims ordered (channel bytes, output channels, taps)
+      const uint64_t dims[3] = {(uint64_t)g.Cp, (uint64_t)g.Cout, (uint64_t)taps};
+      const uint64_t strides[2] = {(uint64_t)taps * g.Cp, (uint64_t)g.Cp};
+      const uint32_t box[3] = {(uint32_t)p.b_mn, (uint32_t)p.KB, (uint32_t)taps};
+      if (!encode_tensor_map_u8(&map_w, w_stored, 3, dims, strides, box, nullptr, p.b_mn)) return MQ_ERR_CUDA;
+    } else if (p.fused) {
       // all taps of the weight tile in one box: dims ordered (channel bytes, rows, taps)
       const uint64_t rb = (uint64_t)pl.rowbytes;
       const uint64_t dims[3] = {rb, (uint64_t)pl.rows_b, (uint64_t)taps};

@@ -1249,7 +1249,12 @@ __device__ __forceinline__ void halo_build_sfb(const ConvTcParams& p, uint8_t* s
       if (q < taps) {
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-          if (j < 4 * atoms_b && 32 * j < p.BN && 32 * j < p.Cd)
+          if (!(j < 4 * atoms_b && 32 * j < p.BN && 32 * j < p.Cd)) continue;
+          if (!FP4 && p.b_mn) {      // the weights as they are stored: a scale line per output channel block of W, which is a K-block here
+#pragma unroll
+            for (int k = 0; k < BPC; ++k)
+              if (k < p.Kblocks) acc[j] |= (unsigned long long)__ldg(p.b_scales + ((long long)k * taps + q) * (p.b_rowbytes >> 5) + j) << (8 * (c * BPC + k));
+          } else
             acc[j] |= load_scale_bytes<BPC, WHOLE>(p.b_scales + ((long long)j * taps + q) * p.Kblocks, 0, p.Kblocks) << (8 * c * BPC);
         }
       }
@@ -1286,6 +1291,10 @@ __device__ __forceinline__ void halo_build_sfb(const ConvTcParams& p, uint8_t* s
 // L2 among them), 700 to issue - against 300 of MMAs; with one warp for each role the chain was what a tile took (us, forward / input
 // gradient, one / several warps, E4M3 3x3: 16 channels 160x160, N = 16, 26.9 / 29.6 -> 16.8 / 20.7; 64 channels 56x56, N = 256,
 // 65.4 / 69.0 -> 53.5 / 58.1, where the fp32 output takes 51 at 4 TB/s; 5x5 32 channels 64x64, N = 64, 35.5 / 38.2 -> 25.6 / 28.6).
+// The input gradient contracts over W's output channels, which the stored order [C_out][taps][C_in] has slowest: 8-bit weights of the
+// fused kernel are loaded as they are and multiplied MN-major (b_mn), without the launch that re-lays them: us, 64 -> 32 channels
+// 32x32, N = 8, 14.0 -> 9.9; 96 <- 64 29x29, N = 64, 17.2 -> 15.1; 64 <- 64 56x56, N = 256, 58.6 -> 55.8.
+// (E2M1 operands are K-major only.)
 // TAPS > 0 fixes the tap count at compile time (the MMA issue loop is then fully unrolled with the tap offsets in
 // registers: the single issuing thread is latency-bound, every instruction between two MMAs counts); 0 = any.
 __host__ __device__ constexpr int HALO_PATCH_BYTES(int bytes_per_pixel) { return bytes_per_pixel == 1 ? 128 : 256; }   // most scale bytes under a halo
@@ -1300,7 +1309,7 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   const int taps = TAPS > 0 ? TAPS : p.Kh * p.Kw;
   const int nsf = p.max_stages;                        // scale chunks (groups of 4 MMAs) per tile
   const int atoms_b = (p.BN + 127) / 128;
-  const int b_bytes = taps * p.BN * KB;
+  const int b_bytes = taps * KB * (p.b_mn ? p.b_rowbytes : p.BN);
   const int sfa_bytes = nsf * 512 * SPA, sfb_bytes = nsf * 512 * SPA * atoms_b;
   const int stage_bytes = p.halo_stage_bytes;
   uint8_t* stage0 = smem + p.halo_b_bytes;             // [weight image | its scale chunks] then the stages
@@ -1333,7 +1342,11 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     pdl_wait();      // everything above touches only this block's shared memory and the kernel parameters
     if (p.fused) {   // the weight tile, all taps: one box, swizzled by the copy engine, while the block finishes setting up
       mbar_arrive_expect_tx(bfull, (uint32_t)b_bytes);
-      tma_load_3d(smem, &map_w, bfull, 0, 0, 0);
+      if (p.b_mn) {
+#pragma unroll 1
+        for (int c = 0; c < p.b_rowbytes; c += p.b_mn) tma_load_3d(smem + taps * KB * c, &map_w, bfull, c, 0, 0);
+      } else
+        tma_load_3d(smem, &map_w, bfull, 0, 0, 0);
     }
   }
   if ((int)threadIdx.x < taps) {
@@ -1344,7 +1357,7 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     const int par = wsh % p.sw_halo;         // column class of the tap's pixels: a box of its own
     const int aoff = (((par * p.Kh) + hrow) * p.TN * p.WH + wsh / p.sw_halo) * KB;
     tap_a[threadIdx.x] = (uint32_t)aoff >> 4;
-    tap_b[threadIdx.x] = (uint32_t)(threadIdx.x * p.BN * KB) >> 4;
+    tap_b[threadIdx.x] = (uint32_t)(threadIdx.x * (p.b_mn ? p.b_mn : p.BN) * KB) >> 4;
     tap_p[threadIdx.x] = (uint32_t)((par * p.Kh + hrow) * p.WH + wsh / p.sw_halo);
   }
   if (warp == 1) { tmem_alloc(tmem_slot, 512); tmem_relinquish(); }
@@ -1402,7 +1415,10 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     {
       const uint32_t first = two_issuers ? (uint32_t)warp - 1u : 0u, step = two_issuers ? 2u : 1u;
       const uint64_t a_desc_base = smem_desc_base(16, (uint32_t)(p.WH * KB), LAYOUT);   // 8-row groups one halo row apart
-      const uint64_t b_desc_base = smem_desc_base(16, 8 * KB, LAYOUT);
+      // weights as stored (b_mn bytes of N per row of K): 8-row groups of K, panels of all taps
+      const uint64_t b_desc_base = p.b_mn ? smem_desc_base((uint32_t)(taps * KB * p.b_mn), 8u * p.b_mn, p.b_mn == 128 ? 2 : (p.b_mn == 64 ? 4 : 6))
+                                          : smem_desc_base(16, 8 * KB, LAYOUT);
+      const uint32_t b_step = p.b_mn ? 2u * p.b_mn : 2u;     // 32 bytes of K further, in 16-byte units
       const uint32_t sb16 = smem_u32(smem) >> 4;
       uint32_t idesc_id[4];
 #pragma unroll
@@ -1460,7 +1476,7 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
             const int atom = (q % G) * APC + ja;
             const int g = (atom * SPA) >> 2, id = (atom * SPA) & 3;
             const uint64_t ad = a_desc_base | (uint64_t)((a16 + 2 * ja) & 0x3FFF);
-            const uint64_t bd = b_desc_base | (uint64_t)((b16 + 2 * ja) & 0x3FFF);
+            const uint64_t bd = b_desc_base | (uint64_t)((b16 + b_step * ja) & 0x3FFF);
             if (FP4) mma_mxf4(d_tmem, ad, bd, idesc_id[id], sfa_t + 4 * g, sfb_t + 4 * g * atoms_b, accumulate);
             else mma_mxf8f6f4(d_tmem, ad, bd, idesc_id[id], sfa_t + 4 * g, sfb_t + 4 * g * atoms_b, accumulate);
             accumulate = 1;

@@ -1,0 +1,37 @@
+"""Input gradient of thin layers on the whole-tile kernel (needs a B200).  Unit strides: 8-bit weights multiplied as they are stored
+(MN-major), in rows of 32, 64 and 128 bytes and three panels of 32, ragged channels both ways, 1 to 25 taps.  Against the CPU
+oracle within the bound of the other GEMM tests; the launches counted say that the route is the one meant."""
+import pytest
+
+from paper_2609_28358_b200 import inputs, mq
+from parity_util import OracleLayer, check_convs, check_quantize
+
+pytestmark = pytest.mark.gpu
+
+# N, C_in, H, W, C_out (E2M1: twice as many), kernel, stride, padding
+CASES = [
+    ("n16", (5, 16, 9, 11, 32, 3, 1, 1)),
+    ("n33", (17, 33, 7, 16, 20, 3, 1, 1)),
+    ("n64_k2", (6, 64, 8, 9, 64, 3, 1, 1)),
+    ("n96_three_panels", (4, 96, 6, 13, 50, 3, 1, 1)),
+    ("n128", (9, 128, 5, 8, 33, 3, 1, 1)),
+    ("n80_pointwise", (33, 80, 6, 7, 64, 1, 1, 0)),
+    ("n40_k5", (3, 40, 9, 9, 32, 5, 1, 2)),
+    ("many_tiles", (40, 32, 21, 40, 64, 3, 1, 1)),
+]
+
+
+@pytest.mark.parametrize("fmts", [(mq.E4M3, mq.E4M3, mq.E5M2), (mq.E2M1,) * 3], ids=["fp8", "fp4"])
+@pytest.mark.parametrize("name,shape", CASES, ids=[c[0] for c in CASES])
+def test_input_gradient(name, shape, fmts):
+    n, cin, h, w, cout, *rest = shape
+    fp4 = fmts[0] == mq.E2M1
+    d = inputs.conv_desc(n, cin, h, w, cout * (2 if fp4 else 1), *rest)
+    ol = OracleLayer(inputs.Layer(name, d, *fmts, "relu", "kaiming", "gauss", 55))
+    qs = check_quantize(ol)
+    before = mq.kernel_launch_count()
+    mq.conv_bwd_data(d, qs[1], qs[2])
+    if rest[0] * rest[0] * min(cout, 64) < 25 * 64:
+        assert mq.kernel_launch_count() - before == (2 if fp4 else 1)
+    check_convs(ol, qs, layouts=(mq.NCHW, mq.HWNC), ops=("dx",))
+    assert mq.last_device_status() == 0
