@@ -263,27 +263,45 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
   // N = 16, 53.2 / 27.8; 32 -> 64 75x75, N = 200, 45.1 / 30.3, 33x33, N = 8, 10.6 / 7.1; E2M1 64 -> 64 80x80, N = 64, 24.0 / 11.7; 100 channels
   // 63x63, N = 200, 52.6 / 31.1; 25 taps of 64 bytes 21.8 / 22.3, the one shape of those measured that it is behind on).
   const int spa_h = fp4 ? 2 : 1, halo_boxes = op == MQ_OP_FWD ? (g.sw < g.Kw ? g.sw : g.Kw) : 1;
-  const int halo_wh = op == MQ_OP_FWD ? 8 + (g.Kw + g.sw - 1) / g.sw - 1 : 8 + g.Kw - 1;
+  // Input gradient: with strides of two the four classes of output pixels together, each in an accumulator of its own (up to 64 channels),
+  // up to nine taps (us, per-tap kernel with its preparation launch / this one: E4M3 16 <- 32 channels 320x320, N = 16, 74.4 / 26.5; 32 <- 64
+  // 52x52, N = 200, 43.0 / 23.7, 33x33, N = 8, 9.6 / 7.7; E2M1 32 <- 64 40x40, N = 100, 16.3 / 13.6; 60 <- 100 63x63, N = 200, 126 / 129; 25 taps 17.3 / 19.2)
+  bool quad = op == MQ_OP_BWD_DATA && layout == MQ_NCHW && !compact && !line && !mx && !ts16 && g.sh == 2 && g.sw == 2 && g.Kh >= 2 && g.Kw >= 2 &&
+              taps <= 9 && p.cpt == 1 && p.KB <= 64 && p.Cd <= 64 && !MQ_ENV("MQ_TC_NO_HALO", 0) && !MQ_ENV("MQ_TC_NO_HALO_S2", 0) && !MQ_ENV("MQ_TC_NO_FUSED", 0) &&
+              !MQ_ENV("MQ_TC_TW", 0) && !MQ_ENV("MQ_TC_BN", 0);
+  // source pixel of tap k relative to the tile's, for the class the tap belongs to; it falls with k
+  auto quad_shift = [](int k, int pad) { return (((k + pad) & 1) + pad - k) / 2; };
+  const int halo_rows = quad ? quad_shift(0, g.ph) - quad_shift(g.Kh - 1, g.ph) + 1 : g.Kh;
+  const int halo_wh = op == MQ_OP_FWD ? 8 + (g.Kw + g.sw - 1) / g.sw - 1 : quad ? 8 + quad_shift(0, g.pw) - quad_shift(g.Kw - 1, g.pw) : 8 + g.Kw - 1;
+  const int patch_bytes = halo_boxes * halo_rows * halo_wh * (p.KB / 32) * spa_h, most_patch_bytes = p.KB / 32 * spa_h == 1 ? 128 : 256;
   // (input gradient: 8-bit weights of a single channel tile are multiplied as they are stored)
   const bool mn_weights = op == MQ_OP_BWD_DATA && !fp4 && !fmt_is_6bit(fmt_w) && !fmt_is_6bit(fmt_x_like) && p.Cd <= 128 && !MQ_ENV("MQ_TC_NO_MN_WEIGHTS", 0);
   auto halo_stages = [&](int bn, bool staged, ConvTcParams* q) {   // stages of the whole-tile kernel (below two: it does not fit)
     const int groups = (taps * p.cpt + p.G - 1) / p.G, atoms_b = (bn + 127) / 128;
     q->WH = halo_wh; q->sw_halo = op == MQ_OP_FWD ? g.sw : 1; q->halo_boxes = halo_boxes;
-    q->halo_box_bytes = g.Kh * halo_wh * 16 * p.KB;
+    q->halo_rows = halo_rows;
+    q->halo_h0 = quad ? quad_shift(g.Kh - 1, g.ph) : g.ph - (g.Kh - 1);
+    q->halo_w0 = quad ? quad_shift(g.Kw - 1, g.pw) : g.pw - (g.Kw - 1);
+    q->halo_box_bytes = halo_rows * halo_wh * 16 * p.KB;
     q->halo_a_bytes = (halo_boxes * q->halo_box_bytes + 1023) / 1024 * 1024;
     q->halo_stage_bytes = (q->halo_a_bytes + groups * 512 * spa_h + 1023) / 1024 * 1024;
     q->halo_b_bytes = (taps * (mn_weights && bn < g.Cp ? g.Cp : bn) * p.KB + groups * 512 * spa_h * atoms_b + 1023) / 1024 * 1024;
     int hst = (227 * 1024 - 4096 - q->halo_b_bytes - (staged ? 65536 : 0)) / q->halo_stage_bytes;
     if (hst > 4) hst = 4;
     // TMEM: accumulator(s), 16 columns per chunk of resident weight scales, 8 per chunk per stage
-    while (hst >= 2 && bn + 16 * groups + 8 * groups * hst > 512) --hst;
+    while (hst >= 2 && (quad ? 4 : 1) * bn + 16 * groups + 8 * groups * hst > 512) --hst;
     return hst;
   };
   if (!line && !mx && !ts16 && op == MQ_OP_FWD && g.sw == 2 && g.sh <= 2 && taps <= 64 && p.cpt == 1 && p.KB <= 64 && p.Cd <= 128 &&
       !(layout == MQ_NCHW && p.Wd % 8 != 0 && big_output && taps == 1) && !MQ_ENV("MQ_TC_NO_HALO", 0) && !MQ_ENV("MQ_TC_NO_HALO_S2", 0) &&
-      halo_boxes * g.Kh * halo_wh * (p.KB / 32) * spa_h <= (p.KB / 32 * spa_h == 1 ? 128 : 256)) {
+      patch_bytes <= most_patch_bytes) {
     ConvTcParams q{};
     thin = halo_stages((p.Cd + 15) / 16 * 16, false, &q) >= 2;
+  }
+  if (quad) {
+    ConvTcParams q{};
+    quad = patch_bytes <= most_patch_bytes && halo_stages((p.Cd + 15) / 16 * 16, false, &q) >= 2;
+    if (quad) { thin = true; p.quad = 1; p.classes = 1; }
   }
   p.line = line ? 1 : 0;
   const int cd16 = mx ? (p.Cd + 31) / 32 * 32 : (p.Cd + 15) / 16 * 16;
@@ -403,10 +421,10 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
   p.n_acc = (2 * p.BN + sf_cols * stages <= 512) ? 2 : 1;
   if (p.n_acc * p.BN + sf_cols * stages > 512) return false;
   p.mma_cp = MQ_ENV("MQ_TC_NO_MMA_CP", 0) ? 0 : 1;   // E2M1 too: the bubble behind a copier warp costs more than the lane's extra issues
-  p.pair = !mx && !p.tma_store && op == MQ_OP_BWD_DATA && g.sw == 2 && layout == MQ_NCHW && p.Wd % 2 == 0 && p.n_acc == 2 && p.total_tiles % 2 == 0 &&
+  p.pair = !mx && !quad && !p.tma_store && op == MQ_OP_BWD_DATA && g.sw == 2 && layout == MQ_NCHW && p.Wd % 2 == 0 && p.n_acc == 2 && p.total_tiles % 2 == 0 &&
            !MQ_ENV("MQ_TC_NO_PAIR", 0);
   const int nkh = op == MQ_OP_FWD ? g.Kh : (g.Kh + g.sh - 1) / g.sh, nkw = op == MQ_OP_FWD ? g.Kw : (g.Kw + g.sw - 1) / g.sw;
-  p.max_stages = (nkh * nkw * p.cpt + p.G - 1) / p.G;
+  p.max_stages = ((quad ? taps : nkh * nkw) * p.cpt + p.G - 1) / p.G;
   // one 256-column accumulator: the epilogue copies it into registers and frees it before storing (with the staged TMA
   // stores only when a tile has at least MQ_TC_SNAP_MIN_STAGES pipeline stages of MMAs to overlap: E2M1 1x1 512 channels, two
   // stages per tile, measured 384-407 us without and 517-601 us with it; E4M3, four stages, 562-567 against 521 us; and only of 256
@@ -434,18 +452,20 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
     if (p.TW == 8 && p.TN == 16) {
       int halo_tma = tma_store_ok && !MQ_ENV("MQ_TC_NO_TMA_STORE", 0) ? 1 : 0;
       int hst = halo_stages(p.BN, halo_tma != 0, &p);
+      if (quad) { halo_tma = 0; hst = halo_stages(p.BN, false, &p); }
       if (hst < 2 && g.sw == 2) { halo_tma = 0; hst = halo_stages(p.BN, false, &p); }   // (the staged stores' 64 KB or the halo: the halo)
       if (hst >= 2 && p.WH <= 256) {
         p.halo = 1;
         p.tma_store = halo_tma;
-        p.fused = p.tiles_c == 1 && p.TN <= 32 && p.halo_boxes * g.Kh * p.WH * (p.KB / 32) * spa_h <= (p.KB / 32 * spa_h == 1 ? 128 : 256) &&
+        p.fused = p.tiles_c == 1 && p.TN <= 32 && patch_bytes <= most_patch_bytes &&
                   !MQ_ENV("MQ_TC_NO_FUSED", 0);
         if (p.fused && mn_weights) p.b_mn = g.Cp % 128 == 0 ? 128 : (g.Cp % 64 == 0 ? 64 : 32);
         p.stages = hst;
-        p.n_acc = (2 * p.BN + 16 * p.max_stages + 8 * p.max_stages * hst <= 512) ? 2 : 1;
+        p.n_acc = ((quad ? 8 : 2) * p.BN + 16 * p.max_stages + 8 * p.max_stages * hst <= 512) ? 2 : 1;
       }
     }
   }
+  if (quad && !(p.halo && p.fused)) return false;   // (the four classes are that kernel's: its conditions were met above)
   // unit strides and one 128-byte chunk per stage: the activation-side scale chunk of (tile, kh) equals that of the tile one
   // output row further with kh - 1, so chunks are stored per source row - Kh times fewer to expand
   p.sfa_dedup = (!p.halo && p.KB == 128 && g.sh == 1 && g.sw == 1 && !MQ_ENV("MQ_TC_NO_SFA_DEDUP", 0)) ? 1 : 0;
@@ -524,7 +544,7 @@ mq_status run_conv_tc(int op, const Geom& g, ConvTcPlan& pl, const mq_qtensor* q
     const uint64_t strides[3] = {(uint64_t)g.N * rb, rb, (uint64_t)p.Ws * g.N * rb};
     const uint32_t wst = op == MQ_OP_FWD ? (uint32_t)g.sw : 1u;
     uint32_t box[4] = {(uint32_t)p.KB, (uint32_t)((p.TW - 1) * wst + 1), (uint32_t)p.TN, 1u};
-    if (p.halo) { box[1] = (uint32_t)((p.WH - 1) * wst + 1); box[3] = (uint32_t)g.Kh; }   // the whole halo of a tile (one class of its columns) in one box
+    if (p.halo) { box[1] = (uint32_t)((p.WH - 1) * wst + 1); box[3] = (uint32_t)p.halo_rows; }   // the whole halo of a tile (one class of its columns) in one box
     const uint32_t es[4] = {1u, wst, 1u, 1u};
     // a packed activation / gradient tensor with rows of whole 128-code boxes is read where it is stored (the copy engine pads
     // each 12-byte group on its way into shared memory): no scratch copy, no pass over the tensor before the GEMM

@@ -869,6 +869,47 @@ __device__ __forceinline__ void epilogue_tma_snap_role(const ConvTcParams& p, co
     if (lane == 0) bulk_wait_group_all();
 }
 
+// Epilogue role of the input gradient with strides of two on the whole-tile kernel (warps 4-11): a tile's four accumulators are the four
+// classes of output pixels over the same 8 source columns x 16 samples.  Warps 4-7 store the even output rows, 8-11 the odd ones, a
+// lane the pixels 2 (w0 + tw) and 2 (w0 + tw) + 1 of its sample: runs of 64 bytes.
+__device__ __forceinline__ void epilogue_quad_role(const ConvTcParams& p, uint32_t tmem, uint64_t* tfull, uint64_t* tempty, volatile int* abort_flag,
+                                                   int warp, int lane, unsigned total) {
+    const int quad = warp & 3, ch = (warp - 4) >> 2;
+    const int tw = lane & 7, tn = 4 * quad + (lane >> 3);
+    const long long cs = (long long)p.Hd * p.Wd;
+    uint32_t tcount = 0;
+    for (unsigned t = blockIdx.x; t < total && !warp_flag(abort_flag); t += gridDim.x, ++tcount) {
+      const Tile tile = decode_tile(p, t);
+      const int acc = acc_index(p, tcount);
+      if (!mbar_wait_warp(&tfull[acc], acc_phase(p, tcount), p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
+      tc_fence_after_sync();
+      const int yo = 2 * tile.h + ch, xo = 2 * (tile.w0 + tw), n = tile.n0 + tn;
+      const bool ok = yo < p.Hd && xo < p.Wd && n < p.N, both = xo + 1 < p.Wd, even = (p.Wd & 1) == 0;
+      const uint32_t taddr = tmem + acc * 4 * p.BN + 2 * ch * p.BN + ((uint32_t)(32 * quad) << 16);
+      float* o = p.out + (((long long)n * p.Cd + tile.c0) * p.Hd + yo) * p.Wd + xo;
+#pragma unroll 1
+      for (int c = 0; c < p.BN; c += 16) {
+        uint32_t v0[16], v1[16];
+        tmem_ld_32x32b_x16(taddr + c, v0);
+        tmem_ld_32x32b_x16(taddr + p.BN + c, v1);
+        tmem_ld_wait();
+        if (ok) {
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            if (tile.c0 + c + j < p.Cd) {
+              if (even) *reinterpret_cast<float2*>(o) = make_float2(__uint_as_float(v0[j]), __uint_as_float(v1[j]));
+              else { o[0] = __uint_as_float(v0[j]); if (both) o[1] = __uint_as_float(v1[j]); }
+            }
+            o += cs;
+          }
+        }
+      }
+      tc_fence_before_sync();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&tempty[acc]);
+    }
+}
+
 // EPI: -1 = fp32 output (the three fp32 epilogue roles, chosen at run time: an instance per role was measured, no
 // change); 0..4 = quantizing epilogue emitting element format EPI
 // registers per thread of the epilogue warpgroups / of the others in the fp32-output kernels (16 warps, 128 per thread at launch)
@@ -1283,6 +1324,9 @@ __device__ __forceinline__ void halo_build_sfb(const ConvTcParams& p, uint8_t* s
 //    one 8-row swizzle group per sample).  With a column stride (forward) the halo is one such box per class of columns that are
 //    sw apart (the copy engine steps over the others): tap kw lies in box kw % sw, kw / sw columns on.
 // Roles and barriers are those of conv_tc_kernel, plus bfull / bempty for the resident weight tile.
+// The input gradient with strides of two (quad) walks the source pixels once for all four classes of output pixels: a tap belongs to one
+// class and adds to that class's accumulator, so the halo of 8 x 16 source pixels yields 16 x 2 x 16
+// outputs, where the per-tap kernel loaded nine boxes for as many (16 <- 32 channels 320x320, N = 16: 74.4 -> 26.5 us).
 // With a single channel tile (p.fused) no preparation kernel runs at all: every block builds the weight image and
 // its scale chunks in shared memory itself at start-up, and warps 3, 12, 13 and 14 expand the tiles' activation scales (the
 // patch of tile scales under the halo: all rows of a tile lie in one 32-sample block) into the scale-vector chunks of the
@@ -1326,7 +1370,8 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   uint32_t* tap_a = tmem_slot + 4;                     // per tap: offset of its A view / B rows, in 16-byte units
   uint32_t* tap_b = tap_a + 64;
   uint32_t* tap_p = tap_b + 64;                        // per tap: first pixel of its view in the tile's scale patch
-  uint8_t* sc_tbl = reinterpret_cast<uint8_t*>(tap_p + 64);   // the patches of raw scale bytes, one per expander warp
+  uint32_t* tap_c = tap_p + 64;                        // per tap: first column of its accumulator; bit 31: not the first tap of that
+  uint8_t* sc_tbl = reinterpret_cast<uint8_t*>(tap_c + 64);   // the patches of raw scale bytes, one per expander warp
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // warp-uniform, see conv_tc_kernel
   const unsigned total = (unsigned)p.total_tiles;
   const unsigned tiles_per_c = (unsigned)(p.classes * p.tiles_w * p.tiles_h);   // tile order: (class, w, h) below the channel tile
@@ -1353,12 +1398,16 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     const int kh = threadIdx.x / p.Kw, kw = threadIdx.x - kh * p.Kw;
     // forward reads halo row kh, column shift kw; the input gradient walks the taps in the same order but its
     // source pixel moves the other way
-    const int hrow = MODE == MQ_OP_FWD ? kh : p.Kh - 1 - kh, wsh = MODE == MQ_OP_FWD ? kw : p.Kw - 1 - kw;
+    // (a stride of two: to the class of output pixels that the tap belongs to, ((class + padding - tap) / 2) source pixels on)
+    const int ch = (kh + p.ph) & 1, cw = (kw + p.pw) & 1;
+    const int hrow = p.quad ? (ch + p.ph - kh) / 2 - p.halo_h0 : (MODE == MQ_OP_FWD ? kh : p.Kh - 1 - kh);
+    const int wsh = p.quad ? (cw + p.pw - kw) / 2 - p.halo_w0 : (MODE == MQ_OP_FWD ? kw : p.Kw - 1 - kw);
     const int par = wsh % p.sw_halo;         // column class of the tap's pixels: a box of its own
-    const int aoff = (((par * p.Kh) + hrow) * p.TN * p.WH + wsh / p.sw_halo) * KB;
+    const int aoff = (((par * p.halo_rows) + hrow) * p.TN * p.WH + wsh / p.sw_halo) * KB;
     tap_a[threadIdx.x] = (uint32_t)aoff >> 4;
     tap_b[threadIdx.x] = (uint32_t)(threadIdx.x * (p.b_mn ? p.b_mn : p.BN) * KB) >> 4;
-    tap_p[threadIdx.x] = (uint32_t)((par * p.Kh + hrow) * p.WH + wsh / p.sw_halo);
+    tap_c[threadIdx.x] = p.quad ? (uint32_t)((2 * ch + cw) * p.BN) | ((kh >= 2 || kw >= 2) ? 1u << 31 : 0u) : (threadIdx.x > 0 ? 1u << 31 : 0u);
+    tap_p[threadIdx.x] = (uint32_t)((par * p.halo_rows + hrow) * p.WH + wsh / p.sw_halo);
   }
   if (warp == 1) { tmem_alloc(tmem_slot, 512); tmem_relinquish(); }
   pdl_wait();
@@ -1371,7 +1420,8 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   tc_fence_after_sync();
   const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
   // TMEM columns: accumulators, the resident weight scale vectors (16 per chunk), then 8 per chunk per stage
-  const uint32_t sfb_base = tmem + p.n_acc * p.BN;
+  const uint32_t acc_cols = (uint32_t)(p.quad ? 4 * p.BN : p.BN);
+  const uint32_t sfb_base = tmem + p.n_acc * acc_cols;
   const uint32_t sfa_base = sfb_base + (uint32_t)nsf * 16;
   const uint32_t sfa_cols_stage = (uint32_t)nsf * 8;
   const bool two_issuers = p.fused && p.mma_cp && p.n_acc == 2;
@@ -1398,8 +1448,8 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         if (!mbar_wait_warp(&empty[s], phase ^ 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
         uint8_t* sa = stage0 + (size_t)s * stage_bytes;
         // first source pixel of the halo: forward (h - ph, w0 - pw); input gradient (h + ph - (Kh-1), w0 + pw - (Kw-1))
-        const int hs = MODE == MQ_OP_FWD ? tile.h * p.sh - p.ph : tile.h + p.ph - (p.Kh - 1);
-        const int ws = MODE == MQ_OP_FWD ? tile.w0 * p.sw - p.pw : tile.w0 + p.pw - (p.Kw - 1);
+        const int hs = MODE == MQ_OP_FWD ? tile.h * p.sh - p.ph : tile.h + p.halo_h0;
+        const int ws = MODE == MQ_OP_FWD ? tile.w0 * p.sw - p.pw : tile.w0 + p.halo_w0;
         if (elect_one()) {
           mbar_arrive_expect_tx(&full[s], (uint32_t)(p.halo_boxes * p.halo_box_bytes + (p.fused ? 0 : sfa_bytes)));
 #pragma unroll 1
@@ -1426,9 +1476,9 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       uint32_t s = first, phase = 0, tcount = first, bcount = 0;
       int cur_ct = -1;
       constexpr int TU = TAPS > 0 ? TAPS : 1;
-      uint32_t ta[TU], tb[TU];
+      uint32_t ta[TU], tb[TU], tc[TU];
 #pragma unroll
-      for (int q = 0; q < TU; ++q) { ta[q] = tap_a[q]; tb[q] = tap_b[q]; }
+      for (int q = 0; q < TU; ++q) { ta[q] = tap_a[q]; tb[q] = tap_b[q]; tc[q] = tap_c[q]; }
       const uint32_t acc_mask = (uint32_t)p.n_acc - 1, acc_shift = (uint32_t)p.n_acc - 1;   // n_acc is 1 or 2
       for (unsigned t = blockIdx.x + first * gridDim.x; t < total && !warp_flag(abort_flag); t += step * gridDim.x, tcount += step) {
         const int ct = p.tiles_c == 1 ? 0 : (int)((t / tiles_per_c) % (unsigned)p.tiles_c);
@@ -1443,7 +1493,7 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         if (!mbar_wait_warp(&tempty[acc], ((tcount >> acc_shift) & 1) ^ 1, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
         if (!mbar_wait_warp(p.mma_cp ? &full[s] : &sffull[s], phase, p.status, MQ_ERR_TIMEOUT)) { *abort_flag = 1; break; }
         tc_fence_after_sync();
-        const uint32_t d_tmem = tmem + acc * p.BN;
+        const uint32_t d_tmem = tmem + acc * acc_cols;
         const uint32_t sa16 = smem_u32(stage0 + (size_t)s * stage_bytes) >> 4;
         const uint32_t sfa_s = sfa_base + s * sfa_cols_stage;
         if (elect_one()) {
@@ -1467,8 +1517,10 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
             for (int g = 0; g < SPA; ++g) tmem_cp_32x128b_warpx4(sfa_s + st * 8 + 4 * g, smem_desc(sf_desc, sfa_sm + (st * SPA + g) * 512));
           }
         }
-        uint32_t accumulate = 0;
-        auto issue_tap = [&](int q, uint32_t a16, uint32_t b16) {
+        auto issue_tap = [&](int q, uint32_t a16, uint32_t b16, uint32_t c) {
+          // (the forward and unit strides: one accumulator, to which all taps but the first add)
+          const uint32_t d = MODE == MQ_OP_BWD_DATA ? d_tmem + (c & 0xffffu) : d_tmem;
+          uint32_t accumulate = MODE == MQ_OP_BWD_DATA ? c >> 31 : (q > 0 ? 1u : 0u);
           const int sfst = q / G;
           const uint32_t sfa_t = sfa_s + sfst * 8, sfb_t = sfb_base + sfst * 16;
 #pragma unroll
@@ -1477,17 +1529,17 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
             const int g = (atom * SPA) >> 2, id = (atom * SPA) & 3;
             const uint64_t ad = a_desc_base | (uint64_t)((a16 + 2 * ja) & 0x3FFF);
             const uint64_t bd = b_desc_base | (uint64_t)((b16 + b_step * ja) & 0x3FFF);
-            if (FP4) mma_mxf4(d_tmem, ad, bd, idesc_id[id], sfa_t + 4 * g, sfb_t + 4 * g * atoms_b, accumulate);
-            else mma_mxf8f6f4(d_tmem, ad, bd, idesc_id[id], sfa_t + 4 * g, sfb_t + 4 * g * atoms_b, accumulate);
+            if (FP4) mma_mxf4(d, ad, bd, idesc_id[id], sfa_t + 4 * g, sfb_t + 4 * g * atoms_b, accumulate);
+            else mma_mxf8f6f4(d, ad, bd, idesc_id[id], sfa_t + 4 * g, sfb_t + 4 * g * atoms_b, accumulate);
             accumulate = 1;
           }
         };
         if (TAPS > 0) {
 #pragma unroll
-          for (int q = 0; q < TU; ++q) issue_tap(q, sa16 + ta[q], sb16 + tb[q]);
+          for (int q = 0; q < TU; ++q) issue_tap(q, sa16 + ta[q], sb16 + tb[q], tc[q]);
         } else {
 #pragma unroll 1
-          for (int q = 0; q < taps; ++q) issue_tap(q, sa16 + tap_a[q], sb16 + tap_b[q]);
+          for (int q = 0; q < taps; ++q) issue_tap(q, sa16 + tap_a[q], sb16 + tap_b[q], tap_c[q]);
         }
         tc_commit(&empty[s]);
         tc_commit(&tfull[acc]);
@@ -1547,13 +1599,13 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       uint8_t* tbl = sc_tbl + 256 * s;
       constexpr int BPC = APC * SPA;                       // scale bytes per tap per row = K-blocks of a tap
       constexpr int NE = HALO_PATCH_BYTES(BPC) / 32;
-      const int npix = p.halo_boxes * p.Kh * p.WH;
+      const int npix = p.halo_boxes * p.halo_rows * p.WH;
       // this lane's patch entries e = lane + 32 i: (column class, halo row, column, K-block), fixed for the whole kernel
       int e_h[NE], e_w[NE], e_k[NE];
 #pragma unroll
       for (int i = 0; i < NE; ++i) {
-        const int e = lane + 32 * i, pe = e / BPC, row = pe / p.WH, par = row / p.Kh;
-        e_k[i] = e - pe * BPC; e_h[i] = row - par * p.Kh; e_w[i] = par + p.sw_halo * (pe - row * p.WH);
+        const int e = lane + 32 * i, pe = e / BPC, row = pe / p.WH, par = row / p.halo_rows;
+        e_k[i] = e - pe * BPC; e_h[i] = row - par * p.halo_rows; e_w[i] = par + p.sw_halo * (pe - row * p.WH);
         if (pe >= npix) e_h[i] = -1;
       }
       int twj[4];
@@ -1562,8 +1614,8 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       uint32_t phase = 0;
       for (unsigned t = blockIdx.x + (unsigned)s * gridDim.x; t < total && !*abort_flag; t += (unsigned)p.stages * gridDim.x, phase ^= 1) {
         const Tile tile = decode_tile(p, t);
-        const int hs = MODE == MQ_OP_FWD ? tile.h * p.sh - p.ph : tile.h + p.ph - (p.Kh - 1);
-        const int ws = MODE == MQ_OP_FWD ? tile.w0 * p.sw - p.pw : tile.w0 + p.pw - (p.Kw - 1);
+        const int hs = MODE == MQ_OP_FWD ? tile.h * p.sh - p.ph : tile.h + p.halo_h0;
+        const int ws = MODE == MQ_OP_FWD ? tile.w0 * p.sw - p.pw : tile.w0 + p.halo_w0;
         const int nblk = tile.n0 >> 5;
         // raw tile scales of the patch (zero outside the image: those codes are zero-filled anyway)
         uint8_t raw[NE];
@@ -1612,7 +1664,8 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       }
     }
   } else if (warp >= 4 && warp < 12) {
-    if (p.tma_store) epilogue_tma_role<MODE>(p, &map_out, staging, tmem, tfull, tempty, abort_flag, warp, lane, total);
+    if (MODE == MQ_OP_BWD_DATA && p.quad) epilogue_quad_role(p, tmem, tfull, tempty, abort_flag, warp, lane, total);
+    else if (p.tma_store) epilogue_tma_role<MODE>(p, &map_out, staging, tmem, tfull, tempty, abort_flag, warp, lane, total);
     else epilogue_role<MODE>(p, tmem, tfull, tempty, abort_flag, warp, lane, total);
   }
   tc_fence_before_sync();
@@ -2122,7 +2175,7 @@ template <int MODE, int KB, bool FP4, int TAPS>
 cudaError_t launch_conv_tc_halo_taps(const ConvTcParams& p, const CUtensorMap& map_a, const CUtensorMap& map_b, const CUtensorMap& map_w, cudaStream_t s) {
   static bool attr_set = false;
   const size_t smem = 1024 + (size_t)p.halo_b_bytes + (size_t)p.stages * p.halo_stage_bytes + (p.tma_store ? EPI_STAGING_BYTES : 0) +
-                      (3 * (size_t)p.stages + 6) * 8 + 16 + 3 * 64 * 4 + 4 * 256;
+                      (3 * (size_t)p.stages + 6) * 8 + 16 + 4 * 64 * 4 + 4 * 256;
   if (!attr_set) {
     cudaError_t e = cudaFuncSetAttribute(conv_tc_halo_kernel<MODE, KB, FP4, TAPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (e != cudaSuccess) return e;

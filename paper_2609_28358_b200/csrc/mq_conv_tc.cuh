@@ -59,8 +59,10 @@ struct ConvTcParams {
   int duo;                  // 1: clusters of two blocks on 256 x 256 tiles (cta_group::2), each loading half of the weight tile
   int snap;                 // 1: 256-column tiles, direct fp32 stores: the epilogue copies the accumulator into registers and frees it before storing
   int a_tx34;               // 1: the activation boxes come from packed 6-bit storage - a box counts 3/4 of its shared-memory bytes on the barrier
+  int quad;                 // 1: input gradient with strides of two, the four classes of output pixels of a tile together (classes is then 1)
+  int halo_rows, halo_h0, halo_w0;   // rows of a halo box; its first row and column relative to the tile's source pixel (input gradient)
   int b_mn;                 // resident weights MN-major: bytes of a row of K (32, 64 or 128; p.b_rowbytes in panels of as many), or 0: K-major
-  int halo_box_bytes;       // bytes of one activation box = Kh * TN * WH * KB (a multiple of 512)
+  int halo_box_bytes;       // bytes of one activation box = halo_rows * TN * WH * KB (a multiple of 512)
   int halo_a_bytes;         // bytes of a tile's activation boxes (rounded up to 1024)
   int halo_stage_bytes;     // bytes of one pipeline stage (activation boxes + A-side scale chunks)
   int halo_b_bytes;         // bytes of the resident weight image + its scale chunks (rounded up to 1024)

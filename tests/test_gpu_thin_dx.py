@@ -1,5 +1,6 @@
 """Input gradient of thin layers on the whole-tile kernel (needs a B200).  Unit strides: 8-bit weights multiplied as they are stored
-(MN-major), in rows of 32, 64 and 128 bytes and three panels of 32, ragged channels both ways, 1 to 25 taps.  Against the CPU
+(MN-major), in rows of 32, 64 and 128 bytes and three panels of 32, ragged channels both ways, 1 to 25 taps.  Strides of two: the four
+classes of output pixels of a tile together, even and odd images, kernels of 4 to 25 taps, one and two accumulator sets.  Against the CPU
 oracle within the bound of the other GEMM tests; the launches counted say that the route is the one meant."""
 import pytest
 
@@ -18,6 +19,14 @@ CASES = [
     ("n80_pointwise", (33, 80, 6, 7, 64, 1, 1, 0)),
     ("n40_k5", (3, 40, 9, 9, 32, 5, 1, 2)),
     ("many_tiles", (40, 32, 21, 40, 64, 3, 1, 1)),
+    ("s2", (5, 16, 9, 12, 32, 3, 2, 1)),
+    ("s2_odd", (18, 33, 10, 15, 20, 3, 2, 1)),
+    ("s2_n64", (17, 64, 12, 18, 64, 3, 2, 1)),              # one set of accumulators
+    ("s2_many_tiles", (33, 16, 41, 70, 32, 3, 2, 1)),
+    ("s2_k2", (6, 20, 8, 34, 32, 2, 2, 0)),
+    ("s2_k4", (6, 20, 9, 17, 32, 4, 2, 1)),
+    ("s2_k5", (4, 32, 11, 13, 32, 5, 2, 2)),
+    ("s2_no_padding", (4, 32, 12, 12, 40, 3, 2, 0)),        # the last row and column reach no output: zeros
 ]
 
 
