@@ -1424,7 +1424,7 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   const uint32_t sfb_base = tmem + p.n_acc * acc_cols;
   const uint32_t sfa_base = sfb_base + (uint32_t)nsf * 16;
   const uint32_t sfa_cols_stage = (uint32_t)nsf * 8;
-  const bool two_issuers = p.fused && p.mma_cp && p.n_acc == 2;
+  const bool two_issuers = p.fused && p.mma_cp && p.n_acc == 2 && !p.paced;
 
   if (warp == 0) {
     // ------------------------------------------------------------------ producer
@@ -1594,9 +1594,9 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     }
   } else if (warp == 3 || warp >= 12) {
     // ------------------------------------------------------------------ activation-scale expanders (fused mode): a warp per stage
-    const int s = warp == 3 ? 0 : warp - 11;
-    if (p.fused && s < p.stages) {
-      uint8_t* tbl = sc_tbl + 256 * s;
+    const int first = warp == 3 ? 0 : warp - 11, expanders = p.paced ? 1 : p.stages;
+    if (p.fused && first < expanders) {
+      uint8_t* tbl = sc_tbl + 256 * first;
       constexpr int BPC = APC * SPA;                       // scale bytes per tap per row = K-blocks of a tap
       constexpr int NE = HALO_PATCH_BYTES(BPC) / 32;
       const int npix = p.halo_boxes * p.halo_rows * p.WH;
@@ -1611,8 +1611,8 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       int twj[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) twj[j] = (32 * j + lane) & (p.TW - 1);
-      uint32_t phase = 0;
-      for (unsigned t = blockIdx.x + (unsigned)s * gridDim.x; t < total && !*abort_flag; t += (unsigned)p.stages * gridDim.x, phase ^= 1) {
+      uint32_t s = (uint32_t)first, phase = 0;
+      for (unsigned t = blockIdx.x + (unsigned)first * gridDim.x; t < total && !*abort_flag; t += (unsigned)expanders * gridDim.x) {
         const Tile tile = decode_tile(p, t);
         const int hs = MODE == MQ_OP_FWD ? tile.h * p.sh - p.ph : tile.h + p.halo_h0;
         const int ws = MODE == MQ_OP_FWD ? tile.w0 * p.sw - p.pw : tile.w0 + p.halo_w0;
@@ -1661,6 +1661,8 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) mbar_arrive(&full[s]);
+        s += (uint32_t)expanders;
+        if (s >= (uint32_t)p.stages) { s -= (uint32_t)p.stages; phase ^= 1; }
       }
     }
   } else if (warp >= 4 && warp < 12) {

@@ -61,6 +61,7 @@ struct ConvTcParams {
   int a_tx34;               // 1: the activation boxes come from packed 6-bit storage - a box counts 3/4 of its shared-memory bytes on the barrier
   int quad;                 // 1: input gradient with strides of two, the four classes of output pixels of a tile together (classes is then 1)
   int halo_rows, halo_h0, halo_w0;   // rows of a halo box; its first row and column relative to the tile's source pixel (input gradient)
+  int paced;                // 1: one warp expands scales and one issues MMAs (fused whole-tile kernel; see the plan)
   int b_mn;                 // resident weights MN-major: bytes of a row of K (32, 64 or 128; p.b_rowbytes in panels of as many), or 0: K-major
   int halo_box_bytes;       // bytes of one activation box = halo_rows * TN * WH * KB (a multiple of 512)
   int halo_a_bytes;         // bytes of a tile's activation boxes (rounded up to 1024)
