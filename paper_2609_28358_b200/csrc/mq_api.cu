@@ -461,9 +461,9 @@ bool conv_tc_plan(int op, const Geom& g, int fmt_x_like, int fmt_w, int layout, 
                   !MQ_ENV("MQ_TC_NO_FUSED", 0);
         // Rows cut inside a sector, beyond what L2 holds: the two parts of a sector come from neighbouring blocks, and where the stores are the
         // bound the blocks drift apart and parts are written out, read back and written again.  One warp for each role keeps the blocks in step
-        // above 32 channels (us, one / several: 32 -> 64 channels 74x74, N = 193, 155 / 216; 64 -> 64 50x50, N = 256, 82 / 95, 53x53, N = 200,
-        // 72 / 91, 75x75, N = 200, 169 / 253; E2M1 96 -> 64 75x75 192 / 250; 32 -> 48 121 / 165, but 32 -> 32 107 / 89; outputs that fit,
-        // 32 -> 64 74x74, N = 50, 41 / 31).  Taking the tiles of a row one after the other in a block does not (95 -> 143).
+        // above 32 channels (us, one / several: 32 -> 64 channels 74x74, N = 193, 162 / 223; 64 -> 64 50x50, N = 256, 87 / 102, 53x53, N = 200,
+        // 77 / 94, 75x75, N = 200, 157 / 260; E2M1 96 -> 64 75x75 189 / 264; 32 -> 48 124 / 156, but 32 -> 32 111 / 71; outputs that fit,
+        // 32 -> 64 74x74, N = 50, 42 / 33).  Taking the tiles of a row one after the other in a block does not (102 -> 145).
         p.paced = layout == MQ_NCHW && p.Wd % 8 != 0 && big_output && p.Cd > 32 ? 1 : 0;
         if (p.fused && mn_weights) p.b_mn = g.Cp % 128 == 0 ? 128 : (g.Cp % 64 == 0 ? 64 : 32);
         p.stages = hst;

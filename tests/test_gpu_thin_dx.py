@@ -1,6 +1,6 @@
 """Input gradient of thin layers on the whole-tile kernel (needs a B200).  Unit strides: 8-bit weights multiplied as they are stored
 (MN-major), in rows of 32, 64 and 128 bytes and three panels of 32, ragged channels both ways, 1 to 25 taps.  Strides of two: the four
-classes of output pixels of a tile together, even and odd images, kernels of 4 to 25 taps, one and two accumulator sets.  Against the CPU
+classes of output pixels of a tile together, even and odd images, kernels of 4 and 9 taps (16 and 25: the per-tap kernel), one and two accumulator sets.  Against the CPU
 oracle within the bound of the other GEMM tests; the launches counted say that the route is the one meant."""
 import pytest
 
@@ -40,7 +40,7 @@ def test_input_gradient(name, shape, fmts):
     qs = check_quantize(ol)
     before = mq.kernel_launch_count()
     mq.conv_bwd_data(d, qs[1], qs[2])
-    if rest[0] * rest[0] * min(cout, 64) < 25 * 64:
+    if rest[1] == 1 or rest[0] <= 3:      # (more taps with strides of two: the per-tap kernel)
         assert mq.kernel_launch_count() - before == (2 if fp4 else 1)
     check_convs(ol, qs, layouts=(mq.NCHW, mq.HWNC), ops=("dx",))
     assert mq.last_device_status() == 0
