@@ -1402,12 +1402,12 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     const int ch = (kh + p.ph) & 1, cw = (kw + p.pw) & 1;
     const int hrow = p.quad ? (ch + p.ph - kh) / 2 - p.halo_h0 : (MODE == MQ_OP_FWD ? kh : p.Kh - 1 - kh);
     const int wsh = p.quad ? (cw + p.pw - kw) / 2 - p.halo_w0 : (MODE == MQ_OP_FWD ? kw : p.Kw - 1 - kw);
-    const int par = wsh % p.sw_halo;         // column class of the tap's pixels: a box of its own
-    const int aoff = (((par * p.halo_rows) + hrow) * p.TN * p.WH + wsh / p.sw_halo) * KB;
+    const int par = wsh & (p.sw_halo - 1);   // (strides of one or two)         // column class of the tap's pixels: a box of its own
+    const int aoff = (((par * p.halo_rows) + hrow) * p.TN * p.WH + (wsh >> (p.sw_halo - 1))) * KB;
     tap_a[threadIdx.x] = (uint32_t)aoff >> 4;
     tap_b[threadIdx.x] = (uint32_t)(threadIdx.x * (p.b_mn ? p.b_mn : p.BN) * KB) >> 4;
     tap_c[threadIdx.x] = p.quad ? (uint32_t)((2 * ch + cw) * p.BN) | ((kh >= 2 || kw >= 2) ? 1u << 31 : 0u) : (threadIdx.x > 0 ? 1u << 31 : 0u);
-    tap_p[threadIdx.x] = (uint32_t)((par * p.halo_rows + hrow) * p.WH + wsh / p.sw_halo);
+    tap_p[threadIdx.x] = (uint32_t)((par * p.halo_rows + hrow) * p.WH + (wsh >> (p.sw_halo - 1)));
   }
   if (warp == 1) { tmem_alloc(tmem_slot, 512); tmem_relinquish(); }
   pdl_wait();
@@ -1600,13 +1600,18 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       constexpr int BPC = APC * SPA;                       // scale bytes per tap per row = K-blocks of a tap
       constexpr int NE = HALO_PATCH_BYTES(BPC) / 32;
       const int npix = p.halo_boxes * p.halo_rows * p.WH;
-      // this lane's patch entries e = lane + 32 i: (column class, halo row, column, K-block), fixed for the whole kernel
-      int e_h[NE], e_w[NE], e_k[NE];
+      // this lane's patch entries e = lane + 32 i: (column class, halo row, column, K-block), fixed for the whole kernel; walked by
+      // counters (two divisions an entry were a microsecond of a small layer's call)
+      const int ek = lane & (BPC - 1);
+      int e_h[NE], e_w[NE];
+      {
+        int pe = lane / BPC, col = pe, row = 0, par = 0;
 #pragma unroll
-      for (int i = 0; i < NE; ++i) {
-        const int e = lane + 32 * i, pe = e / BPC, row = pe / p.WH, par = row / p.halo_rows;
-        e_k[i] = e - pe * BPC; e_h[i] = row - par * p.halo_rows; e_w[i] = par + p.sw_halo * (pe - row * p.WH);
-        if (pe >= npix) e_h[i] = -1;
+        for (int i = 0; i < NE; ++i) {
+          while (col >= p.WH) { col -= p.WH; if (++row == p.halo_rows) { row = 0; ++par; } }
+          e_h[i] = pe < npix ? row : -1; e_w[i] = par + p.sw_halo * col;
+          pe += 32 / BPC; col += 32 / BPC;
+        }
       }
       int twj[4];
 #pragma unroll
@@ -1623,8 +1628,8 @@ conv_tc_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         for (int i = 0; i < NE; ++i) {
           const int hh = hs + e_h[i], ww = ws + e_w[i];
           raw[i] = 0;
-          if (e_h[i] >= 0 && e_k[i] < p.Kblocks && hh >= 0 && hh < p.Hs && ww >= 0 && ww < p.Ws)
-            raw[i] = __ldg(p.a_scales + (((long long)hh * p.Ws + ww) * p.Nt + nblk) * p.Kblocks + e_k[i]);
+          if (e_h[i] >= 0 && ek < p.Kblocks && hh >= 0 && hh < p.Hs && ww >= 0 && ww < p.Ws)
+            raw[i] = __ldg(p.a_scales + (((long long)hh * p.Ws + ww) * p.Nt + nblk) * p.Kblocks + ek);
         }
         bool ok = true;
         if (lane == 0) ok = mbar_wait(&empty[s], phase ^ 1, p.status, MQ_ERR_TIMEOUT);
